@@ -42,6 +42,9 @@ struct FftRes {
     Plan plN{}, plH{};
     PlainPlans pp;
     void *tw = nullptr;       // Cx<T>[n], exp(-2 pi i t / n)
+    int4 *ftab = nullptr;     // FP64: stage twiddles of every plan of length n,
+    const int4 *fix[17] = {}; // and where those of E elements per thread start
+    FixPlan fixed(const Plan &pl) const { return FixPlan{pl, fix[pl.E]}; }
     void *scratch = nullptr;  // one half-layout field (c2r)
 };
 
@@ -143,6 +146,19 @@ template <typename P> cudaError_t dalloc(P **p, size_t bytes) {
     return dev_malloc((void **)p, bytes);
 }
 
+// Untuned shapes of the FP64 passes (the standalone transforms'): the plans
+// the tuner finds for most lengths.
+PlainPlans fix_defaults(int n) {
+    PlainPlans q;
+    for (int E : {8, 12, 16, 9, 6, 4})
+        if (make_plan_e(n, E, &q.inv)) break;
+    q.fwd = q.zc = q.zr = q.inv;
+    int ct = 8;
+    while (ct > 1 && fix_threads(n, q.inv.E, ct) > 256) ct /= 2;
+    q.ct_inv = q.ct_fwd = ct;
+    return q;
+}
+
 // Per-n transform resources (plans, twiddles, c2r scratch), created once.
 ns_status get_fft(ns_ctx *c, int n, FftRes **out) {
     auto it = c->fft.find(n);
@@ -155,11 +171,21 @@ ns_status get_fft(ns_ctx *c, int n, FftRes **out) {
     if (!make_plan(n, &f.plN) || !make_plan(n / 2, &f.plH)) return NS_ERR_UNSUPPORTED_N;
     f.pp.inv = f.pp.fwd = f.plN;
     f.pp.zc = f.pp.zr = f.plH;
-    f.pp.ct_inv = f.pp.ct_fwd = default_ct(c->prec == NS_FP64 ? 16 : 8, n);
+    f.pp.ct_inv = f.pp.ct_fwd = default_ct(n);
     cudaError_t e;
-    if (c->prec == NS_FP64) f.tw = make_twiddles<double>(n, &e);
-    else f.tw = make_twiddles<float>(n, &e);
-    if (!f.tw) return fail_cuda(c, e);
+    if (c->prec == NS_FP64) {
+        f.tw = make_twiddles<double>(n, &e);
+        if (!f.tw) return fail_cuda(c, e);
+        if ((e = make_fix_tables(n, &f.ftab, f.fix)) != cudaSuccess) {
+            dev_free(f.tw);
+            if (f.ftab) dev_free(f.ftab);
+            return fail_cuda(c, e);
+        }
+        f.pp = fix_defaults(n);
+    } else {
+        f.tw = make_twiddles<float>(n, &e);
+        if (!f.tw) return fail_cuda(c, e);
+    }
     c->fft[n] = f;
     *out = &c->fft[n];
     return NS_OK;
@@ -230,6 +256,39 @@ static void prune_sels(const Grid &g, const PlainPrune &p, StridedSel *sx, Strid
     sy->gap_hi = std::max(g.ny - p.ky, sy->gap_lo);
 }
 
+// One pass along an axis with transform resources f: FP64 in block fixed
+// point (fft_fix.cuh), FP32 in floating point.
+template <typename T>
+cudaError_t pass_strided(const FftRes &f, const typename Cx<T>::type *in, typename Cx<T>::type *out, long ncols,
+                         long es, long ps, int planes, int dir, const Plan &pl, int ct, cudaStream_t s,
+                         const StridedSel *sel = nullptr) {
+    if constexpr (std::is_same<T, double>::value)
+        return fix_strided(in, out, ncols, es, ps, ps, planes, dir, f.fixed(pl), ct, s, sel);
+    else
+        return fft_strided<T>(in, out, ncols, es, ps, ps, planes, dir, pl, (const typename Cx<T>::type *)f.tw, f.n,
+                              ct, s, sel);
+}
+template <typename T>
+cudaError_t pass_z_c2r(const FftRes &f, const typename Cx<T>::type *in, T *out, long nlines, const Plan &pl,
+                       cudaStream_t s, int kzk = -1) {
+    if constexpr (std::is_same<T, double>::value)
+        if (pl.n == f.n) return fix_z_c2r(in, out, f.n, nlines, f.fixed(pl), s, kzk);
+    return fft_z_c2r<T>(in, out, f.n, nlines, pl, (const typename Cx<T>::type *)f.tw, s, kzk);
+}
+template <typename T>
+cudaError_t pass_z_r2c(const FftRes &f, const T *in, typename Cx<T>::type *out, long nlines, const Plan &pl,
+                       cudaStream_t s, int kzk = -1) {
+    if constexpr (std::is_same<T, double>::value)
+        if (pl.n == f.n) return fix_z_r2c(in, out, f.n, nlines, f.fixed(pl), s, kzk);
+    return fft_z_r2c<T>(in, out, f.n, nlines, pl, (const typename Cx<T>::type *)f.tw, s, kzk);
+}
+// Columns per CTA that the kernels of the precision take for a plan.
+template <typename T> bool ct_fits(const Plan &pl, int ct) {
+    const int t = pl.n / pl.E * ct;
+    if (std::is_same<T, double>::value) return fix_threads(pl.n, pl.E, ct) <= 512;
+    return t <= 512 && t >= 32;
+}
+
 // c2r of ncomp half fields [ncomp][N_x][N_y][N_z/2+1]: x pass (in -> tmp), y
 // pass (tmp in place), z pass (tmp -> out [ncomp][N_x][N_y][N_z]).  FP32 on
 // compiled lengths: the standalone kernels, one field at a time through tmp.
@@ -256,16 +315,15 @@ cudaError_t c2r_batch(const typename Cx<T>::type *in, typename Cx<T>::type *tmp,
     StridedSel sx, sy;
     if (pruned) prune_sels(g, *pr, &sx, &sy);
     cudaError_t e = NSK_TIMED(tr, "fft_x_inverse",
-                              fft_strided<T>(in, tmp, plane, plane, M, M, ncomp, +1, qx.inv, (const C *)f.x->tw,
-                                             g.nx, qx.ct_inv, s, pruned ? &sx : nullptr));
+                              pass_strided<T>(*f.x, in, tmp, plane, plane, M, ncomp, +1, qx.inv, qx.ct_inv, s,
+                                              pruned ? &sx : nullptr));
     if (e != cudaSuccess) return e;
     e = NSK_TIMED(tr, "fft_y_inverse",
-                  fft_strided<T>(tmp, tmp, nh, nh, plane, plane, ncomp * g.nx, +1, qy.inv, (const C *)f.y->tw,
-                                 g.ny, qy.ct_inv, s, pruned ? &sy : nullptr));
+                  pass_strided<T>(*f.y, tmp, tmp, nh, nh, plane, ncomp * g.nx, +1, qy.inv, qy.ct_inv, s,
+                                  pruned ? &sy : nullptr));
     if (e != cudaSuccess) return e;
     return NSK_TIMED(tr, "fft_z_c2r",
-                     fft_z_c2r<T>(tmp, out, g.nz, (long)ncomp * g.nx * g.ny, qz.zc, (const C *)f.z->tw, s,
-                                  pruned ? pr->kz + 1 : -1));
+                     pass_z_c2r<T>(*f.z, tmp, out, (long)ncomp * g.nx * g.ny, qz.zc, s, pruned ? pr->kz + 1 : -1));
 }
 
 // r2c of ncomp real fields: z pass (in -> out), y and x passes in place.
@@ -288,16 +346,16 @@ cudaError_t r2c_batch(const T *in, typename Cx<T>::type *out, const Grid &g, int
     StridedSel sx, sy;
     if (pruned) prune_sels(g, *pr, &sx, &sy);
     cudaError_t e = NSK_TIMED(tr, "fft_z_r2c",
-                              fft_z_r2c<T>(in, out, g.nz, (long)ncomp * g.nx * g.ny, qz.zr, (const C *)f.z->tw, s,
-                                           pruned ? pr->kz + 1 : -1));
+                              pass_z_r2c<T>(*f.z, in, out, (long)ncomp * g.nx * g.ny, qz.zr, s,
+                                            pruned ? pr->kz + 1 : -1));
     if (e != cudaSuccess) return e;
     e = NSK_TIMED(tr, "fft_y_forward",
-                  fft_strided<T>(out, out, nh, nh, plane, plane, ncomp * g.nx, -1, qy.fwd, (const C *)f.y->tw,
-                                 g.ny, qy.ct_fwd, s, pruned ? &sy : nullptr));
+                  pass_strided<T>(*f.y, out, out, nh, nh, plane, ncomp * g.nx, -1, qy.fwd, qy.ct_fwd, s,
+                                  pruned ? &sy : nullptr));
     if (e != cudaSuccess) return e;
     return NSK_TIMED(tr, "fft_x_forward",
-                     fft_strided<T>(out, out, plane, plane, M, M, ncomp, -1, qx.fwd, (const C *)f.x->tw, g.nx,
-                                    qx.ct_fwd, s, pruned ? &sx : nullptr));
+                     pass_strided<T>(*f.x, out, out, plane, plane, M, ncomp, -1, qx.fwd, qx.ct_fwd, s,
+                                     pruned ? &sx : nullptr));
 }
 
 // The transforms of a run: the resources of its axis lengths with their plans
@@ -493,6 +551,14 @@ static int plain_z_mode() {
     return v && (v[0] == '1' || v[0] == '2') ? v[0] - '0' : 0;
 }
 
+// Is a z pass of the plain form a candidate?  The FP64 one-line form exists in
+// floating point only, which the fixed-point two-line form beats at every
+// length, so it runs on request alone.
+template <typename T> static bool z_candidate(int zmode, bool paired) {
+    if (zmode) return paired == (zmode == 2);
+    return paired || std::is_same<T, float>::value;
+}
+
 template <typename T> ns_status tune_plain(ns_ctx *c, Run &r, FftRes *f) {
     typedef typename Cx<T>::type C;
     static std::mutex mu;
@@ -515,39 +581,36 @@ template <typename T> ns_status tune_plain(ns_ctx *c, Run &r, FftRes *f) {
     if (f->pp.tuned && !zmode) return NS_OK;
     const int n = r.n;
     const long nh = n / 2 + 1, plane = (long)n * nh, M = (long)n * plane, lines = 3L * n * n;
-    const C *tw = (const C *)f->tw;
     cudaStream_t s = c->stream;
     C *in = (C *)r.un, *tmp = (C *)r.work, *half = (C *)r.wn;
     T *phys = (T *)r.phys;
-    const int bound = sizeof(T) == 8 ? 384 : 512;
     PlainPlans best = f->pp;
     float bi = -1.f, bf = -1.f, bc = -1.f, br = -1.f;
     const int Es[] = {16, 12, 9, 8, 6, 4};
     for (int E : Es) {
         Plan pl;
         if (make_plan_e(n, E, &pl) && pl.nst <= 4) {
-            const int Tn = n / E;
             for (int ct = 2; ct <= 32; ct *= 2) {
-                if (ct * Tn > bound || ct * Tn < 32) continue;
+                if (!ct_fits<T>(pl, ct)) continue;
                 const float ti = plain_time([&]() {
-                    return fft_strided<T>(in, tmp, plane, plane, M, M, 3, +1, pl, tw, n, ct, s);
+                    return pass_strided<T>(*f, in, tmp, plane, plane, M, 3, +1, pl, ct, s);
                 }, s);
                 if (ti > 0.f && (bi < 0.f || ti < bi)) { bi = ti; best.inv = pl; best.ct_inv = ct; }
                 const float tf = plain_time([&]() {
-                    return fft_strided<T>(half, half, plane, plane, M, M, 3, -1, pl, tw, n, ct, s);
+                    return pass_strided<T>(*f, half, half, plane, plane, M, 3, -1, pl, ct, s);
                 }, s);
                 if (tf > 0.f && (bf < 0.f || tf < bf)) { bf = tf; best.fwd = pl; best.ct_fwd = ct; }
             }
         }
-        // z passes: one line per transform of length n/2 (even/odd packing), or
-        // two lines per transform of length n
+        // z passes: one line per transform of length n/2 (even/odd packing; FP32,
+        // or on request), or two lines per transform of length n
         for (int len : {n / 2, n}) {
             Plan ph;
-            if ((zmode == 1 && len == n) || (zmode == 2 && len != n)) continue;
+            if (!z_candidate<T>(zmode, len == n)) continue;
             if (!make_plan_e(len, E, &ph) || ph.nst > 4) continue;
-            const float tc = plain_time([&]() { return fft_z_c2r<T>(tmp, phys, n, lines, ph, tw, s); }, s);
+            const float tc = plain_time([&]() { return pass_z_c2r<T>(*f, tmp, phys, lines, ph, s); }, s);
             if (tc > 0.f && (bc < 0.f || tc < bc)) { bc = tc; best.zc = ph; }
-            const float tr = plain_time([&]() { return fft_z_r2c<T>(phys, half, n, lines, ph, tw, s); }, s);
+            const float tr = plain_time([&]() { return pass_z_r2c<T>(*f, phys, half, lines, ph, s); }, s);
             if (tr > 0.f && (br < 0.f || tr < br)) { br = tr; best.zr = ph; }
         }
     }
@@ -585,24 +648,21 @@ template <typename T> ns_status tune_plain_grid(ns_ctx *c, Run &r, FftRes *f[3])
     cudaStream_t s = c->stream;
     C *in = (C *)r.un, *tmp = (C *)r.work, *half = (C *)r.wn;
     T *phys = (T *)r.phys;
-    const int bound = sizeof(T) == 8 ? 384 : 512;
     const int Es[] = {16, 12, 9, 8, 6, 4};
     for (int a = 0; a < 3; a++) r.gp[a] = f[a]->pp;
     for (int a = 0; a < 2; a++) {   // x pass, y pass
         const int n = a == 0 ? g.nx : g.ny;
-        const C *tw = (const C *)f[a]->tw;
         auto pass = [&](const C *src, C *dst, int dir, const Plan &pl, int ct) {
-            return a == 0 ? fft_strided<T>(src, dst, plane, plane, M, M, 3, dir, pl, tw, n, ct, s)
-                          : fft_strided<T>(src, dst, nh, nh, plane, plane, 3 * g.nx, dir, pl, tw, n, ct, s);
+            return a == 0 ? pass_strided<T>(*f[a], src, dst, plane, plane, M, 3, dir, pl, ct, s)
+                          : pass_strided<T>(*f[a], src, dst, nh, nh, plane, 3 * g.nx, dir, pl, ct, s);
         };
         PlainPlans &best = r.gp[a];
         float bi = -1.f, bf = -1.f;
         for (int E : Es) {
             Plan pl;
             if (!make_plan_e(n, E, &pl) || pl.nst > 4) continue;
-            const int Tn = n / E;
             for (int ct = 2; ct <= 32; ct *= 2) {
-                if (ct * Tn > bound || ct * Tn < 32) continue;
+                if (!ct_fits<T>(pl, ct)) continue;
                 const float ti = plain_time([&]() { return pass(a == 0 ? in : tmp, tmp, +1, pl, ct); }, s);
                 if (ti > 0.f && (bi < 0.f || ti < bi)) { bi = ti; best.inv = pl; best.ct_inv = ct; }
                 const float tf = plain_time([&]() { return pass(half, half, -1, pl, ct); }, s);
@@ -611,17 +671,16 @@ template <typename T> ns_status tune_plain_grid(ns_ctx *c, Run &r, FftRes *f[3])
         }
     }
     {   // z passes
-        const C *tw = (const C *)f[2]->tw;
         PlainPlans &best = r.gp[2];
         float bc = -1.f, br = -1.f;
         for (int E : Es)
             for (int len : {g.nz / 2, g.nz}) {
                 Plan ph;
-                if ((zmode == 1 && len == g.nz) || (zmode == 2 && len != g.nz)) continue;
+                if (!z_candidate<T>(zmode, len == g.nz)) continue;
                 if (!make_plan_e(len, E, &ph) || ph.nst > 4) continue;
-                const float tc = plain_time([&]() { return fft_z_c2r<T>(tmp, phys, g.nz, lines, ph, tw, s); }, s);
+                const float tc = plain_time([&]() { return pass_z_c2r<T>(*f[2], tmp, phys, lines, ph, s); }, s);
                 if (tc > 0.f && (bc < 0.f || tc < bc)) { bc = tc; best.zc = ph; }
-                const float tr = plain_time([&]() { return fft_z_r2c<T>(phys, half, g.nz, lines, ph, tw, s); }, s);
+                const float tr = plain_time([&]() { return pass_z_r2c<T>(*f[2], phys, half, lines, ph, s); }, s);
                 if (tr > 0.f && (br < 0.f || tr < br)) { br = tr; best.zr = ph; }
             }
     }
@@ -1113,6 +1172,7 @@ void ns_destroy(ns_ctx *c) {
     for (FusedRun &g : c->groups) fused_free(g);
     for (auto &kv : c->fft) {
         if (kv.second.tw) dev_free(kv.second.tw);
+        if (kv.second.ftab) dev_free(kv.second.ftab);
         if (kv.second.scratch) dev_free(kv.second.scratch);
     }
     if (c->flags) dev_free(c->flags);

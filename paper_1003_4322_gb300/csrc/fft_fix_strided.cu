@@ -1,0 +1,99 @@
+// fft_fix_strided.cu -- the x and y passes of the FP64 transforms (1D FFTs
+// along a strided axis, Sec. 2) in block fixed point (fft_fix.cuh).
+//
+// One CTA: 2^cl contiguous columns of one plane, T = n/E threads per column,
+// lanes along columns (rows of 2^cl 16-byte values); the exchange tile
+// holds element (e, c) at (e + (e >> SK)) 2^cl + c, one row of padding every E
+// elements, so that the stride-E stores of stage 0 spread over the banks.
+#include "fft_fix_line.cuh"
+
+namespace nsk {
+
+template <int E> struct SkewE { enum { shift = E == 4 ? 2 : E == 16 ? 4 : 3 }; };
+
+template <int E, int DIR>
+__global__ void __launch_bounds__(512)
+k_fix_strided(const longlong2 *in, longlong2 *out, SelK sel, long es, long ps_in, long ps_out, FixK pl, int cl) {
+    extern __shared__ __align__(16) unsigned char smraw[];
+    __shared__ unsigned red[512];
+    L2 *sm = reinterpret_cast<L2 *>(smraw);
+    const int T = pl.n / E, ct = 1 << cl;
+    const int c = threadIdx.x & (ct - 1), slot = threadIdx.x >> cl;
+    const bool active = slot < T;   // the CTA is rounded up to whole warps
+    const int ro = blockIdx.x / sel.tpr;
+    const long inner = (long)(blockIdx.x - ro * sel.tpr) * ct + c;
+    const long col = (long)(ro < sel.o1 ? ro : ro - sel.o1 + sel.o2) * sel.inner + inner;
+    const bool valid = active && inner < sel.keep;
+    const longlong2 *src = in + (long)blockIdx.y * ps_in + col;
+    longlong2 *dst = out + (long)blockIdx.y * ps_out + col;
+    auto in_gap = [&](int e) { return e >= sel.gap_lo && e < sel.gap_hi; };
+    L2 v[E];
+#pragma unroll
+    for (int q = 0; q < E; q++) {
+        const int e = slot + q * T;
+        v[q] = mkl(0, 0);
+        if (valid && (DIR < 0 || !in_gap(e))) {
+            const longlong2 t = src[e * es];
+            v[q] = mkl(t.x, t.y);
+        }
+    }
+    LineGeo g{kCols, cl, 0, c};
+    const LineScale sc = line_scale<E, false>(v, g, red);
+#pragma unroll
+    for (int q = 0; q < E; q++) v[q] = fix_from_raw(v[q], sc.top);
+    const int ebase = sc.top + 1 + (pl.nst > 1 ? 2 : 0);
+    auto at = [&](int e) { return ((e + (e >> SkewE<E>::shift)) << cl) + c; };
+    auto sl = [&](int e) { return sm[at(e)]; };
+    auto ss = [&](int e, L2 x) { sm[at(e)] = x; };
+    auto gs = [&](int e, L2 x) {
+        if (valid && (DIR > 0 || !in_gap(e)))
+            reinterpret_cast<double2 *>(dst)[e * es] =
+                make_double2(fix_double(x.x, ebase, sc.mul), fix_double(x.y, ebase, sc.mul));
+    };
+    fix_line<E, DIR, false>(v, active, slot, T, pl, false, sl, ss, gs);
+}
+
+template <int DIR> static const void *kernel_of(int E) {
+    switch (E) {
+    case 4: return (const void *)k_fix_strided<4, DIR>;
+    case 6: return (const void *)k_fix_strided<6, DIR>;
+    case 8: return (const void *)k_fix_strided<8, DIR>;
+    case 9: return (const void *)k_fix_strided<9, DIR>;
+    case 12: return (const void *)k_fix_strided<12, DIR>;
+    case 16: return (const void *)k_fix_strided<16, DIR>;
+    }
+    return nullptr;
+}
+
+cudaError_t prepare_fix_strided() {
+    for (int E : {4, 6, 8, 9, 12, 16})
+        for (const void *k : {kernel_of<-1>(E), kernel_of<1>(E)}) {
+            cudaError_t e = allow_smem(k, 48 * 1024 + 1);
+            if (e != cudaSuccess) return e;
+        }
+    return cudaSuccess;
+}
+
+int fix_threads(int n, int E, int ct) { return (n / E * ct + 31) / 32 * 32; }
+
+cudaError_t fix_strided(const double2 *in, double2 *out, long ncols, long es, long ps_in, long ps_out, int planes,
+                        int dir, const FixPlan &fp, int ct, cudaStream_t s, const StridedSel *sel) {
+    const Plan &pl = fp.pl;
+    const void *k = dir < 0 ? kernel_of<-1>(pl.E) : kernel_of<1>(pl.E);
+    int cl = 0;
+    while ((1 << cl) < ct) cl++;
+    const int threads = fix_threads(pl.n, pl.E, ct);
+    if (!k || !fp.tab || (1 << cl) != ct || ct > 32 || threads > 512) return cudaErrorInvalidValue;
+    SelK sk;
+    unsigned nx;
+    cudaError_t e = strided_selection(ncols, planes, pl.n, ct, sel, &sk, &nx);
+    if (e != cudaSuccess || nx == 0) return e;
+    const size_t smem = (size_t)(pl.n + pl.n / 4 + 1) * ct * sizeof(L2);
+    if ((e = allow_smem(k, smem)) != cudaSuccess) return e;
+    FixK kp{pl.n, pl.nst, pl.radix, fp.tab};
+    void *args[] = {(void *)&in, (void *)&out, (void *)&sk, (void *)&es, (void *)&ps_in, (void *)&ps_out,
+                    (void *)&kp, (void *)&cl};
+    return cudaLaunchKernel(k, dim3(nx, (unsigned)planes), dim3(threads), args, smem, s);
+}
+
+}  // namespace nsk

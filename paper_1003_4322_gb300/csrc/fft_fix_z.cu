@@ -1,0 +1,162 @@
+// fft_fix_z.cu -- the z passes of the FP64 transforms (real lines, Sec. 2,
+// Fig. 1) in block fixed point (fft_fix.cuh): lines 2p and 2p + 1 through one
+// complex transform of length N.
+//  c2r: Z[k] = X1[k] + i X2[k] and Z[N-k] = conj X1[k] + i conj X2[k] from the
+//       half spectra (imaginary parts of X[0] and X[N/2] dropped); the inverse
+//       transform of Z is x1 + i x2.
+//  r2c: the transform Z of x1 + i x2 gives X1[k] = (Z[k] + conj Z[N-k]) / 2
+//       and X2[k] = (Z[k] - conj Z[N-k]) / 2i.
+// The pairing adds are fixed-point too, and c2r converts each loaded entry
+// once for both of its places.  A missing second line (odd line count) reads
+// as zero and is not written.  Entries kz >= kzk are not read (c2r) or not
+// written (r2c).
+#include "fft_fix_line.cuh"
+
+namespace nsk {
+
+// One CTA holds lb line pairs, T = N/E threads each; the shared line is
+// skewed by one element in eight.
+NSK_DEV int zat(int e) { return e + (e >> 3); }
+
+NSK_DEV LineGeo z_geo(int T, int li) {
+    if (T <= 32 && (T & (T - 1)) == 0) return LineGeo{kSub, 31 - __clz(T), 0, li};
+    if (T % 32 == 0) return LineGeo{kWarps, 0, T / 32, li};
+    return LineGeo{kAny, 0, T, li};
+}
+
+template <int E>
+__global__ void __launch_bounds__(256)
+k_fix_r2c2(const i64 *__restrict__ in, double2 *__restrict__ out, int N, long nlines, FixK pl, int kzk) {
+    extern __shared__ __align__(16) unsigned char smraw[];
+    __shared__ unsigned red[256];
+    const int nh = N / 2, T = N / E;
+    const int slot = threadIdx.x % T, li = threadIdx.x / T, lb = blockDim.x / T;
+    const long l1 = 2 * ((long)blockIdx.x * lb + li), l2 = l1 + 1;
+    const bool v1 = l1 < nlines, v2 = l2 < nlines;
+    L2 *ls = reinterpret_cast<L2 *>(smraw) + li * (zat(N) + 1);
+    const i64 *s1 = in + l1 * N, *s2 = in + l2 * N;
+    L2 v[E];
+#pragma unroll
+    for (int q = 0; q < E; q++) v[q] = mkl(v1 ? s1[slot + q * T] : 0, v2 ? s2[slot + q * T] : 0);
+    const LineScale sc = line_scale<E, false>(v, z_geo(T, li), red);
+#pragma unroll
+    for (int q = 0; q < E; q++) v[q] = fix_from_raw(v[q], sc.top);
+    auto sl = [&](int e) { return ls[zat(e)]; };
+    auto ss = [&](int e, L2 x) { ls[zat(e)] = x; };
+    fix_line<E, -1, true>(v, true, slot, T, pl, false, sl, ss, ss);
+    double2 *d1 = out + l1 * (nh + 1), *d2 = out + l2 * (nh + 1);
+    // the halves of the pairing fall to the exponent; with one stage the
+    // values use all 63 bits, so that half is taken before the sum
+    const int pre = pl.nst > 1 ? 0 : 1, eb = sc.top + (pl.nst > 1 ? 2 : 1);
+    for (int k = slot; k <= nh && k < kzk; k += T) {
+        const L2 a = sl(k), b = sl(k == 0 ? 0 : N - k);
+        const i64 ax = a.x >> pre, ay = a.y >> pre, bx = b.x >> pre, by = b.y >> pre;
+        if (v1) d1[k] = make_double2(fix_double(ax + bx, eb, sc.mul), fix_double(ay - by, eb, sc.mul));
+        if (v2) d2[k] = make_double2(fix_double(ay + by, eb, sc.mul), fix_double(bx - ax, eb, sc.mul));
+    }
+}
+
+template <int E>
+__global__ void __launch_bounds__(256)
+k_fix_c2r2(const longlong2 *__restrict__ in, double *__restrict__ out, int N, long nlines, FixK pl, int kzk) {
+    extern __shared__ __align__(16) unsigned char smraw[];
+    __shared__ unsigned red[256];
+    const int nh = N / 2, T = N / E;
+    const int slot = threadIdx.x % T, li = threadIdx.x / T, lb = blockDim.x / T;
+    const long l1 = 2 * ((long)blockIdx.x * lb + li), l2 = l1 + 1;
+    const bool v1 = l1 < nlines, v2 = l2 < nlines;
+    L2 *ls = reinterpret_cast<L2 *>(smraw) + li * (zat(N) + 1);
+    auto sl = [&](int e) { return ls[zat(e)]; };
+    auto ss = [&](int e, L2 x) { ls[zat(e)] = x; };
+    const longlong2 *s1 = in + l1 * (nh + 1), *s2 = in + l2 * (nh + 1);
+    // the thread's entries m = slot + j T <= N/2 of both spectra
+    constexpr int H = E / 2 + 1;
+    const int top_m = kzk <= nh ? kzk : nh + 1;
+    L2 w[2 * H];
+#pragma unroll
+    for (int j = 0; j < H; j++) {
+        const int m = slot + j * T;
+        longlong2 a{0, 0}, b{0, 0};
+        if (m < top_m) {
+            if (v1) a = s1[m];
+            if (v2) b = s2[m];
+        }
+        if (m == 0 || m == nh) a.y = b.y = 0;
+        w[2 * j] = mkl(a.x, a.y);
+        w[2 * j + 1] = mkl(b.x, b.y);
+    }
+    const LineScale sc = line_scale<2 * H, true>(w, z_geo(T, li), red);
+#pragma unroll
+    for (int j = 0; j < H; j++) {
+        const int m = slot + j * T;
+        if (m < top_m) {
+            const L2 a = fix_from_raw(w[2 * j], sc.top), b = fix_from_raw(w[2 * j + 1], sc.top);
+            ss(m, mkl(a.x - b.y, a.y + b.x));
+            if (m != 0 && m != nh) ss(N - m, mkl(a.x + b.y, b.x - a.y));
+        }
+    }
+    __syncthreads();
+    L2 v[E];
+#pragma unroll
+    for (int q = 0; q < E; q++) {
+        const int e = slot + q * T;
+        v[q] = e < top_m || N - e < top_m ? sl(e) : mkl(0, 0);
+    }
+    double *d1 = out + l1 * N, *d2 = out + l2 * N;
+    const int ebase = sc.top + 1 + (pl.nst > 1 ? 2 : 0);
+    auto gs = [&](int e, L2 x) {
+        if (v1) d1[e] = fix_double(x.x, ebase, sc.mul);
+        if (v2) d2[e] = fix_double(x.y, ebase, sc.mul);
+    };
+    fix_line<E, 1, false>(v, true, slot, T, pl, true, sl, ss, gs);
+}
+
+template <bool R2C> static const void *kernel_of(int E) {
+#define NSK_FZ(EE) case EE: return R2C ? (const void *)k_fix_r2c2<EE> : (const void *)k_fix_c2r2<EE>;
+    switch (E) {
+        NSK_FZ(4)
+        NSK_FZ(6)
+        NSK_FZ(8)
+        NSK_FZ(9)
+        NSK_FZ(12)
+        NSK_FZ(16)
+    }
+#undef NSK_FZ
+    return nullptr;
+}
+
+cudaError_t prepare_fix_z() {
+    for (int E : {4, 6, 8, 9, 12, 16})
+        for (const void *k : {kernel_of<true>(E), kernel_of<false>(E)}) {
+            cudaError_t e = allow_smem(k, 48 * 1024 + 1);
+            if (e != cudaSuccess) return e;
+        }
+    return cudaSuccess;
+}
+
+template <bool R2C>
+static cudaError_t launch(const void *in, void *out, int N, long nlines, const FixPlan &fp, cudaStream_t s, int kzk) {
+    const Plan &pl = fp.pl;
+    const void *k = kernel_of<R2C>(pl.E);
+    if (!k || !fp.tab || pl.n != N || nlines < 1) return cudaErrorInvalidValue;
+    if (kzk < 0 || kzk > N / 2 + 1) kzk = N / 2 + 1;   // every entry
+    const int T = N / pl.E, lb = 256 / T;
+    if (lb < 1) return cudaErrorInvalidValue;
+    const size_t smem = (size_t)lb * (N + (N >> 3) + 1) * sizeof(L2);
+    cudaError_t e = allow_smem(k, smem);
+    if (e != cudaSuccess) return e;
+    const long blocks = ((nlines + 1) / 2 + lb - 1) / lb;
+    if (blocks > 0x7fffffffL) return cudaErrorInvalidValue;
+    FixK kp{pl.n, pl.nst, pl.radix, fp.tab};
+    void *args[] = {(void *)&in, (void *)&out, (void *)&N, (void *)&nlines, (void *)&kp, (void *)&kzk};
+    return cudaLaunchKernel(k, dim3((unsigned)blocks), dim3(lb * T), args, smem, s);
+}
+
+cudaError_t fix_z_r2c(const double *in, double2 *out, int N, long nlines, const FixPlan &fp, cudaStream_t s, int kzk) {
+    return launch<true>(in, out, N, nlines, fp, s, kzk);
+}
+cudaError_t fix_z_c2r(const double2 *in, double *out, int N, long nlines, const FixPlan &fp, cudaStream_t s, int kzk) {
+    return launch<false>(in, out, N, nlines, fp, s, kzk);
+}
+
+}  // namespace nsk

@@ -1,13 +1,16 @@
 // fft_passes.cu -- the axis passes of the unpruned 3D r2c / c2r transforms
 // (Sec. 2, Fig. 1: 1D FFTs along each direction of the N^3 box with the
 // (N/2+1) x N x N half storage).  On one GPU the slab transposes of the
-// paper become the data layout of these passes: the strided passes read and
-// write rows of contiguous columns (coalesced 128-byte rows), so no separate
+// paper become the data layout of these passes (FP32 here; the FP64 ones are
+// fft_fix_strided.cu and fft_fix_z.cu): the strided passes read and write
+// rows of contiguous columns (coalesced 128-byte rows), so no separate
 // transpose ever touches HBM.
 #include <math.h>
 
+#include <map>
 #include <mutex>
 #include <set>
+#include <type_traits>
 #include <vector>
 
 #include "ns_internal.h"
@@ -66,15 +69,13 @@ bool supported_n(int n) {
     return make_plan(n, &p) && make_plan(n / 2, &p);
 }
 
-int default_ct(int elem_bytes, int n) {
+int default_ct(int n) {
     // 128-byte rows, within the thread bound of the strided kernel
-    // (512 threads for float, 384 for double: no register spills).
-    int ct = 128 / elem_bytes;
-    const int bound = elem_bytes == 8 ? 512 : 384;
+    int ct = 16;
     Plan p;
     if (make_plan(n, &p)) {
         const int T = n / p.E;
-        while (ct > 1 && ct * T > bound) ct /= 2;
+        while (ct > 1 && ct * T > 512) ct /= 2;
     }
     return ct;
 }
@@ -129,27 +130,90 @@ template <typename T> typename Cx<T>::type *make_twiddles(int n, cudaError_t *er
 template float2 *make_twiddles<float>(int, cudaError_t *);
 template double2 *make_twiddles<double>(int, cudaError_t *);
 
+// exp(-2 pi i t / n) in the format of fft_fix.cuh, w = H 2^-30 + L 2^-60 per
+// part, from long double values (64 mantissa bits or more).
+static int4 fix_twiddle(int t, int n) {
+    const long double a = 6.283185307179586476925286766559005768L * t / n, one = 1073741824.0L;
+    const long double part[2] = {4 * t == n || 4 * t == 3 * n ? 0.0L : cosl(a),
+                                 t == 0 || 2 * t == n ? 0.0L : -sinl(a)};
+    int h[2], l[2];
+    for (int i = 0; i < 2; i++) {
+        h[i] = (int)llroundl(part[i] * one);
+        l[i] = (int)llroundl((part[i] * one - h[i]) * one);
+    }
+    return make_int4(h[0], l[0], h[1], l[1]);
+}
+
+// Host side of make_fix_tables: computed once per length for the life of the
+// process (at most 16 (6 n) bytes for each supported length).
+struct FixTables {
+    std::vector<int4> all;
+    long off[17];
+};
+static const FixTables &fix_tables(int n) {
+    static std::mutex mu;
+    static std::map<int, FixTables> done;
+    std::lock_guard<std::mutex> g(mu);
+    auto it = done.find(n);
+    if (it != done.end()) return it->second;   // entries never move
+    std::vector<int4> base(n);
+    for (int t = 0; t < n; t++) base[t] = fix_twiddle(t, n);
+    FixTables f;
+    for (int E = 0; E <= 16; E++) {
+        Plan pl;
+        f.off[E] = -1;
+        if (!make_plan_e(n, E, &pl)) continue;
+        f.off[E] = (long)f.all.size();
+        for (int s = 1, p = E; s < pl.nst; p *= pl.rad(s++)) {
+            const int R = pl.rad(s), stride = n / (p * R);
+            for (int q = 1; q < R; q++)
+                for (int k = 0; k < p; k++) f.all.push_back(base[(long)q * k * stride]);
+        }
+    }
+    if (f.all.empty()) f.all.push_back(base[0]);   // single-stage plans read no twiddles
+    return done[n] = std::move(f);
+}
+
+cudaError_t make_fix_tables(int n, int4 **buf, const int4 *tab[17]) {
+    const FixTables &f = fix_tables(n);
+    cudaError_t e = dev_malloc((void **)buf, f.all.size() * sizeof(int4));
+    if (e != cudaSuccess) return e;
+    e = cudaMemcpy(*buf, f.all.data(), f.all.size() * sizeof(int4), cudaMemcpyHostToDevice);
+    for (int E = 0; E <= 16; E++) tab[E] = f.off[E] >= 0 ? *buf + f.off[E] : nullptr;
+    return e;
+}
+
 // ---------------------------------------------------------------- strided pass
 
-template <typename T> struct Bounds;
-template <> struct Bounds<float> { enum { threads = 512 }; };
-template <> struct Bounds<double> { enum { threads = 384 }; };
-
-// The columns of a plane a strided launch transforms, as the kernel sees
-// them: the plane is nouter rows of `inner` columns, of which rows [0, o1)
-// and [o2, nouter) and the first `keep` columns of each are done, tpr tiles
-// of ct columns per row; rows e of the transform axis in [gap_lo, gap_hi)
-// read as zero (inverse) or are not written (forward).
-struct SelK {
-    long inner;
-    int keep, tpr, o1, o2, gap_lo, gap_hi;
-};
+cudaError_t strided_selection(long ncols, int planes, int n, int ct, const StridedSel *sel, SelK *out,
+                              unsigned *tiles) {
+    *tiles = 0;
+    if (planes < 1 || planes > 65535 || ct < 1) return cudaErrorInvalidValue;
+    if (ncols < 1 || ncols > 0x7fff0000L) return cudaErrorInvalidValue;
+    SelK sk{ncols, (int)ncols, 0, 1, 1, 0, 0};
+    int nrows = 1;
+    if (sel) {
+        if (sel->nouter < 1 || sel->inner < 1 || sel->keep < 0 || sel->keep > sel->inner ||
+            sel->inner * sel->nouter != ncols || sel->o1 < 0 || sel->o1 > sel->o2 || sel->o2 > sel->nouter ||
+            sel->gap_lo < 0 || sel->gap_lo > sel->gap_hi || sel->gap_hi > n)
+            return cudaErrorInvalidValue;
+        sk = SelK{sel->inner, sel->keep, 0, sel->o1, sel->o2, sel->gap_lo, sel->gap_hi};
+        nrows = sel->o1 + sel->nouter - sel->o2;
+    }
+    if (sk.keep > 0x7fffffffL - ct) return cudaErrorInvalidValue;
+    sk.tpr = (sk.keep + ct - 1) / ct;
+    *out = sk;
+    if (nrows < 1 || sk.tpr < 1) return cudaSuccess;   // nothing selected
+    if ((long)nrows * sk.tpr > 0x7fffffffL) return cudaErrorInvalidValue;
+    *tiles = (unsigned)(nrows * sk.tpr);
+    return cudaSuccess;
+}
 
 // One CTA: ct contiguous columns of one plane, T = n/E threads per column,
 // lanes along columns (coalesced rows).  Shared tile: element (e, c) at
 // e * ct + c.
 template <typename T, int E, int DIR>
-__global__ void __launch_bounds__(Bounds<T>::threads)
+__global__ void __launch_bounds__(512)
 k_fft_strided(const typename Cx<T>::type *__restrict__ in, typename Cx<T>::type *out, SelK sel,
               long es, long ps_in, long ps_out, Plan pl, const typename Cx<T>::type *__restrict__ tw,
               int ntab) {
@@ -195,28 +259,16 @@ cudaError_t fft_strided(const typename Cx<T>::type *in, typename Cx<T>::type *ou
                         const StridedSel *sel) {
     typedef typename Cx<T>::type C;
     const void *k = dir < 0 ? strided_kernel<T, -1>(pl.E) : strided_kernel<T, +1>(pl.E);
-    if (!k || planes < 1 || planes > 65535) return cudaErrorInvalidValue;
     const int T_ = pl.n / pl.E;
-    if (ct < 1 || ct * T_ > (int)Bounds<T>::threads) return cudaErrorInvalidValue;
-    if (ncols < 1 || ncols > 0x7fff0000L) return cudaErrorInvalidValue;
-    SelK sk{ncols, (int)ncols, 0, 1, 1, 0, 0};
-    int nrows = 1;
-    if (sel) {
-        if (sel->nouter < 1 || sel->inner < 1 || sel->keep < 0 || sel->keep > sel->inner ||
-            sel->inner * sel->nouter != ncols || sel->o1 < 0 || sel->o1 > sel->o2 || sel->o2 > sel->nouter ||
-            sel->gap_lo < 0 || sel->gap_lo > sel->gap_hi || sel->gap_hi > pl.n)
-            return cudaErrorInvalidValue;
-        sk = SelK{sel->inner, sel->keep, 0, sel->o1, sel->o2, sel->gap_lo, sel->gap_hi};
-        nrows = sel->o1 + sel->nouter - sel->o2;
-    }
-    if (sk.keep > 0x7fffffffL - ct) return cudaErrorInvalidValue;
-    sk.tpr = (sk.keep + ct - 1) / ct;
-    if (nrows < 1 || sk.tpr < 1) return cudaSuccess;   // nothing selected
-    if ((long)nrows * sk.tpr > 0x7fffffffL) return cudaErrorInvalidValue;
+    if (!k || ct < 1 || ct * T_ > 512) return cudaErrorInvalidValue;
+    SelK sk;
+    unsigned tiles;
+    cudaError_t e = strided_selection(ncols, planes, pl.n, ct, sel, &sk, &tiles);
+    if (e != cudaSuccess || tiles == 0) return e;
     const size_t smem = (size_t)pl.n * ct * sizeof(C);
-    cudaError_t e = allow_smem(k, smem);
+    e = allow_smem(k, smem);
     if (e != cudaSuccess) return e;
-    dim3 grid((unsigned)(nrows * sk.tpr), (unsigned)planes);
+    dim3 grid(tiles, (unsigned)planes);
     Plan p = pl;
     void *args[] = {(void *)&in, (void *)&out, (void *)&sk, (void *)&es, (void *)&ps_in,
                     (void *)&ps_out, (void *)&p, (void *)&tw, (void *)&ntab};
@@ -225,10 +277,6 @@ cudaError_t fft_strided(const typename Cx<T>::type *in, typename Cx<T>::type *ou
 template cudaError_t fft_strided<float>(const float2 *, float2 *, long, long, long, long, int, int,
                                         const Plan &, const float2 *, int, int, cudaStream_t,
                                         const StridedSel *);
-template cudaError_t fft_strided<double>(const double2 *, double2 *, long, long, long, long, int,
-                                         int, const Plan &, const double2 *, int, int,
-                                         cudaStream_t, const StridedSel *);
-
 // ---------------------------------------------------------------- z passes
 
 // Shared-memory line with a skew of one element every 128 bytes, so that the
@@ -423,7 +471,9 @@ static cudaError_t launch_z(const void *in, void *out, int N, long nlines, const
                             const typename Cx<T>::type *tw, cudaStream_t s, int kzk) {
     typedef typename Cx<T>::type C;
     const bool paired = pl.n == N;
-    const void *k = paired ? z_kernel2<T, R2C>(pl.E) : z_kernel<T, R2C>(pl.E);
+    const void *k = nullptr;
+    if (!paired) k = z_kernel<T, R2C>(pl.E);
+    else if constexpr (std::is_same<T, float>::value) k = z_kernel2<T, R2C>(pl.E);   // FP64: fft_fix_z.cu
     if (!k || (!paired && pl.n * 2 != N) || nlines < 1) return cudaErrorInvalidValue;
     if (kzk < 0 || kzk > N / 2 + 1) kzk = N / 2 + 1;   // every entry
     const int Tn = pl.n / pl.E;
@@ -456,17 +506,16 @@ cudaError_t prepare_fft_kernels() {
     const int Es[] = {4, 6, 8, 9, 12, 16};
     for (int E : Es) {
         const void *ks[] = {strided_kernel<float, -1>(E), strided_kernel<float, 1>(E),
-                            strided_kernel<double, -1>(E), strided_kernel<double, 1>(E),
                             z_kernel<float, true>(E), z_kernel<float, false>(E),
                             z_kernel<double, true>(E), z_kernel<double, false>(E),
-                            z_kernel2<float, true>(E), z_kernel2<float, false>(E),
-                            z_kernel2<double, true>(E), z_kernel2<double, false>(E)};
+                            z_kernel2<float, true>(E), z_kernel2<float, false>(E)};
         for (const void *k : ks) {
             cudaError_t e = allow_smem(k, big);
             if (e != cudaSuccess) return e;
         }
     }
-    return cudaSuccess;
+    const cudaError_t e = prepare_fix_strided();
+    return e != cudaSuccess ? e : prepare_fix_z();
 }
 
 template cudaError_t fft_z_r2c<float>(const float *, float2 *, int, long, const Plan &,

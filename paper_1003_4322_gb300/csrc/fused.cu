@@ -1219,7 +1219,7 @@ cudaError_t fused_alloc(FusedRun &f, const std::vector<ns_run_params> &runs, con
     if ((e = dev_malloc((void **)&f.counter, nr * sizeof(unsigned long long))) != cudaSuccess) return e;
     if ((e = cudaMemsetAsync(f.counter, 0, nr * sizeof(unsigned long long), s)) != cudaSuccess) return e;
     if ((e = prepare_fused_kernels()) != cudaSuccess) return e;
-    const int ct = default_ct(sizeof(float2), f.n);
+    const int ct = default_ct(f.n);
     for (int i = 0; i < 4; i++) f.sp[i] = PassCfg{pass_plan(f, i), ct};
     f.zc = PassCfg{f.plH, std::max(1, 192 / (6 * (f.nz / 2 / f.plH.E)))};
     cudaError_t e2 = fused_autotune(f, s);

@@ -110,7 +110,7 @@ extern "C" ns_status ns_fft_c2r_noalloc(int n, int ncomp, const void *in, void *
     const float2 *tw = dev.twiddles + off;
 
     const long nh = n / 2 + 1, plane = (long)n * nh, M = (long)n * plane, V = (long)n * n * n;
-    const int ct = default_ct(sizeof(float2), n);
+    const int ct = default_ct(n);
     const float2 *src = (const float2 *)in;
     float *dst = (float *)out;
     for (int c = 0; c < ncomp; c++) {

@@ -100,6 +100,17 @@ struct StridedSel {
     int gap_lo = 0, gap_hi = 0;
 };
 
+// The same as the kernels see it: tpr tiles of ct columns per row.
+struct SelK {
+    long inner;
+    int keep, tpr, o1, o2, gap_lo, gap_hi;
+};
+// Checks a selection (nullptr: all ncols columns) of a strided pass of length
+// n over `planes` planes and forms *sk and the CTAs per plane (0: nothing
+// selected).
+cudaError_t strided_selection(long ncols, int planes, int n, int ct, const StridedSel *sel, SelK *sk,
+                              unsigned *tiles);
+
 // Batched FFT along a strided axis.  Element e (< pl.n) of column c (< ncols)
 // of plane b (< planes) sits at base + b * plane_stride + e * es + c (in
 // complex units); columns are contiguous.  dir = -1 forward, +1 inverse.
@@ -126,8 +137,32 @@ template <typename T>
 cudaError_t fft_z_c2r(const typename Cx<T>::type *in, T *out, int N, long nlines,
                       const Plan &pl, const typename Cx<T>::type *tw, cudaStream_t s, int kzk = -1);
 
-// Columns per CTA of the strided pass for a given precision and length.
-int default_ct(int elem_bytes, int n);
+// Columns per CTA of the FP32 strided pass for a length.
+int default_ct(int n);
+
+// A plan of the FP64 transforms with its stage twiddles on the device, in the
+// fixed-point format of fft_fix.cuh.
+struct FixPlan {
+    Plan pl{};
+    const int4 *tab = nullptr;
+};
+// The stage twiddles of length n for every E that suits it, in one device
+// array: tab[E] points at those of make_plan_e(n, E) (nullptr: no such plan).
+// *buf receives the array (freed with dev_free).
+cudaError_t make_fix_tables(int n, int4 **buf, const int4 *tab[17]);
+
+// The FP64 passes (fft_fix_strided.cu, fft_fix_z.cu), arguments as those of
+// fft_strided, fft_z_r2c and fft_z_c2r; the z plans have length N (two lines
+// per transform).  ct: a power of two up to 32, fix_threads(n, E, ct) <= 512.
+int fix_threads(int n, int E, int ct);
+cudaError_t fix_strided(const double2 *in, double2 *out, long ncols, long es, long ps_in, long ps_out, int planes,
+                        int dir, const FixPlan &fp, int ct, cudaStream_t s, const StridedSel *sel = nullptr);
+cudaError_t fix_z_r2c(const double *in, double2 *out, int N, long nlines, const FixPlan &fp, cudaStream_t s,
+                      int kzk = -1);
+cudaError_t fix_z_c2r(const double2 *in, double *out, int N, long nlines, const FixPlan &fp, cudaStream_t s,
+                      int kzk = -1);
+cudaError_t prepare_fix_strided();
+cudaError_t prepare_fix_z();
 
 // Opt a kernel into more than 48 KB of dynamic shared memory (once per
 // device); fails if bytes exceeds the device's opt-in maximum.
