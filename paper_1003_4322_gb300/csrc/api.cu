@@ -285,7 +285,7 @@ cudaError_t pass_z_r2c(const FftRes &f, const T *in, typename Cx<T>::type *out, 
 // Columns per CTA that the kernels of the precision take for a plan.
 template <typename T> bool ct_fits(const Plan &pl, int ct) {
     const int t = pl.n / pl.E * ct;
-    if (std::is_same<T, double>::value) return fix_threads(pl.n, pl.E, ct) <= 512;
+    if (std::is_same<T, double>::value) return fix_threads(pl.n, pl.E, ct) <= 256;
     return t <= 512 && t >= 32;
 }
 

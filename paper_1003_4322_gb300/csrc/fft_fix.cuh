@@ -5,12 +5,12 @@
 // rate, and the FP64 passes sat on that limit (FP64 pipe 85 % busy, 17 clocks
 // per point and SM where a point's bytes take 1.2).  Integer instructions run
 // at 64 per SM and clock on each of two pipes: measured per SM and clock, a
-// 64-bit add 60 against 1.7 FP64 additions, the complex product cmul_w 2.1
+// 64-bit add 60 against 1.7 FP64 additions, the complex product cmul_w 2.0
 // against 0.4.  A Fourier transform of a line is linear with unit-modulus
 // factors, so one power-of-two scale per line serves every intermediate value,
 // and 63 bits under that scale are more than the 53 of a double.  At 512^3
 // (three components) the passes went from 11.5 / 6.7 / 4.5 ms (z c2r, y, x)
-// in FP64 to 2.8 / 1.9 / 1.3 ms.
+// in FP64 to 2.4 / 1.6 / 1.1 ms, bound by integer instruction issue.
 //
 // The scale: with S >= sum |x_j| over the line, every sub-transform of every
 // stage is bounded by S in modulus (it is a sum of x_j times unit factors), so
@@ -59,7 +59,44 @@ template <int S> NSK_FIX L2 ladd_i(L2 a, L2 b) {
 
 NSK_FIX int lhi(i64 a) { return (int)(a >> 32); }
 NSK_FIX unsigned llo(i64 a) { return (unsigned)(unsigned long long)a; }
-NSK_FIX i64 mulw(int a, int b) { return (i64)a * b; }   // one wide multiply(-add)
+// One wide multiply(-add) each.  The instruction is spelled out because the
+// compiler otherwise turns a (-b) + c into c - a b, which takes three
+// instructions (a complex product 57 instead of 28, 0.76 against 0.50 clocks
+// per SM).
+NSK_FIX i64 madw(int a, int b, i64 c) {
+#ifdef __CUDA_ARCH__
+    i64 d;
+    asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(d) : "r"(a), "r"(b), "l"(c));
+    return d;
+#else
+    return (i64)a * b + c;
+#endif
+}
+NSK_FIX i64 mulw(int a, int b) {
+#ifdef __CUDA_ARCH__
+    i64 d;
+    asm("mul.wide.s32 %0, %1, %2;" : "=l"(d) : "r"(a), "r"(b));
+    return d;
+#else
+    return (i64)a * b;
+#endif
+}
+// Lower word of (hi:lo) shifted right by s < 32.
+NSK_FIX unsigned fshr(unsigned lo, unsigned hi, int s) {
+#ifdef __CUDA_ARCH__
+    return __funnelshift_r(lo, hi, s);
+#else
+    return s ? (lo >> s) | (hi << (32 - s)) : lo;
+#endif
+}
+// Upper word of (hi:lo) shifted left by s < 32.
+NSK_FIX unsigned fshl(unsigned lo, unsigned hi, int s) {
+#ifdef __CUDA_ARCH__
+    return __funnelshift_l(lo, hi, s);
+#else
+    return s ? (hi << s) | (lo >> (32 - s)) : hi;
+#endif
+}
 
 // A constant c in (0, 1) as add + H 2^-32 + L 2^-62.
 struct FixC {
@@ -77,7 +114,7 @@ __host__ __device__ constexpr FixC fixcos(int key) {
     case 32: return FixC{1, -1004831466, 513831524};
     case 36: return FixC{1, -1257966796, -25716447};
     case 40: return FixC{1, -1534215534, -131319465};
-    case 48: return FixC{1, -2147483647 - 1, 0};
+    case 48: return FixC{0, 2147483647, 1073741824};   // 1/2; -H must not overflow
     case 54: return FixC{0, 1643612827, -290889006};
     case 56: return FixC{0, 1468965330, 168555869};
     case 64: return FixC{0, 745813244, 96060625};
@@ -88,8 +125,8 @@ __host__ __device__ constexpr FixC fixcos(int key) {
 // x c for a constant c, |x| < 2^63.
 NSK_FIX i64 mulc(i64 x, FixC c) {
     const int xh = lhi(x), xl = (int)(llo(x) >> 2);
-    const i64 t = mulw(xl, c.H) + (1 << 29) + mulw(xh, c.L);
-    return mulw(xh, c.H) + ((t >> 30) + (c.add ? x : 0));
+    const i64 t = c.L ? madw(xh, c.L, mulw(xl, c.H)) : mulw(xl, c.H);
+    return madw(xh, c.H, (t >> 30) + (c.add ? x : 0));
 }
 
 // v exp(DIR 2 pi i m / R), m and R compile-time constants once unrolled.
@@ -108,10 +145,10 @@ template <int R, int DIR> NSK_FIX L2 lrot(L2 v, int m) {
     }
     const FixC c = fixcos(r), s = fixcos(72 - r);
     const int xh = lhi(v.x), xl = (int)(llo(v.x) >> 2), yh = lhi(v.y), yl = (int)(llo(v.y) >> 2);
-    const i64 tx = mulw(xl, c.H) + (1 << 29) + mulw(xh, c.L) - (mulw(yl, s.H) + mulw(yh, s.L));
-    const i64 ty = mulw(yl, c.H) + (1 << 29) + mulw(yh, c.L) + (mulw(xl, s.H) + mulw(xh, s.L));
-    i64 rx = mulw(xh, c.H) - mulw(yh, s.H) + (tx >> 30);
-    i64 ry = mulw(yh, c.H) + mulw(xh, s.H) + (ty >> 30);
+    const i64 tx = madw(yh, -s.L, madw(yl, -s.H, madw(xh, c.L, mulw(xl, c.H))));
+    const i64 ty = madw(xh, s.L, madw(xl, s.H, madw(yh, c.L, mulw(yl, c.H))));
+    i64 rx = madw(xh, c.H, madw(yh, -s.H, tx >> 30));
+    i64 ry = madw(yh, c.H, madw(xh, s.H, ty >> 30));
     if (c.add) {
         rx += v.x;
         ry += v.y;
@@ -134,16 +171,15 @@ template <int DIR> NSK_FIX L2 cmul_w(L2 v, int4 w, bool first) {
         xl = llo(v.x) >> 2;
         yl = llo(v.y) >> 2;
     } else {
-        xh = (int)(v.x >> 30);
-        yh = (int)(v.y >> 30);
+        xh = (int)fshr(llo(v.x), (unsigned)lhi(v.x), 30);
+        yh = (int)fshr(llo(v.y), (unsigned)lhi(v.y), 30);
         xl = llo(v.x) & 0x3fffffffu;
         yl = llo(v.y) & 0x3fffffffu;
     }
     const int ih = DIR < 0 ? w.z : -w.z, il = DIR < 0 ? w.w : -w.w;
-    const i64 half = 1 << 29;
-    const i64 tx = mulw((int)xl, w.x) + half + mulw(xh, w.y) + mulw((int)yl, -ih) + mulw(yh, -il);
-    const i64 ty = mulw((int)yl, w.x) + half + mulw(yh, w.y) + mulw((int)xl, ih) + mulw(xh, il);
-    return mkl(mulw(xh, w.x) + mulw(yh, -ih) + (tx >> 30), mulw(yh, w.x) + mulw(xh, ih) + (ty >> 30));
+    const i64 tx = madw(yh, -il, madw((int)yl, -ih, madw(xh, w.y, mulw((int)xl, w.x))));
+    const i64 ty = madw(xh, il, madw((int)xl, ih, madw(yh, w.y, mulw((int)yl, w.x))));
+    return mkl(madw(xh, w.x, madw(yh, -ih, tx >> 30)), madw(yh, w.x, madw(xh, ih, ty >> 30)));
 }
 
 // Register DFTs, the decompositions of fft_core.cuh in this arithmetic.
@@ -207,11 +243,11 @@ template <int DIR> struct LDft<16, DIR> : LDftComposite<4, 4, DIR> {};
 
 // ---------------------------------------------------------------- conversions
 
-NSK_FIX int fix_clz64(unsigned long long a) {
+NSK_FIX int fix_clz(unsigned a) {
 #ifdef __CUDA_ARCH__
-    return __clzll((long long)a);
+    return __clz((int)a);
 #else
-    return a ? __builtin_clzll(a) : 64;
+    return a ? __builtin_clz(a) : 32;
 #endif
 }
 NSK_FIX float fix_u2f(unsigned u) {
@@ -264,22 +300,26 @@ NSK_FIX i64 fix_from(int hi, unsigned lo, int top) {
     const unsigned e = ((unsigned)hi >> 20) & 0x7ffu, m = ((unsigned)hi & 0xfffffu) | 0x100000u;
     const unsigned long long M = ((unsigned long long)m << 42) | ((unsigned long long)lo << 10);
     unsigned r = (unsigned)top - e;
-    r = r < 63u ? r : 63u;
+#ifndef __CUDA_ARCH__
+    r = r < 63u ? r : 63u;   // the device's shift yields zero beyond 63
+#endif
     const i64 t = (i64)(M >> r), s = (i64)(hi >> 31);
     return (t ^ s) - s;
 }
 
 // The double nearest v, scaled so that a leading bit at bit 63 gives the
 // biased exponent ebase (bit 62: ebase - 1, ...); halves round up in
-// magnitude.  The result must be a normal number or zero.
+// magnitude, and negative values go through their one's complement (off by one
+// unit of v).  The result must be a normal number or zero.
 NSK_FIX void fix_to(i64 v, int ebase, unsigned &hi, unsigned &lo) {
-    const i64 s = v >> 63;
-    const unsigned long long a = (unsigned long long)((v ^ s) - s);
-    const int z = fix_clz64(a);
-    const unsigned long long t = a << (z & 63);
-    const unsigned long long r = ((t >> 10) + 1) >> 1;   // 53 bits, or 2^53 after a carry
-    const unsigned h = (unsigned)(r >> 32) + ((unsigned)(ebase - z - 1) << 20);
-    hi = (a ? h : 0u) | ((unsigned)(s >> 32) & 0x80000000u);
+    const unsigned s = (unsigned)(lhi(v) >> 31), ah = (unsigned)lhi(v) ^ s, al = llo(v) ^ s;
+    const bool high = ah != 0;
+    const unsigned a = high ? ah : al, b = high ? al : 0u;
+    const int z = fix_clz(a);   // 32 for zero: the shifts then see a = b = 0
+    const unsigned nh = fshl(b, a, z & 31), nl = b << (z & 31);
+    const unsigned long long r = (((((unsigned long long)nh << 32) | nl) >> 1) + 0x200) >> 10;
+    const unsigned e = (unsigned)((high ? ebase - 1 : ebase - 33) - z) << 20;
+    hi = (a ? (unsigned)(r >> 32) + e : 0u) | (s & 0x80000000u);
     lo = (unsigned)r;
 }
 

@@ -73,11 +73,12 @@ template <class Op> NSK_DEV unsigned line_reduce(unsigned v, const LineGeo &g, u
     return v;
 }
 
-// Scale of one line: `top` (fix_from) and a factor that the results are
-// multiplied by (1, except for lines outside the range of the FP32 sum).
+// Scale of one line: `top` (fix_from) and, for lines outside the range of the
+// FP32 sum (odd), a factor that the results are multiplied by.
 struct LineScale {
     int top;
-    double mul;
+    bool any;    // some line of the CTA is odd
+    double mul;  // 1 for the others
 };
 
 // The raw value x times the power of two f (a line outside the FP32 range).
@@ -87,15 +88,19 @@ NSK_DEV i64 raw_scaled(i64 x, double f) { return __double_as_longlong(__longlong
 // they count twice in the sum (both members of a Hermitian pair).  A line of
 // entries in 2^-80 .. 2^100 needs one reduction.  Others (CTA-uniform branch)
 // are first brought to about 1 by a power of two taken from their largest
-// entry; a line with a NaN or an infinity gets the factor NaN.
-template <int NV, bool TWICE> NSK_DEV LineScale line_scale(L2 (&v)[NV], const LineGeo &g, unsigned *sh) {
+// entry; a line with a NaN or an infinity gets the factor NaN.  skip(i)
+// (CTA-uniform): v[i] is zero in the whole CTA.
+template <int NV, bool TWICE, class Skip>
+NSK_DEV LineScale line_scale(L2 (&v)[NV], const LineGeo &g, unsigned *sh, Skip skip) {
     auto sum = [&](unsigned &mx) {
         float s = 0.f;
-#pragma unroll
-        for (int i = 0; i < NV; i++) s += fix_mag(lhi(v[i].x), lhi(v[i].y), mx);
         unsigned low = 0;   // the smallest subnormals have an empty upper word
 #pragma unroll
-        for (int i = 0; i < NV; i++) low |= llo(v[i].x) | llo(v[i].y);
+        for (int i = 0; i < NV; i++) {
+            if (skip(i)) continue;
+            s += fix_mag(lhi(v[i].x), lhi(v[i].y), mx);
+            low |= llo(v[i].x) | llo(v[i].y);
+        }
         if (mx == 0 && low != 0) mx = 1;
         if (mx != 0 && s < 7.8886091e-31f) s = 7.8886091e-31f;   // 2^-100: not a zero line
         if (mx >= (1100u << 20)) s = 2.f * NSK_FIX_HIGH;
@@ -103,10 +108,9 @@ template <int NV, bool TWICE> NSK_DEV LineScale line_scale(L2 (&v)[NV], const Li
     };
     unsigned mx = 0;
     float S = __uint_as_float(line_reduce<OpAdd>(__float_as_uint(sum(mx)), g, sh));
-    LineScale r;
-    r.mul = 1.0;
     const bool odd = S != 0.f && !(S >= NSK_FIX_LOW && S <= NSK_FIX_HIGH);
-    if (__syncthreads_or(odd)) {
+    LineScale r{0, __syncthreads_or(odd) != 0, 1.0};
+    if (r.any) {
         const unsigned lm = line_reduce<OpMax>(mx, g, sh);
         if (odd) {
             const int e = (int)(lm >> 20);
@@ -132,12 +136,23 @@ template <int NV, bool TWICE> NSK_DEV LineScale line_scale(L2 (&v)[NV], const Li
 NSK_DEV i64 fix_from_raw(i64 raw, int top) { return fix_from(lhi(raw), llo(raw), top); }
 NSK_DEV L2 fix_from_raw(L2 raw, int top) { return mkl(fix_from_raw(raw.x, top), fix_from_raw(raw.y, top)); }
 
-NSK_DEV double fix_double(i64 v, int ebase, double mul) {
-    unsigned hi, lo;
-    fix_to(v, ebase, hi, lo);
-    const double d = __hiloint2double((int)hi, (int)lo);
-    return mul == 1.0 ? d : d * mul;
-}
+// Conversion of a line's results; ebase as fix_to's.  On the integer pipes (23
+// instructions a value): two FP64 additions can do it too, but all of a CTA's
+// conversions come together at its end, where the FP64 pipe made the passes
+// 20 % slower (an eighth to a quarter of the values there: 0.6 % faster).
+struct FixOut {
+    int ebase;
+    NSK_DEV double operator()(i64 v) const {
+        unsigned hi, lo;
+        fix_to(v, ebase, hi, lo);
+        return __hiloint2double((int)hi, (int)lo);
+    }
+};
+
+// CTAs of 256 threads an SM is to hold, by the registers E values take; more
+// or fewer change a 512^3 step by less than 1 %, the passes being bound by
+// instruction issue.
+template <int E> struct MinCtas { enum { n = E >= 9 ? 2 : E == 8 ? 3 : 4 }; };
 
 // Multiply by the stage twiddles and run the radix-R DFT of butterfly b.
 template <int R, int E, int DIR>
@@ -152,67 +167,72 @@ NSK_DEV void fix_butterfly(L2 (&v)[E], int b, int k, int p, const int4 *__restri
     LDft<R, DIR>::run(&v[b * R]);
 }
 
-// One stage s >= 1: every value of the line comes from sl and goes to st.
-template <int R, int E, int DIR, class SL, class ST>
+// One stage s >= 1.  The line comes from sl; every stage but the last writes
+// it back through ss (between barriers); the last leaves its results in v, in
+// the order of the line: v[j] is element slot + j T.
+template <int R, int E, int DIR, class SL, class SS>
 NSK_DEV void fix_stage(L2 (&v)[E], bool active, int slot, int T, int p, const int4 *__restrict__ tab,
-                       bool first, SL sl, ST st, bool sync_mid) {
-    const int nR = T * (E / R);
+                       bool first, bool last, SL sl, SS ss) {
+    constexpr int B = E / R;
+    const int nR = T * B;
     const unsigned magic = 0xffffffffu / (unsigned)p + 1u;   // i / p for i p < 2^32
     if (active) {
 #pragma unroll
-        for (int b = 0; b < E / R; b++)
+        for (int b = 0; b < B; b++)
 #pragma unroll
             for (int q = 0; q < R; q++) v[b * R + q] = sl(slot + b * T + q * nR);
 #pragma unroll
-        for (int b = 0; b < E / R; b++) {
+        for (int b = 0; b < B; b++) {
             const int i = slot + b * T;
             fix_butterfly<R, E, DIR>(v, b, i - p * (int)__umulhi((unsigned)i, magic), p, tab, first);
         }
     }
-    if (sync_mid) __syncthreads();
+    if (last) {   // p = n / R: butterfly i writes element i + q p = slot + (b + q B) T
+        L2 w[E];
+#pragma unroll
+        for (int j = 0; j < E; j++) w[j] = v[j];
+#pragma unroll
+        for (int b = 0; b < B; b++)
+#pragma unroll
+            for (int q = 0; q < R; q++) v[b + q * B] = w[b * R + q];
+        return;
+    }
+    __syncthreads();
     if (active) {
 #pragma unroll
-        for (int b = 0; b < E / R; b++) {
+        for (int b = 0; b < B; b++) {
             const int i = slot + b * T;
             const int k = i - p * (int)__umulhi((unsigned)i, magic);
             const int j = (i - k) * R + k;
 #pragma unroll
-            for (int q = 0; q < R; q++) st(j + q * p, v[b * R + q]);
+            for (int q = 0; q < R; q++) ss(j + q * p, v[b * R + q]);
         }
     }
+    __syncthreads();
 }
 
-// The stages of one line.  v holds the fixed-point inputs slot + q T (stage 0's
-// operands) on entry.  sl / ss: the shared line; gs: the final store, into
-// the shared line as well if LAST_SMEM (then a barrier ends the function).
-// smem_read: the inputs came from the shared line, so a barrier must precede
-// the first store into it.
-template <int E, int DIR, bool LAST_SMEM, class SL, class SS, class GS>
-NSK_DEV void fix_line(L2 (&v)[E], bool active, int slot, int T, const FixK &pl, bool smem_read, SL sl, SS ss,
-                      GS gs) {
+// The stages of one line.  v holds the fixed-point elements slot + q T on
+// entry and the transform's on return.  sl / ss: the shared line.  smem_read:
+// the inputs came from it, so a barrier must precede the first store.
+template <int E, int DIR, class SL, class SS>
+NSK_DEV void fix_line(L2 (&v)[E], bool active, int slot, int T, const FixK &pl, bool smem_read, SL sl, SS ss) {
     const int nst = pl.nst;
     if (active) LDft<E, DIR>::run(v);
-    if (smem_read && (LAST_SMEM || nst > 1)) __syncthreads();
+    if (nst == 1) return;   // T = 1: element q is v[q]
+    if (smem_read) __syncthreads();
     if (active) {
 #pragma unroll
-        for (int q = 0; q < E; q++) {
-            if (nst == 1) gs(slot * E + q, v[q]);
-            else ss(slot * E + q, v[q]);
-        }
+        for (int q = 0; q < E; q++) ss(slot * E + q, v[q]);
     }
-    if (LAST_SMEM || nst > 1) __syncthreads();
+    __syncthreads();
     int p = E;
     const int4 *tab = pl.tab;
     for (int s = 1; s < nst; s++) {
-        const bool last = s == nst - 1, wr = LAST_SMEM || !last;
-        auto st = [&](int e, L2 x) {
-            if (last) gs(e, x);
-            else ss(e, x);
-        };
+        const bool last = s == nst - 1;
         const int R = pl.rad(s);
-#define NSK_FIX_ST(RR)                                                                              \
-    case RR:                                                                                        \
-        if constexpr (E % RR == 0) fix_stage<RR, E, DIR>(v, active, slot, T, p, tab, s == 1, sl, st, wr); \
+#define NSK_FIX_ST(RR)                                                                                   \
+    case RR:                                                                                             \
+        if constexpr (E % RR == 0) fix_stage<RR, E, DIR>(v, active, slot, T, p, tab, s == 1, last, sl, ss); \
         break;
         switch (R) {
             NSK_FIX_ST(2)
@@ -225,7 +245,6 @@ NSK_DEV void fix_line(L2 (&v)[E], bool active, int slot, int T, const FixK &pl, 
             NSK_FIX_ST(16)
         }
 #undef NSK_FIX_ST
-        if (wr) __syncthreads();
         tab += (R - 1) * p;
         p *= R;
     }

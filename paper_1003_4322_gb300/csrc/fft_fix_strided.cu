@@ -12,10 +12,10 @@ namespace nsk {
 template <int E> struct SkewE { enum { shift = E == 4 ? 2 : E == 16 ? 4 : 3 }; };
 
 template <int E, int DIR>
-__global__ void __launch_bounds__(512)
+__global__ void __launch_bounds__(256, MinCtas<E>::n)
 k_fix_strided(const longlong2 *in, longlong2 *out, SelK sel, long es, long ps_in, long ps_out, FixK pl, int cl) {
     extern __shared__ __align__(16) unsigned char smraw[];
-    __shared__ unsigned red[512];
+    __shared__ unsigned red[256];
     L2 *sm = reinterpret_cast<L2 *>(smraw);
     const int T = pl.n / E, ct = 1 << cl;
     const int c = threadIdx.x & (ct - 1), slot = threadIdx.x >> cl;
@@ -27,30 +27,38 @@ k_fix_strided(const longlong2 *in, longlong2 *out, SelK sel, long es, long ps_in
     const longlong2 *src = in + (long)blockIdx.y * ps_in + col;
     longlong2 *dst = out + (long)blockIdx.y * ps_out + col;
     auto in_gap = [&](int e) { return e >= sel.gap_lo && e < sel.gap_hi; };
+    // elements q T .. (q + 1) T - 1 all in the gap: zeros that need no work
+    auto skip = [&](int q) { return DIR > 0 && q * T >= sel.gap_lo && (q + 1) * T <= sel.gap_hi; };
     L2 v[E];
 #pragma unroll
     for (int q = 0; q < E; q++) {
         const int e = slot + q * T;
         v[q] = mkl(0, 0);
+        if (skip(q)) continue;
         if (valid && (DIR < 0 || !in_gap(e))) {
             const longlong2 t = src[e * es];
             v[q] = mkl(t.x, t.y);
         }
     }
     LineGeo g{kCols, cl, 0, c};
-    const LineScale sc = line_scale<E, false>(v, g, red);
+    const LineScale sc = line_scale<E, false>(v, g, red, skip);
 #pragma unroll
-    for (int q = 0; q < E; q++) v[q] = fix_from_raw(v[q], sc.top);
-    const int ebase = sc.top + 1 + (pl.nst > 1 ? 2 : 0);
+    for (int q = 0; q < E; q++)
+        if (!skip(q)) v[q] = fix_from_raw(v[q], sc.top);
     auto at = [&](int e) { return ((e + (e >> SkewE<E>::shift)) << cl) + c; };
     auto sl = [&](int e) { return sm[at(e)]; };
     auto ss = [&](int e, L2 x) { sm[at(e)] = x; };
-    auto gs = [&](int e, L2 x) {
-        if (valid && (DIR > 0 || !in_gap(e)))
-            reinterpret_cast<double2 *>(dst)[e * es] =
-                make_double2(fix_double(x.x, ebase, sc.mul), fix_double(x.y, ebase, sc.mul));
-    };
-    fix_line<E, DIR, false>(v, active, slot, T, pl, false, sl, ss, gs);
+    fix_line<E, DIR>(v, active, slot, T, pl, false, sl, ss);
+    if (!valid) return;
+    const FixOut fo{sc.top + 1 + (pl.nst > 1 ? 2 : 0)};
+#pragma unroll
+    for (int q = 0; q < E; q++) {
+        const int e = slot + q * T;
+        if (DIR < 0 && in_gap(e)) continue;
+        double2 d = make_double2(fo(v[q].x), fo(v[q].y));
+        if (sc.any) d = make_double2(d.x * sc.mul, d.y * sc.mul);
+        reinterpret_cast<double2 *>(dst)[e * es] = d;
+    }
 }
 
 template <int DIR> static const void *kernel_of(int E) {
@@ -83,7 +91,7 @@ cudaError_t fix_strided(const double2 *in, double2 *out, long ncols, long es, lo
     int cl = 0;
     while ((1 << cl) < ct) cl++;
     const int threads = fix_threads(pl.n, pl.E, ct);
-    if (!k || !fp.tab || (1 << cl) != ct || ct > 32 || threads > 512) return cudaErrorInvalidValue;
+    if (!k || !fp.tab || (1 << cl) != ct || ct > 32 || threads > 256) return cudaErrorInvalidValue;
     SelK sk;
     unsigned nx;
     cudaError_t e = strided_selection(ncols, planes, pl.n, ct, sel, &sk, &nx);

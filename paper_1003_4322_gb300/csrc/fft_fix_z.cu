@@ -25,7 +25,7 @@ NSK_DEV LineGeo z_geo(int T, int li) {
 }
 
 template <int E>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, MinCtas<E>::n)
 k_fix_r2c2(const i64 *__restrict__ in, double2 *__restrict__ out, int N, long nlines, FixK pl, int kzk) {
     extern __shared__ __align__(16) unsigned char smraw[];
     __shared__ unsigned red[256];
@@ -38,26 +38,36 @@ k_fix_r2c2(const i64 *__restrict__ in, double2 *__restrict__ out, int N, long nl
     L2 v[E];
 #pragma unroll
     for (int q = 0; q < E; q++) v[q] = mkl(v1 ? s1[slot + q * T] : 0, v2 ? s2[slot + q * T] : 0);
-    const LineScale sc = line_scale<E, false>(v, z_geo(T, li), red);
+    const LineScale sc = line_scale<E, false>(v, z_geo(T, li), red, [](int) { return false; });
 #pragma unroll
     for (int q = 0; q < E; q++) v[q] = fix_from_raw(v[q], sc.top);
     auto sl = [&](int e) { return ls[zat(e)]; };
     auto ss = [&](int e, L2 x) { ls[zat(e)] = x; };
-    fix_line<E, -1, true>(v, true, slot, T, pl, false, sl, ss, ss);
+    fix_line<E, -1>(v, true, slot, T, pl, false, sl, ss);
+    if (pl.nst > 1) __syncthreads();
+#pragma unroll
+    for (int q = 0; q < E; q++) ss(slot + q * T, v[q]);
+    __syncthreads();
     double2 *d1 = out + l1 * (nh + 1), *d2 = out + l2 * (nh + 1);
     // the halves of the pairing fall to the exponent; with one stage the
     // values use all 63 bits, so that half is taken before the sum
-    const int pre = pl.nst > 1 ? 0 : 1, eb = sc.top + (pl.nst > 1 ? 2 : 1);
+    const int pre = pl.nst > 1 ? 0 : 1;
+    const FixOut fo{sc.top + (pl.nst > 1 ? 2 : 1)};
     for (int k = slot; k <= nh && k < kzk; k += T) {
         const L2 a = sl(k), b = sl(k == 0 ? 0 : N - k);
         const i64 ax = a.x >> pre, ay = a.y >> pre, bx = b.x >> pre, by = b.y >> pre;
-        if (v1) d1[k] = make_double2(fix_double(ax + bx, eb, sc.mul), fix_double(ay - by, eb, sc.mul));
-        if (v2) d2[k] = make_double2(fix_double(ay + by, eb, sc.mul), fix_double(bx - ax, eb, sc.mul));
+        double2 x1 = make_double2(fo(ax + bx), fo(ay - by)), x2 = make_double2(fo(ay + by), fo(bx - ax));
+        if (sc.any) {
+            x1 = make_double2(x1.x * sc.mul, x1.y * sc.mul);
+            x2 = make_double2(x2.x * sc.mul, x2.y * sc.mul);
+        }
+        if (v1) d1[k] = x1;
+        if (v2) d2[k] = x2;
     }
 }
 
 template <int E>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, MinCtas<E>::n)
 k_fix_c2r2(const longlong2 *__restrict__ in, double *__restrict__ out, int N, long nlines, FixK pl, int kzk) {
     extern __shared__ __align__(16) unsigned char smraw[];
     __shared__ unsigned red[256];
@@ -77,7 +87,7 @@ k_fix_c2r2(const longlong2 *__restrict__ in, double *__restrict__ out, int N, lo
     for (int j = 0; j < H; j++) {
         const int m = slot + j * T;
         longlong2 a{0, 0}, b{0, 0};
-        if (m < top_m) {
+        if (j * T < top_m && m < top_m) {
             if (v1) a = s1[m];
             if (v2) b = s2[m];
         }
@@ -85,7 +95,7 @@ k_fix_c2r2(const longlong2 *__restrict__ in, double *__restrict__ out, int N, lo
         w[2 * j] = mkl(a.x, a.y);
         w[2 * j + 1] = mkl(b.x, b.y);
     }
-    const LineScale sc = line_scale<2 * H, true>(w, z_geo(T, li), red);
+    const LineScale sc = line_scale<2 * H, true>(w, z_geo(T, li), red, [&](int i) { return (i / 2) * T >= top_m; });
 #pragma unroll
     for (int j = 0; j < H; j++) {
         const int m = slot + j * T;
@@ -103,12 +113,19 @@ k_fix_c2r2(const longlong2 *__restrict__ in, double *__restrict__ out, int N, lo
         v[q] = e < top_m || N - e < top_m ? sl(e) : mkl(0, 0);
     }
     double *d1 = out + l1 * N, *d2 = out + l2 * N;
-    const int ebase = sc.top + 1 + (pl.nst > 1 ? 2 : 0);
-    auto gs = [&](int e, L2 x) {
-        if (v1) d1[e] = fix_double(x.x, ebase, sc.mul);
-        if (v2) d2[e] = fix_double(x.y, ebase, sc.mul);
-    };
-    fix_line<E, 1, false>(v, true, slot, T, pl, true, sl, ss, gs);
+    fix_line<E, 1>(v, true, slot, T, pl, true, sl, ss);
+    const FixOut fo{sc.top + 1 + (pl.nst > 1 ? 2 : 0)};
+#pragma unroll
+    for (int q = 0; q < E; q++) {
+        const int e = slot + q * T;
+        double x1 = fo(v[q].x), x2 = fo(v[q].y);
+        if (sc.any) {
+            x1 *= sc.mul;
+            x2 *= sc.mul;
+        }
+        if (v1) d1[e] = x1;
+        if (v2) d2[e] = x2;
+    }
 }
 
 template <bool R2C> static const void *kernel_of(int E) {

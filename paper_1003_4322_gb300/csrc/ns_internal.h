@@ -153,7 +153,7 @@ cudaError_t make_fix_tables(int n, int4 **buf, const int4 *tab[17]);
 
 // The FP64 passes (fft_fix_strided.cu, fft_fix_z.cu), arguments as those of
 // fft_strided, fft_z_r2c and fft_z_c2r; the z plans have length N (two lines
-// per transform).  ct: a power of two up to 32, fix_threads(n, E, ct) <= 512.
+// per transform).  ct: a power of two up to 32, fix_threads(n, E, ct) <= 256.
 int fix_threads(int n, int E, int ct);
 cudaError_t fix_strided(const double2 *in, double2 *out, long ncols, long es, long ps_in, long ps_out, int planes,
                         int dir, const FixPlan &fp, int ct, cudaStream_t s, const StridedSel *sel = nullptr);
