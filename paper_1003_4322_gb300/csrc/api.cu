@@ -60,6 +60,7 @@ struct Run {
     int n = 0;    // N_x (the N of a cubic run)
     Grid g;       // grid and box
     PlainPlans gp[3];   // grid runs: the run's own plans for the x, y and z passes
+    Reach reach{};      // the largest |m_i| that the run's rule keeps
     PlainPrune prune;   // lines of the step's transforms that are skipped
     long M = 0;   // modes per component, half layout
     long V = 0;   // grid points per component
@@ -97,7 +98,8 @@ struct ns_ctx {
     int *flags = nullptr;            // device error word (bit 0: non-finite energy, bit 1: a bounded
                                      // device wait gave up)
     double *spec = nullptr, *ens = nullptr;
-    int spec_cap = 0;
+    int spec_cap = 0;                // shells of the run that has the most
+    size_t spec_slice = 0;           // results and partial sums of one run's spectrum
     void *staging = nullptr;
     size_t staging_bytes = 0;
     bool plain_only = false;         // a run the fused form does not cover (MHD at a size
@@ -713,10 +715,10 @@ static bool plain_prune_enabled() {
 
 template <typename T> ns_status plain_alloc(ns_ctx *c, Run &r) {
     typedef typename Cx<T>::type C;
-    r.prune.kx = axis_keep(r.g, 0, r.p.dealias);
-    r.prune.ky = axis_keep(r.g, 1, r.p.dealias);
-    r.prune.kz = axis_keep(r.g, 2, r.p.dealias);
-    r.prune.on = plain_prune_enabled() && r.prune.kx >= 0 && r.prune.ky >= 0 && r.prune.kz >= 0;
+    r.prune.kx = r.reach.x;
+    r.prune.ky = r.reach.y;
+    r.prune.kz = r.reach.z;
+    r.prune.on = plain_prune_enabled();
     const size_t half = (size_t)r.M * sizeof(C), real = (size_t)r.V * sizeof(T);
     const int nc = r.p.mhd ? 6 : 3;   // state components: u, or u and b
     NS_CK(dalloc(&r.un, nc * half));
@@ -969,8 +971,8 @@ cudaError_t fused_grid_spectrum(ns_ctx *c, const Run &r, int field, int nb, doub
     FusedRun &g = c->groups[r.group];
     cudaError_t e = fused_expand(g, r.gidx, field, g.bbuf, c->stream);
     if (e != cudaSuccess) return e;
-    return hel ? plain_helicity<float>(g.bbuf, r.g, nb, spec, aux, c->stream)
-               : plain_spectrum<float>(g.bbuf, r.g, nb, spec, aux, c->stream);
+    return hel ? plain_helicity<float>(g.bbuf, r.g, r.reach, nb, spec, aux, c->stream)
+               : plain_spectrum<float>(g.bbuf, r.g, r.reach, nb, spec, aux, c->stream);
 }
 
 ns_status check_flags(ns_ctx *c) {
@@ -1092,10 +1094,14 @@ ns_status ns_init(const ns_run_params *runs, int nruns, ns_prec prec, void *cuda
         r.p = runs[i];
         r.n = r.p.n;
         r.g = run_grid(r.p);
+        r.reach = Reach{axis_keep(r.g, 0, r.p.dealias), axis_keep(r.g, 1, r.p.dealias),
+                        axis_keep(r.g, 2, r.p.dealias)};
         r.M = r.g.M();
         r.V = r.g.V();
         r.nparts = energy_nparts(r.M);
-        maxbins = std::max(maxbins, grid_nbins(r.g));
+        const int nb = grid_nbins(r.g);
+        maxbins = std::max(maxbins, nb);
+        c->spec_slice = std::max(c->spec_slice, (size_t)nb * (1 + shell_parts(nb)));
         FftRes *f[3];
         if ((st = get_fft3(c, r.g, f)) != NS_OK) return bail(st);
         if (use_fused(c)) continue;   // grouped below
@@ -1141,9 +1147,9 @@ ns_status ns_init(const ns_run_params *runs, int nruns, ns_prec prec, void *cuda
             }
         }
     }
-    // nbins results, then kShellParts partials per shell
-    if ((e = dalloc(&c->spec, sizeof(double) * maxbins * (1 + kShellParts))) != cudaSuccess ||
-        (e = dalloc(&c->ens, sizeof(double) * maxbins * (1 + kShellParts))) != cudaSuccess)
+    c->spec_slice = std::max(c->spec_slice, (size_t)maxbins);
+    if ((e = dalloc(&c->spec, sizeof(double) * c->spec_slice)) != cudaSuccess ||
+        (e = dalloc(&c->ens, sizeof(double) * c->spec_slice)) != cudaSuccess)
         return bail(fail_cuda(nullptr, e));
     c->spec_cap = maxbins;
     // streams for concurrent units of the step graph (ensembles)
@@ -1409,9 +1415,9 @@ ns_status ns_field_spectrum(ns_ctx *c, int run, int field, double *spec, int nbi
     else if (use_fused(c))   // a grid or box: the shells of the plain form on the expanded state
         NS_CK(fused_grid_spectrum(c, r, field, nb, c->spec, c->ens, false));
     else if (c->prec == NS_FP64)
-        NS_CK(plain_spectrum<double>((const double2 *)r.un + off, r.g, nb, c->spec, c->ens, c->stream));
+        NS_CK(plain_spectrum<double>((const double2 *)r.un + off, r.g, r.reach, nb, c->spec, c->ens, c->stream));
     else
-        NS_CK(plain_spectrum<float>((const float2 *)r.un + off, r.g, nb, c->spec, c->ens, c->stream));
+        NS_CK(plain_spectrum<float>((const float2 *)r.un + off, r.g, r.reach, nb, c->spec, c->ens, c->stream));
     std::vector<double> hs(nb), he(nb);
     NS_CK(cudaMemcpyAsync(hs.data(), c->spec, nb * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
     NS_CK(cudaMemcpyAsync(he.data(), c->ens, nb * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
@@ -1440,7 +1446,7 @@ ns_status ns_energy_spectra(ns_ctx *c, int first, int count, double *spec, int n
     if (first < 0 || count < 1 || first + count > (int)c->runs.size() || nbins < 0 || (nbins > 0 && !spec))
         return NS_ERR_ARG;
     // one device slice per run: spec_cap results then partials, for spec and ens
-    const size_t slice = (size_t)c->spec_cap * (1 + kShellParts);
+    const size_t slice = c->spec_slice;
     if (c->bspec_runs < (size_t)count) {
         NS_CK(cudaStreamSynchronize(c->stream));
         if (c->bspec) dev_free(c->bspec);
@@ -1458,9 +1464,9 @@ ns_status ns_energy_spectra(ns_ctx *c, int first, int count, double *spec, int n
         else if (use_fused(c))
             NS_CK(fused_grid_spectrum(c, r, 0, nb, sp, en, false));
         else if (c->prec == NS_FP64)
-            NS_CK(plain_spectrum<double>((const double2 *)r.un, r.g, nb, sp, en, c->stream));
+            NS_CK(plain_spectrum<double>((const double2 *)r.un, r.g, r.reach, nb, sp, en, c->stream));
         else
-            NS_CK(plain_spectrum<float>((const float2 *)r.un, r.g, nb, sp, en, c->stream));
+            NS_CK(plain_spectrum<float>((const float2 *)r.un, r.g, r.reach, nb, sp, en, c->stream));
     }
     // the results of every run (spec, then ens, of each slice) in one copy
     std::vector<double> h((size_t)2 * count * c->spec_cap);
@@ -1526,9 +1532,9 @@ ns_status ns_helicity(ns_ctx *c, int run, double *spec, int nbins, double *helic
     else if (use_fused(c))
         NS_CK(fused_grid_spectrum(c, r, 0, nb, c->spec, c->ens, true));
     else if (c->prec == NS_FP64)
-        NS_CK(plain_helicity<double>((const double2 *)r.un, r.g, nb, c->spec, c->ens, c->stream));
+        NS_CK(plain_helicity<double>((const double2 *)r.un, r.g, r.reach, nb, c->spec, c->ens, c->stream));
     else
-        NS_CK(plain_helicity<float>((const float2 *)r.un, r.g, nb, c->spec, c->ens, c->stream));
+        NS_CK(plain_helicity<float>((const float2 *)r.un, r.g, r.reach, nb, c->spec, c->ens, c->stream));
     std::vector<double> hs(nb);
     NS_CK(cudaMemcpyAsync(hs.data(), c->spec, nb * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
     NS_CK(cudaStreamSynchronize(c->stream));

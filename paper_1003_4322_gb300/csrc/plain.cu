@@ -570,21 +570,25 @@ cudaError_t plain_energy_partials(const typename Cx<T>::type *a, const Grid &g, 
 }
 
 template <typename T>
-cudaError_t plain_spectrum(const typename Cx<T>::type *a, const Grid &g, int nbins, double *spec,
+cudaError_t plain_spectrum(const typename Cx<T>::type *a, const Grid &g, const Reach &rc, int nbins, double *spec,
                            double *ens, cudaStream_t s) {
-    if (g.cube)
-        return shell_launch(k_shell_spectrum<HalfAcc<T>>, nbins, spec, ens, s, HalfAcc<T>{a, g.nx, g.M()}, g.nx,
-                            nbins);
-    return shell_launch(k_grid_spectrum<GridAcc<T>>, nbins, spec, ens, s, GridAcc<T>{a, g}, g, nbins);
+    const HalfAcc<T> cube{a, g.nx, g.M()};
+    const GridAcc<T> any{a, g};
+    if (nbins <= kRowBins)
+        return g.cube ? shell_rows(cube, CubeShells{g.nx}, rc, nbins, spec, ens, s)
+                      : shell_rows(any, GridShells{g}, rc, nbins, spec, ens, s);
+    return shell_launch(k_grid_spectrum<GridAcc<T>>, nbins, spec, ens, s, any, g, nbins);
 }
 
 template <typename T>
-cudaError_t plain_helicity(const typename Cx<T>::type *a, const Grid &g, int nbins, double *spec,
+cudaError_t plain_helicity(const typename Cx<T>::type *a, const Grid &g, const Reach &rc, int nbins, double *spec,
                            double *aux, cudaStream_t s) {
-    if (g.cube)
-        return shell_launch(k_shell_spectrum<HalfHelAcc<T>>, nbins, spec, aux, s, HalfHelAcc<T>{a, g.nx, g.M()},
-                            g.nx, nbins);
-    return shell_launch(k_grid_spectrum<GridHelAcc<T>>, nbins, spec, aux, s, GridHelAcc<T>{a, g}, g, nbins);
+    const HalfHelAcc<T> cube{a, g.nx, g.M()};
+    const GridHelAcc<T> any{a, g};
+    if (nbins <= kRowBins)
+        return g.cube ? shell_rows(cube, CubeShells{g.nx}, rc, nbins, spec, aux, s)
+                      : shell_rows(any, GridShells{g}, rc, nbins, spec, aux, s);
+    return shell_launch(k_grid_spectrum<GridHelAcc<T>>, nbins, spec, aux, s, any, g, nbins);
 }
 
 cudaError_t energy_final(const double *part, int nparts, double *series, int cap,
@@ -610,10 +614,10 @@ cudaError_t energy_final(const double *part, int nparts, double *series, int cap
                                          cudaStream_t);                                           \
     template cudaError_t plain_energy_partials<T>(const Cx<T>::type *, const Grid &, double *,    \
                                                   const Rect &, cudaStream_t);                    \
-    template cudaError_t plain_spectrum<T>(const Cx<T>::type *, const Grid &, int, double *, double *, \
-                                           cudaStream_t);                                         \
-    template cudaError_t plain_helicity<T>(const Cx<T>::type *, const Grid &, int, double *, double *, \
-                                           cudaStream_t);
+    template cudaError_t plain_spectrum<T>(const Cx<T>::type *, const Grid &, const Reach &, int, double *, \
+                                           double *, cudaStream_t);                               \
+    template cudaError_t plain_helicity<T>(const Cx<T>::type *, const Grid &, const Reach &, int, double *, \
+                                           double *, cudaStream_t);
 NSK_INST(float)
 NSK_INST(double)
 #undef NSK_INST

@@ -1,6 +1,7 @@
 // plain.h -- launchers of the plain-form pointwise kernels and reductions.
 #pragma once
 #include "grid.cuh"
+#include "reduce.cuh"
 #include "ns_internal.h"
 
 namespace nsk {
@@ -58,10 +59,10 @@ template <typename T>
 cudaError_t plain_energy_partials(const typename Cx<T>::type *a, const Grid &g, double *part, const Rect &rc,
                                   cudaStream_t s);
 template <typename T>
-cudaError_t plain_spectrum(const typename Cx<T>::type *a, const Grid &g, int nbins, double *spec,
+cudaError_t plain_spectrum(const typename Cx<T>::type *a, const Grid &g, const Reach &rc, int nbins, double *spec,
                            double *ens, cudaStream_t s);
 template <typename T>
-cudaError_t plain_helicity(const typename Cx<T>::type *a, const Grid &g, int nbins, double *spec,
+cudaError_t plain_helicity(const typename Cx<T>::type *a, const Grid &g, const Reach &rc, int nbins, double *spec,
                            double *aux, cudaStream_t s);
 cudaError_t energy_final(const double *part, int nparts, double *series, int cap,
                          unsigned long long *counter, int *flags, cudaStream_t s);
