@@ -20,12 +20,13 @@ struct UpdateArgs {
     int mfx, mfy, mfz;   // grid index of kf along each axis (kf l_i)
     int dealias;
     double rot;       // rotation rate about z (Coriolis -2 rot z x u)
+    double gdt, rn;   // dt / N^3 and 2 rot N^3 (set by plain_update)
 };
 
-// rc (the curl, both updates, the energy partials): the rectangle of the
-// half layout outside which the state is zero and which alone the (pruned)
-// transforms read; with rc.on the curl and the updates touch only its modes,
-// and the partials load only its modes (in the same summation order).
+// rc (the curl, both updates): the rectangle of the half layout outside which
+// the state is zero and which alone the (pruned) transforms read; with rc.on
+// they touch only its modes.  The energy partials take the rectangle of the
+// kept modes whether or not the transforms are pruned.
 template <typename T>
 cudaError_t plain_curl(const typename Cx<T>::type *a, typename Cx<T>::type *w, const Grid &g, const Rect &rc,
                        cudaStream_t s);
@@ -44,8 +45,8 @@ cudaError_t plain_phase_avg(typename Cx<T>::type *acc, const typename Cx<T>::typ
                             const typename Cx<T>::type *ph, const Grid &g, cudaStream_t s);
 // MHD induction update of b (stage 1: b1 = E (b + dt N_b); stage 2: b = E b/2 +
 // (b1 + dt N_b)/2) from nb = transform of u x b.  Factor tables (etab here,
-// and the update's): exp(-c k^2 dt) by integer |k|^2 on a unit box, else the
-// per-axis factors exp(-c k_i^2 dt) by array position, [N_x | N_y | N_z/2+1].
+// and the update's): exp(-c k^2 dt) by integer |k|^2 on a unit box (the
+// update's as pairs with 1/|k|^2), else the per-axis factors exp(-c k_i^2 dt) by array position, [N_x | N_y | N_z/2+1].
 template <typename T>
 cudaError_t plain_update_b(typename Cx<T>::type *b, typename Cx<T>::type *b1,
                            const typename Cx<T>::type *nb, const T *etab, const Grid &g, int stage,
