@@ -263,9 +263,9 @@ static void prune_sels(const Grid &g, const PlainPrune &p, StridedSel *sx, Strid
 template <typename T>
 cudaError_t pass_strided(const FftRes &f, const typename Cx<T>::type *in, typename Cx<T>::type *out, long ncols,
                          long es, long ps, int planes, int dir, const Plan &pl, int ct, cudaStream_t s,
-                         const StridedSel *sel = nullptr) {
+                         const StridedSel *sel = nullptr, const FixCurl *curl = nullptr) {
     if constexpr (std::is_same<T, double>::value)
-        return fix_strided(in, out, ncols, es, ps, ps, planes, dir, f.fixed(pl), ct, s, sel);
+        return fix_strided(in, out, ncols, es, ps, ps, planes, dir, f.fixed(pl), ct, s, sel, curl);
     else
         return fft_strided<T>(in, out, ncols, es, ps, ps, planes, dir, pl, (const typename Cx<T>::type *)f.tw, f.n,
                               ct, s, sel);
@@ -281,7 +281,7 @@ template <typename T>
 cudaError_t pass_z_r2c(const FftRes &f, const T *in, typename Cx<T>::type *out, long nlines, const Plan &pl,
                        cudaStream_t s, int kzk = -1) {
     if constexpr (std::is_same<T, double>::value)
-        if (pl.n == f.n) return fix_z_r2c(in, out, f.n, nlines, f.fixed(pl), s, kzk);
+        if (pl.n == f.n) return fix_z_r2c(FixProduct{{in}}, out, f.n, nlines, f.fixed(pl), s, kzk);
     return fft_z_r2c<T>(in, out, f.n, nlines, pl, (const typename Cx<T>::type *)f.tw, s, kzk);
 }
 // Columns per CTA that the kernels of the precision take for a plan.
@@ -296,10 +296,11 @@ template <typename T> bool ct_fits(const Plan &pl, int ct) {
 // compiled lengths: the standalone kernels, one field at a time through tmp.
 // pr (on): the fields lie inside the run's Pi, and only the lines that can be
 // nonzero are transformed (the rest of tmp is neither read nor written).
+// curl (FP64, ncomp = 3): the transform of i k x in.
 template <typename T>
 cudaError_t c2r_batch(const typename Cx<T>::type *in, typename Cx<T>::type *tmp, T *out, const Grid &g,
                       int ncomp, const Fft3 &f, cudaStream_t s, Tracer *tr = nullptr,
-                      const PlainPrune *pr = nullptr) {
+                      const PlainPrune *pr = nullptr, bool curl = false) {
     typedef typename Cx<T>::type C;
     if constexpr (std::is_same<T, float>::value) {
         const StdGrid sg = std_grid(g, f);
@@ -316,9 +317,10 @@ cudaError_t c2r_batch(const typename Cx<T>::type *in, typename Cx<T>::type *tmp,
     const bool pruned = pr && pr->on;
     StridedSel sx, sy;
     if (pruned) prune_sels(g, *pr, &sx, &sy);
-    cudaError_t e = NSK_TIMED(tr, "fft_x_inverse",
+    const FixCurl cu{g.ny, (int)nh, g.ilx, g.ily, g.ilz};
+    cudaError_t e = NSK_TIMED(tr, curl ? "curl_x_inverse" : "fft_x_inverse",
                               pass_strided<T>(*f.x, in, tmp, plane, plane, M, ncomp, +1, qx.inv, qx.ct_inv, s,
-                                              pruned ? &sx : nullptr));
+                                              pruned ? &sx : nullptr, curl ? &cu : nullptr));
     if (e != cudaSuccess) return e;
     e = NSK_TIMED(tr, "fft_y_inverse",
                   pass_strided<T>(*f.y, tmp, tmp, nh, nh, plane, ncomp * g.nx, +1, qy.inv, qy.ct_inv, s,
@@ -328,13 +330,40 @@ cudaError_t c2r_batch(const typename Cx<T>::type *in, typename Cx<T>::type *tmp,
                      pass_z_c2r<T>(*f.z, tmp, out, (long)ncomp * g.nx * g.ny, qz.zc, s, pruned ? pr->kz + 1 : -1));
 }
 
+// The vorticity i k x a of three components on the grid: FP64 forms it in the
+// x pass's loads, FP32 in a kernel of its own through w.
+template <typename T>
+cudaError_t c2r_curl(const typename Cx<T>::type *a, typename Cx<T>::type *w, typename Cx<T>::type *tmp, T *out,
+                     const Grid &g, const Rect &rc, const Fft3 &f, cudaStream_t s, Tracer *tr, const PlainPrune *pr) {
+    if (std::is_same<T, double>::value) return c2r_batch<T>(a, tmp, out, g, 3, f, s, tr, pr, true);
+    const cudaError_t e = NSK_TIMED(tr, "curl", plain_curl<T>(a, w, g, rc, s));
+    return e != cudaSuccess ? e : c2r_batch<T>(w, tmp, out, g, 3, f, s, tr, pr);
+}
+
+// The y and x passes of r2c, in place.
+template <typename T>
+cudaError_t r2c_yx(typename Cx<T>::type *out, const Grid &g, int ncomp, const Fft3 &f, cudaStream_t s, Tracer *tr,
+                   const PlainPrune *pr) {
+    const long nh = g.nzh(), plane = (long)g.ny * nh, M = (long)g.nx * plane;
+    const PlainPlans &qx = *f.px, &qy = *f.py;
+    const bool pruned = pr && pr->on;
+    StridedSel sx, sy;
+    if (pruned) prune_sels(g, *pr, &sx, &sy);
+    const cudaError_t e = NSK_TIMED(tr, "fft_y_forward",
+                                    pass_strided<T>(*f.y, out, out, nh, nh, plane, ncomp * g.nx, -1, qy.fwd,
+                                                    qy.ct_fwd, s, pruned ? &sy : nullptr));
+    if (e != cudaSuccess) return e;
+    return NSK_TIMED(tr, "fft_x_forward",
+                     pass_strided<T>(*f.x, out, out, plane, plane, M, ncomp, -1, qx.fwd, qx.ct_fwd, s,
+                                     pruned ? &sx : nullptr));
+}
+
 // r2c of ncomp real fields: z pass (in -> out), y and x passes in place.
 // pr (on): only the modes inside the run's Pi are wanted; the others are left
 // partly transformed or untouched.
 template <typename T>
 cudaError_t r2c_batch(const T *in, typename Cx<T>::type *out, const Grid &g, int ncomp, const Fft3 &f,
                       cudaStream_t s, Tracer *tr = nullptr, const PlainPrune *pr = nullptr) {
-    typedef typename Cx<T>::type C;
     if constexpr (std::is_same<T, float>::value) {
         cudaError_t e = cudaSuccess;
         if (tr) tr->begin("fft_r2c_std");
@@ -342,22 +371,52 @@ cudaError_t r2c_batch(const T *in, typename Cx<T>::type *out, const Grid &g, int
         if (tr) tr->end();
         if (done) return e;
     }
-    const long nh = g.nzh(), plane = (long)g.ny * nh, M = (long)g.nx * plane;
-    const PlainPlans &qx = *f.px, &qy = *f.py, &qz = *f.pz;
-    const bool pruned = pr && pr->on;
-    StridedSel sx, sy;
-    if (pruned) prune_sels(g, *pr, &sx, &sy);
-    cudaError_t e = NSK_TIMED(tr, "fft_z_r2c",
-                              pass_z_r2c<T>(*f.z, in, out, (long)ncomp * g.nx * g.ny, qz.zr, s,
-                                            pruned ? pr->kz + 1 : -1));
-    if (e != cudaSuccess) return e;
-    e = NSK_TIMED(tr, "fft_y_forward",
-                  pass_strided<T>(*f.y, out, out, nh, nh, plane, ncomp * g.nx, -1, qy.fwd, qy.ct_fwd, s,
-                                  pruned ? &sy : nullptr));
-    if (e != cudaSuccess) return e;
-    return NSK_TIMED(tr, "fft_x_forward",
-                     pass_strided<T>(*f.x, out, out, plane, plane, M, ncomp, -1, qx.fwd, qx.ct_fwd, s,
-                                     pruned ? &sx : nullptr));
+    const cudaError_t e = NSK_TIMED(tr, "fft_z_r2c",
+                                    pass_z_r2c<T>(*f.z, in, out, (long)ncomp * g.nx * g.ny, f.pz->zr, s,
+                                                  pr && pr->on ? pr->kz + 1 : -1));
+    return e != cudaSuccess ? e : r2c_yx<T>(out, g, ncomp, f, s, tr, pr);
+}
+
+// r2c of the products u x w (and, with j, u x w + j x b): FP64 forms them in
+// the z pass's loads; the general way is the product kernel, over u, and the
+// transform of its result.
+template <typename T>
+cudaError_t r2c_cross(T *u, const T *w, typename Cx<T>::type *out, const Grid &g, const Fft3 &f, cudaStream_t s,
+                      Tracer *tr, const PlainPrune *pr) {
+    if constexpr (std::is_same<T, double>::value)
+        if (f.pz->zr.n == g.nz) {
+            const FixProduct p{{u, w}, g.V(), 1};
+            const cudaError_t e = NSK_TIMED(tr, "cross_z_r2c",
+                                            fix_z_r2c(p, out, g.nz, 3L * g.nx * g.ny, f.z->fixed(f.pz->zr), s,
+                                                      pr && pr->on ? pr->kz + 1 : -1));
+            return e != cudaSuccess ? e : r2c_yx<T>(out, g, 3, f, s, tr, pr);
+        }
+    const cudaError_t e = NSK_TIMED(tr, "cross", plain_cross<T>(u, w, g, s));
+    return e != cudaSuccess ? e : r2c_batch<T>(u, out, g, 3, f, s, tr, pr);
+}
+
+// The same for MHD: phys = [u, w, b, j] -> nu = r2c(u x w + j x b), nb = r2c(u x b).
+template <typename T>
+cudaError_t r2c_cross_mhd(T *phys, typename Cx<T>::type *nu, typename Cx<T>::type *nb, const Grid &g, const Fft3 &f,
+                          cudaStream_t s, Tracer *tr, const PlainPrune *pr) {
+    const long V3 = 3 * g.V();
+    cudaError_t e;
+    if constexpr (std::is_same<T, double>::value)
+        if (f.pz->zr.n == g.nz) {
+            const double *u = phys, *w = phys + V3, *b = phys + 2 * V3, *j = phys + 3 * V3;
+            const FixProduct p[2] = {{{u, w, j, b}, g.V(), 2}, {{u, b}, g.V(), 1}};
+            typename Cx<T>::type *out[2] = {nu, nb};
+            for (int i = 0; i < 2; i++) {
+                e = NSK_TIMED(tr, i ? "cross_z_r2c" : "cross2_z_r2c",
+                              fix_z_r2c(p[i], out[i], g.nz, 3L * g.nx * g.ny, f.z->fixed(f.pz->zr), s,
+                                        pr && pr->on ? pr->kz + 1 : -1));
+                if (e != cudaSuccess || (e = r2c_yx<T>(out[i], g, 3, f, s, tr, pr)) != cudaSuccess) return e;
+            }
+            return cudaSuccess;
+        }
+    e = NSK_TIMED(tr, "cross_mhd", plain_cross_mhd<T>(phys, g, s));
+    if (e != cudaSuccess || (e = r2c_batch<T>(phys, nu, g, 3, f, s, tr, pr)) != cudaSuccess) return e;
+    return r2c_batch<T>(phys + V3, nb, g, 3, f, s, tr, pr);
 }
 
 // The transforms of a run: the resources of its axis lengths with their plans
@@ -576,6 +635,17 @@ template <typename T> static bool z_candidate(int zmode, bool paired) {
     return paired || std::is_same<T, float>::value;
 }
 
+// The z r2c pass as the step runs it: in FP64 (two lines per transform) of the
+// products u x w, on the fields at phys and phys + V3.
+template <typename T>
+static cudaError_t tune_r2c(const FftRes &f, const T *phys, long V3, typename Cx<T>::type *out, long lines,
+                            const Plan &pl, cudaStream_t s) {
+    if constexpr (std::is_same<T, double>::value)
+        if (pl.n == f.n)
+            return fix_z_r2c(FixProduct{{phys, phys + V3}, V3 / 3, 1}, out, f.n, lines, f.fixed(pl), s);
+    return pass_z_r2c<T>(f, phys, out, lines, pl, s);
+}
+
 template <typename T> ns_status tune_plain(ns_ctx *c, Run &r, FftRes *f) {
     typedef typename Cx<T>::type C;
     static std::mutex mu;
@@ -597,7 +667,7 @@ template <typename T> ns_status tune_plain(ns_ctx *c, Run &r, FftRes *f) {
     }
     if (f->pp.tuned && !zmode) return NS_OK;
     const int n = r.n;
-    const long nh = n / 2 + 1, plane = (long)n * nh, M = (long)n * plane, lines = 3L * n * n;
+    const long nh = n / 2 + 1, plane = (long)n * nh, M = (long)n * plane, lines = 3L * n * n, V3 = 3 * r.V;
     cudaStream_t s = c->stream;
     C *in = (C *)r.un, *tmp = (C *)r.work, *half = (C *)r.wn;
     T *phys = (T *)r.phys;
@@ -627,7 +697,7 @@ template <typename T> ns_status tune_plain(ns_ctx *c, Run &r, FftRes *f) {
             if (!make_plan_e(len, E, &ph) || ph.nst > 4) continue;
             const float tc = plain_time([&]() { return pass_z_c2r<T>(*f, tmp, phys, lines, ph, s); }, s);
             if (tc > 0.f && (bc < 0.f || tc < bc)) { bc = tc; best.zc = ph; }
-            const float tr = plain_time([&]() { return pass_z_r2c<T>(*f, phys, half, lines, ph, s); }, s);
+            const float tr = plain_time([&]() { return tune_r2c<T>(*f, phys, V3, half, lines, ph, s); }, s);
             if (tr > 0.f && (br < 0.f || tr < br)) { br = tr; best.zr = ph; }
         }
     }
@@ -661,7 +731,7 @@ template <typename T> ns_status tune_plain_grid(ns_ctx *c, Run &r, FftRes *f[3])
             return NS_OK;
         }
     }
-    const long nh = g.nzh(), plane = (long)g.ny * nh, M = (long)g.nx * plane, lines = 3L * g.nx * g.ny;
+    const long nh = g.nzh(), plane = (long)g.ny * nh, M = (long)g.nx * plane, lines = 3L * g.nx * g.ny, V3 = 3 * r.V;
     cudaStream_t s = c->stream;
     C *in = (C *)r.un, *tmp = (C *)r.work, *half = (C *)r.wn;
     T *phys = (T *)r.phys;
@@ -697,7 +767,7 @@ template <typename T> ns_status tune_plain_grid(ns_ctx *c, Run &r, FftRes *f[3])
                 if (!make_plan_e(len, E, &ph) || ph.nst > 4) continue;
                 const float tc = plain_time([&]() { return pass_z_c2r<T>(*f[2], tmp, phys, lines, ph, s); }, s);
                 if (tc > 0.f && (bc < 0.f || tc < bc)) { bc = tc; best.zc = ph; }
-                const float tr = plain_time([&]() { return pass_z_r2c<T>(*f[2], phys, half, lines, ph, s); }, s);
+                const float tr = plain_time([&]() { return tune_r2c<T>(*f[2], phys, V3, half, lines, ph, s); }, s);
                 if (tr > 0.f && (br < 0.f || tr < br)) { br = tr; best.zr = ph; }
             }
     }
@@ -850,15 +920,11 @@ template <typename T> ns_status plain_step(ns_ctx *c, Run &r, cudaStream_t s, Tr
         // grid -> u x w + j x b, u x b -> their transforms -> the two updates
         C *src = (C *)(stage == 1 ? r.un : r.u1);
         C *wj = (C *)r.wn;
-        NS_CK(NSK_TIMED(tr, "curl", plain_curl<T>(src, wj, g, rc, s)));
-        NS_CK(NSK_TIMED(tr, "curl", plain_curl<T>(src + M3, wj + M3, g, rc, s)));
         NS_CK(c2r_batch<T>(src, (C *)r.work, phys, g, 3, f, s, tr, &r.prune));
-        NS_CK(c2r_batch<T>(wj, (C *)r.work, phys + V3, g, 3, f, s, tr, &r.prune));
+        NS_CK(c2r_curl<T>(src, wj, (C *)r.work, phys + V3, g, rc, f, s, tr, &r.prune));
         NS_CK(c2r_batch<T>(src + M3, (C *)r.work, phys + 2 * V3, g, 3, f, s, tr, &r.prune));
-        NS_CK(c2r_batch<T>(wj + M3, (C *)r.work, phys + 3 * V3, g, 3, f, s, tr, &r.prune));
-        NS_CK(NSK_TIMED(tr, "cross_mhd", plain_cross_mhd<T>(phys, g, s)));
-        NS_CK(r2c_batch<T>(phys, wj, g, 3, f, s, tr, &r.prune));
-        NS_CK(r2c_batch<T>(phys + V3, wj + M3, g, 3, f, s, tr, &r.prune));
+        NS_CK(c2r_curl<T>(src + M3, wj + M3, (C *)r.work, phys + 3 * V3, g, rc, f, s, tr, &r.prune));
+        NS_CK(r2c_cross_mhd<T>(phys, wj, wj + M3, g, f, s, tr, &r.prune));
         const UpdateArgs ua = update_args(r, stage);
         NS_CK(NSK_TIMED(tr, "update",
                         plain_update<T>((C *)r.un, (C *)r.u1, (const C *)wj, (const T *)r.etab, g, ua, rc, s)));
@@ -869,19 +935,15 @@ template <typename T> ns_status plain_step(ns_ctx *c, Run &r, cudaStream_t s, Tr
     }
     for (int stage = 1; stage <= 2 && !r.p.mhd; stage++) {
         C *src = (C *)(stage == 1 ? r.un : r.u1);
-        NS_CK(NSK_TIMED(tr, "curl", plain_curl<T>(src, (C *)r.wn, g, rc, s)));
         NS_CK(c2r_batch<T>(src, (C *)r.work, phys, g, 3, f, s, tr, &r.prune));
-        NS_CK(c2r_batch<T>((C *)r.wn, (C *)r.work, phys + 3 * r.V, g, 3, f, s, tr, &r.prune));
-        NS_CK(NSK_TIMED(tr, "cross", plain_cross<T>(phys, phys + 3 * r.V, g, s)));
-        NS_CK(r2c_batch<T>(phys, (C *)r.wn, g, 3, f, s, tr, &r.prune));
+        NS_CK(c2r_curl<T>(src, (C *)r.wn, (C *)r.work, phys + 3 * r.V, g, rc, f, s, tr, &r.prune));
+        NS_CK(r2c_cross<T>(phys, phys + 3 * r.V, (C *)r.wn, g, f, s, tr, &r.prune));
         if (r.p.dealias == 2) {   // the same on the grid shifted by half a spacing, averaged
             C *sh = (C *)r.sh, *sh2 = (C *)r.sh2;
             NS_CK(NSK_TIMED(tr, "phase", plain_phase<T>(src, sh, (const C *)r.phtab, g, s)));
-            NS_CK(NSK_TIMED(tr, "curl", plain_curl<T>(sh, sh2, g, rc, s)));
             NS_CK(c2r_batch<T>(sh, (C *)r.work, phys, g, 3, f, s, tr, &r.prune));
-            NS_CK(c2r_batch<T>(sh2, (C *)r.work, phys + 3 * r.V, g, 3, f, s, tr, &r.prune));
-            NS_CK(NSK_TIMED(tr, "cross", plain_cross<T>(phys, phys + 3 * r.V, g, s)));
-            NS_CK(r2c_batch<T>(phys, sh2, g, 3, f, s, tr, &r.prune));
+            NS_CK(c2r_curl<T>(sh, sh2, (C *)r.work, phys + 3 * r.V, g, rc, f, s, tr, &r.prune));
+            NS_CK(r2c_cross<T>(phys, phys + 3 * r.V, sh2, g, f, s, tr, &r.prune));
             NS_CK(NSK_TIMED(tr, "phase", plain_phase_avg<T>((C *)r.wn, sh2, (const C *)r.phtab, g, s)));
         }
         const UpdateArgs ua = update_args(r, stage);

@@ -24,20 +24,53 @@ NSK_DEV LineGeo z_geo(int T, int li) {
     return LineGeo{kAny, 0, T, li};
 }
 
-template <int E>
+// r2c's input: one field, or the products of the nonlinear term formed from
+// the fields as they are loaded (component c of f0 x f1, or of f0 x f1 + f2 x f3,
+// with f_i = 3 fields of V points).  A pass of products alone runs at the FP64
+// pipe's limit (two instructions a value: 1.45 ms at 512^3) while the
+// transform leaves that pipe idle; together they take 2.84 ms where the two took
+// 3.65.  The lines of a product's three components go to neighbouring
+// transforms, whose loads of the same lines meet in L1 and L2.
+template <int KIND>
+NSK_DEV double product_at(const FixProduct &f, long base, long o1, long o2, int e) {
+    // o1, o2: offsets of the components (c + 1) % 3 and (c + 2) % 3
+    const long i = base + e;
+    if constexpr (KIND == 0) return f.f[0][i];
+    double t = f.f[0][o1 + i] * f.f[1][o2 + i] - f.f[0][o2 + i] * f.f[1][o1 + i];
+    if constexpr (KIND == 2) t += f.f[2][o1 + i] * f.f[3][o2 + i] - f.f[2][o2 + i] * f.f[3][o1 + i];
+    return t;
+}
+
+template <int E, int KIND>
 __global__ void __launch_bounds__(256, MinCtas<E>::n)
-k_fix_r2c2(const i64 *__restrict__ in, double2 *__restrict__ out, int N, long nlines, FixK pl, int kzk) {
+k_fix_r2c2(FixProduct in, double2 *__restrict__ out, int N, long nlines, FixK pl, int kzk) {
     extern __shared__ __align__(16) unsigned char smraw[];
     __shared__ unsigned red[256];
     const int nh = N / 2, T = N / E;
     const int slot = threadIdx.x % T, li = threadIdx.x / T, lb = blockDim.x / T;
-    const long l1 = 2 * ((long)blockIdx.x * lb + li), l2 = l1 + 1;
-    const bool v1 = l1 < nlines, v2 = l2 < nlines;
+    // products: pairs of lines of the components in turn (the lines of one
+    // component are even in number)
+    long pair = (long)blockIdx.x * lb + li, base = 0, o1 = 0, o2 = 0;
+    if constexpr (KIND > 0) {
+        const int c = (int)(pair % 3);
+        base = 2 * (pair / 3) * N;
+        o1 = (c + 1) % 3 * in.V;
+        o2 = (c + 2) % 3 * in.V;
+        pair = c * (nlines / 6) + pair / 3;
+    } else {
+        base = 2 * pair * N;
+    }
+    const long l1 = 2 * pair, l2 = l1 + 1;
+    const bool v1 = KIND > 0 ? (long)blockIdx.x * lb + li < nlines / 2 : l1 < nlines;
+    const bool v2 = KIND > 0 ? v1 : l2 < nlines;
     L2 *ls = reinterpret_cast<L2 *>(smraw) + li * (zat(N) + 1);
-    const i64 *s1 = in + l1 * N, *s2 = in + l2 * N;
     L2 v[E];
 #pragma unroll
-    for (int q = 0; q < E; q++) v[q] = mkl(v1 ? s1[slot + q * T] : 0, v2 ? s2[slot + q * T] : 0);
+    for (int q = 0; q < E; q++) {
+        const int e = slot + q * T;
+        v[q] = mkl(v1 ? __double_as_longlong(product_at<KIND>(in, base, o1, o2, e)) : 0,
+                   v2 ? __double_as_longlong(product_at<KIND>(in, base + N, o1, o2, e)) : 0);
+    }
     const LineScale sc = line_scale<E, false>(v, z_geo(T, li), red, [](int) { return false; });
 #pragma unroll
     for (int q = 0; q < E; q++) v[q] = fix_from_raw(v[q], sc.top);
@@ -128,8 +161,18 @@ k_fix_c2r2(const longlong2 *__restrict__ in, double *__restrict__ out, int N, lo
     }
 }
 
-template <bool R2C> static const void *kernel_of(int E) {
-#define NSK_FZ(EE) case EE: return R2C ? (const void *)k_fix_r2c2<EE> : (const void *)k_fix_c2r2<EE>;
+// Threads per CTA (one line pair at least).  Smaller CTAs drift apart, so that
+// one's FP64 products and another's integer stages share an SM: 256 threads
+// took 3.25 ms for the product pass at 512^3, 128 take 2.84, 64 2.76 but more
+// elsewhere (c2r 2.36 / 2.26 / 2.28).
+static const int kThreads = 128;
+
+// kind: -1 c2r, else the r2c of that kind of input.
+static const void *kernel_of(int kind, int E) {
+#define NSK_FZ(EE)                                                                                    \
+    case EE:                                                                                          \
+        return kind < 0 ? (const void *)k_fix_c2r2<EE> : kind == 0 ? (const void *)k_fix_r2c2<EE, 0>  \
+             : kind == 1 ? (const void *)k_fix_r2c2<EE, 1> : (const void *)k_fix_r2c2<EE, 2>;
     switch (E) {
         NSK_FZ(4)
         NSK_FZ(6)
@@ -144,36 +187,38 @@ template <bool R2C> static const void *kernel_of(int E) {
 
 cudaError_t prepare_fix_z() {
     for (int E : {4, 6, 8, 9, 12, 16})
-        for (const void *k : {kernel_of<true>(E), kernel_of<false>(E)}) {
-            cudaError_t e = allow_smem(k, 48 * 1024 + 1);
+        for (int kind = -1; kind <= 2; kind++) {
+            cudaError_t e = allow_smem(kernel_of(kind, E), 48 * 1024 + 1);
             if (e != cudaSuccess) return e;
         }
     return cudaSuccess;
 }
 
-template <bool R2C>
-static cudaError_t launch(const void *in, void *out, int N, long nlines, const FixPlan &fp, cudaStream_t s, int kzk) {
+static cudaError_t launch(int kind, const void *in, void *out, int N, long nlines, const FixPlan &fp, cudaStream_t s,
+                          int kzk) {
     const Plan &pl = fp.pl;
-    const void *k = kernel_of<R2C>(pl.E);
-    if (!k || !fp.tab || pl.n != N || nlines < 1) return cudaErrorInvalidValue;
+    const void *k = kernel_of(kind, pl.E);
+    if (!k || !fp.tab || pl.n != N || nlines < 1 || (kind > 0 && nlines % 6)) return cudaErrorInvalidValue;
     if (kzk < 0 || kzk > N / 2 + 1) kzk = N / 2 + 1;   // every entry
-    const int T = N / pl.E, lb = 256 / T;
-    if (lb < 1) return cudaErrorInvalidValue;
+    const int T = N / pl.E, lb = T > kThreads ? 1 : kThreads / T;
+    if (T > 256) return cudaErrorInvalidValue;
     const size_t smem = (size_t)lb * (N + (N >> 3) + 1) * sizeof(L2);
     cudaError_t e = allow_smem(k, smem);
     if (e != cudaSuccess) return e;
     const long blocks = ((nlines + 1) / 2 + lb - 1) / lb;
     if (blocks > 0x7fffffffL) return cudaErrorInvalidValue;
     FixK kp{pl.n, pl.nst, pl.radix, fp.tab};
-    void *args[] = {(void *)&in, (void *)&out, (void *)&N, (void *)&nlines, (void *)&kp, (void *)&kzk};
+    // in: the argument itself (a FixProduct), or where the pointer argument is
+    void *args[] = {(void *)in, (void *)&out, (void *)&N, (void *)&nlines, (void *)&kp, (void *)&kzk};
     return cudaLaunchKernel(k, dim3((unsigned)blocks), dim3(lb * T), args, smem, s);
 }
 
-cudaError_t fix_z_r2c(const double *in, double2 *out, int N, long nlines, const FixPlan &fp, cudaStream_t s, int kzk) {
-    return launch<true>(in, out, N, nlines, fp, s, kzk);
+cudaError_t fix_z_r2c(const FixProduct &in, double2 *out, int N, long nlines, const FixPlan &fp, cudaStream_t s,
+                      int kzk) {
+    return launch(in.kind, &in, out, N, nlines, fp, s, kzk);
 }
 cudaError_t fix_z_c2r(const double2 *in, double *out, int N, long nlines, const FixPlan &fp, cudaStream_t s, int kzk) {
-    return launch<false>(in, out, N, nlines, fp, s, kzk);
+    return launch(-1, &in, out, N, nlines, fp, s, kzk);
 }
 
 }  // namespace nsk

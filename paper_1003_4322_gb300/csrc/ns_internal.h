@@ -155,9 +155,25 @@ cudaError_t make_fix_tables(int n, int4 **buf, const int4 *tab[17]);
 // fft_strided, fft_z_r2c and fft_z_c2r; the z plans have length N (two lines
 // per transform).  ct: a power of two up to 32, fix_threads(n, E, ct) <= 256.
 int fix_threads(int n, int E, int ct);
+// The x pass of a vorticity (dir +1, planes = the 3 components, ps_in apart):
+// transforms i k x a instead of a, formed on load.  The plane is ny rows of
+// nz columns; ix, iy, iz: wavenumber per index.
+struct FixCurl {
+    int ny = 0, nz = 0;
+    double ix = 1.0, iy = 1.0, iz = 1.0;
+};
 cudaError_t fix_strided(const double2 *in, double2 *out, long ncols, long es, long ps_in, long ps_out, int planes,
-                        int dir, const FixPlan &fp, int ct, cudaStream_t s, const StridedSel *sel = nullptr);
-cudaError_t fix_z_r2c(const double *in, double2 *out, int N, long nlines, const FixPlan &fp, cudaStream_t s,
+                        int dir, const FixPlan &fp, int ct, cudaStream_t s, const StridedSel *sel = nullptr,
+                        const FixCurl *curl = nullptr);
+// The input of the r2c pass: f[0] (kind 0), or products of 3-component fields of
+// V points each, formed on load: f[0] x f[1] (kind 1), f[0] x f[1] + f[2] x f[3]
+// (kind 2; nlines then covers the three components, a multiple of 6).
+struct FixProduct {
+    const double *f[4] = {nullptr, nullptr, nullptr, nullptr};
+    long V = 0;
+    int kind = 0;
+};
+cudaError_t fix_z_r2c(const FixProduct &in, double2 *out, int N, long nlines, const FixPlan &fp, cudaStream_t s,
                       int kzk = -1);
 cudaError_t fix_z_c2r(const double2 *in, double *out, int N, long nlines, const FixPlan &fp, cudaStream_t s,
                       int kzk = -1);
