@@ -20,6 +20,15 @@ namespace nsk {
 
 #define NSK_DEV __device__ __forceinline__
 
+// First statement of every kernel that launch_dep (ns_internal.h) starts: such
+// a kernel may be resident before the one ahead of it in the stream has ended,
+// so it waits for that one's end (its memory operations are then visible)
+// before anything else, and from here lets the next one become resident.
+NSK_DEV void grid_dep() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 template <typename T> struct Cx;
 template <> struct Cx<float> { typedef float2 type; };
 template <> struct Cx<double> { typedef double2 type; };

@@ -22,6 +22,7 @@ template <int E, int DIR, int KIND>
 __global__ void __launch_bounds__(256, MinCtas<E>::n)
 k_fix_strided(const longlong2 *in, longlong2 *out, SelK sel, long es, long ps_in, long ps_out, FixK pl, int cl,
               FixCurl cu) {
+    grid_dep();
     extern __shared__ __align__(16) unsigned char smraw[];
     __shared__ unsigned red[256];
     L2 *sm = reinterpret_cast<L2 *>(smraw);
@@ -132,7 +133,7 @@ cudaError_t fix_strided(const double2 *in, double2 *out, long ncols, long es, lo
     FixCurl cu = curl ? *curl : FixCurl{};
     void *args[] = {(void *)&in, (void *)&out, (void *)&sk, (void *)&es, (void *)&ps_in, (void *)&ps_out,
                     (void *)&kp, (void *)&cl, (void *)&cu};
-    return cudaLaunchKernel(k, dim3(nx, (unsigned)planes), dim3(threads), args, smem, s);
+    return launch_dep(k, dim3(nx, (unsigned)planes), dim3(threads), args, smem, s);
 }
 
 }  // namespace nsk

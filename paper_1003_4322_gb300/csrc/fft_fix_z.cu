@@ -44,6 +44,7 @@ NSK_DEV double product_at(const FixProduct &f, long base, long o1, long o2, int 
 template <int E, int KIND>
 __global__ void __launch_bounds__(256, MinCtas<E>::n)
 k_fix_r2c2(FixProduct in, double2 *__restrict__ out, int N, long nlines, FixK pl, int kzk) {
+    grid_dep();
     extern __shared__ __align__(16) unsigned char smraw[];
     __shared__ unsigned red[256];
     const int nh = N / 2, T = N / E;
@@ -102,6 +103,7 @@ k_fix_r2c2(FixProduct in, double2 *__restrict__ out, int N, long nlines, FixK pl
 template <int E>
 __global__ void __launch_bounds__(256, MinCtas<E>::n)
 k_fix_c2r2(const longlong2 *__restrict__ in, double *__restrict__ out, int N, long nlines, FixK pl, int kzk) {
+    grid_dep();
     extern __shared__ __align__(16) unsigned char smraw[];
     __shared__ unsigned red[256];
     const int nh = N / 2, T = N / E;
@@ -210,7 +212,7 @@ static cudaError_t launch(int kind, const void *in, void *out, int N, long nline
     FixK kp{pl.n, pl.nst, pl.radix, fp.tab};
     // in: the argument itself (a FixProduct), or where the pointer argument is
     void *args[] = {(void *)in, (void *)&out, (void *)&N, (void *)&nlines, (void *)&kp, (void *)&kzk};
-    return cudaLaunchKernel(k, dim3((unsigned)blocks), dim3(lb * T), args, smem, s);
+    return launch_dep(k, dim3((unsigned)blocks), dim3(lb * T), args, smem, s);
 }
 
 cudaError_t fix_z_r2c(const FixProduct &in, double2 *out, int N, long nlines, const FixPlan &fp, cudaStream_t s,

@@ -80,6 +80,23 @@ int default_ct(int n) {
     return ct;
 }
 
+cudaError_t launch_dep(const void *kernel, dim3 grid, dim3 block, void **args, size_t smem, cudaStream_t s) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusActive;
+    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone)
+        return cudaLaunchKernel(kernel, grid, block, args, smem, s);
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelExC(&cfg, kernel, args);
+}
+
 // Raise a kernel's dynamic shared-memory opt-in to the device maximum, once
 // per (device, kernel).  Occupancy depends on what a launch asks for, not on
 // this limit, so one setting serves every launch size.
@@ -217,6 +234,7 @@ __global__ void __launch_bounds__(512)
 k_fft_strided(const typename Cx<T>::type *__restrict__ in, typename Cx<T>::type *out, SelK sel,
               long es, long ps_in, long ps_out, Plan pl, const typename Cx<T>::type *__restrict__ tw,
               int ntab) {
+    grid_dep();
     typedef typename Cx<T>::type C;
     extern __shared__ __align__(16) unsigned char smraw[];
     C *sm = reinterpret_cast<C *>(smraw);
@@ -272,7 +290,7 @@ cudaError_t fft_strided(const typename Cx<T>::type *in, typename Cx<T>::type *ou
     Plan p = pl;
     void *args[] = {(void *)&in, (void *)&out, (void *)&sk, (void *)&es, (void *)&ps_in,
                     (void *)&ps_out, (void *)&p, (void *)&tw, (void *)&ntab};
-    return cudaLaunchKernel(k, grid, dim3(ct * T_), args, smem, s);
+    return launch_dep(k, grid, dim3(ct * T_), args, smem, s);
 }
 template cudaError_t fft_strided<float>(const float2 *, float2 *, long, long, long, long, int, int,
                                         const Plan &, const float2 *, int, int, cudaStream_t,
@@ -297,6 +315,7 @@ template <typename T, int E>
 __global__ void __launch_bounds__(256)
 k_fft_z_r2c(const T *__restrict__ in, typename Cx<T>::type *__restrict__ out, int N, long nlines,
             Plan pl, const typename Cx<T>::type *__restrict__ tw, int kzk) {
+    grid_dep();
     typedef typename Cx<T>::type C;
     extern __shared__ __align__(16) unsigned char smraw[];
     const int n = N / 2, Tn = n / E;
@@ -325,6 +344,7 @@ template <typename T, int E>
 __global__ void __launch_bounds__(256)
 k_fft_z_c2r(const typename Cx<T>::type *__restrict__ in, T *__restrict__ out, int N, long nlines,
             Plan pl, const typename Cx<T>::type *__restrict__ tw, int kzk) {
+    grid_dep();
     typedef typename Cx<T>::type C;
     extern __shared__ __align__(16) unsigned char smraw[];
     const int n = N / 2, Tn = n / E;
@@ -375,6 +395,7 @@ template <typename T, int E>
 __global__ void __launch_bounds__(256)
 k_fft_z_r2c2(const T *__restrict__ in, typename Cx<T>::type *__restrict__ out, int N, long nlines,
              Plan pl, const typename Cx<T>::type *__restrict__ tw, int kzk) {
+    grid_dep();
     typedef typename Cx<T>::type C;
     extern __shared__ __align__(16) unsigned char smraw[];
     const int nh = N / 2, Tn = N / E;
@@ -402,6 +423,7 @@ template <typename T, int E>
 __global__ void __launch_bounds__(256)
 k_fft_z_c2r2(const typename Cx<T>::type *__restrict__ in, T *__restrict__ out, int N, long nlines,
              Plan pl, const typename Cx<T>::type *__restrict__ tw, int kzk) {
+    grid_dep();
     typedef typename Cx<T>::type C;
     extern __shared__ __align__(16) unsigned char smraw[];
     const int nh = N / 2, Tn = N / E;
@@ -488,7 +510,7 @@ static cudaError_t launch_z(const void *in, void *out, int N, long nlines, const
     Plan p = pl;
     void *args[] = {(void *)&in, (void *)&out, (void *)&N, (void *)&nlines, (void *)&p,
                     (void *)&tw, (void *)&kzk};
-    return cudaLaunchKernel(k, dim3((unsigned)blocks), dim3(lb * Tn), args, smem, s);
+    return launch_dep(k, dim3((unsigned)blocks), dim3(lb * Tn), args, smem, s);
 }
 
 template <typename T>

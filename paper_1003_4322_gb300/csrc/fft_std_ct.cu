@@ -32,6 +32,7 @@ template <int N, int E, int WPB>
 __global__ void __launch_bounds__(32 * WPB)
 k_z_r2c_ct(const float *__restrict__ in, float2 *__restrict__ out, long nlines,
            const float2 *__restrict__ tw) {
+    grid_dep();
     typedef ZStdShape<N, E> Z;
     constexpr int n = Z::n, T = Z::T, LPW = Z::LPW, LS = Z::LS;
     extern __shared__ __align__(16) unsigned char smraw[];
@@ -72,6 +73,7 @@ template <int N, int E, int WPB>
 __global__ void __launch_bounds__(32 * WPB)
 k_z_c2r_ct(const float2 *__restrict__ in, float *__restrict__ out, long nlines,
            const float2 *__restrict__ tw) {
+    grid_dep();
     typedef ZStdShape<N, E> Z;
     constexpr int n = Z::n, T = Z::T, LPW = Z::LPW, LS = Z::LS;
     extern __shared__ __align__(16) unsigned char smraw[];
@@ -158,7 +160,7 @@ static cudaError_t launch_zstd(const ZctKernel &z, const void *in, void *out, lo
     if (e != cudaSuccess) return e;
     const long blocks = (nlines + z.lines_per_block - 1) / z.lines_per_block;
     void *args[] = {(void *)&in, (void *)&out, (void *)&nlines, (void *)&tw};
-    return cudaLaunchKernel(z.k, dim3((unsigned)blocks), dim3(z.threads), args, z.smem, s);
+    return launch_dep(z.k, dim3((unsigned)blocks), dim3(z.threads), args, z.smem, s);
 }
 
 static cudaError_t launch_col(const FzsKernel &k, const FzPass &ps, int ct, const float2 *tw,
@@ -168,7 +170,7 @@ static cudaError_t launch_col(const FzsKernel &k, const FzPass &ps, int ct, cons
     const long blocks = (ps.ncols + ct - 1) / ct * ps.nfields;
     FzPass p = ps;
     void *args[] = {(void *)&p, (void *)&tw};
-    return cudaLaunchKernel(k.k, dim3((unsigned)blocks), dim3(k.threads), args, k.smem, s);
+    return launch_dep(k.k, dim3((unsigned)blocks), dim3(k.threads), args, k.smem, s);
 }
 
 // Tuned shapes of the standalone transform for one (N, direction): the x

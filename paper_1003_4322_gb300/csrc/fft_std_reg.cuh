@@ -75,6 +75,7 @@ template <int N, int E, int WPB>
 __global__ void __launch_bounds__(32 * WPB)
 k_z_r2c_reg(const float *__restrict__ in, float2 *__restrict__ out, long nlines,
             const float2 *__restrict__ tw) {
+    grid_dep();
     typedef ZRegShape<N, E> Z;
     constexpr int n = Z::n, T = Z::T, LPW = Z::LPW, LS = Z::LS;
     extern __shared__ __align__(16) unsigned char smraw[];
@@ -103,6 +104,7 @@ template <int N, int E, int WPB>
 __global__ void __launch_bounds__(32 * WPB)
 k_z_c2r_reg(const float2 *__restrict__ in, float *__restrict__ out, long nlines,
             const float2 *__restrict__ tw) {
+    grid_dep();
     typedef ZRegShape<N, E> Z;
     constexpr int n = Z::n, T = Z::T, LPW = Z::LPW, LS = Z::LS;
     extern __shared__ __align__(16) unsigned char smraw[];
@@ -139,6 +141,7 @@ template <int N, int E, int WPB, int IT>
 __global__ void __launch_bounds__(32 * WPB)
 k_z_r2c_pf(const float *__restrict__ in, float2 *__restrict__ out, long nlines,
            const float2 *__restrict__ tw) {
+    grid_dep();
     typedef ZRegShape<N, E> Z;
     constexpr int n = Z::n, T = Z::T, LPW = Z::LPW, LS = Z::LS;
     extern __shared__ __align__(16) unsigned char smraw[];
@@ -178,6 +181,7 @@ template <int N, int E, int WPB, int IT>
 __global__ void __launch_bounds__(32 * WPB)
 k_z_c2r_pf(const float2 *__restrict__ in, float *__restrict__ out, long nlines,
            const float2 *__restrict__ tw) {
+    grid_dep();
     typedef ZRegShape<N, E> Z;
     constexpr int n = Z::n, T = Z::T, LPW = Z::LPW, LS = Z::LS;
     extern __shared__ __align__(16) unsigned char smraw[];

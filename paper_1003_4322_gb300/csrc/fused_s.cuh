@@ -27,6 +27,7 @@ template <int E, int CT> struct TileIndex {
 template <int N, int E, int CT, int DIR, bool IN_C, bool OUT_C, bool CURL>
 __global__ void __launch_bounds__(CT *(N / E))
 k_fzs_ct(FzPass ps, const float2 *__restrict__ tw) {
+    grid_dep();
     extern __shared__ __align__(16) unsigned char smraw[];
     float2 *sm = reinterpret_cast<float2 *>(smraw);
     const int c = threadIdx.x % CT, slot = threadIdx.x / CT;
