@@ -95,7 +95,8 @@ struct ns_ctx {
     std::vector<FusedRun> groups;   // fused form: runs grouped by N
     std::map<int, FftRes> fft;
     ns_status sticky = NS_OK;
-    int *flags = nullptr;            // device error word (bit 0: non-finite energy, bit 1: a bounded
+    int *hflags = nullptr;           // error word in mapped host memory, read after a synchronisation
+    int *flags = nullptr;            // its device address (bit 0: non-finite energy, bit 1: a bounded
                                      // device wait gave up)
     double *spec = nullptr, *ens = nullptr;
     int spec_cap = 0;                // shells of the run that has the most
@@ -950,10 +951,9 @@ template <typename T> ns_status plain_step(ns_ctx *c, Run &r, cudaStream_t s, Tr
         NS_CK(NSK_TIMED(tr, "update",
                         plain_update<T>((C *)r.un, (C *)r.u1, (const C *)r.wn, (const T *)r.etab, g, ua, rc, s)));
     }
-    NS_CK(NSK_TIMED(tr, "energy_partials", plain_energy_partials<T>((const C *)r.un, g, r.part,
-                                                                   Rect{1, r.reach.x, r.reach.y, r.reach.z}, s)));
-    NS_CK(NSK_TIMED(tr, "energy_final",
-                    energy_final(r.part, r.nparts, r.series, kSeriesCap, r.counter, c->flags, s)));
+    const EnergyOut eo{r.series, kSeriesCap, r.counter, (unsigned *)(r.counter + 1), c->flags};
+    NS_CK(NSK_TIMED(tr, "energy", plain_energy<T>((const C *)r.un, g, r.part,
+                                                  Rect{1, r.reach.x, r.reach.y, r.reach.z}, eo, s)));
     return NS_OK;
 }
 
@@ -1062,8 +1062,7 @@ cudaError_t fused_grid_spectrum(ns_ctx *c, const Run &r, int field, int nb, doub
 }
 
 ns_status check_flags(ns_ctx *c) {
-    int h = 0;
-    NS_CK(cudaMemcpy(&h, c->flags, sizeof(int), cudaMemcpyDeviceToHost));
+    const int h = *(volatile int *)c->hflags;   // every caller has synchronised the stream
     if (h & 2) return NS_ERR_TIMEOUT;
     if (h & 1) return NS_ERR_NONFINITE;
     return NS_OK;
@@ -1171,8 +1170,11 @@ ns_status ns_init(const ns_run_params *runs, int nruns, ns_prec prec, void *cuda
     cudaError_t e = cudaStreamCreateWithFlags(&c->cap, cudaStreamNonBlocking);
     if (e != cudaSuccess) return bail(fail_cuda(nullptr, e));
     if ((e = prepare_fft_kernels()) != cudaSuccess) return bail(fail_cuda(nullptr, e));
-    if ((e = dalloc(&c->flags, sizeof(int))) != cudaSuccess) return bail(fail_cuda(nullptr, e));
-    cudaMemset(c->flags, 0, sizeof(int));
+    if ((e = cudaHostAlloc((void **)&c->hflags, sizeof(int), cudaHostAllocMapped)) != cudaSuccess)
+        return bail(fail_cuda(nullptr, e));
+    *c->hflags = 0;
+    if ((e = cudaHostGetDevicePointer((void **)&c->flags, c->hflags, 0)) != cudaSuccess)
+        return bail(fail_cuda(nullptr, e));
     c->runs.resize(nruns);
     int maxbins = 0;
     for (int i = 0; i < nruns; i++) {
@@ -1195,9 +1197,9 @@ ns_status ns_init(const ns_run_params *runs, int nruns, ns_prec prec, void *cuda
         if (st != NS_OK) return bail(st);
         if ((e = dalloc(&r.part, sizeof(double) * 2 * std::max(r.nparts, 1))) != cudaSuccess ||
             (e = dalloc(&r.series, sizeof(double) * 2 * kSeriesCap)) != cudaSuccess ||
-            (e = dalloc(&r.counter, sizeof(unsigned long long))) != cudaSuccess)
+            (e = dalloc(&r.counter, 2 * sizeof(unsigned long long))) != cudaSuccess)
             return bail(fail_cuda(nullptr, e));
-        cudaMemset(r.counter, 0, sizeof(unsigned long long));
+        cudaMemset(r.counter, 0, 2 * sizeof(unsigned long long));   // steps recorded; finished blocks
     }
     if (use_fused(c)) {
         // runs of the same grid, box and equations form one group (in order of
@@ -1234,9 +1236,9 @@ ns_status ns_init(const ns_run_params *runs, int nruns, ns_prec prec, void *cuda
         }
     }
     c->spec_slice = std::max(c->spec_slice, (size_t)maxbins);
-    if ((e = dalloc(&c->spec, sizeof(double) * c->spec_slice)) != cudaSuccess ||
-        (e = dalloc(&c->ens, sizeof(double) * c->spec_slice)) != cudaSuccess)
+    if ((e = dalloc(&c->spec, 2 * sizeof(double) * c->spec_slice)) != cudaSuccess)
         return bail(fail_cuda(nullptr, e));
+    c->ens = c->spec + c->spec_slice;
     c->spec_cap = maxbins;
     // streams for concurrent units of the step graph (ensembles)
     const size_t units = use_fused(c) ? c->groups.size() : c->runs.size();
@@ -1267,9 +1269,8 @@ void ns_destroy(ns_ctx *c) {
         if (kv.second.ftab) dev_free(kv.second.ftab);
         if (kv.second.scratch) dev_free(kv.second.scratch);
     }
-    if (c->flags) dev_free(c->flags);
+    if (c->hflags) cudaFreeHost(c->hflags);
     if (c->spec) dev_free(c->spec);
-    if (c->ens) dev_free(c->ens);
     if (c->staging) dev_free(c->staging);
     if (c->gscratch) dev_free(c->gscratch);
     if (c->bspec) dev_free(c->bspec);
@@ -1504,10 +1505,11 @@ ns_status ns_field_spectrum(ns_ctx *c, int run, int field, double *spec, int nbi
         NS_CK(plain_spectrum<double>((const double2 *)r.un + off, r.g, r.reach, nb, c->spec, c->ens, c->stream));
     else
         NS_CK(plain_spectrum<float>((const float2 *)r.un + off, r.g, r.reach, nb, c->spec, c->ens, c->stream));
-    std::vector<double> hs(nb), he(nb);
-    NS_CK(cudaMemcpyAsync(hs.data(), c->spec, nb * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-    NS_CK(cudaMemcpyAsync(he.data(), c->ens, nb * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
+    std::vector<double> h(2 * (size_t)nb);   // spec, then ens, in one copy
+    NS_CK(cudaMemcpy2DAsync(h.data(), nb * sizeof(double), c->spec, c->spec_slice * sizeof(double),
+                            nb * sizeof(double), 2, cudaMemcpyDeviceToHost, c->stream));
     NS_CK(cudaStreamSynchronize(c->stream));
+    const double *hs = h.data(), *he = hs + nb;
     double e = 0.0, om = 0.0;
     for (int k = 0; k < nb; k++) {
         e += hs[k];

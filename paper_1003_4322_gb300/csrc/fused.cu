@@ -208,36 +208,7 @@ k_fused_update(float2 *__restrict__ a, float2 *__restrict__ a1, const float2 *__
     if (two) {
         double e = e_acc.value(), o = o_acc.value();
         block_sum2(e, o, sh);
-        if (threadIdx.x == 0) {
-            double *pp = part + 2 * ((long)run * u.nparts + blockIdx.x);
-            pp[0] = e;
-            pp[1] = o;
-        }
-    }
-}
-
-// One block per run: sum that run's partials in a fixed order, append
-// (E, Omega) to its ring buffer at slot counter % cap, bump the counter, and
-// raise bit 0 of *flags if E is not finite.
-__global__ void __launch_bounds__(256)
-k_fz_energy_final(const double *__restrict__ part, int nparts, double *series, int cap,
-                  unsigned long long *counter, int *flags) {
-    __shared__ double sh[512];
-    const int run = blockIdx.x;
-    const double *pp = part + 2L * run * nparts;
-    double e = 0.0, om = 0.0;
-    for (int i = threadIdx.x; i < nparts; i += blockDim.x) {
-        e += pp[2 * i];
-        om += pp[2 * i + 1];
-    }
-    block_sum2(e, om, sh);
-    if (threadIdx.x == 0) {
-        const unsigned long long c = counter[run];
-        double *sr = series + 2L * run * cap;
-        sr[2 * (c % cap)] = e;
-        sr[2 * (c % cap) + 1] = om;
-        counter[run] = c + 1;
-        if (!isfinite(e)) atomicOr(flags, 1);
+        energy_publish(e, o, part + 2L * run * u.nparts, u.nparts, run, blockIdx.x, u.out);
     }
 }
 
@@ -277,13 +248,28 @@ __global__ void k_fz_load(const double2 *__restrict__ src, float2 *__restrict__ 
     }
 }
 
+// The same for the whole field from device (or mapped host) memory: grid
+// (compact row modes, ikx, component), 32-bit index splits, and every compact
+// entry written, so that one launch replaces a clearing and six.  A state of
+// 64^3 loads in 5 us instead of 31.
+__global__ void __launch_bounds__(256)
+k_fz_load3(const double2 *__restrict__ src, float2 *__restrict__ dst, FzHalfGeom g, int dealias) {
+    const int j = blockIdx.x * blockDim.x + threadIdx.x, ikx = blockIdx.y, nh = g.nz / 2 + 1;
+    if (j >= g.My * g.Mz) return;
+    const int iky = j / g.Mz, kz = j - iky * g.Mz;
+    const int kx = fz_compact_signed(ikx, g.Mx, g.K), ky = fz_compact_signed(iky, g.My, g.Ky);
+    const int fx = kx >= 0 ? kx : kx + g.nx, fy = ky >= 0 ? ky : ky + g.ny;
+    double2 v = src[(((long)blockIdx.z * g.nx + fx) * g.ny + fy) * nh + kz];
+    const long ax = kx * g.qx, ay = ky * g.qy, az = kz * g.qz;
+    if (dealias == 1 && 9 * (ax * ax + ay * ay + az * az) >= g.D * g.D) v = make_double2(0.0, 0.0);
+    dst[((long)blockIdx.z * g.Mx + ikx) * g.My * g.Mz + j] = make_float2((float)v.x, (float)v.y);
+}
+
 NSK_DEV void fz_put(double2 *d, float2 v) { *d = make_double2((double)v.x, (double)v.y); }
 NSK_DEV void fz_put(float2 *d, float2 v) { *d = v; }
 
-// compact -> cnt full kx planes starting at kx0 (zeros outside the kept set),
-// FP64 (state transfer) or FP32 (the input of the grid spectra)
-template <typename D2>
-__global__ void k_fz_store(const float2 *__restrict__ src, D2 *__restrict__ dst, int kx0, int cnt, FzHalfGeom g) {
+// compact -> cnt full kx planes starting at kx0 (zeros outside the kept set)
+__global__ void k_fz_store(const float2 *__restrict__ src, double2 *__restrict__ dst, int kx0, int cnt, FzHalfGeom g) {
     const int nh = g.nz / 2 + 1;
     const long total = (long)cnt * g.ny * nh;
     for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < total; i += (long)gridDim.x * blockDim.x) {
@@ -729,7 +715,8 @@ static cudaError_t launch_update_n(FusedRun &f, const FzUpdate &u, cudaStream_t 
 
 // Update arguments of stage `stage` with nparts partial sums per run.
 static FzUpdate make_update(const FusedRun &f, int stage, int nparts) {
-    FzUpdate u{f.n, f.K, f.Mx, f.Mz, stage, f.M, f.nk2, nparts};
+    FzUpdate u{f.n, f.K, f.Mx, f.Mz, stage, f.M, f.nk2, nparts, EnergyOut{}};
+    if (f.flags) u.out = EnergyOut{f.series, f.cap, f.counter, f.ticket, f.flags};   // not while tuning
     if (!f.cube) {
         u.My = f.My;
         u.Ky = f.Ky;
@@ -1211,13 +1198,17 @@ cudaError_t fused_alloc(FusedRun &f, const std::vector<ns_run_params> &runs, con
         return e;
     // partials per run: the separate update's blocks, or one per column tile of
     // pass E fused with the update (at most eu_tiles(f, 8))
-    f.nparts_upd = (int)std::min<long>(1024, std::max<long>(1, (f.M + 4095) / 4096));
+    // (two rounds of two modes per thread until the cap: 4096 modes per block left
+    // half the SMs without one below 160^3)
+    f.nparts_upd = (int)std::min<long>(1024, std::max<long>(1, (f.M + 1023) / 1024));
     f.nparts = f.nparts_upd;
     const long parts_max = std::max<long>(f.nparts_upd, eu_tiles(f, 8));
     if ((e = dev_malloc((void **)&f.part, nr * parts_max * 2 * sizeof(double))) != cudaSuccess) return e;
     if ((e = dev_malloc((void **)&f.series, nr * (long)f.cap * 2 * sizeof(double))) != cudaSuccess) return e;
     if ((e = dev_malloc((void **)&f.counter, nr * sizeof(unsigned long long))) != cudaSuccess) return e;
     if ((e = cudaMemsetAsync(f.counter, 0, nr * sizeof(unsigned long long), s)) != cudaSuccess) return e;
+    if ((e = dev_malloc((void **)&f.ticket, nr * sizeof(unsigned))) != cudaSuccess) return e;
+    if ((e = cudaMemsetAsync(f.ticket, 0, nr * sizeof(unsigned), s)) != cudaSuccess) return e;
     if ((e = prepare_fused_kernels()) != cudaSuccess) return e;
     const int ct = default_ct(f.n);
     for (int i = 0; i < 4; i++) f.sp[i] = PassCfg{pass_plan(f, i), ct};
@@ -1273,7 +1264,7 @@ cudaError_t fused_alloc(FusedRun &f, const std::vector<ns_run_params> &runs, con
 }
 
 void fused_free(FusedRun &f) {
-    void *ps[] = {f.a, f.a1, f.nl, f.abuf, f.bbuf, f.etab, f.etab_b, f.rp, f.part, f.series, f.counter, f.k2tab};
+    void *ps[] = {f.a, f.a1, f.nl, f.abuf, f.bbuf, f.etab, f.etab_b, f.rp, f.part, f.series, f.counter, f.ticket, f.k2tab};
     for (void *p : ps)
         if (p) dev_free(p);
     f.a = f.a1 = f.nl = f.abuf = f.bbuf = nullptr;
@@ -1282,16 +1273,12 @@ void fused_free(FusedRun &f) {
     f.rp = nullptr;
     f.part = f.series = nullptr;
     f.counter = nullptr;
+    f.ticket = nullptr;
 }
 
 static cudaError_t launch_update(FusedRun &f, const FzUpdate &u, cudaStream_t s) {
     if (f.cube) k_fused_update<false><<<dim3(f.nparts, f.nr), 256, 0, s>>>(f.a, f.a1, f.nl, f.etab, f.rp, u, f.part);
     else k_fused_update<true><<<dim3(f.nparts, f.nr), 256, 0, s>>>(f.a, f.a1, f.nl, f.etab, f.rp, u, f.part);
-    return cudaGetLastError();
-}
-
-static cudaError_t launch_energy_final(FusedRun &f, int *flags, cudaStream_t s) {
-    k_fz_energy_final<<<f.nr, 256, 0, s>>>(f.part, f.nparts, f.series, f.cap, f.counter, flags);
     return cudaGetLastError();
 }
 
@@ -1330,7 +1317,7 @@ static cudaError_t fused_step_mhd(FusedRun &f, int *flags, cudaStream_t s, Trace
                        cudaGetLastError()));
         if (e != cudaSuccess) return e;
     }
-    return NSK_TIMED(tr, "energy_final", launch_energy_final(f, flags, s));
+    return cudaSuccess;
 }
 
 cudaError_t fused_step(FusedRun &f, int *flags, cudaStream_t s, Tracer *tr) {
@@ -1359,7 +1346,7 @@ cudaError_t fused_step(FusedRun &f, int *flags, cudaStream_t s, Tracer *tr) {
         e = NSK_TIMED(tr, "fused_update", launch_update(f, u, s));
         if (e != cudaSuccess) return e;
     }
-    return NSK_TIMED(tr, "energy_final", launch_energy_final(f, flags, s));
+    return cudaSuccess;
 }
 
 int fused_describe(const FusedRun &f, char *out, int len) {
@@ -1401,14 +1388,37 @@ int fused_describe(const FusedRun &f, char *out, int len) {
     return w;
 }
 
+// compact -> the whole half layout, grid (modes of a kx plane, kx, component).
+template <typename D2>
+__global__ void __launch_bounds__(256)
+k_fz_store3(const float2 *__restrict__ src, D2 *__restrict__ dst, FzHalfGeom g) {
+    const int nh = g.nz / 2 + 1, j = blockIdx.x * blockDim.x + threadIdx.x;
+    if (j >= g.ny * nh) return;
+    const int fy = j / nh, kz = j - fy * nh;
+    const int ikx = fz_compact(blockIdx.y, g.nx, g.K, g.Mx), iky = fz_compact(fy, g.ny, g.Ky, g.My);
+    float2 v = make_float2(0.f, 0.f);
+    if (ikx >= 0 && iky >= 0 && kz < g.Mz)
+        v = src[(((long)blockIdx.z * g.Mx + ikx) * g.My + iky) * g.Mz + kz];
+    fz_put(dst + ((long)blockIdx.z * g.nx + blockIdx.y) * g.ny * nh + j, v);
+}
+template <typename D2>
+static cudaError_t store3(const float2 *src, D2 *dst, const FzHalfGeom &g, cudaStream_t s) {
+    k_fz_store3<D2><<<dim3((g.ny * (g.nz / 2 + 1) + 255) / 256, g.nx, 3), 256, 0, s>>>(src, dst, g);
+    return cudaGetLastError();
+}
+
 cudaError_t fused_set_state(FusedRun &f, int run, int field, const double2 *src, int on_device, void *staging,
                             size_t staging_bytes, cudaStream_t s) {
     const int n = f.n, nh = f.nz / 2 + 1;
     const long plane = (long)f.ny * nh, M = (long)n * plane;
-    const int pc = on_device ? n : (int)std::max<size_t>(1, staging_bytes / (plane * sizeof(double2)));
+    const int pc = (int)std::max<size_t>(1, staging_bytes / (plane * sizeof(double2)));
     if (field != 0 && !(field == 1 && f.mhd)) return cudaErrorInvalidValue;
     float2 *a = f.a + field * f.blk_s + (long)run * 3 * f.M;
     const int dealias = f.p[run].dealias;
+    if (on_device) {
+        k_fz_load3<<<dim3((f.My * f.Mz + 255) / 256, f.Mx, 3), 256, 0, s>>>(src, a, half_geom(f), dealias);
+        return cudaGetLastError();
+    }
     cudaError_t e;
     if ((e = cudaMemsetAsync(a, 0, 3 * f.M * sizeof(float2), s)) != cudaSuccess) return e;
     const int ranges[2][2] = {{0, f.K + 1}, {n - f.K, n}};
@@ -1416,18 +1426,14 @@ cudaError_t fused_set_state(FusedRun &f, int run, int field, const double2 *src,
         for (auto &r : ranges) {
             for (int kx0 = r[0]; kx0 < r[1]; kx0 += pc) {
                 const int cnt = std::min(pc, r[1] - kx0);
-                const double2 *p = src + c * M + (long)kx0 * plane;
-                if (!on_device) {
-                    if ((e = cudaMemcpyAsync(staging, p, cnt * plane * sizeof(double2),
-                                             cudaMemcpyHostToDevice, s)) != cudaSuccess)
-                        return e;
-                    p = (const double2 *)staging;
-                }
+                if ((e = cudaMemcpyAsync(staging, src + c * M + (long)kx0 * plane, cnt * plane * sizeof(double2),
+                                         cudaMemcpyHostToDevice, s)) != cudaSuccess)
+                    return e;
                 const long work = (long)cnt * f.My * f.Mz;
-                k_fz_load<<<grid_of(work, 256, 152L * 16), 256, 0, s>>>(p, a + c * f.M, kx0, cnt, half_geom(f),
-                                                                      dealias);
+                k_fz_load<<<grid_of(work, 256, 152L * 16), 256, 0, s>>>((const double2 *)staging, a + c * f.M,
+                                                                      kx0, cnt, half_geom(f), dealias);
                 if ((e = cudaGetLastError()) != cudaSuccess) return e;
-                if (!on_device && (e = cudaStreamSynchronize(s)) != cudaSuccess) return e;
+                if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return e;
             }
         }
     }
@@ -1438,25 +1444,23 @@ cudaError_t fused_get_state(FusedRun &f, int run, int field, double2 *dst, int o
                             size_t staging_bytes, cudaStream_t s) {
     const int n = f.n, nh = f.nz / 2 + 1;
     const long plane = (long)f.ny * nh, M = (long)n * plane;
-    const int pc = on_device ? n : (int)std::max<size_t>(1, staging_bytes / (plane * sizeof(double2)));
+    const int pc = (int)std::max<size_t>(1, staging_bytes / (plane * sizeof(double2)));
     if (field != 0 && !(field == 1 && f.mhd)) return cudaErrorInvalidValue;
     const float2 *a = f.a + field * f.blk_s + (long)run * 3 * f.M;
+    if (on_device) return store3(a, dst, half_geom(f), s);
     cudaError_t e;
     for (int c = 0; c < 3; c++) {
         for (int kx0 = 0; kx0 < n; kx0 += pc) {
             const int cnt = std::min(pc, n - kx0);
             double2 *out = dst + c * M + (long)kx0 * plane;
-            double2 *d = on_device ? out : (double2 *)staging;
+            double2 *d = (double2 *)staging;
             const long work = (long)cnt * plane;
-            k_fz_store<double2><<<grid_of(work, 256, 152L * 16), 256, 0, s>>>(a + c * f.M, d, kx0, cnt,
+            k_fz_store<<<grid_of(work, 256, 152L * 16), 256, 0, s>>>(a + c * f.M, d, kx0, cnt,
                                                                             half_geom(f));
             if ((e = cudaGetLastError()) != cudaSuccess) return e;
-            if (!on_device) {
-                if ((e = cudaMemcpyAsync(out, staging, work * sizeof(double2), cudaMemcpyDeviceToHost,
-                                         s)) != cudaSuccess)
-                    return e;
-                if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return e;
-            }
+            if ((e = cudaMemcpyAsync(out, staging, work * sizeof(double2), cudaMemcpyDeviceToHost, s)) != cudaSuccess)
+                return e;
+            if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return e;
         }
     }
     return cudaSuccess;
@@ -1464,14 +1468,7 @@ cudaError_t fused_get_state(FusedRun &f, int run, int field, double2 *dst, int o
 
 cudaError_t fused_expand(FusedRun &f, int run, int field, float2 *dst, cudaStream_t s) {
     if (field != 0 && !(field == 1 && f.mhd)) return cudaErrorInvalidValue;
-    const float2 *a = f.a + field * f.blk_s + (long)run * 3 * f.M;
-    const long M = (long)f.n * f.ny * (f.nz / 2 + 1);
-    for (int c = 0; c < 3; c++) {
-        k_fz_store<float2><<<grid_of(M, 256, 152L * 16), 256, 0, s>>>(a + c * f.M, dst + c * M, 0, f.n, half_geom(f));
-        cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-    }
-    return cudaSuccess;
+    return store3(f.a + field * f.blk_s + (long)run * 3 * f.M, dst, half_geom(f), s);
 }
 
 cudaError_t fused_spectrum(FusedRun &f, int run, int field, int nbins, double *spec, double *ens,

@@ -129,6 +129,7 @@ struct FusedRun {
     double *part = nullptr;      // [nr][nparts][2]
     double *series = nullptr;    // [nr][cap][2] energy / enstrophy ring buffers
     unsigned long long *counter = nullptr;   // [nr] steps recorded
+    unsigned *ticket = nullptr;              // [nr] blocks of the update that have finished
     int cap = 0;
 };
 

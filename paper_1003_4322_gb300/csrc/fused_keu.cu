@@ -73,11 +73,7 @@ k_fzeu(const float2 *__restrict__ din, float2 *__restrict__ a, float2 *__restric
     if (two) {
         double e = e_acc.value(), o = o_acc.value();
         block_sum2(e, o, red);
-        if (threadIdx.x == 0) {
-            double *pp = part + 2 * ((long)run * u.nparts + blockIdx.x);
-            pp[0] = e;
-            pp[1] = o;
-        }
+        energy_publish(e, o, part + 2L * run * u.nparts, u.nparts, run, blockIdx.x, u.out);
     }
 }
 

@@ -6,6 +6,7 @@
 #pragma once
 #include "fused.h"
 #include "fused_access.cuh"
+#include "reduce.cuh"
 
 namespace nsk {
 
@@ -19,6 +20,7 @@ struct FzUpdate {
     long M;          // compact modes per component
     int nk2;         // entries of one run's factor table
     int nparts;      // partial sums per run
+    EnergyOut out;   // stage 2: where the sums go
     // a grid or a box (fz_update_mode_grid): the y compaction, 1 / (N_x N_y
     // N_z), the wavenumber per grid index 1 / l_i, the sphere in integers
     // (D = lcm N_i, q_i = D / N_i); the factor table is then per axis by

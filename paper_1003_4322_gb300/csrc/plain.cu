@@ -390,14 +390,13 @@ __global__ void k_phase_avg(typename Cx<T>::type *__restrict__ acc, const typena
 
 // ---------------------------------------------------------------- reductions
 
-// Per-block partial energy and enstrophy of a half-layout state, over the
-// rows of the rectangle that holds its nonzero modes: warps take rows in a
+// Energy and enstrophy of a half-layout state, over the rows of the rectangle that holds its nonzero modes: warps take rows in a
 // fixed pattern, a lane sums its modes in order, the block adds up in a fixed
 // tree.  10 FP64 instructions per mode (r2 and 1/2 join once per row): 0.65 ->
 // 0.56 ms at 512^3, 137 -> 75 us at 256^3.
 template <typename T, bool UNIT>
 __global__ void __launch_bounds__(256)
-k_energy_partials(const typename Cx<T>::type *__restrict__ a, Grid g, long M, double *part, Rect rc) {
+k_energy(const typename Cx<T>::type *__restrict__ a, Grid g, long M, double *part, Rect rc, EnergyOut eo) {
     __shared__ double sh[512];
     double e = 0.0, om = 0.0;
     const int lane = threadIdx.x & 31, rows = rect_rows(rc, g), nk = rect_kz(rc, g);
@@ -424,32 +423,7 @@ k_energy_partials(const typename Cx<T>::type *__restrict__ a, Grid g, long M, do
         om += fma(r2, er, zr);
     }
     block_sum2(e, om, sh);
-    if (threadIdx.x == 0) {
-        part[2 * blockIdx.x] = e;
-        part[2 * blockIdx.x + 1] = om;
-    }
-}
-
-// Sum nparts partials in a fixed order, append (E, Omega) to the run's ring
-// buffer series[cap][2] at slot counter % cap, bump the counter, and raise
-// bit 0 of *flags if E is not finite.
-__global__ void __launch_bounds__(256)
-k_energy_final(const double *__restrict__ part, int nparts, double *series, int cap,
-               unsigned long long *counter, int *flags) {
-    __shared__ double sh[512];
-    double e = 0.0, om = 0.0;
-    for (int i = threadIdx.x; i < nparts; i += blockDim.x) {
-        e += part[2 * i];
-        om += part[2 * i + 1];
-    }
-    block_sum2(e, om, sh);
-    if (threadIdx.x == 0) {
-        const unsigned long long c = *counter;
-        series[2 * (c % cap)] = e;
-        series[2 * (c % cap) + 1] = om;
-        *counter = c + 1;
-        if (!isfinite(e)) atomicOr(flags, 1);
-    }
+    energy_publish(e, om, part, gridDim.x, 0, blockIdx.x, eo);
 }
 
 template <typename T> struct HalfAcc {
@@ -626,18 +600,18 @@ cudaError_t plain_update(typename Cx<T>::type *a, typename Cx<T>::type *a1,
 }
 
 int energy_nparts(long M) {
-    long np = (M + 4095) / 4096;
-    if (np > 152 * 4) np = 152 * 4;   // one wave
+    long np = (M + 511) / 512;        // small states: few rows per warp (19 -> 8 us at 32^3)
+    if (np > 152 * 4) np = 152 * 4;   // large ones: one wave
     return (int)(np < 1 ? 1 : np);
 }
 
 template <typename T>
-cudaError_t plain_energy_partials(const typename Cx<T>::type *a, const Grid &g, double *part, const Rect &rc,
-                                  cudaStream_t s) {
+cudaError_t plain_energy(const typename Cx<T>::type *a, const Grid &g, double *part, const Rect &rc,
+                         const EnergyOut &eo, cudaStream_t s) {
     const long M = g.M();
     const int np = energy_nparts(M);
-    if (g.unit) k_energy_partials<T, true><<<np, 256, 0, s>>>(a, g, M, part, rc);
-    else k_energy_partials<T, false><<<np, 256, 0, s>>>(a, g, M, part, rc);
+    if (g.unit) k_energy<T, true><<<np, 256, 0, s>>>(a, g, M, part, rc, eo);
+    else k_energy<T, false><<<np, 256, 0, s>>>(a, g, M, part, rc, eo);
     return cudaGetLastError();
 }
 
@@ -663,12 +637,6 @@ cudaError_t plain_helicity(const typename Cx<T>::type *a, const Grid &g, const R
     return shell_launch(k_grid_spectrum<GridHelAcc<T>>, nbins, spec, aux, s, any, g, nbins);
 }
 
-cudaError_t energy_final(const double *part, int nparts, double *series, int cap,
-                         unsigned long long *counter, int *flags, cudaStream_t s) {
-    k_energy_final<<<1, 256, 0, s>>>(part, nparts, series, cap, counter, flags);
-    return cudaGetLastError();
-}
-
 #define NSK_INST(T)                                                                                \
     template cudaError_t plain_curl<T>(const Cx<T>::type *, Cx<T>::type *, const Grid &, const Rect &,   \
                                        cudaStream_t);                                             \
@@ -684,8 +652,8 @@ cudaError_t energy_final(const double *part, int nparts, double *series, int cap
     template cudaError_t plain_update<T>(Cx<T>::type *, Cx<T>::type *, const Cx<T>::type *,       \
                                          const T *, const Grid &, const UpdateArgs &, const Rect &, \
                                          cudaStream_t);                                           \
-    template cudaError_t plain_energy_partials<T>(const Cx<T>::type *, const Grid &, double *,    \
-                                                  const Rect &, cudaStream_t);                    \
+    template cudaError_t plain_energy<T>(const Cx<T>::type *, const Grid &, double *, const Rect &, \
+                                         const EnergyOut &, cudaStream_t);                        \
     template cudaError_t plain_spectrum<T>(const Cx<T>::type *, const Grid &, const Reach &, int, double *, \
                                            double *, cudaStream_t);                               \
     template cudaError_t plain_helicity<T>(const Cx<T>::type *, const Grid &, const Reach &, int, double *, \

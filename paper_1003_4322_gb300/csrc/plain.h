@@ -25,7 +25,7 @@ struct UpdateArgs {
 
 // rc (the curl, both updates): the rectangle of the half layout outside which
 // the state is zero and which alone the (pruned) transforms read; with rc.on
-// they touch only its modes.  The energy partials take the rectangle of the
+// they touch only its modes.  The energy sums take the rectangle of the
 // kept modes whether or not the transforms are pruned.
 template <typename T>
 cudaError_t plain_curl(const typename Cx<T>::type *a, typename Cx<T>::type *w, const Grid &g, const Rect &rc,
@@ -57,15 +57,13 @@ cudaError_t plain_update(typename Cx<T>::type *a, typename Cx<T>::type *a1,
                          const UpdateArgs &ua, const Rect &rc, cudaStream_t s);
 int energy_nparts(long M);
 template <typename T>
-cudaError_t plain_energy_partials(const typename Cx<T>::type *a, const Grid &g, double *part, const Rect &rc,
-                                  cudaStream_t s);
+cudaError_t plain_energy(const typename Cx<T>::type *a, const Grid &g, double *part, const Rect &rc,
+                         const EnergyOut &eo, cudaStream_t s);
 template <typename T>
 cudaError_t plain_spectrum(const typename Cx<T>::type *a, const Grid &g, const Reach &rc, int nbins, double *spec,
                            double *ens, cudaStream_t s);
 template <typename T>
 cudaError_t plain_helicity(const typename Cx<T>::type *a, const Grid &g, const Reach &rc, int nbins, double *spec,
                            double *aux, cudaStream_t s);
-cudaError_t energy_final(const double *part, int nparts, double *series, int cap,
-                         unsigned long long *counter, int *flags, cudaStream_t s);
 
 }  // namespace nsk

@@ -29,6 +29,59 @@ __device__ __forceinline__ void block_sum2(double &s0, double &s1, double *sh) {
     s1 = sh[1];
 }
 
+// Where a step's energy and enstrophy go: ring buffer series[run][cap][2] at
+// slot counter[run] % cap; ticket[run] counts the blocks that have finished.
+// counter null: nothing is recorded (tuning).
+struct EnergyOut {
+    double *series = nullptr;
+    int cap = 0;
+    unsigned long long *counter = nullptr;
+    unsigned *ticket = nullptr;
+    int *flags = nullptr;   // bit 0: E is not finite
+};
+
+// End of a kernel whose blocks each hold a partial (e, om) in thread 0: the
+// run's last block adds the nparts partials part[block][2] in a fixed order
+// (independent of which block is last) and records them.  One launch less per
+// step than a kernel of its own, which is 4 us of a step of 64^3 (48 us).
+// Every thread of the block calls it; at least one warp.
+__device__ __forceinline__ void energy_publish(double e, double om, double *part, int nparts, int run, int block,
+                                               const EnergyOut &eo) {
+    __shared__ unsigned last;
+    if (threadIdx.x == 0) {
+        part[2 * block] = e;
+        part[2 * block + 1] = om;
+        if (eo.counter) {
+            __threadfence();
+            last = atomicAdd(eo.ticket + run, 1u) == (unsigned)nparts - 1;
+        } else {
+            last = 0;
+        }
+    }
+    __syncthreads();
+    if (!last || threadIdx.x >= 32) return;
+    __threadfence();
+    double s0 = 0.0, s1 = 0.0;
+#pragma unroll 4
+    for (int i = threadIdx.x; i < nparts; i += 32) {
+        s0 += __ldcg(part + 2 * i);
+        s1 += __ldcg(part + 2 * i + 1);
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        s0 += __shfl_down_sync(0xffffffffu, s0, o);
+        s1 += __shfl_down_sync(0xffffffffu, s1, o);
+    }
+    if (threadIdx.x == 0) {
+        const unsigned long long c = eo.counter[run];
+        double *sr = eo.series + 2L * run * eo.cap;
+        sr[2 * (c % eo.cap)] = s0;
+        sr[2 * (c % eo.cap) + 1] = s1;
+        eo.counter[run] = c + 1;
+        eo.ticket[run] = 0;
+        if (!isfinite(s0)) atomicOr(eo.flags, 1);
+    }
+}
+
 // The spectrum kernels leave partial sums after the nbins results in spec and
 // ens, which hold nbins (1 + shell_parts(nbins)) doubles each; a second kernel
 // adds them in a fixed order.  Up to kRowBins shells, k_shell_rows: one block
