@@ -93,8 +93,8 @@ def load_peaks():
 # Kernel sources of each form, for telling whether a committed ncu capture
 # still describes the kernels that run.
 KERNEL_SOURCES = {
-    "fp64": ("fft_core.cuh", "fft_passes.cu", "fft_fix.cuh", "fft_fix_line.cuh", "fft_fix_strided.cu",
-             "fft_fix_z.cu", "plain.cu", "plain.h", "grid.cuh", "reduce.cuh", "api.cu"),
+    "fp64": ("fft_core.cuh", "fft_passes.cu", "fft_fix.cuh", "fft_fix_line.cuh", "fft_fix_strided.cuh",
+             "fft_fix_inv.cu", "fft_fix_fwd.cu", "fft_fix_z.cu", "plain.cu", "plain.h", "grid.cuh", "reduce.cuh", "api.cu"),
     "fp32": ("fft_core.cuh", "fft_ct.cuh", "reduce.cuh", "fused.cu", "fused.h", "fused_access.cuh",
              "fused_s.cuh", "fused_k.cuh", "fused_kA.cu", "fused_kB.cu", "fused_kD.cu",
              "fused_kE.cu", "fused_keu.cu", "fused_update.cuh", "fused_sA.cu", "fused_sB.cu",

@@ -48,6 +48,20 @@ struct FftRes {
     void *scratch = nullptr;  // one half-layout field (c2r)
 };
 
+// Line exponents of the FP64 transforms between their passes: those of x lines
+// or of z lines in a, of y lines in b.
+struct FixBufs {
+    int *a = nullptr, *b = nullptr;
+    static size_t ints(const Grid &g, int ncomp) {   // both, one allocation
+        return a_ints(g, ncomp) + (size_t)ncomp * g.nx * g.nzh();
+    }
+    static size_t a_ints(const Grid &g, int ncomp) {
+        return (size_t)ncomp * std::max(g.ny * g.nzh(), (long)g.nx * g.ny);
+    }
+    FixBufs() = default;
+    FixBufs(int *p, const Grid &g, int ncomp) : a(p), b(p ? p + a_ints(g, ncomp) : nullptr) {}
+};
+
 // The largest |m_i| per axis that a run's dealiasing rule keeps: the plain
 // form's transforms skip the lines beyond them (on = false: every line).
 struct PlainPrune {
@@ -67,6 +81,7 @@ struct Run {
     // plain form (full half layout)
     void *un = nullptr, *u1 = nullptr, *wn = nullptr, *work = nullptr, *phys = nullptr;
     void *sh = nullptr, *sh2 = nullptr;   // phase-shift dealiasing: shifted state, its product
+    int *ftx = nullptr;                   // FP64: line exponents of a transform of three components
     void *phtab = nullptr;                // per-axis shift factors exp(i pi m / N_i)
     void *etab = nullptr;   // exp(-nu k^2 dt), 1/k^2 by integer k^2 (unit boxes), or per axis
     void *etab_b = nullptr; // MHD: exp(-eta k^2 dt); un, u1, wn then hold [u; b] (6 components)
@@ -108,6 +123,8 @@ struct ns_ctx {
                                      // or a grid or box other than the cube)
     void *gscratch = nullptr;        // c2r scratch of the grid transforms
     size_t gscratch_bytes = 0;
+    int *ftx = nullptr;              // line exponents of the standalone FP64 transforms
+    size_t ftx_ints = 0;
     double *bspec = nullptr;         // batched spectra: per run nbins results + partials, twice
     size_t bspec_runs = 0;
     cudaGraphExec_t graph = nullptr;
@@ -260,30 +277,66 @@ static void prune_sels(const Grid &g, const PlainPrune &p, StridedSel *sx, Strid
 }
 
 // One pass along an axis with transform resources f: FP64 in block fixed
-// point (fft_fix.cuh), FP32 in floating point.
+// point (fft_fix.cuh), FP32 in floating point.  io: the FP64 pass's formats.
 template <typename T>
 cudaError_t pass_strided(const FftRes &f, const typename Cx<T>::type *in, typename Cx<T>::type *out, long ncols,
                          long es, long ps, int planes, int dir, const Plan &pl, int ct, cudaStream_t s,
-                         const StridedSel *sel = nullptr, const FixCurl *curl = nullptr) {
+                         const StridedSel *sel, const FixIo &io) {
     if constexpr (std::is_same<T, double>::value)
-        return fix_strided(in, out, ncols, es, ps, ps, planes, dir, f.fixed(pl), ct, s, sel, curl);
+        return fix_strided(in, out, ncols, es, ps, planes, dir, f.fixed(pl), ct, s, sel, io);
     else
         return fft_strided<T>(in, out, ncols, es, ps, ps, planes, dir, pl, (const typename Cx<T>::type *)f.tw, f.n,
                               ct, s, sel);
 }
 template <typename T>
 cudaError_t pass_z_c2r(const FftRes &f, const typename Cx<T>::type *in, T *out, long nlines, const Plan &pl,
-                       cudaStream_t s, int kzk = -1) {
+                       cudaStream_t s, int kzk, const FixBufs &fb, int ny) {
     if constexpr (std::is_same<T, double>::value)
-        if (pl.n == f.n) return fix_z_c2r(in, out, f.n, nlines, f.fixed(pl), s, kzk);
+        if (pl.n == f.n) return fix_z_c2r(in, fb.b, ny, out, f.n, nlines, f.fixed(pl), s, kzk);
     return fft_z_c2r<T>(in, out, f.n, nlines, pl, (const typename Cx<T>::type *)f.tw, s, kzk);
 }
 template <typename T>
 cudaError_t pass_z_r2c(const FftRes &f, const T *in, typename Cx<T>::type *out, long nlines, const Plan &pl,
-                       cudaStream_t s, int kzk = -1) {
+                       cudaStream_t s, int kzk, const FixBufs &fb) {
     if constexpr (std::is_same<T, double>::value)
-        if (pl.n == f.n) return fix_z_r2c(FixProduct{{in}}, out, f.n, nlines, f.fixed(pl), s, kzk);
+        if (pl.n == f.n) return fix_z_r2c(FixProduct{{in}}, out, fb.a, f.n, nlines, f.fixed(pl), s, kzk);
     return fft_z_r2c<T>(in, out, f.n, nlines, pl, (const typename Cx<T>::type *)f.tw, s, kzk);
+}
+// Formats of the strided FP64 passes of a grid (axis 0: x, 1: y): fixed point
+// between the passes, doubles at the ends.  fixed = false: doubles throughout,
+// around a z pass that takes them.
+FixIo fix_io(const Grid &g, int axis, int dir, const FixBufs &fb, bool fixed = true, bool curl = false) {
+    FixIo io;
+    io.nzh = (int)g.nzh();
+    io.ny = g.ny;
+    io.ix = g.ilx;
+    io.iy = g.ily;
+    io.iz = g.ilz;
+    if (!fixed) return io;
+    if (axis == 0 && dir > 0) {          // x lines -> a
+        io.in = curl ? kIoCurl : kIoDouble;
+        io.out = kIoFixed;
+        io.tout = fb.a;
+        return io;
+    }
+    io.in = kIoFixed;
+    io.out = axis == 1 ? kIoFixed : kIoDouble;
+    io.tout = fb.b;                      // y lines -> b
+    io.tin = axis == 1 ? fb.a : fb.b;
+    if (axis == 0) {                     // element x of a column (y, kz): y line (x, kz)
+        io.eps = g.nx * g.nzh();
+        io.estride = (int)g.nzh();
+        io.ecol = 1;
+    } else if (dir > 0) {                // element ky of (x, kz): x line (ky, kz)
+        io.pdiv = g.nx;
+        io.eps = g.ny * g.nzh();
+        io.estride = (int)g.nzh();
+        io.ecol = 1;
+    } else {                             // element y of (x, kz): z line (x, y)
+        io.eps = g.ny;
+        io.estride = 1;
+    }
+    return io;
 }
 // Columns per CTA that the kernels of the precision take for a plan.
 template <typename T> bool ct_fits(const Plan &pl, int ct) {
@@ -300,7 +353,7 @@ template <typename T> bool ct_fits(const Plan &pl, int ct) {
 // curl (FP64, ncomp = 3): the transform of i k x in.
 template <typename T>
 cudaError_t c2r_batch(const typename Cx<T>::type *in, typename Cx<T>::type *tmp, T *out, const Grid &g,
-                      int ncomp, const Fft3 &f, cudaStream_t s, Tracer *tr = nullptr,
+                      int ncomp, const Fft3 &f, cudaStream_t s, const FixBufs &fb, Tracer *tr = nullptr,
                       const PlainPrune *pr = nullptr, bool curl = false) {
     typedef typename Cx<T>::type C;
     if constexpr (std::is_same<T, float>::value) {
@@ -318,45 +371,49 @@ cudaError_t c2r_batch(const typename Cx<T>::type *in, typename Cx<T>::type *tmp,
     const bool pruned = pr && pr->on;
     StridedSel sx, sy;
     if (pruned) prune_sels(g, *pr, &sx, &sy);
-    const FixCurl cu{g.ny, (int)nh, g.ilx, g.ily, g.ilz};
+    const bool fixed = qz.zc.n == g.nz;
     cudaError_t e = NSK_TIMED(tr, curl ? "curl_x_inverse" : "fft_x_inverse",
                               pass_strided<T>(*f.x, in, tmp, plane, plane, M, ncomp, +1, qx.inv, qx.ct_inv, s,
-                                              pruned ? &sx : nullptr, curl ? &cu : nullptr));
+                                              pruned ? &sx : nullptr, fix_io(g, 0, +1, fb, fixed, curl)));
     if (e != cudaSuccess) return e;
     e = NSK_TIMED(tr, "fft_y_inverse",
                   pass_strided<T>(*f.y, tmp, tmp, nh, nh, plane, ncomp * g.nx, +1, qy.inv, qy.ct_inv, s,
-                                  pruned ? &sy : nullptr));
+                                  pruned ? &sy : nullptr, fix_io(g, 1, +1, fb, fixed)));
     if (e != cudaSuccess) return e;
     return NSK_TIMED(tr, "fft_z_c2r",
-                     pass_z_c2r<T>(*f.z, tmp, out, (long)ncomp * g.nx * g.ny, qz.zc, s, pruned ? pr->kz + 1 : -1));
+                     pass_z_c2r<T>(*f.z, tmp, out, (long)ncomp * g.nx * g.ny, qz.zc, s,
+                                   pruned ? pr->kz + 1 : -1, fb, g.ny));
 }
 
 // The vorticity i k x a of three components on the grid: FP64 forms it in the
 // x pass's loads, FP32 in a kernel of its own through w.
 template <typename T>
 cudaError_t c2r_curl(const typename Cx<T>::type *a, typename Cx<T>::type *w, typename Cx<T>::type *tmp, T *out,
-                     const Grid &g, const Rect &rc, const Fft3 &f, cudaStream_t s, Tracer *tr, const PlainPrune *pr) {
-    if (std::is_same<T, double>::value) return c2r_batch<T>(a, tmp, out, g, 3, f, s, tr, pr, true);
+                     const Grid &g, const Rect &rc, const Fft3 &f, cudaStream_t s, const FixBufs &fb, Tracer *tr,
+                     const PlainPrune *pr) {
+    if (std::is_same<T, double>::value && f.pz->zc.n == g.nz)
+        return c2r_batch<T>(a, tmp, out, g, 3, f, s, fb, tr, pr, true);
     const cudaError_t e = NSK_TIMED(tr, "curl", plain_curl<T>(a, w, g, rc, s));
-    return e != cudaSuccess ? e : c2r_batch<T>(w, tmp, out, g, 3, f, s, tr, pr);
+    return e != cudaSuccess ? e : c2r_batch<T>(w, tmp, out, g, 3, f, s, fb, tr, pr);
 }
 
 // The y and x passes of r2c, in place.
 template <typename T>
-cudaError_t r2c_yx(typename Cx<T>::type *out, const Grid &g, int ncomp, const Fft3 &f, cudaStream_t s, Tracer *tr,
-                   const PlainPrune *pr) {
+cudaError_t r2c_yx(typename Cx<T>::type *out, const Grid &g, int ncomp, const Fft3 &f, cudaStream_t s,
+                   const FixBufs &fb, Tracer *tr, const PlainPrune *pr) {
     const long nh = g.nzh(), plane = (long)g.ny * nh, M = (long)g.nx * plane;
     const PlainPlans &qx = *f.px, &qy = *f.py;
-    const bool pruned = pr && pr->on;
+    const bool pruned = pr && pr->on, fixed = f.pz->zr.n == g.nz;
     StridedSel sx, sy;
     if (pruned) prune_sels(g, *pr, &sx, &sy);
     const cudaError_t e = NSK_TIMED(tr, "fft_y_forward",
                                     pass_strided<T>(*f.y, out, out, nh, nh, plane, ncomp * g.nx, -1, qy.fwd,
-                                                    qy.ct_fwd, s, pruned ? &sy : nullptr));
+                                                    qy.ct_fwd, s, pruned ? &sy : nullptr,
+                                                    fix_io(g, 1, -1, fb, fixed)));
     if (e != cudaSuccess) return e;
     return NSK_TIMED(tr, "fft_x_forward",
                      pass_strided<T>(*f.x, out, out, plane, plane, M, ncomp, -1, qx.fwd, qx.ct_fwd, s,
-                                     pruned ? &sx : nullptr));
+                                     pruned ? &sx : nullptr, fix_io(g, 0, -1, fb, fixed)));
 }
 
 // r2c of ncomp real fields: z pass (in -> out), y and x passes in place.
@@ -364,7 +421,7 @@ cudaError_t r2c_yx(typename Cx<T>::type *out, const Grid &g, int ncomp, const Ff
 // partly transformed or untouched.
 template <typename T>
 cudaError_t r2c_batch(const T *in, typename Cx<T>::type *out, const Grid &g, int ncomp, const Fft3 &f,
-                      cudaStream_t s, Tracer *tr = nullptr, const PlainPrune *pr = nullptr) {
+                      cudaStream_t s, const FixBufs &fb, Tracer *tr = nullptr, const PlainPrune *pr = nullptr) {
     if constexpr (std::is_same<T, float>::value) {
         cudaError_t e = cudaSuccess;
         if (tr) tr->begin("fft_r2c_std");
@@ -374,8 +431,8 @@ cudaError_t r2c_batch(const T *in, typename Cx<T>::type *out, const Grid &g, int
     }
     const cudaError_t e = NSK_TIMED(tr, "fft_z_r2c",
                                     pass_z_r2c<T>(*f.z, in, out, (long)ncomp * g.nx * g.ny, f.pz->zr, s,
-                                                  pr && pr->on ? pr->kz + 1 : -1));
-    return e != cudaSuccess ? e : r2c_yx<T>(out, g, ncomp, f, s, tr, pr);
+                                                  pr && pr->on ? pr->kz + 1 : -1, fb));
+    return e != cudaSuccess ? e : r2c_yx<T>(out, g, ncomp, f, s, fb, tr, pr);
 }
 
 // r2c of the products u x w (and, with j, u x w + j x b): FP64 forms them in
@@ -383,23 +440,23 @@ cudaError_t r2c_batch(const T *in, typename Cx<T>::type *out, const Grid &g, int
 // transform of its result.
 template <typename T>
 cudaError_t r2c_cross(T *u, const T *w, typename Cx<T>::type *out, const Grid &g, const Fft3 &f, cudaStream_t s,
-                      Tracer *tr, const PlainPrune *pr) {
+                      const FixBufs &fb, Tracer *tr, const PlainPrune *pr) {
     if constexpr (std::is_same<T, double>::value)
         if (f.pz->zr.n == g.nz) {
             const FixProduct p{{u, w}, g.V(), 1};
             const cudaError_t e = NSK_TIMED(tr, "cross_z_r2c",
-                                            fix_z_r2c(p, out, g.nz, 3L * g.nx * g.ny, f.z->fixed(f.pz->zr), s,
+                                            fix_z_r2c(p, out, fb.a, g.nz, 3L * g.nx * g.ny, f.z->fixed(f.pz->zr), s,
                                                       pr && pr->on ? pr->kz + 1 : -1));
-            return e != cudaSuccess ? e : r2c_yx<T>(out, g, 3, f, s, tr, pr);
+            return e != cudaSuccess ? e : r2c_yx<T>(out, g, 3, f, s, fb, tr, pr);
         }
     const cudaError_t e = NSK_TIMED(tr, "cross", plain_cross<T>(u, w, g, s));
-    return e != cudaSuccess ? e : r2c_batch<T>(u, out, g, 3, f, s, tr, pr);
+    return e != cudaSuccess ? e : r2c_batch<T>(u, out, g, 3, f, s, fb, tr, pr);
 }
 
 // The same for MHD: phys = [u, w, b, j] -> nu = r2c(u x w + j x b), nb = r2c(u x b).
 template <typename T>
 cudaError_t r2c_cross_mhd(T *phys, typename Cx<T>::type *nu, typename Cx<T>::type *nb, const Grid &g, const Fft3 &f,
-                          cudaStream_t s, Tracer *tr, const PlainPrune *pr) {
+                          cudaStream_t s, const FixBufs &fb, Tracer *tr, const PlainPrune *pr) {
     const long V3 = 3 * g.V();
     cudaError_t e;
     if constexpr (std::is_same<T, double>::value)
@@ -409,15 +466,15 @@ cudaError_t r2c_cross_mhd(T *phys, typename Cx<T>::type *nu, typename Cx<T>::typ
             typename Cx<T>::type *out[2] = {nu, nb};
             for (int i = 0; i < 2; i++) {
                 e = NSK_TIMED(tr, i ? "cross_z_r2c" : "cross2_z_r2c",
-                              fix_z_r2c(p[i], out[i], g.nz, 3L * g.nx * g.ny, f.z->fixed(f.pz->zr), s,
+                              fix_z_r2c(p[i], out[i], fb.a, g.nz, 3L * g.nx * g.ny, f.z->fixed(f.pz->zr), s,
                                         pr && pr->on ? pr->kz + 1 : -1));
-                if (e != cudaSuccess || (e = r2c_yx<T>(out[i], g, 3, f, s, tr, pr)) != cudaSuccess) return e;
+                if (e != cudaSuccess || (e = r2c_yx<T>(out[i], g, 3, f, s, fb, tr, pr)) != cudaSuccess) return e;
             }
             return cudaSuccess;
         }
     e = NSK_TIMED(tr, "cross_mhd", plain_cross_mhd<T>(phys, g, s));
-    if (e != cudaSuccess || (e = r2c_batch<T>(phys, nu, g, 3, f, s, tr, pr)) != cudaSuccess) return e;
-    return r2c_batch<T>(phys + V3, nb, g, 3, f, s, tr, pr);
+    if (e != cudaSuccess || (e = r2c_batch<T>(phys, nu, g, 3, f, s, fb, tr, pr)) != cudaSuccess) return e;
+    return r2c_batch<T>(phys + V3, nb, g, 3, f, s, fb, tr, pr);
 }
 
 // The transforms of a run: the resources of its axis lengths with their plans
@@ -640,11 +697,12 @@ template <typename T> static bool z_candidate(int zmode, bool paired) {
 // products u x w, on the fields at phys and phys + V3.
 template <typename T>
 static cudaError_t tune_r2c(const FftRes &f, const T *phys, long V3, typename Cx<T>::type *out, long lines,
-                            const Plan &pl, cudaStream_t s) {
+                            const Plan &pl, cudaStream_t s, int kzk, const FixBufs &fb) {
     if constexpr (std::is_same<T, double>::value)
         if (pl.n == f.n)
-            return fix_z_r2c(FixProduct{{phys, phys + V3}, V3 / 3, 1}, out, f.n, lines, f.fixed(pl), s);
-    return pass_z_r2c<T>(f, phys, out, lines, pl, s);
+            return fix_z_r2c(FixProduct{{phys, phys + V3}, V3 / 3, 1}, out, fb.a, f.n, lines, f.fixed(pl), s,
+                             kzk);
+    return pass_z_r2c<T>(f, phys, out, lines, pl, s, kzk, fb);
 }
 
 template <typename T> ns_status tune_plain(ns_ctx *c, Run &r, FftRes *f) {
@@ -672,6 +730,10 @@ template <typename T> ns_status tune_plain(ns_ctx *c, Run &r, FftRes *f) {
     cudaStream_t s = c->stream;
     C *in = (C *)r.un, *tmp = (C *)r.work, *half = (C *)r.wn;
     T *phys = (T *)r.phys;
+    const FixBufs fb(r.ftx, r.g, 3);
+    StridedSel sx, sy;
+    prune_sels(r.g, r.prune, &sx, &sy);
+    const int kzk = std::is_same<T, double>::value && r.prune.on ? r.prune.kz + 1 : -1;
     PlainPlans best = f->pp;
     float bi = -1.f, bf = -1.f, bc = -1.f, br = -1.f;
     const int Es[] = {16, 12, 9, 8, 6, 4};
@@ -680,13 +742,26 @@ template <typename T> ns_status tune_plain(ns_ctx *c, Run &r, FftRes *f) {
         if (make_plan_e(n, E, &pl) && pl.nst <= 4) {
             for (int ct = 2; ct <= 32; ct *= 2) {
                 if (!ct_fits<T>(pl, ct)) continue;
-                const float ti = plain_time([&]() {
-                    return pass_strided<T>(*f, in, tmp, plane, plane, M, 3, +1, pl, ct, s);
-                }, s);
+                // One shape serves the x and the y passes of a direction.  FP64 times
+                // them as the step runs them: on the pruned lines, the x pass of
+                // the velocity and of the vorticity and the y pass of both.
+                auto both = [&](const C *src, C *dst, int dir) {
+                    if (!std::is_same<T, double>::value)
+                        return pass_strided<T>(*f, src, dst, plane, plane, M, 3, dir, pl, ct, s, nullptr, FixIo());
+                    const StridedSel *px = r.prune.on ? &sx : nullptr, *py = r.prune.on ? &sy : nullptr;
+                    cudaError_t e = cudaSuccess;
+                    for (int i = 0; i < (dir > 0 ? 2 : 1) && e == cudaSuccess; i++) {
+                        e = pass_strided<T>(*f, src, dst, plane, plane, M, 3, dir, pl, ct, s, px,
+                                            fix_io(r.g, 0, dir, fb, true, i == 1));
+                        if (e == cudaSuccess)
+                            e = pass_strided<T>(*f, dst, dst, nh, nh, plane, 3 * n, dir, pl, ct, s, py,
+                                                fix_io(r.g, 1, dir, fb));
+                    }
+                    return e;
+                };
+                const float ti = plain_time([&]() { return both(in, tmp, +1); }, s);
                 if (ti > 0.f && (bi < 0.f || ti < bi)) { bi = ti; best.inv = pl; best.ct_inv = ct; }
-                const float tf = plain_time([&]() {
-                    return pass_strided<T>(*f, half, half, plane, plane, M, 3, -1, pl, ct, s);
-                }, s);
+                const float tf = plain_time([&]() { return both(half, half, -1); }, s);
                 if (tf > 0.f && (bf < 0.f || tf < bf)) { bf = tf; best.fwd = pl; best.ct_fwd = ct; }
             }
         }
@@ -696,9 +771,9 @@ template <typename T> ns_status tune_plain(ns_ctx *c, Run &r, FftRes *f) {
             Plan ph;
             if (!z_candidate<T>(zmode, len == n)) continue;
             if (!make_plan_e(len, E, &ph) || ph.nst > 4) continue;
-            const float tc = plain_time([&]() { return pass_z_c2r<T>(*f, tmp, phys, lines, ph, s); }, s);
+            const float tc = plain_time([&]() { return pass_z_c2r<T>(*f, tmp, phys, lines, ph, s, kzk, fb, n); }, s);
             if (tc > 0.f && (bc < 0.f || tc < bc)) { bc = tc; best.zc = ph; }
-            const float tr = plain_time([&]() { return tune_r2c<T>(*f, phys, V3, half, lines, ph, s); }, s);
+            const float tr = plain_time([&]() { return tune_r2c<T>(*f, phys, V3, half, lines, ph, s, kzk, fb); }, s);
             if (tr > 0.f && (br < 0.f || tr < br)) { br = tr; best.zr = ph; }
         }
     }
@@ -737,12 +812,24 @@ template <typename T> ns_status tune_plain_grid(ns_ctx *c, Run &r, FftRes *f[3])
     C *in = (C *)r.un, *tmp = (C *)r.work, *half = (C *)r.wn;
     T *phys = (T *)r.phys;
     const int Es[] = {16, 12, 9, 8, 6, 4};
+    const FixBufs fb(r.ftx, g, 3);
+    StridedSel sx, sy;
+    prune_sels(g, r.prune, &sx, &sy);
+    const int kzk = std::is_same<T, double>::value && r.prune.on ? r.prune.kz + 1 : -1;
     for (int a = 0; a < 3; a++) r.gp[a] = f[a]->pp;
     for (int a = 0; a < 2; a++) {   // x pass, y pass
         const int n = a == 0 ? g.nx : g.ny;
         auto pass = [&](const C *src, C *dst, int dir, const Plan &pl, int ct) {
-            return a == 0 ? pass_strided<T>(*f[a], src, dst, plane, plane, M, 3, dir, pl, ct, s)
-                          : pass_strided<T>(*f[a], src, dst, nh, nh, plane, 3 * g.nx, dir, pl, ct, s);
+            // FP64 as the step runs them (see tune_plain)
+            const bool dbl = std::is_same<T, double>::value;
+            const StridedSel *sel = dbl && r.prune.on ? (a == 0 ? &sx : &sy) : nullptr;
+            cudaError_t e = cudaSuccess;
+            for (int i = 0; i < (a == 0 && dir > 0 && dbl ? 2 : 1) && e == cudaSuccess; i++) {
+                const FixIo io = fix_io(g, a, dir, fb, true, i == 1);
+                e = a == 0 ? pass_strided<T>(*f[a], src, dst, plane, plane, M, 3, dir, pl, ct, s, sel, io)
+                           : pass_strided<T>(*f[a], src, dst, nh, nh, plane, 3 * g.nx, dir, pl, ct, s, sel, io);
+            }
+            return e;
         };
         PlainPlans &best = r.gp[a];
         float bi = -1.f, bf = -1.f;
@@ -766,9 +853,9 @@ template <typename T> ns_status tune_plain_grid(ns_ctx *c, Run &r, FftRes *f[3])
                 Plan ph;
                 if (!z_candidate<T>(zmode, len == g.nz)) continue;
                 if (!make_plan_e(len, E, &ph) || ph.nst > 4) continue;
-                const float tc = plain_time([&]() { return pass_z_c2r<T>(*f[2], tmp, phys, lines, ph, s); }, s);
+                const float tc = plain_time([&]() { return pass_z_c2r<T>(*f[2], tmp, phys, lines, ph, s, kzk, fb, g.ny); }, s);
                 if (tc > 0.f && (bc < 0.f || tc < bc)) { bc = tc; best.zc = ph; }
-                const float tr = plain_time([&]() { return tune_r2c<T>(*f[2], phys, V3, half, lines, ph, s); }, s);
+                const float tr = plain_time([&]() { return tune_r2c<T>(*f[2], phys, V3, half, lines, ph, s, kzk, fb); }, s);
                 if (tr > 0.f && (br < 0.f || tr < br)) { br = tr; best.zr = ph; }
             }
     }
@@ -811,6 +898,10 @@ template <typename T> ns_status plain_alloc(ns_ctx *c, Run &r) {
     NS_CK(dalloc(&r.u1, nc * half));
     NS_CK(dalloc(&r.wn, nc * half));
     NS_CK(dalloc(&r.work, 3 * half));
+    if (std::is_same<T, double>::value) {
+        NS_CK(dalloc(&r.ftx, FixBufs::ints(r.g, 3) * sizeof(int)));
+        NS_CK(cudaMemsetAsync(r.ftx, 0, FixBufs::ints(r.g, 3) * sizeof(int), c->stream));
+    }
     NS_CK(dalloc(&r.phys, 2 * nc * real));
     if (r.p.dealias == 2) {
         NS_CK(dalloc(&r.sh, 3 * half));
@@ -881,8 +972,8 @@ template <typename T> ns_status plain_alloc(ns_ctx *c, Run &r) {
         // choose the standalone kernels' shapes now, outside any graph capture
         // (on the run's own buffers, whose contents the first step overwrites)
         const Fft3 f3 = run_fft3(r, f);
-        NS_CK(r2c_batch<T>((const T *)r.phys, (C *)r.wn, r.g, 3, f3, c->stream));
-        NS_CK(c2r_batch<T>((const C *)r.wn, (C *)r.work, (T *)r.phys, r.g, 3, f3, c->stream));
+        NS_CK(r2c_batch<T>((const T *)r.phys, (C *)r.wn, r.g, 3, f3, c->stream, FixBufs()));
+        NS_CK(c2r_batch<T>((const C *)r.wn, (C *)r.work, (T *)r.phys, r.g, 3, f3, c->stream, FixBufs()));
         NS_CK(cudaStreamSynchronize(c->stream));
     }
     return NS_OK;
@@ -911,6 +1002,7 @@ template <typename T> ns_status plain_step(ns_ctx *c, Run &r, cudaStream_t s, Tr
     const Fft3 f = run_fft3(r, fr);
     const Grid &g = r.g;
     T *phys = (T *)r.phys;
+    const FixBufs fb(r.ftx, g, 3);
     const long M3 = 3 * r.M, V3 = 3 * r.V;
     // the pointwise kernels may skip the modes outside the kept rectangle only
     // where every transform that reads their output is pruned: the FP64 path
@@ -921,11 +1013,11 @@ template <typename T> ns_status plain_step(ns_ctx *c, Run &r, cudaStream_t s, Tr
         // grid -> u x w + j x b, u x b -> their transforms -> the two updates
         C *src = (C *)(stage == 1 ? r.un : r.u1);
         C *wj = (C *)r.wn;
-        NS_CK(c2r_batch<T>(src, (C *)r.work, phys, g, 3, f, s, tr, &r.prune));
-        NS_CK(c2r_curl<T>(src, wj, (C *)r.work, phys + V3, g, rc, f, s, tr, &r.prune));
-        NS_CK(c2r_batch<T>(src + M3, (C *)r.work, phys + 2 * V3, g, 3, f, s, tr, &r.prune));
-        NS_CK(c2r_curl<T>(src + M3, wj + M3, (C *)r.work, phys + 3 * V3, g, rc, f, s, tr, &r.prune));
-        NS_CK(r2c_cross_mhd<T>(phys, wj, wj + M3, g, f, s, tr, &r.prune));
+        NS_CK(c2r_batch<T>(src, (C *)r.work, phys, g, 3, f, s, fb, tr, &r.prune));
+        NS_CK(c2r_curl<T>(src, wj, (C *)r.work, phys + V3, g, rc, f, s, fb, tr, &r.prune));
+        NS_CK(c2r_batch<T>(src + M3, (C *)r.work, phys + 2 * V3, g, 3, f, s, fb, tr, &r.prune));
+        NS_CK(c2r_curl<T>(src + M3, wj + M3, (C *)r.work, phys + 3 * V3, g, rc, f, s, fb, tr, &r.prune));
+        NS_CK(r2c_cross_mhd<T>(phys, wj, wj + M3, g, f, s, fb, tr, &r.prune));
         const UpdateArgs ua = update_args(r, stage);
         NS_CK(NSK_TIMED(tr, "update",
                         plain_update<T>((C *)r.un, (C *)r.u1, (const C *)wj, (const T *)r.etab, g, ua, rc, s)));
@@ -936,15 +1028,15 @@ template <typename T> ns_status plain_step(ns_ctx *c, Run &r, cudaStream_t s, Tr
     }
     for (int stage = 1; stage <= 2 && !r.p.mhd; stage++) {
         C *src = (C *)(stage == 1 ? r.un : r.u1);
-        NS_CK(c2r_batch<T>(src, (C *)r.work, phys, g, 3, f, s, tr, &r.prune));
-        NS_CK(c2r_curl<T>(src, (C *)r.wn, (C *)r.work, phys + 3 * r.V, g, rc, f, s, tr, &r.prune));
-        NS_CK(r2c_cross<T>(phys, phys + 3 * r.V, (C *)r.wn, g, f, s, tr, &r.prune));
+        NS_CK(c2r_batch<T>(src, (C *)r.work, phys, g, 3, f, s, fb, tr, &r.prune));
+        NS_CK(c2r_curl<T>(src, (C *)r.wn, (C *)r.work, phys + 3 * r.V, g, rc, f, s, fb, tr, &r.prune));
+        NS_CK(r2c_cross<T>(phys, phys + 3 * r.V, (C *)r.wn, g, f, s, fb, tr, &r.prune));
         if (r.p.dealias == 2) {   // the same on the grid shifted by half a spacing, averaged
             C *sh = (C *)r.sh, *sh2 = (C *)r.sh2;
             NS_CK(NSK_TIMED(tr, "phase", plain_phase<T>(src, sh, (const C *)r.phtab, g, s)));
-            NS_CK(c2r_batch<T>(sh, (C *)r.work, phys, g, 3, f, s, tr, &r.prune));
-            NS_CK(c2r_curl<T>(sh, sh2, (C *)r.work, phys + 3 * r.V, g, rc, f, s, tr, &r.prune));
-            NS_CK(r2c_cross<T>(phys, phys + 3 * r.V, sh2, g, f, s, tr, &r.prune));
+            NS_CK(c2r_batch<T>(sh, (C *)r.work, phys, g, 3, f, s, fb, tr, &r.prune));
+            NS_CK(c2r_curl<T>(sh, sh2, (C *)r.work, phys + 3 * r.V, g, rc, f, s, fb, tr, &r.prune));
+            NS_CK(r2c_cross<T>(phys, phys + 3 * r.V, sh2, g, f, s, fb, tr, &r.prune));
             NS_CK(NSK_TIMED(tr, "phase", plain_phase_avg<T>((C *)r.wn, sh2, (const C *)r.phtab, g, s)));
         }
         const UpdateArgs ua = update_args(r, stage);
@@ -1029,7 +1121,7 @@ ns_status build_graph(ns_ctx *c) {
 }
 
 void free_run(Run &r) {
-    void *ps[] = {r.un, r.u1, r.wn, r.work, r.phys, r.etab, r.etab_b, r.sh, r.sh2, r.phtab};
+    void *ps[] = {r.un, r.u1, r.wn, r.work, r.ftx, r.phys, r.etab, r.etab_b, r.sh, r.sh2, r.phtab};
     for (void *p : ps)
         if (p) dev_free(p);
     if (r.owns_diag) {
@@ -1066,6 +1158,56 @@ ns_status check_flags(ns_ctx *c) {
     if (h & 2) return NS_ERR_TIMEOUT;
     if (h & 1) return NS_ERR_NONFINITE;
     return NS_OK;
+}
+
+// Line exponents for up to kFtxComp components of a standalone FP64 transform,
+// grown to the largest grid asked for.  Where they cannot be had (the stream is
+// being captured, or no memory is left), the transform keeps doubles between
+// its passes around the one-line z passes, which need none: *f3 then takes
+// `plain` for the z axis.
+const int kFtxComp = 3;
+FixBufs standalone_bufs(ns_ctx *c, const Grid &g, Fft3 *f3, PlainPlans *plain) {
+    const size_t need = FixBufs::ints(g, kFtxComp);
+    if (c->ftx_ints < need) {
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusActive;
+        int *p = nullptr;
+        if (cudaStreamIsCapturing(c->stream, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone &&
+            cudaStreamSynchronize(c->stream) == cudaSuccess && dalloc(&p, need * sizeof(int)) == cudaSuccess) {
+            if (c->ftx) dev_free(c->ftx);
+            c->ftx = p;
+            c->ftx_ints = need;
+        } else {
+            (void)cudaGetLastError();
+            *plain = *f3->pz;
+            plain->zc = plain->zr = f3->z->plH;
+            f3->pz = plain;
+            return FixBufs();
+        }
+    }
+    return FixBufs(c->ftx, g, kFtxComp);
+}
+
+// r2c of any number of components, kFtxComp at a time.
+cudaError_t standalone_r2c(ns_ctx *c, const double *in, double2 *out, const Grid &g, int ncomp, Fft3 f3) {
+    PlainPlans plain;
+    const FixBufs fb = standalone_bufs(c, g, &f3, &plain);
+    for (int k = 0; k < ncomp; k += kFtxComp) {
+        const cudaError_t e = r2c_batch<double>(in + k * g.V(), out + k * g.M(), g, std::min(kFtxComp, ncomp - k), f3,
+                                                c->stream, fb);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
+// c2r through tmp, one component at a time.
+cudaError_t standalone_c2r(ns_ctx *c, const double2 *in, double2 *tmp, double *out, const Grid &g, int ncomp, Fft3 f3) {
+    PlainPlans plain;
+    const FixBufs fb = standalone_bufs(c, g, &f3, &plain);
+    for (int k = 0; k < ncomp; k++) {
+        const cudaError_t e = c2r_batch<double>(in + k * g.M(), tmp, out + k * g.V(), g, 1, f3, c->stream, fb);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 }  // namespace
@@ -1273,6 +1415,7 @@ void ns_destroy(ns_ctx *c) {
     if (c->spec) dev_free(c->spec);
     if (c->staging) dev_free(c->staging);
     if (c->gscratch) dev_free(c->gscratch);
+    if (c->ftx) dev_free(c->ftx);
     if (c->bspec) dev_free(c->bspec);
     if (c->cap) cudaStreamDestroy(c->cap);
     for (cudaStream_t q : c->par) cudaStreamDestroy(q);
@@ -1380,13 +1523,13 @@ ns_status ns_fft_r2c(ns_ctx *c, int n, int ncomp, const void *in, void *out) {
     const Grid g = make_grid(n, n, n, 1.0, 1.0, 1.0);
     const Fft3 f3{f, f, f, &f->pp, &f->pp, &f->pp};
     if (c->prec == NS_FP64) {
-        NS_CK(r2c_batch<double>((const double *)in, (double2 *)out, g, ncomp, f3, c->stream));
+        NS_CK(standalone_r2c(c, (const double *)in, (double2 *)out, g, ncomp, f3));
     } else {
         cudaError_t e = cudaSuccess;
         if (std_r2c_fp32((const float *)in, (float2 *)out, n, ncomp, (const float2 *)f->tw, c->stream, &e))
             NS_CK(e);
         else
-            NS_CK(r2c_batch<float>((const float *)in, (float2 *)out, g, ncomp, f3, c->stream));
+            NS_CK(r2c_batch<float>((const float *)in, (float2 *)out, g, ncomp, f3, c->stream, FixBufs()));
     }
     return NS_OK;
 }
@@ -1402,19 +1545,18 @@ ns_status ns_fft_c2r(ns_ctx *c, int n, int ncomp, const void *in, void *out) {
     const Grid g = make_grid(n, n, n, 1.0, 1.0, 1.0);
     const Fft3 f3{f, f, f, &f->pp, &f->pp, &f->pp};
     const long M = g.M(), V = g.V();
+    if (c->prec == NS_FP64) {
+        NS_CK(standalone_c2r(c, (const double2 *)in, (double2 *)f->scratch, (double *)out, g, ncomp, f3));
+        return NS_OK;
+    }
     for (int k = 0; k < ncomp; k++) {
-        if (c->prec == NS_FP64)
-            NS_CK(c2r_batch<double>((const double2 *)in + k * M, (double2 *)f->scratch,
-                                    (double *)out + k * V, g, 1, f3, c->stream));
-        else {
-            cudaError_t e = cudaSuccess;
-            if (std_c2r_fp32((const float2 *)in + k * M, (float2 *)f->scratch, (float *)out + k * V, n,
-                             (const float2 *)f->tw, c->stream, &e))
-                NS_CK(e);
-            else
-                NS_CK(c2r_batch<float>((const float2 *)in + k * M, (float2 *)f->scratch,
-                                       (float *)out + k * V, g, 1, f3, c->stream));
-        }
+        cudaError_t e = cudaSuccess;
+        if (std_c2r_fp32((const float2 *)in + k * M, (float2 *)f->scratch, (float *)out + k * V, n,
+                         (const float2 *)f->tw, c->stream, &e))
+            NS_CK(e);
+        else
+            NS_CK(c2r_batch<float>((const float2 *)in + k * M, (float2 *)f->scratch, (float *)out + k * V, g, 1, f3,
+                                   c->stream, FixBufs()));
     }
     return NS_OK;
 }
@@ -1436,7 +1578,7 @@ ns_status ns_fft_r2c_grid(ns_ctx *c, int nx, int ny, int nz, int ncomp, const vo
     ns_status st = grid_fft_args(c, nx, ny, nz, ncomp, in, out, &g, &f3);
     if (st != NS_OK) return st;
     if (c->prec == NS_FP64) {
-        NS_CK(r2c_batch<double>((const double *)in, (double2 *)out, g, ncomp, f3, c->stream));
+        NS_CK(standalone_r2c(c, (const double *)in, (double2 *)out, g, ncomp, f3));
     } else {
         const StdGrid sg{nx, ny, nz, (const float2 *)f3.x->tw, (const float2 *)f3.y->tw,
                          (const float2 *)f3.z->tw};
@@ -1444,7 +1586,7 @@ ns_status ns_fft_r2c_grid(ns_ctx *c, int nx, int ny, int nz, int ncomp, const vo
         if (std_r2c_fp32_grid((const float *)in, (float2 *)out, sg, ncomp, c->stream, &e))
             NS_CK(e);
         else
-            NS_CK(r2c_batch<float>((const float *)in, (float2 *)out, g, ncomp, f3, c->stream));
+            NS_CK(r2c_batch<float>((const float *)in, (float2 *)out, g, ncomp, f3, c->stream, FixBufs()));
     }
     return NS_OK;
 }
@@ -1465,19 +1607,18 @@ ns_status ns_fft_c2r_grid(ns_ctx *c, int nx, int ny, int nz, int ncomp, const vo
     }
     const long M = g.M(), V = g.V();
     const StdGrid sg{nx, ny, nz, (const float2 *)f3.x->tw, (const float2 *)f3.y->tw, (const float2 *)f3.z->tw};
+    if (c->prec == NS_FP64) {
+        NS_CK(standalone_c2r(c, (const double2 *)in, (double2 *)c->gscratch, (double *)out, g, ncomp, f3));
+        return NS_OK;
+    }
     for (int k = 0; k < ncomp; k++) {
-        if (c->prec == NS_FP64) {
-            NS_CK(c2r_batch<double>((const double2 *)in + k * M, (double2 *)c->gscratch, (double *)out + k * V,
-                                    g, 1, f3, c->stream));
-        } else {
-            cudaError_t e = cudaSuccess;
-            if (std_c2r_fp32_grid((const float2 *)in + k * M, (float2 *)c->gscratch, (float *)out + k * V, sg,
-                                  c->stream, &e))
-                NS_CK(e);
-            else
-                NS_CK(c2r_batch<float>((const float2 *)in + k * M, (float2 *)c->gscratch, (float *)out + k * V,
-                                       g, 1, f3, c->stream));
-        }
+        cudaError_t e = cudaSuccess;
+        if (std_c2r_fp32_grid((const float2 *)in + k * M, (float2 *)c->gscratch, (float *)out + k * V, sg, c->stream,
+                              &e))
+            NS_CK(e);
+        else
+            NS_CK(c2r_batch<float>((const float2 *)in + k * M, (float2 *)c->gscratch, (float *)out + k * V, g, 1, f3,
+                                   c->stream, FixBufs()));
     }
     return NS_OK;
 }

@@ -10,7 +10,7 @@
 // factors, so one power-of-two scale per line serves every intermediate value,
 // and 63 bits under that scale are more than the 53 of a double.  At 512^3
 // (three components) the passes went from 11.5 / 6.7 / 4.5 ms (z c2r, y, x)
-// in FP64 to 2.4 / 1.6 / 1.1 ms, bound by integer instruction issue.
+// in FP64 to 2.35 / 1.44 / 0.98 ms, bound by integer instruction issue.
 //
 // The scale: with S >= sum |x_j| over the line, every sub-transform of every
 // stage is bounded by S in modulus (it is a sum of x_j times unit factors), so

@@ -73,12 +73,21 @@ template <class Op> NSK_DEV unsigned line_reduce(unsigned v, const LineGeo &g, u
     return v;
 }
 
-// Scale of one line: `top` (fix_from) and, for lines outside the range of the
-// FP32 sum (odd), a factor that the results are multiplied by.
+// Between the passes of a transform values stay in fixed point: 64-bit
+// integers v with one exponent t per line, value = v 2^(t - 1085) (t is the
+// biased double exponent of bit 62).  That saves a conversion to double (23
+// instructions a value) at the end of one pass and one from it (17, and the
+// line sum) at the start of the next, for shifts, and two roundings to 53 bits
+// (512^3: x inverse 1.10 -> 0.98 ms, y inverse 1.60 -> 1.44, r2c with products
+// 2.84 -> 2.49, y forward 1.52 -> 1.32).  kZeroT: a line of zeros; kNanT: a line with a NaN or an
+// infinity; both stay beyond +-kEdgeT through the small steps the passes add.
+constexpr int kZeroT = -(1 << 20), kNanT = 1 << 20, kEdgeT = 1 << 19;
+
+// Scale of a line read as doubles: `top` for fix_from (of the entries, which
+// line_scale has multiplied by a power of two if the line lies outside the
+// range of the FP32 sum) and the line's t.
 struct LineScale {
-    int top;
-    bool any;    // some line of the CTA is odd
-    double mul;  // 1 for the others
+    int top, t;
 };
 
 // The raw value x times the power of two f (a line outside the FP32 range).
@@ -109,16 +118,15 @@ NSK_DEV LineScale line_scale(L2 (&v)[NV], const LineGeo &g, unsigned *sh, Skip s
     unsigned mx = 0;
     float S = __uint_as_float(line_reduce<OpAdd>(__float_as_uint(sum(mx)), g, sh));
     const bool odd = S != 0.f && !(S >= NSK_FIX_LOW && S <= NSK_FIX_HIGH);
-    LineScale r{0, __syncthreads_or(odd) != 0, 1.0};
-    if (r.any) {
+    LineScale r{0, 0};
+    if (__syncthreads_or(odd)) {
         const unsigned lm = line_reduce<OpMax>(mx, g, sh);
         if (odd) {
             const int e = (int)(lm >> 20);
             int a = 1023 - e;
             a = a < -1000 ? -1000 : a > 1000 ? 1000 : a;
             const double f = __longlong_as_double((i64)(1023 + a) << 52);
-            r.mul = e == 0x7ff ? __longlong_as_double(0x7ff8000000000000LL)
-                               : __longlong_as_double((i64)(1023 - a) << 52);
+            r.t = e == 0x7ff ? kNanT : -a;
 #pragma unroll
             for (int i = 0; i < NV; i++) v[i] = mkl(raw_scaled(v[i].x, f), raw_scaled(v[i].y, f));
         }
@@ -130,57 +138,143 @@ NSK_DEV LineScale line_scale(L2 (&v)[NV], const LineGeo &g, unsigned *sh, Skip s
         __syncthreads();
     }
     r.top = fix_top(S);
+    r.t = S == 0.f ? kZeroT : r.t + r.top;
     return r;
+}
+
+// Scale of a line read in fixed point: v[i] with exponents t[i], brought to a
+// common one, which is returned.  The common exponent is at least the largest
+// t (an entry is not known below its own lines' unit), and leaves the line sum
+// below 2^63.  sh holds two words per thread.
+template <int NV, bool TWICE, class Skip>
+NSK_DEV int line_scale_fixed(L2 (&v)[NV], const int (&t)[NV], const LineGeo &g, unsigned *sh, Skip skip) {
+    int tm = kZeroT;
+#pragma unroll
+    for (int i = 0; i < NV; i++)
+        if (!skip(i)) tm = max(tm, t[i]);
+    tm = (int)line_reduce<OpMax>((unsigned)(tm + (1 << 22)), g, sh) - (1 << 22);
+    float s = 0.f;
+#pragma unroll
+    for (int i = 0; i < NV; i++) {
+        if (skip(i)) continue;
+        // in units of 2^32; 1.5 covers the lower words (while R below is zero,
+        // S plays no part, and it is large against them otherwise)
+        const float a = fabsf((float)lhi(v[i].x)), b = fabsf((float)lhi(v[i].y));
+        const float f = __uint_as_float((unsigned)(max(t[i] - tm, -127) + 127) << 23);
+        s = fmaf(fmaf(0.41421360f, fminf(a, b), fmaxf(a, b) + 1.5f), f, s);
+    }
+    if (TWICE) s *= 2.f;
+    const float S = __uint_as_float(line_reduce<OpAdd>(__float_as_uint(s), g, sh + blockDim.x));
+    const int R = max((int)(__float_as_uint(S * 1.001f) >> 23) + 32 - (127 + 62), 0);
+#pragma unroll
+    for (int i = 0; i < NV; i++) {
+        if (skip(i)) continue;
+        const int r = min(R + tm - t[i], 63);
+        v[i] = mkl(v[i].x >> r, v[i].y >> r);
+    }
+    return tm + R;
 }
 
 NSK_DEV i64 fix_from_raw(i64 raw, int top) { return fix_from(lhi(raw), llo(raw), top); }
 NSK_DEV L2 fix_from_raw(L2 raw, int top) { return mkl(fix_from_raw(raw.x, top), fix_from_raw(raw.y, top)); }
 
-// Conversion of a line's results; ebase as fix_to's.  On the integer pipes (23
-// instructions a value): two FP64 additions can do it too, but all of a CTA's
-// conversions come together at its end, where the FP64 pipe made the passes
-// 20 % slower (an eighth to a quarter of the values there: 0.6 % faster).
+// Conversion of a line's results with exponent t to double, on the integer
+// pipes (23 instructions a value): two FP64 additions can do it too, but all of
+// a CTA's conversions come together at its end, where the FP64 pipe made the
+// passes 20 % slower (an eighth to a quarter of the values there: 0.6 %
+// faster).  Lines whose results could leave the range of normal numbers
+// convert about 1 and are multiplied by two factors.
 struct FixOut {
     int ebase;
-    NSK_DEV double operator()(i64 v) const {
-        unsigned hi, lo;
-        fix_to(v, ebase, hi, lo);
-        return __hiloint2double((int)hi, (int)lo);
+    bool odd;
+    double f1, f2;
+    NSK_DEV explicit FixOut(int t) {
+        odd = t < 70 || t > 1980;
+        ebase = odd ? 1024 : t + 1;   // of a leading bit at bit 63
+        f1 = f2 = 1.0;
+        if (odd && t > -kEdgeT) {
+            const int h = (t - 1023) / 2;
+            f1 = t > kEdgeT ? __longlong_as_double(0x7ff8000000000000LL) : power(h);
+            f2 = t > kEdgeT ? 1.0 : power(t - 1023 - h);
+        }
+    }
+    static NSK_DEV double power(int e) {   // 2^e, |e| <= 1022
+        e = e < -1022 ? -1022 : e > 1023 ? 1023 : e;
+        return __longlong_as_double((i64)(1023 + e) << 52);
+    }
+    // The bits of the doubles, in place.  The factors are a branch of their own:
+    // as a predicated multiplication per value they kept the FP64 pipe busy for
+    // two clocks a point.
+    template <int NV> NSK_DEV void run(L2 (&v)[NV]) const {
+#pragma unroll
+        for (int i = 0; i < NV; i++) {
+            unsigned hi, lo;
+            fix_to(v[i].x, ebase, hi, lo);
+            v[i].x = (i64)(((unsigned long long)hi << 32) | lo);
+            fix_to(v[i].y, ebase, hi, lo);
+            v[i].y = (i64)(((unsigned long long)hi << 32) | lo);
+        }
+        if (odd) {
+#pragma unroll 1
+            for (int i = 0; i < 2; i++) {
+                const double f = i ? f2 : f1;
+#pragma unroll
+                for (int j = 0; j < NV; j++) v[j] = mkl(raw_scaled(v[j].x, f), raw_scaled(v[j].y, f));
+            }
+        }
     }
 };
 
-// CTAs of 256 threads an SM is to hold, by the registers E values take; more
-// or fewer change a 512^3 step by less than 1 %, the passes being bound by
-// instruction issue.
-template <int E> struct MinCtas { enum { n = E >= 9 ? 2 : E == 8 ? 3 : 4 }; };
+// CTAs of 256 threads an SM is to hold, by the registers that E values take.
+// At E = 8 the passes that wait for their loads most (the inverse strided ones
+// and the product r2c) want 64 registers and the warps of four CTAs, the
+// others 80 (512^3, four against three: y inverse 1.43 / 1.51 ms, product r2c
+// 2.49 / 2.67, but y forward 1.46 / 1.34, c2r the same; two: 1.60, 3.28, 1.43).
+template <int E, bool MANY> struct MinCtas { enum { n = E >= 9 ? 2 : E == 8 && !MANY ? 3 : 4 }; };
+
+// The shared line of a transform with E elements per thread: element e at
+// index (e + e / E) << cl, one entry of padding after every E so that the
+// stride-E stores of stage 0 spread over the banks.  Every later stage reads
+// with stride n / R and writes with stride p, both multiples of E, so the
+// entries of a butterfly lie one constant step apart.
+template <int E> struct LineAt {
+    L2 *base;
+    int cl;
+    NSK_DEV int step(int stride) const { return (stride + stride / E) << cl; }   // stride % E == 0
+    NSK_DEV L2 *at(int e) const { return base + ((e + e / E) << cl); }
+    static size_t entries(int n) { return (size_t)n + n / E; }
+};
 
 // Multiply by the stage twiddles and run the radix-R DFT of butterfly b.
 template <int R, int E, int DIR>
 NSK_DEV void fix_butterfly(L2 (&v)[E], int b, int k, int p, const int4 *__restrict__ tab, bool first) {
     const int sh = first ? 2 : 0;
     v[b * R] = mkl(v[b * R].x >> sh, v[b * R].y >> sh);
+    const int4 *w = tab + k;
 #pragma unroll
     for (int q = 1; q < R; q++) {
-        const int4 w = __ldg(tab + (q - 1) * p + k);
-        v[b * R + q] = cmul_w<DIR>(v[b * R + q], w, first);
+        v[b * R + q] = cmul_w<DIR>(v[b * R + q], __ldg(w + (q - 1) * p), first);
     }
     LDft<R, DIR>::run(&v[b * R]);
 }
 
-// One stage s >= 1.  The line comes from sl; every stage but the last writes
-// it back through ss (between barriers); the last leaves its results in v, in
-// the order of the line: v[j] is element slot + j T.
-template <int R, int E, int DIR, class SL, class SS>
+// One stage s >= 1.  The line comes from ln; every stage but the last writes it
+// back there (between barriers); the last leaves its results in v, in the
+// order of the line: v[j] is element slot + j T.
+template <int R, int E, int DIR>
 NSK_DEV void fix_stage(L2 (&v)[E], bool active, int slot, int T, int p, const int4 *__restrict__ tab,
-                       bool first, bool last, SL sl, SS ss) {
+                       bool first, bool last, const LineAt<E> &ln) {
     constexpr int B = E / R;
     const int nR = T * B;
     const unsigned magic = 0xffffffffu / (unsigned)p + 1u;   // i / p for i p < 2^32
     if (active) {
+        const int step = ln.step(nR);
 #pragma unroll
-        for (int b = 0; b < B; b++)
+        for (int b = 0; b < B; b++) {
+            const L2 *x = ln.at(slot + b * T);
 #pragma unroll
-            for (int q = 0; q < R; q++) v[b * R + q] = sl(slot + b * T + q * nR);
+            for (int q = 0; q < R; q++) v[b * R + q] = x[q * step];
+        }
 #pragma unroll
         for (int b = 0; b < B; b++) {
             const int i = slot + b * T;
@@ -199,30 +293,32 @@ NSK_DEV void fix_stage(L2 (&v)[E], bool active, int slot, int T, int p, const in
     }
     __syncthreads();
     if (active) {
+        const int step = ln.step(p);
 #pragma unroll
         for (int b = 0; b < B; b++) {
             const int i = slot + b * T;
             const int k = i - p * (int)__umulhi((unsigned)i, magic);
-            const int j = (i - k) * R + k;
+            L2 *x = ln.at((i - k) * R + k);
 #pragma unroll
-            for (int q = 0; q < R; q++) ss(j + q * p, v[b * R + q]);
+            for (int q = 0; q < R; q++) x[q * step] = v[b * R + q];
         }
     }
     __syncthreads();
 }
 
 // The stages of one line.  v holds the fixed-point elements slot + q T on
-// entry and the transform's on return.  sl / ss: the shared line.  smem_read:
-// the inputs came from it, so a barrier must precede the first store.
-template <int E, int DIR, class SL, class SS>
-NSK_DEV void fix_line(L2 (&v)[E], bool active, int slot, int T, const FixK &pl, bool smem_read, SL sl, SS ss) {
+// entry and the transform's on return.  smem_read: the inputs came from the
+// shared line, so a barrier must precede the first store.
+template <int E, int DIR>
+NSK_DEV void fix_line(L2 (&v)[E], bool active, int slot, int T, const FixK &pl, bool smem_read, const LineAt<E> &ln) {
     const int nst = pl.nst;
     if (active) LDft<E, DIR>::run(v);
     if (nst == 1) return;   // T = 1: element q is v[q]
     if (smem_read) __syncthreads();
     if (active) {
+        L2 *x = ln.base + ((slot * (E + 1)) << ln.cl);
 #pragma unroll
-        for (int q = 0; q < E; q++) ss(slot * E + q, v[q]);
+        for (int q = 0; q < E; q++) x[q << ln.cl] = v[q];
     }
     __syncthreads();
     int p = E;
@@ -230,9 +326,9 @@ NSK_DEV void fix_line(L2 (&v)[E], bool active, int slot, int T, const FixK &pl, 
     for (int s = 1; s < nst; s++) {
         const bool last = s == nst - 1;
         const int R = pl.rad(s);
-#define NSK_FIX_ST(RR)                                                                                   \
-    case RR:                                                                                             \
-        if constexpr (E % RR == 0) fix_stage<RR, E, DIR>(v, active, slot, T, p, tab, s == 1, last, sl, ss); \
+#define NSK_FIX_ST(RR)                                                                                  \
+    case RR:                                                                                            \
+        if constexpr (E % RR == 0) fix_stage<RR, E, DIR>(v, active, slot, T, p, tab, s == 1, last, ln); \
         break;
         switch (R) {
             NSK_FIX_ST(2)

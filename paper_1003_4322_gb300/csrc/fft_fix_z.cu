@@ -7,17 +7,14 @@
 //  r2c: the transform Z of x1 + i x2 gives X1[k] = (Z[k] + conj Z[N-k]) / 2
 //       and X2[k] = (Z[k] - conj Z[N-k]) / 2i.
 // The pairing adds are fixed-point too, and c2r converts each loaded entry
-// once for both of its places.  A missing second line (odd line count) reads
-// as zero and is not written.  Entries kz >= kzk are not read (c2r) or not
+// once for both of its places.  The spectra are in fixed point with their
+// lines' exponents.  Entries kz >= kzk are not read (c2r) or not
 // written (r2c).
 #include "fft_fix_line.cuh"
 
 namespace nsk {
 
-// One CTA holds lb line pairs, T = N/E threads each; the shared line is
-// skewed by one element in eight.
-NSK_DEV int zat(int e) { return e + (e >> 3); }
-
+// One CTA holds lb line pairs, T = N/E threads each.
 NSK_DEV LineGeo z_geo(int T, int li) {
     if (T <= 32 && (T & (T - 1)) == 0) return LineGeo{kSub, 31 - __clz(T), 0, li};
     if (T % 32 == 0) return LineGeo{kWarps, 0, T / 32, li};
@@ -42,11 +39,11 @@ NSK_DEV double product_at(const FixProduct &f, long base, long o1, long o2, int 
 }
 
 template <int E, int KIND>
-__global__ void __launch_bounds__(256, MinCtas<E>::n)
-k_fix_r2c2(FixProduct in, double2 *__restrict__ out, int N, long nlines, FixK pl, int kzk) {
+__global__ void __launch_bounds__(256, MinCtas<E, true>::n)
+k_fix_r2c2(FixProduct in, longlong2 *__restrict__ out, int *__restrict__ tout, int N, long nlines, FixK pl, int kzk) {
     grid_dep();
     extern __shared__ __align__(16) unsigned char smraw[];
-    __shared__ unsigned red[256];
+    __shared__ unsigned red[512];
     const int nh = N / 2, T = N / E;
     const int slot = threadIdx.x % T, li = threadIdx.x / T, lb = blockDim.x / T;
     // products: pairs of lines of the components in turn (the lines of one
@@ -62,82 +59,81 @@ k_fix_r2c2(FixProduct in, double2 *__restrict__ out, int N, long nlines, FixK pl
         base = 2 * pair * N;
     }
     const long l1 = 2 * pair, l2 = l1 + 1;
-    const bool v1 = KIND > 0 ? (long)blockIdx.x * lb + li < nlines / 2 : l1 < nlines;
-    const bool v2 = KIND > 0 ? v1 : l2 < nlines;
-    L2 *ls = reinterpret_cast<L2 *>(smraw) + li * (zat(N) + 1);
+    const bool valid = (long)blockIdx.x * lb + li < nlines / 2;
+    const LineAt<E> ln{reinterpret_cast<L2 *>(smraw) + li * (N + T), 0};
     L2 v[E];
 #pragma unroll
     for (int q = 0; q < E; q++) {
         const int e = slot + q * T;
-        v[q] = mkl(v1 ? __double_as_longlong(product_at<KIND>(in, base, o1, o2, e)) : 0,
-                   v2 ? __double_as_longlong(product_at<KIND>(in, base + N, o1, o2, e)) : 0);
+        v[q] = mkl(valid ? __double_as_longlong(product_at<KIND>(in, base, o1, o2, e)) : 0,
+                   valid ? __double_as_longlong(product_at<KIND>(in, base + N, o1, o2, e)) : 0);
     }
     const LineScale sc = line_scale<E, false>(v, z_geo(T, li), red, [](int) { return false; });
 #pragma unroll
     for (int q = 0; q < E; q++) v[q] = fix_from_raw(v[q], sc.top);
-    auto sl = [&](int e) { return ls[zat(e)]; };
-    auto ss = [&](int e, L2 x) { ls[zat(e)] = x; };
-    fix_line<E, -1>(v, true, slot, T, pl, false, sl, ss);
+    fix_line<E, -1>(v, true, slot, T, pl, false, ln);
     if (pl.nst > 1) __syncthreads();
 #pragma unroll
-    for (int q = 0; q < E; q++) ss(slot + q * T, v[q]);
+    for (int q = 0; q < E; q++) *ln.at(slot + q * T) = v[q];
     __syncthreads();
-    double2 *d1 = out + l1 * (nh + 1), *d2 = out + l2 * (nh + 1);
+    if (!valid) return;
+    longlong2 *d1 = out + l1 * (nh + 1), *d2 = out + l2 * (nh + 1);
     // the halves of the pairing fall to the exponent; with one stage the
     // values use all 63 bits, so that half is taken before the sum
     const int pre = pl.nst > 1 ? 0 : 1;
-    const FixOut fo{sc.top + (pl.nst > 1 ? 2 : 1)};
+    if (slot < 2) tout[l1 + slot] = sc.t + (pl.nst > 1 ? 1 : 0);
+    if (T == 1) tout[l2] = sc.t + (pl.nst > 1 ? 1 : 0);
     for (int k = slot; k <= nh && k < kzk; k += T) {
-        const L2 a = sl(k), b = sl(k == 0 ? 0 : N - k);
+        const L2 a = *ln.at(k), b = *ln.at(k == 0 ? 0 : N - k);
         const i64 ax = a.x >> pre, ay = a.y >> pre, bx = b.x >> pre, by = b.y >> pre;
-        double2 x1 = make_double2(fo(ax + bx), fo(ay - by)), x2 = make_double2(fo(ay + by), fo(bx - ax));
-        if (sc.any) {
-            x1 = make_double2(x1.x * sc.mul, x1.y * sc.mul);
-            x2 = make_double2(x2.x * sc.mul, x2.y * sc.mul);
-        }
-        if (v1) d1[k] = x1;
-        if (v2) d2[k] = x2;
+        d1[k] = longlong2{ax + bx, ay - by};
+        d2[k] = longlong2{ay + by, bx - ax};
     }
 }
 
 template <int E>
-__global__ void __launch_bounds__(256, MinCtas<E>::n)
-k_fix_c2r2(const longlong2 *__restrict__ in, double *__restrict__ out, int N, long nlines, FixK pl, int kzk) {
+__global__ void __launch_bounds__(256, MinCtas<E, false>::n)
+k_fix_c2r2(const longlong2 *__restrict__ in, const int *__restrict__ tin, int ny, double *__restrict__ out, int N,
+           long nlines, FixK pl, int kzk) {
     grid_dep();
     extern __shared__ __align__(16) unsigned char smraw[];
-    __shared__ unsigned red[256];
+    __shared__ unsigned red[512];
     const int nh = N / 2, T = N / E;
     const int slot = threadIdx.x % T, li = threadIdx.x / T, lb = blockDim.x / T;
     const long l1 = 2 * ((long)blockIdx.x * lb + li), l2 = l1 + 1;
-    const bool v1 = l1 < nlines, v2 = l2 < nlines;
-    L2 *ls = reinterpret_cast<L2 *>(smraw) + li * (zat(N) + 1);
-    auto sl = [&](int e) { return ls[zat(e)]; };
-    auto ss = [&](int e, L2 x) { ls[zat(e)] = x; };
+    const bool valid = l1 < nlines;
+    const LineAt<E> ln{reinterpret_cast<L2 *>(smraw) + li * (N + T), 0};
     const longlong2 *s1 = in + l1 * (nh + 1), *s2 = in + l2 * (nh + 1);
     // the thread's entries m = slot + j T <= N/2 of both spectra
     constexpr int H = E / 2 + 1;
     const int top_m = kzk <= nh ? kzk : nh + 1;
+    const int *tl = tin + l1 / ny * (nh + 1);
     L2 w[2 * H];
+    int t[2 * H];
 #pragma unroll
     for (int j = 0; j < H; j++) {
         const int m = slot + j * T;
         longlong2 a{0, 0}, b{0, 0};
-        if (j * T < top_m && m < top_m) {
-            if (v1) a = s1[m];
-            if (v2) b = s2[m];
+        t[2 * j] = kZeroT;
+        if (j * T < top_m && m < top_m && valid) {
+            a = s1[m];
+            b = s2[m];
+            t[2 * j] = tl[m];
         }
+        t[2 * j + 1] = t[2 * j];
         if (m == 0 || m == nh) a.y = b.y = 0;
         w[2 * j] = mkl(a.x, a.y);
         w[2 * j + 1] = mkl(b.x, b.y);
     }
-    const LineScale sc = line_scale<2 * H, true>(w, z_geo(T, li), red, [&](int i) { return (i / 2) * T >= top_m; });
+    const int tz =
+        line_scale_fixed<2 * H, true>(w, t, z_geo(T, li), red, [&](int i) { return (i / 2) * T >= top_m; });
 #pragma unroll
     for (int j = 0; j < H; j++) {
         const int m = slot + j * T;
         if (m < top_m) {
-            const L2 a = fix_from_raw(w[2 * j], sc.top), b = fix_from_raw(w[2 * j + 1], sc.top);
-            ss(m, mkl(a.x - b.y, a.y + b.x));
-            if (m != 0 && m != nh) ss(N - m, mkl(a.x + b.y, b.x - a.y));
+            const L2 a = w[2 * j], b = w[2 * j + 1];
+            *ln.at(m) = mkl(a.x - b.y, a.y + b.x);
+            if (m != 0 && m != nh) *ln.at(N - m) = mkl(a.x + b.y, b.x - a.y);
         }
     }
     __syncthreads();
@@ -145,21 +141,17 @@ k_fix_c2r2(const longlong2 *__restrict__ in, double *__restrict__ out, int N, lo
 #pragma unroll
     for (int q = 0; q < E; q++) {
         const int e = slot + q * T;
-        v[q] = e < top_m || N - e < top_m ? sl(e) : mkl(0, 0);
+        v[q] = e < top_m || N - e < top_m ? *ln.at(e) : mkl(0, 0);
     }
     double *d1 = out + l1 * N, *d2 = out + l2 * N;
-    fix_line<E, 1>(v, true, slot, T, pl, true, sl, ss);
-    const FixOut fo{sc.top + 1 + (pl.nst > 1 ? 2 : 0)};
+    fix_line<E, 1>(v, true, slot, T, pl, true, ln);
+    if (!valid) return;
+    FixOut(tz + (pl.nst > 1 ? 2 : 0)).run(v);
 #pragma unroll
     for (int q = 0; q < E; q++) {
         const int e = slot + q * T;
-        double x1 = fo(v[q].x), x2 = fo(v[q].y);
-        if (sc.any) {
-            x1 *= sc.mul;
-            x2 *= sc.mul;
-        }
-        if (v1) d1[e] = x1;
-        if (v2) d2[e] = x2;
+        d1[e] = __longlong_as_double(v[q].x);
+        d2[e] = __longlong_as_double(v[q].y);
     }
 }
 
@@ -196,31 +188,36 @@ cudaError_t prepare_fix_z() {
     return cudaSuccess;
 }
 
-static cudaError_t launch(int kind, const void *in, void *out, int N, long nlines, const FixPlan &fp, cudaStream_t s,
-                          int kzk) {
+static cudaError_t launch(int kind, void **args, int N, long *nlines, const FixPlan &fp, cudaStream_t s) {
     const Plan &pl = fp.pl;
     const void *k = kernel_of(kind, pl.E);
-    if (!k || !fp.tab || pl.n != N || nlines < 1 || (kind > 0 && nlines % 6)) return cudaErrorInvalidValue;
-    if (kzk < 0 || kzk > N / 2 + 1) kzk = N / 2 + 1;   // every entry
+    if (!k || !fp.tab || pl.n != N || *nlines < 2 || *nlines % 2 || (kind > 0 && *nlines % 6))
+        return cudaErrorInvalidValue;
     const int T = N / pl.E, lb = T > kThreads ? 1 : kThreads / T;
     if (T > 256) return cudaErrorInvalidValue;
-    const size_t smem = (size_t)lb * (N + (N >> 3) + 1) * sizeof(L2);
+    const size_t smem = (size_t)lb * (N + T) * sizeof(L2);   // LineAt
     cudaError_t e = allow_smem(k, smem);
     if (e != cudaSuccess) return e;
-    const long blocks = ((nlines + 1) / 2 + lb - 1) / lb;
+    const long blocks = (*nlines / 2 + lb - 1) / lb;
     if (blocks > 0x7fffffffL) return cudaErrorInvalidValue;
-    FixK kp{pl.n, pl.nst, pl.radix, fp.tab};
-    // in: the argument itself (a FixProduct), or where the pointer argument is
-    void *args[] = {(void *)in, (void *)&out, (void *)&N, (void *)&nlines, (void *)&kp, (void *)&kzk};
     return launch_dep(k, dim3((unsigned)blocks), dim3(lb * T), args, smem, s);
 }
 
-cudaError_t fix_z_r2c(const FixProduct &in, double2 *out, int N, long nlines, const FixPlan &fp, cudaStream_t s,
-                      int kzk) {
-    return launch(in.kind, &in, out, N, nlines, fp, s, kzk);
+cudaError_t fix_z_r2c(const FixProduct &in, void *out, int *tout, int N, long nlines, const FixPlan &fp,
+                      cudaStream_t s, int kzk) {
+    if (kzk < 0 || kzk > N / 2 + 1) kzk = N / 2 + 1;   // every entry
+    FixK kp{fp.pl.n, fp.pl.nst, fp.pl.radix, fp.tab};
+    void *args[] = {(void *)&in, (void *)&out, (void *)&tout, (void *)&N, (void *)&nlines, (void *)&kp, (void *)&kzk};
+    return launch(in.kind, args, N, &nlines, fp, s);
 }
-cudaError_t fix_z_c2r(const double2 *in, double *out, int N, long nlines, const FixPlan &fp, cudaStream_t s, int kzk) {
-    return launch(-1, &in, out, N, nlines, fp, s, kzk);
+cudaError_t fix_z_c2r(const void *in, const int *tin, int ny, double *out, int N, long nlines, const FixPlan &fp,
+                      cudaStream_t s, int kzk) {
+    if (ny < 2 || ny % 2) return cudaErrorInvalidValue;
+    if (kzk < 0 || kzk > N / 2 + 1) kzk = N / 2 + 1;
+    FixK kp{fp.pl.n, fp.pl.nst, fp.pl.radix, fp.tab};
+    void *args[] = {(void *)&in, (void *)&tin, (void *)&ny, (void *)&out, (void *)&N, (void *)&nlines, (void *)&kp,
+                    (void *)&kzk};
+    return launch(-1, args, N, &nlines, fp, s);
 }
 
 }  // namespace nsk

@@ -2,7 +2,7 @@
 // (Sec. 2, Fig. 1: 1D FFTs along each direction of the N^3 box with the
 // (N/2+1) x N x N half storage).  On one GPU the slab transposes of the
 // paper become the data layout of these passes (FP32 here; the FP64 ones are
-// fft_fix_strided.cu and fft_fix_z.cu): the strided passes read and write
+// fft_fix_strided.cuh and fft_fix_z.cu): the strided passes read and write
 // rows of contiguous columns (coalesced 128-byte rows), so no separate
 // transpose ever touches HBM.
 #include <math.h>

@@ -151,20 +151,31 @@ struct FixPlan {
 // *buf receives the array (freed with dev_free).
 cudaError_t make_fix_tables(int n, int4 **buf, const int4 *tab[17]);
 
-// The FP64 passes (fft_fix_strided.cu, fft_fix_z.cu), arguments as those of
-// fft_strided, fft_z_r2c and fft_z_c2r; the z plans have length N (two lines
-// per transform).  ct: a power of two up to 32, fix_threads(n, E, ct) <= 256.
-int fix_threads(int n, int E, int ct);
-// The x pass of a vorticity (dir +1, planes = the 3 components, ps_in apart):
-// transforms i k x a instead of a, formed on load.  The plane is ny rows of
-// nz columns; ix, iy, iz: wavenumber per index.
-struct FixCurl {
-    int ny = 0, nz = 0;
+// The FP64 passes (fft_fix_strided.cuh, fft_fix_z.cu).  Arrays of complex
+// values hold doubles, or fixed-point integers in the same 16 bytes with one
+// exponent per line in an array of their own.
+enum { kIoDouble = 0, kIoCurl = 1, kIoFixed = 2 };
+// Input and output of a strided pass.  Input exponents: those of the lines
+// that the pass before went along; element e of column (.., kz) of plane b
+// belongs to tin[(b / pdiv) eps + e estride + (ecol ? kz : 0)], kz = column mod
+// nzh.  Output exponents: tout[b ncols + column].
+// kIoCurl (x pass, dir +1, planes = the 3 components, ps apart): transforms
+// i k x a of the doubles a, formed on load; the plane is ny rows of nzh columns
+// and ix, iy, iz are the wavenumbers per index.
+struct FixIo {
+    int in = kIoDouble, out = kIoDouble;
+    const int *tin = nullptr;
+    int *tout = nullptr;
+    int pdiv = 1, estride = 0, ecol = 0, nzh = 1;
+    long eps = 0;
+    int ny = 0;
     double ix = 1.0, iy = 1.0, iz = 1.0;
 };
-cudaError_t fix_strided(const double2 *in, double2 *out, long ncols, long es, long ps_in, long ps_out, int planes,
-                        int dir, const FixPlan &fp, int ct, cudaStream_t s, const StridedSel *sel = nullptr,
-                        const FixCurl *curl = nullptr);
+// Arguments as those of fft_strided.  ct: a power of two up to 32,
+// fix_threads(n, E, ct) <= 256.
+int fix_threads(int n, int E, int ct);
+cudaError_t fix_strided(const void *in, void *out, long ncols, long es, long ps, int planes, int dir,
+                        const FixPlan &fp, int ct, cudaStream_t s, const StridedSel *sel, const FixIo &io);
 // The input of the r2c pass: f[0] (kind 0), or products of 3-component fields of
 // V points each, formed on load: f[0] x f[1] (kind 1), f[0] x f[1] + f[2] x f[3]
 // (kind 2; nlines then covers the three components, a multiple of 6).
@@ -173,10 +184,14 @@ struct FixProduct {
     long V = 0;
     int kind = 0;
 };
-cudaError_t fix_z_r2c(const FixProduct &in, double2 *out, int N, long nlines, const FixPlan &fp, cudaStream_t s,
-                      int kzk = -1);
-cudaError_t fix_z_c2r(const double2 *in, double *out, int N, long nlines, const FixPlan &fp, cudaStream_t s,
-                      int kzk = -1);
+// As fft_z_r2c and fft_z_c2r, with plans of length N (two lines, of the same x,
+// per transform; an even number of lines).  The spectra are in fixed point:
+// r2c writes the exponent of every line to tout[line]; c2r reads that of
+// entry kz of a line from tin[(line / ny) (N/2 + 1) + kz].
+cudaError_t fix_z_r2c(const FixProduct &in, void *out, int *tout, int N, long nlines, const FixPlan &fp,
+                      cudaStream_t s, int kzk = -1);
+cudaError_t fix_z_c2r(const void *in, const int *tin, int ny, double *out, int N, long nlines, const FixPlan &fp,
+                      cudaStream_t s, int kzk = -1);
 cudaError_t prepare_fix_strided();
 cudaError_t prepare_fix_z();
 

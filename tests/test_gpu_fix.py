@@ -95,3 +95,35 @@ def test_non_finite_entries_spread(ns, bad):
     X, v = _both(ns, u, x)
     assert np.isfinite(X[0]).all() and np.isfinite(v[0]).all()
     assert not np.isfinite(X[1]).any() and not np.isfinite(v[1]).any()
+
+
+def test_capture_without_exponent_buffers(ns):
+    """Under capture nothing is allocated: a grid larger than any before keeps
+    doubles between its passes (and, replayed, gives the same transform)."""
+    import torch
+    stream = torch.cuda.Stream()
+    ctx = ns.ns_init([dict(n=8, dt=1e-3)], ns.NS_FP64, stream)
+    try:
+        for dims in ((24, 8, 16), (8, 24, 16)):   # the tables of 8, 16, 24
+            small = torch.zeros((1,) + dims, dtype=torch.float64, device="cuda")
+            o = torch.empty((1,) + dims[:2] + (9,), dtype=torch.complex128, device="cuda")
+            torch.cuda.synchronize()
+            ns.ns_fft_r2c_grid(ctx, *dims, 1, small, o)
+            ns.ns_sync(ctx)
+        u, _ = _inputs((24, 24, 24), 3, nc=4)
+        ud = torch.zeros(u.shape, dtype=torch.float64, device="cuda")
+        out = torch.empty((4, 24, 24, 13), dtype=torch.complex128, device="cuda")
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=stream):
+            ns.ns_fft_r2c(ctx, 24, 4, ud, out)
+        ud.copy_(torch.from_numpy(u))
+        graph.replay()
+        torch.cuda.synchronize()
+        ref = oracle.fft3_r2c(u)
+        assert _rel(out.cpu().numpy(), ref) < TOL
+        ns.ns_fft_r2c(ctx, 24, 4, ud, out)   # the ordinary way, components in groups of three
+        ns.ns_sync(ctx)
+        assert _rel(out.cpu().numpy(), ref) < TOL
+    finally:
+        ns.ns_destroy(ctx)
