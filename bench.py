@@ -96,7 +96,7 @@ KERNEL_SOURCES = {
     "fp64": ("fft_core.cuh", "fft_passes.cu", "fft_fix.cuh", "fft_fix_line.cuh", "fft_fix_strided.cuh",
              "fft_fix_inv.cu", "fft_fix_fwd.cu", "fft_fix_z.cu", "plain.cu", "plain.h", "grid.cuh", "reduce.cuh", "api.cu"),
     "fp32": ("fft_core.cuh", "fft_ct.cuh", "reduce.cuh", "fused.cu", "fused.h", "fused_access.cuh",
-             "fused_s.cuh", "fused_k.cuh", "fused_kA.cu", "fused_kB.cu", "fused_kD.cu",
+             "fused_s.cuh", "fused_k.cuh", "fused_kA.cu", "fused_kA3.cu", "fused_kB.cu", "fused_kD.cu",
              "fused_kE.cu", "fused_keu.cu", "fused_update.cuh", "fused_sA.cu", "fused_sB.cu",
              "fused_sDE.cu", "fused_z.cu", "fused_zr.cuh", "fused_zr2.cu", "fused_zr3.cu",
              "fused_zr4.cu", "fused_zr5.cu", "fused_zm.cu"),

@@ -377,6 +377,11 @@ static bool fzk_for(const FusedRun &f, int pass, int E, int CT, FzsKernel *o) {
     if (!f.cube && f.n == f.ny && f.n == f.nz) return false;
     return fzk_lookup(pass, f.n, f.ny, f.nz, E, CT, o);
 }
+// Pass A with shared transforms (kind 3).
+static bool fza3_for(const FusedRun &f, int E, int CT, FzsKernel *o) {
+    if (!f.cube && f.n == f.ny && f.n == f.nz) return false;
+    return fza3_lookup(f.n, f.ny, f.nz, E, CT, o);
+}
 
 cudaError_t prepare_fused_kernels() {
     const int Ns[] = {32, 64, 96, 128, 192, 256, 384, 512, 768, 1024};
@@ -422,14 +427,20 @@ cudaError_t prepare_fused_kernels() {
                         if (e != cudaSuccess) return e;
                     }
                 }
+                FzsKernel z;
+                if (fza3_lookup(N, N, N, E, ct, &z)) {
+                    cudaError_t e = allow_smem(z.k, 48 * 1024 + 1);
+                    if (e != cudaSuccess) return e;
+                }
             }
 #define NSK_CASE(nx_, ny_, nz_, e_, ct_) {nx_, ny_, nz_, e_, ct_},
     static const int grids[][5] = {NSK_FZK_GRIDS(NSK_CASE)};
 #undef NSK_CASE
     for (const auto &g : grids)
-        for (int pass = 0; pass < 4; pass++) {
+        for (int pass = 0; pass < 5; pass++) {
             FzsKernel z;
-            if (fzk_lookup(pass, g[0], g[1], g[2], g[3], g[4], &z)) {
+            if (pass < 4 ? fzk_lookup(pass, g[0], g[1], g[2], g[3], g[4], &z)
+                         : fza3_lookup(g[0], g[1], g[2], g[3], g[4], &z)) {
                 cudaError_t e = allow_smem(z.k, 48 * 1024 + 1);
                 if (e != cudaSuccess) return e;
             }
@@ -611,11 +622,13 @@ static cudaError_t run_pass_ct(FusedRun &f, int pass, const PassCfg &cfg, const 
 
 static cudaError_t run_pass_k(FusedRun &f, int pass, const PassCfg &cfg, const FzPass &ps, cudaStream_t s) {
     FzsKernel z;
-    if (!fzk_for(f, pass, cfg.pl.E, cfg.ct, &z)) return cudaErrorInvalidValue;
+    const bool shared = cfg.kind == 3;   // pass A with shared transforms: two CTAs per tile
+    if (shared ? pass != 0 || !fza3_for(f, cfg.pl.E, cfg.ct, &z) : !fzk_for(f, pass, cfg.pl.E, cfg.ct, &z))
+        return cudaErrorInvalidValue;
     cudaError_t e = allow_smem(z.k, z.smem);
     if (e != cudaSuccess) return e;
     const long tiles = (ps.ncols + cfg.ct - 1) / cfg.ct;
-    const long blocks = tiles * ps.nfields;
+    const long blocks = tiles * (shared ? 2 : ps.nfields);
     if (blocks > 0x7fffffffL) return cudaErrorInvalidValue;
     const float2 *in = ps.in, *tw = pass_tw(f, pass);
     float2 *out = ps.out;
@@ -626,7 +639,7 @@ static cudaError_t run_pass_k(FusedRun &f, int pass, const PassCfg &cfg, const F
 
 // Pass 0..3 (A, B, D, E) with configuration cfg on the buffers of ps.
 static cudaError_t run_pass(FusedRun &f, int pass, const PassCfg &cfg, const FzPass &ps, cudaStream_t s) {
-    if (cfg.kind == 2) return run_pass_k(f, pass, cfg, ps, s);
+    if (cfg.kind >= 2) return run_pass_k(f, pass, cfg, ps, s);
     const int which = pass < 2 ? pass : 2;
     if (cfg.kind == 1) return run_pass_ct(f, pass, cfg, ps, s);
     const int E = cfg.pl.E;
@@ -825,7 +838,7 @@ template <class F> static float time_launch(F launch, cudaStream_t s, int reps) 
 static bool cfg_from_triple(int n, int kind, int E, int tile, bool zpass, PassCfg &out) {
     Plan pl;
     const int len = zpass ? n / 2 : n;
-    if (kind == 1 || kind == 2) {
+    if (kind == 1 || kind == 2 || (kind == 3 && !zpass)) {
         if (!make_plan(len, &pl)) return false;
         pl.E = E;   // compile-time kernels carry their own plan; E names the shape
     } else if (!make_plan_e(len, E, &pl)) {
@@ -967,11 +980,13 @@ static cudaError_t fused_autotune(FusedRun &f, cudaStream_t s) {
         };
         const int Es[] = {8, 12, 16, 32};
         const int len = pass_len(f, i);
-        for (int kind = 2; kind >= 1; kind--)
+        for (int kind = i == 0 ? 3 : 2; kind >= 1; kind--)
             for (int E : Es)
                 for (int ct = 8; ct <= 16; ct *= 2) {
                     FzsKernel z;
-                    if (kind == 1 ? !fzs_lookup(which[i], len, E, ct, &z) : !fzk_for(f, i, E, ct, &z))
+                    if (kind == 1   ? !fzs_lookup(which[i], len, E, ct, &z)
+                        : kind == 2 ? !fzk_for(f, i, E, ct, &z)
+                                    : !fza3_for(f, E, ct, &z))
                         continue;
                     PassCfg cfg{pass_plan(f, i), ct, kind};
                     cfg.pl.E = E;
@@ -1247,15 +1262,17 @@ cudaError_t fused_alloc(FusedRun &f, const std::vector<ns_run_params> &runs, con
         }
     }
     // The same for the strided passes A, B, D, E: NS_FORCE_STRIDED="kind,E,ct"
-    // (kind 1 or 2) applies to each pass that has such a kernel compiled.
+    // (kind 1 or 2; 3 for pass A alone) applies to each pass that has such a
+    // kernel compiled.
     if (const char *fs = getenv("NS_FORCE_STRIDED")) {
         int kind = -1, E = 0, ct = 0;
-        if (sscanf(fs, "%d,%d,%d", &kind, &E, &ct) == 3 && (kind == 1 || kind == 2))
+        if (sscanf(fs, "%d,%d,%d", &kind, &E, &ct) == 3 && kind >= 1 && kind <= 3)
             for (int i = 0; i < 4; i++) {
                 FzsKernel z;
                 PassCfg ci;
                 if (!cfg_from_triple(pass_len(f, i), kind, E, ct, false, ci)) continue;
-                const bool ok = kind == 2 ? fzk_for(f, i, E, ct, &z)
+                const bool ok = kind == 3   ? i == 0 && fza3_for(f, E, ct, &z)
+                                : kind == 2 ? fzk_for(f, i, E, ct, &z)
                                           : fzs_lookup(i < 2 ? i : 2, pass_len(f, i), E, ct, &z);
                 if (ok) f.sp[i] = ci;
             }
@@ -1355,7 +1372,8 @@ int fused_describe(const FusedRun &f, char *out, int len) {
     for (int i = 0; i < 4 && w < len; i++)
         w += snprintf(out + w, len - w,
                       "\"%s\": {\"kernel\": \"%s\", \"E\": %d, \"cols_per_cta\": %d}, ", names[i],
-                      f.sp[i].kind == 2   ? "constant geometry"
+                      f.sp[i].kind == 3   ? "constant geometry, shared transforms"
+                      : f.sp[i].kind == 2 ? "constant geometry"
                       : f.sp[i].kind == 1 ? "compile-time length"
                                           : "runtime length",
                       f.sp[i].pl.E,

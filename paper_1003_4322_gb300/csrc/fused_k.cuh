@@ -147,6 +147,8 @@ bool fzk_lookup_A(int NX, int NY, int NZ, int E, int CT, FzsKernel *o);
 bool fzk_lookup_B(int NX, int NY, int NZ, int E, int CT, FzsKernel *o);
 bool fzk_lookup_D(int NX, int NY, int NZ, int E, int CT, FzsKernel *o);
 bool fzk_lookup_E(int NX, int NY, int NZ, int E, int CT, FzsKernel *o);
+// Pass A with shared transforms (fused_kA3.cu); grid x = 2 ceil(My Mz / CT).
+bool fza3_lookup(int NX, int NY, int NZ, int E, int CT, FzsKernel *o);
 // Pass E fused with the update (fused_keu.cu); grid x = ceil(Mx Mz / CT)
 // column tiles, one energy partial per CTA.
 bool fzeu_lookup(int N, int E, int CT, FzsKernel *o);
