@@ -80,6 +80,7 @@ struct Run {
     long V = 0;   // grid points per component
     // plain form (full half layout)
     void *un = nullptr, *u1 = nullptr, *wn = nullptr, *work = nullptr, *phys = nullptr;
+    int work_comps = 3;                   // components that work holds
     void *sh = nullptr, *sh2 = nullptr;   // phase-shift dealiasing: shifted state, its product
     int *ftx = nullptr;                   // FP64: line exponents of a transform of three components
     void *phtab = nullptr;                // per-axis shift factors exp(i pi m / N_i)
@@ -305,7 +306,7 @@ cudaError_t pass_z_r2c(const FftRes &f, const T *in, typename Cx<T>::type *out, 
 // Formats of the strided FP64 passes of a grid (axis 0: x, 1: y): fixed point
 // between the passes, doubles at the ends.  fixed = false: doubles throughout,
 // around a z pass that takes them.
-FixIo fix_io(const Grid &g, int axis, int dir, const FixBufs &fb, bool fixed = true, bool curl = false) {
+FixIo fix_io(const Grid &g, int axis, int dir, const FixBufs &fb, bool fixed = true, int curl = 0) {
     FixIo io;
     io.nzh = (int)g.nzh();
     io.ny = g.ny;
@@ -315,6 +316,7 @@ FixIo fix_io(const Grid &g, int axis, int dir, const FixBufs &fb, bool fixed = t
     if (!fixed) return io;
     if (axis == 0 && dir > 0) {          // x lines -> a
         io.in = curl ? kIoCurl : kIoDouble;
+        io.both = curl == 2;
         io.out = kIoFixed;
         io.tout = fb.a;
         return io;
@@ -350,11 +352,12 @@ template <typename T> bool ct_fits(const Plan &pl, int ct) {
 // compiled lengths: the standalone kernels, one field at a time through tmp.
 // pr (on): the fields lie inside the run's Pi, and only the lines that can be
 // nonzero are transformed (the rest of tmp is neither read nor written).
-// curl (FP64, ncomp = 3): the transform of i k x in.
+// curl (FP64): 1, the transform of i k x in (ncomp = 3); 2, those of in and of
+// i k x in (ncomp = 6, in of three components).
 template <typename T>
 cudaError_t c2r_batch(const typename Cx<T>::type *in, typename Cx<T>::type *tmp, T *out, const Grid &g,
                       int ncomp, const Fft3 &f, cudaStream_t s, const FixBufs &fb, Tracer *tr = nullptr,
-                      const PlainPrune *pr = nullptr, bool curl = false) {
+                      const PlainPrune *pr = nullptr, int curl = 0) {
     typedef typename Cx<T>::type C;
     if constexpr (std::is_same<T, float>::value) {
         const StdGrid sg = std_grid(g, f);
@@ -392,9 +395,21 @@ cudaError_t c2r_curl(const typename Cx<T>::type *a, typename Cx<T>::type *w, typ
                      const Grid &g, const Rect &rc, const Fft3 &f, cudaStream_t s, const FixBufs &fb, Tracer *tr,
                      const PlainPrune *pr) {
     if (std::is_same<T, double>::value && f.pz->zc.n == g.nz)
-        return c2r_batch<T>(a, tmp, out, g, 3, f, s, fb, tr, pr, true);
+        return c2r_batch<T>(a, tmp, out, g, 3, f, s, fb, tr, pr, 1);
     const cudaError_t e = NSK_TIMED(tr, "curl", plain_curl<T>(a, w, g, rc, s));
     return e != cudaSuccess ? e : c2r_batch<T>(w, tmp, out, g, 3, f, s, fb, tr, pr);
+}
+
+// a and its vorticity on the grid, out = [a, i k x a].  Where the run's buffers
+// hold six components (comps), FP64 takes them through the same launches.
+template <typename T>
+cudaError_t c2r_both(const typename Cx<T>::type *a, typename Cx<T>::type *w, typename Cx<T>::type *tmp, T *out,
+                     const Grid &g, const Rect &rc, const Fft3 &f, cudaStream_t s, const FixBufs &fb, int comps,
+                     Tracer *tr, const PlainPrune *pr) {
+    if (std::is_same<T, double>::value && comps == 6 && f.pz->zc.n == g.nz)
+        return c2r_batch<T>(a, tmp, out, g, 6, f, s, fb, tr, pr, 2);
+    const cudaError_t e = c2r_batch<T>(a, tmp, out, g, 3, f, s, fb, tr, pr);
+    return e != cudaSuccess ? e : c2r_curl<T>(a, w, tmp, out + 3 * g.V(), g, rc, f, s, fb, tr, pr);
 }
 
 // The y and x passes of r2c, in place.
@@ -730,7 +745,7 @@ template <typename T> ns_status tune_plain(ns_ctx *c, Run &r, FftRes *f) {
     cudaStream_t s = c->stream;
     C *in = (C *)r.un, *tmp = (C *)r.work, *half = (C *)r.wn;
     T *phys = (T *)r.phys;
-    const FixBufs fb(r.ftx, r.g, 3);
+    const FixBufs fb(r.ftx, r.g, r.work_comps);
     StridedSel sx, sy;
     prune_sels(r.g, r.prune, &sx, &sy);
     const int kzk = std::is_same<T, double>::value && r.prune.on ? r.prune.kz + 1 : -1;
@@ -812,7 +827,7 @@ template <typename T> ns_status tune_plain_grid(ns_ctx *c, Run &r, FftRes *f[3])
     C *in = (C *)r.un, *tmp = (C *)r.work, *half = (C *)r.wn;
     T *phys = (T *)r.phys;
     const int Es[] = {16, 12, 9, 8, 6, 4};
-    const FixBufs fb(r.ftx, g, 3);
+    const FixBufs fb(r.ftx, g, r.work_comps);
     StridedSel sx, sy;
     prune_sels(g, r.prune, &sx, &sy);
     const int kzk = std::is_same<T, double>::value && r.prune.on ? r.prune.kz + 1 : -1;
@@ -886,6 +901,13 @@ static bool plain_prune_enabled() {
     return !(v && v[0] == '0');
 }
 
+// FP64 runs up to this many modes per component (256^3) transform u and w
+// through the same launches, which takes a work buffer of six components
+// (32^3: 947 -> 747 us for ten steps with state transfer and spectrum, 96 x
+// 144 x 192: 0.95 -> 0.89 ms per step).  Larger ones fill the GPU with three and
+// keep the memory.
+const long kBothModes = 256L * 256 * 129;
+
 template <typename T> ns_status plain_alloc(ns_ctx *c, Run &r) {
     typedef typename Cx<T>::type C;
     r.prune.kx = r.reach.x;
@@ -897,10 +919,12 @@ template <typename T> ns_status plain_alloc(ns_ctx *c, Run &r) {
     NS_CK(dalloc(&r.un, nc * half));
     NS_CK(dalloc(&r.u1, nc * half));
     NS_CK(dalloc(&r.wn, nc * half));
-    NS_CK(dalloc(&r.work, 3 * half));
+    r.work_comps = std::is_same<T, double>::value && r.M <= kBothModes ? 6 : 3;
+    NS_CK(dalloc(&r.work, r.work_comps * half));
     if (std::is_same<T, double>::value) {
-        NS_CK(dalloc(&r.ftx, FixBufs::ints(r.g, 3) * sizeof(int)));
-        NS_CK(cudaMemsetAsync(r.ftx, 0, FixBufs::ints(r.g, 3) * sizeof(int), c->stream));
+        const size_t ints = FixBufs::ints(r.g, r.work_comps);
+        NS_CK(dalloc(&r.ftx, ints * sizeof(int)));
+        NS_CK(cudaMemsetAsync(r.ftx, 0, ints * sizeof(int), c->stream));
     }
     NS_CK(dalloc(&r.phys, 2 * nc * real));
     if (r.p.dealias == 2) {
@@ -1002,7 +1026,7 @@ template <typename T> ns_status plain_step(ns_ctx *c, Run &r, cudaStream_t s, Tr
     const Fft3 f = run_fft3(r, fr);
     const Grid &g = r.g;
     T *phys = (T *)r.phys;
-    const FixBufs fb(r.ftx, g, 3);
+    const FixBufs fb(r.ftx, g, r.work_comps);
     const long M3 = 3 * r.M, V3 = 3 * r.V;
     // the pointwise kernels may skip the modes outside the kept rectangle only
     // where every transform that reads their output is pruned: the FP64 path
@@ -1013,10 +1037,8 @@ template <typename T> ns_status plain_step(ns_ctx *c, Run &r, cudaStream_t s, Tr
         // grid -> u x w + j x b, u x b -> their transforms -> the two updates
         C *src = (C *)(stage == 1 ? r.un : r.u1);
         C *wj = (C *)r.wn;
-        NS_CK(c2r_batch<T>(src, (C *)r.work, phys, g, 3, f, s, fb, tr, &r.prune));
-        NS_CK(c2r_curl<T>(src, wj, (C *)r.work, phys + V3, g, rc, f, s, fb, tr, &r.prune));
-        NS_CK(c2r_batch<T>(src + M3, (C *)r.work, phys + 2 * V3, g, 3, f, s, fb, tr, &r.prune));
-        NS_CK(c2r_curl<T>(src + M3, wj + M3, (C *)r.work, phys + 3 * V3, g, rc, f, s, fb, tr, &r.prune));
+        NS_CK(c2r_both<T>(src, wj, (C *)r.work, phys, g, rc, f, s, fb, r.work_comps, tr, &r.prune));
+        NS_CK(c2r_both<T>(src + M3, wj + M3, (C *)r.work, phys + 2 * V3, g, rc, f, s, fb, r.work_comps, tr, &r.prune));
         NS_CK(r2c_cross_mhd<T>(phys, wj, wj + M3, g, f, s, fb, tr, &r.prune));
         const UpdateArgs ua = update_args(r, stage);
         NS_CK(NSK_TIMED(tr, "update",
@@ -1028,14 +1050,12 @@ template <typename T> ns_status plain_step(ns_ctx *c, Run &r, cudaStream_t s, Tr
     }
     for (int stage = 1; stage <= 2 && !r.p.mhd; stage++) {
         C *src = (C *)(stage == 1 ? r.un : r.u1);
-        NS_CK(c2r_batch<T>(src, (C *)r.work, phys, g, 3, f, s, fb, tr, &r.prune));
-        NS_CK(c2r_curl<T>(src, (C *)r.wn, (C *)r.work, phys + 3 * r.V, g, rc, f, s, fb, tr, &r.prune));
+        NS_CK(c2r_both<T>(src, (C *)r.wn, (C *)r.work, phys, g, rc, f, s, fb, r.work_comps, tr, &r.prune));
         NS_CK(r2c_cross<T>(phys, phys + 3 * r.V, (C *)r.wn, g, f, s, fb, tr, &r.prune));
         if (r.p.dealias == 2) {   // the same on the grid shifted by half a spacing, averaged
             C *sh = (C *)r.sh, *sh2 = (C *)r.sh2;
             NS_CK(NSK_TIMED(tr, "phase", plain_phase<T>(src, sh, (const C *)r.phtab, g, s)));
-            NS_CK(c2r_batch<T>(sh, (C *)r.work, phys, g, 3, f, s, fb, tr, &r.prune));
-            NS_CK(c2r_curl<T>(sh, sh2, (C *)r.work, phys + 3 * r.V, g, rc, f, s, fb, tr, &r.prune));
+            NS_CK(c2r_both<T>(sh, sh2, (C *)r.work, phys, g, rc, f, s, fb, r.work_comps, tr, &r.prune));
             NS_CK(r2c_cross<T>(phys, phys + 3 * r.V, sh2, g, f, s, fb, tr, &r.prune));
             NS_CK(NSK_TIMED(tr, "phase", plain_phase_avg<T>((C *)r.wn, sh2, (const C *)r.phtab, g, s)));
         }

@@ -33,7 +33,7 @@ cudaError_t fix_strided(const void *in, void *out, long ncols, long es, long ps,
     const int threads = fix_threads(pl.n, pl.E, ct);
     if (!k || !fp.tab || (1 << cl) != ct || ct > 32 || threads > 256) return cudaErrorInvalidValue;
     if ((io.in == kIoFixed && !io.tin) || (io.out == kIoFixed && !io.tout) || io.nzh < 1 || io.pdiv < 1 ||
-        (io.in == kIoCurl && planes != 3))
+        (io.in == kIoCurl && planes != (io.both ? 6 : 3)))
         return cudaErrorInvalidValue;
     StridedK sk{SelK{}, es, ps, ncols, cl, io};
     unsigned tiles;

@@ -38,7 +38,9 @@ k_fix_strided(const longlong2 *in, longlong2 *out, FixK pl, StridedK k) {
     const int inner = (blockIdx.x - ro * sel.tpr) * ct + c;
     const long col = (long)(ro < sel.o1 ? ro : ro - sel.o1 + sel.o2) * sel.inner + inner;
     const bool valid = active && inner < sel.keep;
-    const longlong2 *src = in + (IN == kIoCurl ? 0 : b * k.ps) + col;
+    const bool plain = IN != kIoCurl || (io.both && b < 3);
+    const int d = IN == kIoCurl && b >= 3 ? b - 3 : b;   // component of the curl
+    const longlong2 *src = in + (plain ? b * k.ps : 0) + col;
     longlong2 *dst = out + b * k.ps + col;
     auto in_gap = [&](int e) { return e >= sel.gap_lo && e < sel.gap_hi; };
     // elements q T .. (q + 1) T - 1 all in the gap: zeros that need no work
@@ -47,11 +49,11 @@ k_fix_strided(const longlong2 *in, longlong2 *out, FixK pl, StridedK k) {
     long o1 = 0, o2 = 0;
     double k1 = 0.0, k2 = 0.0;
     if constexpr (IN == kIoCurl) {
-        o1 = (b + 1) % 3 * k.ps;
-        o2 = (b + 2) % 3 * k.ps;
+        o1 = (d + 1) % 3 * k.ps;
+        o2 = (d + 2) % 3 * k.ps;
         const double ky = io.iy * (2 * yi < io.ny ? yi : yi - io.ny), kzz = io.iz * kz;
-        k1 = b == 0 ? ky : kzz;   // b = 1: k2, b = 2: k1 are k_x, which varies along the line
-        k2 = b == 0 ? kzz : ky;
+        k1 = d == 0 ? ky : kzz;   // d = 1: k2, d = 2: k1 are k_x, which varies along the line
+        k2 = d == 0 ? kzz : ky;
     }
     const long gstep = T * k.es;   // element slot + q T: q steps on
     const int *tin = nullptr;
@@ -69,11 +71,11 @@ k_fix_strided(const longlong2 *in, longlong2 *out, FixK pl, StridedK k) {
         v[q] = mkl(0, 0);
         t[q] = kZeroT;
         if (!skip(q) && valid && (DIR < 0 || !in_gap(e))) {
-            if constexpr (IN == kIoCurl) {
+            if (!plain) {
                 const double2 a1 = reinterpret_cast<const double2 *>(src)[o1];
                 const double2 a2 = reinterpret_cast<const double2 *>(src)[o2];
                 const double kx = io.ix * (2 * e < pl.n ? e : e - pl.n);
-                const double p1 = b == 2 ? kx : k1, p2 = b == 1 ? kx : k2;
+                const double p1 = d == 2 ? kx : k1, p2 = d == 1 ? kx : k2;
                 v[q] = mkl(__double_as_longlong(p2 * a1.y - p1 * a2.y),
                            __double_as_longlong(p1 * a2.x - p2 * a1.x));
             } else {

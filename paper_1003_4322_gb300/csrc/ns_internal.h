@@ -161,12 +161,13 @@ enum { kIoDouble = 0, kIoCurl = 1, kIoFixed = 2 };
 // nzh.  Output exponents: tout[b ncols + column].
 // kIoCurl (x pass, dir +1, planes = the 3 components, ps apart): transforms
 // i k x a of the doubles a, formed on load; the plane is ny rows of nzh columns
-// and ix, iy, iz are the wavenumbers per index.
+// and ix, iy, iz are the wavenumbers per index.  both: planes 0 .. 2 transform a
+// itself, planes 3 .. 5 its curl.
 struct FixIo {
     int in = kIoDouble, out = kIoDouble;
     const int *tin = nullptr;
     int *tout = nullptr;
-    int pdiv = 1, estride = 0, ecol = 0, nzh = 1;
+    int pdiv = 1, estride = 0, ecol = 0, nzh = 1, both = 0;
     long eps = 0;
     int ny = 0;
     double ix = 1.0, iy = 1.0, iz = 1.0;
