@@ -92,7 +92,6 @@ struct Run {
     double *part = nullptr;
     double *series = nullptr;
     unsigned long long *counter = nullptr;
-    int nparts = 0;
     bool owns_diag = true;
 };
 
@@ -1027,6 +1026,7 @@ template <typename T> ns_status plain_step(ns_ctx *c, Run &r, cudaStream_t s, Tr
     const Grid &g = r.g;
     T *phys = (T *)r.phys;
     const FixBufs fb(r.ftx, g, r.work_comps);
+    const EnergyOut eo{r.series, kSeriesCap, r.counter, (unsigned *)(r.counter + 1), c->flags};
     const long M3 = 3 * r.M, V3 = 3 * r.V;
     // the pointwise kernels may skip the modes outside the kept rectangle only
     // where every transform that reads their output is pruned: the FP64 path
@@ -1042,7 +1042,7 @@ template <typename T> ns_status plain_step(ns_ctx *c, Run &r, cudaStream_t s, Tr
         NS_CK(r2c_cross_mhd<T>(phys, wj, wj + M3, g, f, s, fb, tr, &r.prune));
         const UpdateArgs ua = update_args(r, stage);
         NS_CK(NSK_TIMED(tr, "update",
-                        plain_update<T>((C *)r.un, (C *)r.u1, (const C *)wj, (const T *)r.etab, g, ua, rc, s)));
+                        plain_update<T>((C *)r.un, (C *)r.u1, (const C *)wj, (const T *)r.etab, g, ua, rc, r.part, eo, s)));
         NS_CK(NSK_TIMED(tr, "update_b",
                         plain_update_b<T>((C *)r.un + M3, (C *)r.u1 + M3, (const C *)wj + M3,
                                           (const T *)r.etab_b, g, stage, r.p.dt,
@@ -1061,11 +1061,8 @@ template <typename T> ns_status plain_step(ns_ctx *c, Run &r, cudaStream_t s, Tr
         }
         const UpdateArgs ua = update_args(r, stage);
         NS_CK(NSK_TIMED(tr, "update",
-                        plain_update<T>((C *)r.un, (C *)r.u1, (const C *)r.wn, (const T *)r.etab, g, ua, rc, s)));
+                        plain_update<T>((C *)r.un, (C *)r.u1, (const C *)r.wn, (const T *)r.etab, g, ua, rc, r.part, eo, s)));
     }
-    const EnergyOut eo{r.series, kSeriesCap, r.counter, (unsigned *)(r.counter + 1), c->flags};
-    NS_CK(NSK_TIMED(tr, "energy", plain_energy<T>((const C *)r.un, g, r.part,
-                                                  Rect{1, r.reach.x, r.reach.y, r.reach.z}, eo, s)));
     return NS_OK;
 }
 
@@ -1348,7 +1345,6 @@ ns_status ns_init(const ns_run_params *runs, int nruns, ns_prec prec, void *cuda
                         axis_keep(r.g, 2, r.p.dealias)};
         r.M = r.g.M();
         r.V = r.g.V();
-        r.nparts = energy_nparts(r.M);
         const int nb = grid_nbins(r.g);
         maxbins = std::max(maxbins, nb);
         c->spec_slice = std::max(c->spec_slice, (size_t)nb * (1 + shell_parts(nb)));
@@ -1357,7 +1353,7 @@ ns_status ns_init(const ns_run_params *runs, int nruns, ns_prec prec, void *cuda
         if (use_fused(c)) continue;   // grouped below
         st = prec == NS_FP64 ? plain_alloc<double>(c, r) : plain_alloc<float>(c, r);
         if (st != NS_OK) return bail(st);
-        if ((e = dalloc(&r.part, sizeof(double) * 2 * std::max(r.nparts, 1))) != cudaSuccess ||
+        if ((e = dalloc(&r.part, sizeof(double) * 2 * kEnergyParts)) != cudaSuccess ||
             (e = dalloc(&r.series, sizeof(double) * 2 * kSeriesCap)) != cudaSuccess ||
             (e = dalloc(&r.counter, 2 * sizeof(unsigned long long))) != cudaSuccess)
             return bail(fail_cuda(nullptr, e));

@@ -9,6 +9,8 @@
 // wavenumber m / l_i, and the 2/3 rule holds per axis in grid indices.
 #include <math.h>
 
+#include <algorithm>
+
 #include "ns_internal.h"
 #include "plain.h"
 #include "reduce.cuh"
@@ -237,70 +239,96 @@ __device__ __forceinline__ void abc_forcing(const Idx &k, const UpdateArgs &ua, 
 // On the unit box the table holds pairs (E, 1/|k|^2) by integer |k|^2, and a
 // mode takes 26 FP64 instructions in either stage and one conversion (60 with a
 // division, the conversions of k and the halvings as multiplications): 1.80 ->
-// 1.54 ms at 512^3.
+// 1.54 ms at 512^3.  Stage 2 also sums the new state's energy and enstrophy
+// (9 more FP64 instructions a mode; a lane adds its modes in order, the block in
+// a fixed tree, the last block the partials): 1.85 ms with them, and the pass of
+// 0.56 ms that read the state again is gone (32^3: 747 -> 724 us for ten steps).
 template <typename T, bool UNIT>
 __global__ void __launch_bounds__(256)
 k_update(typename Cx<T>::type *__restrict__ a, typename Cx<T>::type *__restrict__ a1,
          const typename Cx<T>::type *__restrict__ nl, const T *__restrict__ etab, Grid g, long M, UpdateArgs ua,
-         Rect rc) {
+         Rect rc, double *part, EnergyOut eo) {
     typedef typename Cx<T>::type C;
-    const int row = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
-    if (row >= rect_rows(rc, g)) return;
-    const RowIdx q = row_at(row, rc, g);
-    const RowWave<T, UNIT> k(q, g, etab);
-    const T gdt = (T)ua.gdt, dt = (T)ua.dt, F = (T)ua.force_amp;
-    const T rn = (T)ua.rn;   // the Coriolis factor in the units of nl
-    const T kx = k.kx, ky = k.ky;
-    const bool every = all_kept(rc, ua.dealias);
-    const int nk = rect_kz(rc, g);
-    for (int z = threadIdx.x & 31; z < nk; z += 32) {
-        const long m = q.m0 + z;
-        const Idx id{q.x, q.y, z};
-        C o0 = czero<C>(), o1 = czero<C>(), o2 = czero<C>();
-        if ((every || kept(id, g, ua.dealias)) && (q.x | q.y | z) != 0) {
-            // v = N^3 (nl / N^3 + Coriolis), in the units of nl
-            C vx = nl[m], vy = nl[M + m], vz = nl[2 * M + m];
-            if (ua.rot != 0.0) {   // Coriolis -2 rot z x u of the stage's state, before P
-                const C *cur = ua.stage == 1 ? a : a1;
-                vx = cadd(vx, cscale(cur[M + m], rn));
-                vy = csub(vy, cscale(cur[m], rn));
+    __shared__ double sh[512];
+    double en = 0.0, om = 0.0;   // stage 2: energy and enstrophy of the new state
+    const int rows = rect_rows(rc, g);
+    for (int row = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5); row < rows;
+         row += (int)(gridDim.x * blockDim.x) >> 5) {
+        const RowIdx q = row_at(row, rc, g);
+        const RowWave<T, UNIT> k(q, g, etab);
+        double er = 0.0, zr = 0.0;   // sums of w |a|^2 and k_z^2 w |a|^2 of the row
+        const T gdt = (T)ua.gdt, dt = (T)ua.dt, F = (T)ua.force_amp;
+        const T rn = (T)ua.rn;   // the Coriolis factor in the units of nl
+        const T kx = k.kx, ky = k.ky;
+        const bool every = all_kept(rc, ua.dealias);
+        const int nk = rect_kz(rc, g);
+        for (int z = threadIdx.x & 31; z < nk; z += 32) {
+            const long m = q.m0 + z;
+            const Idx id{q.x, q.y, z};
+            C o0 = czero<C>(), o1 = czero<C>(), o2 = czero<C>();
+            if ((every || kept(id, g, ua.dealias)) && (q.x | q.y | z) != 0) {
+                // v = N^3 (nl / N^3 + Coriolis), in the units of nl
+                C vx = nl[m], vy = nl[M + m], vz = nl[2 * M + m];
+                if (ua.rot != 0.0) {   // Coriolis -2 rot z x u of the stage's state, before P
+                    const C *cur = ua.stage == 1 ? a : a1;
+                    vx = cadd(vx, cscale(cur[M + m], rn));
+                    vy = csub(vy, cscale(cur[m], rn));
+                }
+                const T kz = k.kz(z, g);
+                T ik2;
+                if constexpr (UNIT) ik2 = etab[2 * (k.i2 + z * z) + 1];
+                else {
+                    const double dz = kmul(z, g.ilz);
+                    ik2 = (T)1 / (T)(k.r2 + dz * dz);
+                }
+                const T e = k.template factor<UNIT ? 2 : 1>(z, etab, g);
+                const C s = cscale(mkc(vx.x * kx + vy.x * ky + vz.x * kz, vx.y * kx + vy.y * ky + vz.y * kz), ik2);
+                vx = mkc(vx.x - kx * s.x, vx.y - kx * s.y);   // P(k) v = v - k (k.v) / k^2
+                vy = mkc(vy.x - ky * s.x, vy.y - ky * s.y);
+                vz = mkc(vz.x - kz * s.x, vz.y - kz * s.y);
+                const C f0 = a[m], f1 = a[M + m], f2 = a[2 * M + m];
+                if (ua.stage == 1) {   // E (a + (dt/N^3) v + dt f)
+                    C t0 = mkc(f0.x + gdt * vx.x, f0.y + gdt * vx.y);
+                    C t1 = mkc(f1.x + gdt * vy.x, f1.y + gdt * vy.y);
+                    C t2 = mkc(f2.x + gdt * vz.x, f2.y + gdt * vz.y);
+                    abc_forcing(id, ua, F * dt, t0, t1, t2);
+                    o0 = cscale(t0, e);
+                    o1 = cscale(t1, e);
+                    o2 = cscale(t2, e);
+                } else {               // (E a + a1 + (dt/N^3) v + dt f) / 2
+                    const C g0 = a1[m], g1 = a1[M + m], g2 = a1[2 * M + m];
+                    o0 = mkc(e * f0.x + g0.x + gdt * vx.x, e * f0.y + g0.y + gdt * vx.y);
+                    o1 = mkc(e * f1.x + g1.x + gdt * vy.x, e * f1.y + g1.y + gdt * vy.y);
+                    o2 = mkc(e * f2.x + g2.x + gdt * vz.x, e * f2.y + g2.y + gdt * vz.y);
+                    abc_forcing(id, ua, F * dt, o0, o1, o2);
+                    o0 = mkc(halve(o0.x), halve(o0.y));
+                    o1 = mkc(halve(o1.x), halve(o1.y));
+                    o2 = mkc(halve(o2.x), halve(o2.y));
+                }
             }
-            const T kz = k.kz(z, g);
-            T ik2;
-            if constexpr (UNIT) ik2 = etab[2 * (k.i2 + z * z) + 1];
-            else {
-                const double dz = kmul(z, g.ilz);
-                ik2 = (T)1 / (T)(k.r2 + dz * dz);
-            }
-            const T e = k.template factor<UNIT ? 2 : 1>(z, etab, g);
-            const C s = cscale(mkc(vx.x * kx + vy.x * ky + vz.x * kz, vx.y * kx + vy.y * ky + vz.y * kz), ik2);
-            vx = mkc(vx.x - kx * s.x, vx.y - kx * s.y);   // P(k) v = v - k (k.v) / k^2
-            vy = mkc(vy.x - ky * s.x, vy.y - ky * s.y);
-            vz = mkc(vz.x - kz * s.x, vz.y - kz * s.y);
-            const C f0 = a[m], f1 = a[M + m], f2 = a[2 * M + m];
-            if (ua.stage == 1) {   // E (a + (dt/N^3) v + dt f)
-                C t0 = mkc(f0.x + gdt * vx.x, f0.y + gdt * vx.y);
-                C t1 = mkc(f1.x + gdt * vy.x, f1.y + gdt * vy.y);
-                C t2 = mkc(f2.x + gdt * vz.x, f2.y + gdt * vz.y);
-                abc_forcing(id, ua, F * dt, t0, t1, t2);
-                o0 = cscale(t0, e);
-                o1 = cscale(t1, e);
-                o2 = cscale(t2, e);
-            } else {               // (E a + a1 + (dt/N^3) v + dt f) / 2
-                const C g0 = a1[m], g1 = a1[M + m], g2 = a1[2 * M + m];
-                o0 = mkc(e * f0.x + g0.x + gdt * vx.x, e * f0.y + g0.y + gdt * vx.y);
-                o1 = mkc(e * f1.x + g1.x + gdt * vy.x, e * f1.y + g1.y + gdt * vy.y);
-                o2 = mkc(e * f2.x + g2.x + gdt * vz.x, e * f2.y + g2.y + gdt * vz.y);
-                abc_forcing(id, ua, F * dt, o0, o1, o2);
-                o0 = mkc(halve(o0.x), halve(o0.y));
-                o1 = mkc(halve(o1.x), halve(o1.y));
-                o2 = mkc(halve(o2.x), halve(o2.y));
+            C *dst = ua.stage == 1 ? a1 : a;
+            dst[m] = o0;
+            dst[M + m] = o1;
+            dst[2 * M + m] = o2;
+            if (ua.stage == 2) {
+                double a2 = (double)o0.x * o0.x;
+                a2 = fma((double)o0.y, (double)o0.y, a2);
+                a2 = fma((double)o1.x, (double)o1.x, a2);
+                a2 = fma((double)o1.y, (double)o1.y, a2);
+                a2 = fma((double)o2.x, (double)o2.x, a2);
+                a2 = fma((double)o2.y, (double)o2.y, a2);
+                if (z == 0 || 2 * z == g.nz) a2 = halve(a2);   // 1/2 * multiplicity
+                const double kz = UNIT ? (double)z : kmul(z, g.ilz);
+                er += a2;
+                zr = fma(kz * kz, a2, zr);
             }
         }
-        C *dst = ua.stage == 1 ? a1 : a;
-        dst[m] = o0;
-        dst[M + m] = o1;
-        dst[2 * M + m] = o2;
+        en += er;
+        om += fma(UNIT ? (double)k.i2 : k.r2, er, zr);
+    }
+    if (ua.stage == 2) {
+        block_sum2(en, om, sh);
+        energy_publish(en, om, part, gridDim.x, 0, blockIdx.x, eo);
     }
 }
 
@@ -389,42 +417,6 @@ __global__ void k_phase_avg(typename Cx<T>::type *__restrict__ acc, const typena
 }
 
 // ---------------------------------------------------------------- reductions
-
-// Energy and enstrophy of a half-layout state, over the rows of the rectangle that holds its nonzero modes: warps take rows in a
-// fixed pattern, a lane sums its modes in order, the block adds up in a fixed
-// tree.  10 FP64 instructions per mode (r2 and 1/2 join once per row): 0.65 ->
-// 0.56 ms at 512^3, 137 -> 75 us at 256^3.
-template <typename T, bool UNIT>
-__global__ void __launch_bounds__(256)
-k_energy(const typename Cx<T>::type *__restrict__ a, Grid g, long M, double *part, Rect rc, EnergyOut eo) {
-    __shared__ double sh[512];
-    double e = 0.0, om = 0.0;
-    const int lane = threadIdx.x & 31, rows = rect_rows(rc, g), nk = rect_kz(rc, g);
-    for (int row = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5); row < rows;
-         row += (int)(gridDim.x * blockDim.x) >> 5) {
-        const RowIdx q = row_at(row, rc, g);
-        const RowWave<double, UNIT> k(q, g, nullptr);
-        const double r2 = UNIT ? (double)k.i2 : k.r2;
-        double er = 0.0, zr = 0.0;   // sums of w |a|^2 and kz^2 w |a|^2
-        for (int z = lane; z < nk; z += 32) {
-            const long m = q.m0 + z;
-            double a2 = 0.0;
-#pragma unroll
-            for (int c = 0; c < 3; c++) {
-                const double re = (double)a[c * M + m].x, im = (double)a[c * M + m].y;
-                a2 = fma(im, im, fma(re, re, a2));
-            }
-            if (z == 0 || 2 * z == g.nz) a2 = 0.5 * a2;   // 1/2 * multiplicity
-            const double kz = k.kz(z, g);
-            er += a2;
-            zr = fma(kz * kz, a2, zr);
-        }
-        e += er;
-        om += fma(r2, er, zr);
-    }
-    block_sum2(e, om, sh);
-    energy_publish(e, om, part, gridDim.x, 0, blockIdx.x, eo);
-}
 
 template <typename T> struct HalfAcc {
     const typename Cx<T>::type *a;
@@ -589,29 +581,15 @@ cudaError_t plain_phase_avg(typename Cx<T>::type *acc, const typename Cx<T>::typ
 template <typename T>
 cudaError_t plain_update(typename Cx<T>::type *a, typename Cx<T>::type *a1,
                          const typename Cx<T>::type *nl, const T *etab, const Grid &g,
-                         const UpdateArgs &args, const Rect &rc, cudaStream_t s) {
+                         const UpdateArgs &args, const Rect &rc, double *part, const EnergyOut &eo,
+                         cudaStream_t s) {
     const long M = g.M();
+    const unsigned blocks = std::min(rows_grid(rc, g), (unsigned)kEnergyParts);
     UpdateArgs ua = args;
     ua.gdt = ua.dt / (double)g.V();
     ua.rn = 2.0 * ua.rot * (double)g.V();
-    if (g.unit) k_update<T, true><<<rows_grid(rc, g), 256, 0, s>>>(a, a1, nl, etab, g, M, ua, rc);
-    else k_update<T, false><<<rows_grid(rc, g), 256, 0, s>>>(a, a1, nl, etab, g, M, ua, rc);
-    return cudaGetLastError();
-}
-
-int energy_nparts(long M) {
-    long np = (M + 511) / 512;        // small states: few rows per warp (19 -> 8 us at 32^3)
-    if (np > 152 * 4) np = 152 * 4;   // large ones: one wave
-    return (int)(np < 1 ? 1 : np);
-}
-
-template <typename T>
-cudaError_t plain_energy(const typename Cx<T>::type *a, const Grid &g, double *part, const Rect &rc,
-                         const EnergyOut &eo, cudaStream_t s) {
-    const long M = g.M();
-    const int np = energy_nparts(M);
-    if (g.unit) k_energy<T, true><<<np, 256, 0, s>>>(a, g, M, part, rc, eo);
-    else k_energy<T, false><<<np, 256, 0, s>>>(a, g, M, part, rc, eo);
+    if (g.unit) k_update<T, true><<<blocks, 256, 0, s>>>(a, a1, nl, etab, g, M, ua, rc, part, eo);
+    else k_update<T, false><<<blocks, 256, 0, s>>>(a, a1, nl, etab, g, M, ua, rc, part, eo);
     return cudaGetLastError();
 }
 
@@ -651,9 +629,7 @@ cudaError_t plain_helicity(const typename Cx<T>::type *a, const Grid &g, const R
                                            cudaStream_t);                                         \
     template cudaError_t plain_update<T>(Cx<T>::type *, Cx<T>::type *, const Cx<T>::type *,       \
                                          const T *, const Grid &, const UpdateArgs &, const Rect &, \
-                                         cudaStream_t);                                           \
-    template cudaError_t plain_energy<T>(const Cx<T>::type *, const Grid &, double *, const Rect &, \
-                                         const EnergyOut &, cudaStream_t);                        \
+                                         double *, const EnergyOut &, cudaStream_t);              \
     template cudaError_t plain_spectrum<T>(const Cx<T>::type *, const Grid &, const Reach &, int, double *, \
                                            double *, cudaStream_t);                               \
     template cudaError_t plain_helicity<T>(const Cx<T>::type *, const Grid &, const Reach &, int, double *, \

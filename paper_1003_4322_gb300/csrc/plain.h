@@ -25,8 +25,9 @@ struct UpdateArgs {
 
 // rc (the curl, both updates): the rectangle of the half layout outside which
 // the state is zero and which alone the (pruned) transforms read; with rc.on
-// they touch only its modes.  The energy sums take the rectangle of the
-// kept modes whether or not the transforms are pruned.
+// they touch only its modes.  The update's stage 2 leaves partial sums of energy
+// and enstrophy in part ([kEnergyParts][2]) and their totals in eo.
+constexpr int kEnergyParts = 152 * 8;
 template <typename T>
 cudaError_t plain_curl(const typename Cx<T>::type *a, typename Cx<T>::type *w, const Grid &g, const Rect &rc,
                        cudaStream_t s);
@@ -54,11 +55,7 @@ cudaError_t plain_update_b(typename Cx<T>::type *b, typename Cx<T>::type *b1,
 template <typename T>
 cudaError_t plain_update(typename Cx<T>::type *a, typename Cx<T>::type *a1,
                          const typename Cx<T>::type *nl, const T *etab, const Grid &g,
-                         const UpdateArgs &ua, const Rect &rc, cudaStream_t s);
-int energy_nparts(long M);
-template <typename T>
-cudaError_t plain_energy(const typename Cx<T>::type *a, const Grid &g, double *part, const Rect &rc,
-                         const EnergyOut &eo, cudaStream_t s);
+                         const UpdateArgs &ua, const Rect &rc, double *part, const EnergyOut &eo, cudaStream_t s);
 template <typename T>
 cudaError_t plain_spectrum(const typename Cx<T>::type *a, const Grid &g, const Reach &rc, int nbins, double *spec,
                            double *ens, cudaStream_t s);
