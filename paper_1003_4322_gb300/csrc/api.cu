@@ -125,6 +125,7 @@ struct ns_ctx {
     size_t gscratch_bytes = 0;
     int *ftx = nullptr;              // line exponents of the standalone FP64 transforms
     size_t ftx_ints = 0;
+    std::vector<int *> ftx_old;      // outgrown ones, which a graph captured by the caller may hold
     double *bspec = nullptr;         // batched spectra: per run nbins results + partials, twice
     size_t bspec_runs = 0;
     cudaGraphExec_t graph = nullptr;
@@ -374,15 +375,15 @@ cudaError_t c2r_batch(const typename Cx<T>::type *in, typename Cx<T>::type *tmp,
     StridedSel sx, sy;
     if (pruned) prune_sels(g, *pr, &sx, &sy);
     const bool fixed = qz.zc.n == g.nz;
-    cudaError_t e = NSK_TIMED(tr, curl ? "curl_x_inverse" : "fft_x_inverse",
+    cudaError_t e = NSK_TIMED(tr, curl == 2 ? "curl_x_inverse6" : curl ? "curl_x_inverse" : "fft_x_inverse",
                               pass_strided<T>(*f.x, in, tmp, plane, plane, M, ncomp, +1, qx.inv, qx.ct_inv, s,
                                               pruned ? &sx : nullptr, fix_io(g, 0, +1, fb, fixed, curl)));
     if (e != cudaSuccess) return e;
-    e = NSK_TIMED(tr, "fft_y_inverse",
+    e = NSK_TIMED(tr, curl == 2 ? "fft_y_inverse6" : "fft_y_inverse",
                   pass_strided<T>(*f.y, tmp, tmp, nh, nh, plane, ncomp * g.nx, +1, qy.inv, qy.ct_inv, s,
                                   pruned ? &sy : nullptr, fix_io(g, 1, +1, fb, fixed)));
     if (e != cudaSuccess) return e;
-    return NSK_TIMED(tr, "fft_z_c2r",
+    return NSK_TIMED(tr, curl == 2 ? "fft_z_c2r6" : "fft_z_c2r",
                      pass_z_c2r<T>(*f.z, tmp, out, (long)ncomp * g.nx * g.ny, qz.zc, s,
                                    pruned ? pr->kz + 1 : -1, fb, g.ny));
 }
@@ -654,8 +655,14 @@ template <class F> static float plain_time(F launch, cudaStream_t s) {
 // process.  Where nothing runs, the defaults stay.
 // Plain-form plan cache file (environment variable NS_PLAIN_CACHE): one line
 // per (N, bytes of the real type): "N bytes E_inv ct_inv E_fwd ct_fwd E_zc2r
-// E_zr2c".  Entries found there are used as they are; newly tuned ones are
-// written back, so that profiled runs execute the same kernels as plain ones.
+// E_zr2c".  Entries found there are used as they are, if the precision's
+// kernels take them (a file may be older than they are: FP64 z passes of one
+// line per transform, or more columns per CTA); newly tuned ones are written
+// back, so that profiled runs execute the same kernels as plain ones.
+static bool fix_takes(const Plan &pl, int ct) {
+    return ct >= 1 && ct <= 32 && (ct & (ct - 1)) == 0 && ct_fits<double>(pl, ct);
+}
+
 static void plain_cache_read(std::map<std::pair<int, int>, PlainPlans> &cache) {
     const char *path = getenv("NS_PLAIN_CACHE");
     FILE *fp = path ? fopen(path, "r") : nullptr;
@@ -668,7 +675,9 @@ static void plain_cache_read(std::map<std::pair<int, int>, PlainPlans> &cache) {
             return code >= 100 ? make_plan_e(n, code - 100, pl) : make_plan_e(n / 2, code, pl);
         };
         if (make_plan_e(n, ei, &q.inv) && make_plan_e(n, ef, &q.fwd) && zplan(ec, &q.zc) &&
-            zplan(er, &q.zr) && ci > 0 && cf > 0) {
+            zplan(er, &q.zr) &&
+            (b == (int)sizeof(double) ? fix_takes(q.inv, ci) && fix_takes(q.fwd, cf) && ec >= 100 && er >= 100
+                                      : ci > 0 && cf > 0)) {
             q.ct_inv = ci;
             q.ct_fwd = cf;
             q.tuned = true;
@@ -904,8 +913,36 @@ static bool plain_prune_enabled() {
 // through the same launches, which takes a work buffer of six components
 // (32^3: 947 -> 747 us for ten steps with state transfer and spectrum, 96 x
 // 144 x 192: 0.95 -> 0.89 ms per step).  Larger ones fill the GPU with three and
-// keep the memory.
+// keep the memory.  The buffers are widened once every run has its own, and
+// only within a sixteenth of the memory still free: a context that fits with
+// three components still fits.
 const long kBothModes = 256L * 256 * 129;
+
+void plain_widen(ns_ctx *c) {
+    size_t extra = 0, avail = 0, total = 0;
+    for (const Run &r : c->runs)
+        if (r.M <= kBothModes) extra += 3 * r.M * sizeof(double2);
+    if (!extra || cudaMemGetInfo(&avail, &total) != cudaSuccess || extra > avail / 16) return;
+    for (Run &r : c->runs) {
+        if (r.M > kBothModes) continue;
+        void *work = nullptr;
+        int *ftx = nullptr;
+        const size_t ints = FixBufs::ints(r.g, 6);
+        if (dalloc(&work, 6 * r.M * sizeof(double2)) != cudaSuccess ||
+            dalloc(&ftx, ints * sizeof(int)) != cudaSuccess ||
+            cudaMemsetAsync(ftx, 0, ints * sizeof(int), c->stream) != cudaSuccess) {
+            (void)cudaGetLastError();
+            if (work) dev_free(work);
+            if (ftx) dev_free(ftx);
+            return;
+        }
+        dev_free(r.work);   // nothing but the clearing of ftx has been queued on either
+        dev_free(r.ftx);
+        r.work = work;
+        r.ftx = ftx;
+        r.work_comps = 6;
+    }
+}
 
 template <typename T> ns_status plain_alloc(ns_ctx *c, Run &r) {
     typedef typename Cx<T>::type C;
@@ -918,10 +955,9 @@ template <typename T> ns_status plain_alloc(ns_ctx *c, Run &r) {
     NS_CK(dalloc(&r.un, nc * half));
     NS_CK(dalloc(&r.u1, nc * half));
     NS_CK(dalloc(&r.wn, nc * half));
-    r.work_comps = std::is_same<T, double>::value && r.M <= kBothModes ? 6 : 3;
-    NS_CK(dalloc(&r.work, r.work_comps * half));
+    NS_CK(dalloc(&r.work, 3 * half));
     if (std::is_same<T, double>::value) {
-        const size_t ints = FixBufs::ints(r.g, r.work_comps);
+        const size_t ints = FixBufs::ints(r.g, 3);
         NS_CK(dalloc(&r.ftx, ints * sizeof(int)));
         NS_CK(cudaMemsetAsync(r.ftx, 0, ints * sizeof(int), c->stream));
     }
@@ -1178,19 +1214,22 @@ ns_status check_flags(ns_ctx *c) {
 }
 
 // Line exponents for up to kFtxComp components of a standalone FP64 transform,
-// grown to the largest grid asked for.  Where they cannot be had (the stream is
+// at least doubled for a larger grid; the outgrown buffers (together no larger)
+// live as long as the context, as a graph captured by the caller may hold them.
+// Where they cannot be had (the stream is
 // being captured, or no memory is left), the transform keeps doubles between
 // its passes around the one-line z passes, which need none: *f3 then takes
 // `plain` for the z axis.
 const int kFtxComp = 3;
 FixBufs standalone_bufs(ns_ctx *c, const Grid &g, Fft3 *f3, PlainPlans *plain) {
-    const size_t need = FixBufs::ints(g, kFtxComp);
+    size_t need = FixBufs::ints(g, kFtxComp);
     if (c->ftx_ints < need) {
+        need = std::max(need, 2 * c->ftx_ints);
         cudaStreamCaptureStatus cap = cudaStreamCaptureStatusActive;
         int *p = nullptr;
         if (cudaStreamIsCapturing(c->stream, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone &&
-            cudaStreamSynchronize(c->stream) == cudaSuccess && dalloc(&p, need * sizeof(int)) == cudaSuccess) {
-            if (c->ftx) dev_free(c->ftx);
+            dalloc(&p, need * sizeof(int)) == cudaSuccess) {
+            if (c->ftx) c->ftx_old.push_back(c->ftx);
             c->ftx = p;
             c->ftx_ints = need;
         } else {
@@ -1359,6 +1398,7 @@ ns_status ns_init(const ns_run_params *runs, int nruns, ns_prec prec, void *cuda
             return bail(fail_cuda(nullptr, e));
         cudaMemset(r.counter, 0, 2 * sizeof(unsigned long long));   // steps recorded; finished blocks
     }
+    if (prec == NS_FP64) plain_widen(c);
     if (use_fused(c)) {
         // runs of the same grid, box and equations form one group (in order of
         // first appearance); an MHD group carries a magnetic block beside the
@@ -1432,6 +1472,7 @@ void ns_destroy(ns_ctx *c) {
     if (c->staging) dev_free(c->staging);
     if (c->gscratch) dev_free(c->gscratch);
     if (c->ftx) dev_free(c->ftx);
+    for (int *p : c->ftx_old) dev_free(p);
     if (c->bspec) dev_free(c->bspec);
     if (c->cap) cudaStreamDestroy(c->cap);
     for (cudaStream_t q : c->par) cudaStreamDestroy(q);

@@ -834,7 +834,8 @@ template <class F> static float time_launch(F launch, cudaStream_t s, int reps) 
 
 // Plan cache file (environment variable NS_PLAN_CACHE): one JSON object
 // mapping N to five [kind, E, tile] triples (passes A, B, D, E, C).  Entries
-// found there are used as they are; newly tuned sizes are written back.
+// found there are used as they are (kind 3 where pass A has such a kernel);
+// newly tuned sizes are written back.
 static bool cfg_from_triple(int n, int kind, int E, int tile, bool zpass, PassCfg &out) {
     Plan pl;
     const int len = zpass ? n / 2 : n;
@@ -874,9 +875,11 @@ static void plan_cache_read(std::map<int, TunedCfgs> &cache) {
                            &v[11], &v[12], &v[13], &v[14], &used) == 16 && used > 0)) {
             TunedCfgs t;
             bool ok = true;
-            for (int i = 0; i < 4 && ok; i++) ok = cfg_from_triple(n, v[3 * i], v[3 * i + 1], v[3 * i + 2], false, t.s[i]);
-            ok = ok && cfg_from_triple(n, v[12], v[13], v[14], true, t.c);
             FzsKernel z;
+            for (int i = 0; i < 4 && ok; i++)
+                ok = cfg_from_triple(n, v[3 * i], v[3 * i + 1], v[3 * i + 2], false, t.s[i]) &&
+                     (v[3 * i] != 3 || (i == 0 && fza3_lookup(n, n, n, v[1], v[2], &z)));
+            ok = ok && cfg_from_triple(n, v[12], v[13], v[14], true, t.c);
             if (v[15] == 3 && fzeu_lookup(n, v[16], v[17], &z)) {
                 t.eu_E = v[16];
                 t.eu_ct = v[17];
