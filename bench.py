@@ -193,7 +193,8 @@ def plain_keep(dims, dealias=0):
 
 
 PLAIN_KERNELS = ("fft_x_inverse", "fft_x_forward", "fft_y_inverse", "fft_y_forward", "fft_z_c2r",
-                 "fft_z_r2c")
+                 "fft_z_r2c", "curl_x_inverse", "curl_x_inverse6", "fft_y_inverse6", "fft_z_c2r6",
+                 "cross_z_r2c", "cross2_z_r2c")
 PLAIN_POINTWISE = ("curl", "update", "update_b", "energy_partials")
 
 
@@ -203,7 +204,8 @@ def kernel_model(name, n, prec, keep=None):
     N_z) for the plain kernels).  FFT flops use 5 n log2 n per complex line
     of length n.  keep (plain form): the kept (K_x, K_y, K_z), whose lines
     alone the transforms do and whose rows alone they read (inverse) or
-    write (forward); None: every line."""
+    write (forward); None: every line.  A name ending in 6: u and its curl
+    through the same launch."""
     es = 8 if prec == "fp64" else 4
     nx, ny, nz = (n, n, n) if isinstance(n, int) else n
     n = nx
@@ -222,6 +224,15 @@ def kernel_model(name, n, prec, keep=None):
         return 3 * cy * (ry + ny) * 2 * es, 3 * cy * 5 * ny * math.log2(ny)
     if name in ("fft_z_c2r", "fft_z_r2c"):
         return 3 * (nx * ny * zk * 2 * es + V * es), 3 * nx * ny * f_zline
+    if name in ("fft_y_inverse6", "fft_z_c2r6"):
+        return tuple(2 * v for v in kernel_model(name[:-1], (nx, ny, nz), prec, keep))
+    if name in ("curl_x_inverse", "curl_x_inverse6"):   # the three components of a in, of i k x a (and a) out
+        out = 6 if name[-1] == "6" else 3
+        return cx * (3 * rx + out * nx) * 2 * es, out * cx * 5 * nx * math.log2(nx) + 3 * cx * rx * 6
+    if name in ("cross_z_r2c", "cross2_z_r2c"):   # u x w (and j x b) formed in the transform's loads
+        terms = 1 if name[5] == "_" else 2
+        return (3 * nx * ny * zk * 2 * es + 6 * terms * V * es,
+                3 * nx * ny * f_zline + (12 * terms - 3) * V)
     if name in ("fft_c2r_std", "fft_r2c_std"):   # all three passes of three components
         flops = 3 * (ny * nh * 5 * nx * math.log2(nx) + nx * nh * 5 * ny * math.log2(ny) + nx * ny * f_zline)
         return 3 * (M * 2 * es + V * es) + 2 * (2 * 3 * M * 2 * es), flops
@@ -379,7 +390,10 @@ def time_form(w, prec, mem, steps, warmup, census_steps, dist, keep_states=True)
 
 def roofline_of(census, w, prec, census_steps, peaks, sm_mhz, sizes=None):
     """Dominant kernel (largest share of device time in the census) against
-    HBM or the FP64 ALU roof, whichever its algorithmic model says binds."""
+    HBM or the FP64 ALU roof, whichever its algorithmic model says binds.  The
+    FP64 line transforms run in 64-bit fixed point on the integer pipes, and
+    pass the rate of the FP64 pipe: no roof there, so such a kernel is set
+    against HBM."""
     if not census:
         return None, None
     total = sum(t for _, _, t in census)
@@ -412,7 +426,8 @@ def roofline_of(census, w, prec, census_steps, peaks, sm_mhz, sizes=None):
             src = "FP64 FMA pipes x max SM clock (derived)"
         tflops = flops / (per_launch_ms * 1e-3) / 1e12
         alu_frac = tflops * 1e12 / peak_flops
-        if alu_frac >= hbm_frac:
+        roof["fp64_pipe_frac"] = alu_frac
+        if hbm_frac <= alu_frac <= 1.0:
             roof.update(bound="alu", achieved=tflops, peak=peak_flops / 1e12, unit="TFLOP/s",
                         frac=alu_frac, peak_source=src, hbm_frac=hbm_frac)
             return roof, total
