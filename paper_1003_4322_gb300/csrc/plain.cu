@@ -123,14 +123,33 @@ template <typename T, bool UNIT> struct RowWave {
 // kept set)
 __device__ __forceinline__ bool all_kept(const Rect &rc, int dealias) { return rc.on && dealias == 0; }
 
-// x / 2, through the exponent: an FP64 multiplication costs this pipe as much
-// as 32 integer instructions.
-__device__ __forceinline__ float halve(float x) { return 0.5f * x; }
-__device__ __forceinline__ double halve(double x) {
-    const int hi = __double2hiint(x);
+// x / 2 through the exponent: an FP64 multiplication costs this pipe as much as
+// 32 integer instructions.  False (x left as it is) where the exponent does not
+// give it.  halve3 keeps those multiplications in one branch, as predicated ones
+// occupy the FP64 pipe of a warp that needs none.
+__device__ __forceinline__ bool halves(double &x) {
+    const int hi = __double2hiint(x), lo = __double2loint(x);
     const unsigned e = ((unsigned)hi >> 20) & 0x7ffu;
-    if (e - 2u < 0x7fdu - 1u) return __hiloint2double(hi - 0x100000, __double2loint(x));   // 2 <= e <= 0x7fd
-    return __double2loint(x) == 0 && (hi & 0x7fffffff) == 0 ? x : 0.5 * x;
+    const bool fast = e - 2u < 0x7fdu - 1u, zero = ((hi & 0x7fffffff) | lo) == 0;
+    x = __hiloint2double(fast ? hi - 0x100000 : hi, lo);
+    return fast || zero;
+}
+__device__ __forceinline__ void halve3(float2 &a, float2 &b, float2 &c) {
+    a = cscale(a, 0.5f);
+    b = cscale(b, 0.5f);
+    c = cscale(c, 0.5f);
+}
+__device__ __forceinline__ void halve3(double2 &a, double2 &b, double2 &c) {
+    const bool f0 = halves(a.x), f1 = halves(a.y), f2 = halves(b.x), f3 = halves(b.y), f4 = halves(c.x),
+               f5 = halves(c.y);
+    if (__builtin_expect(!(f0 && f1 && f2 && f3 && f4 && f5), 0)) {
+        if (!f0) a.x *= 0.5;
+        if (!f1) a.y *= 0.5;
+        if (!f2) b.x *= 0.5;
+        if (!f3) b.y *= 0.5;
+        if (!f4) c.x *= 0.5;
+        if (!f5) c.y *= 0.5;
+    }
 }
 
 // ---------------------------------------------------------------- curl
@@ -210,13 +229,19 @@ __global__ void k_cross_mhd(T *g, long V) {
 
 // ---------------------------------------------------------------- update
 
+// Can a mode of the row (kx, ky) be forced?  The same for a whole warp, so that the rows
+// that cannot branch around the additions.
+__device__ __forceinline__ bool forced_row(const RowIdx &q, const UpdateArgs &ua) {
+    return ua.force_k > 0 && ((q.x == 0 && (q.y == 0 || q.y == ua.mfy || q.y == -ua.mfy)) ||
+                              (q.y == 0 && (q.x == ua.mfx || q.x == -ua.mfx)));
+}
+
 // ABC forcing coefficients at signed grid index k (closed form of
 // f = F (sin kf z + cos kf y, sin kf x + cos kf z, sin kf y + cos kf x));
 // kf sits at grid index kf l_i along axis i (mfx, mfy, mfz).
 template <typename C, typename T>
 __device__ __forceinline__ void abc_forcing(const Idx &k, const UpdateArgs &ua, T F, C &fx, C &fy, C &fz) {
     const T h = F * (T)0.5;
-    if (ua.force_k <= 0) return;
     if (k.x == 0 && k.y == 0 && k.z == ua.mfz) {   // e^{i kf z}: sin -> -i/2, cos -> 1/2
         fx = cadd(fx, mkc((T)0, -h));
         fy = cadd(fy, mkc(h, (T)0));
@@ -238,11 +263,13 @@ __device__ __forceinline__ void abc_forcing(const Idx &k, const UpdateArgs &ua, 
 // stage's weights; the forcing enters as dt f_hat at the forced modes only.
 // On the unit box the table holds pairs (E, 1/|k|^2) by integer |k|^2, and a
 // mode takes 26 FP64 instructions in either stage and one conversion (60 with a
-// division, the conversions of k and the halvings as multiplications): 1.80 ->
-// 1.54 ms at 512^3.  Stage 2 also sums the new state's energy and enstrophy
-// (9 more FP64 instructions a mode; a lane adds its modes in order, the block in
-// a fixed tree, the last block the partials): 1.85 ms with them, and the pass of
-// 0.56 ms that read the state again is gone (32^3: 747 -> 724 us for ten steps).
+// division, the conversions of k and the halvings as multiplications).  Stage 2
+// also sums the new state's energy and enstrophy (9 more a mode; a lane adds
+// its modes in order, the block in a fixed tree, the last block the partials),
+// which spares a pass of 0.56 ms over the state and a launch (32^3: 747 -> 724 us
+// for ten steps).  The forcing and the halvings' rare multiplications sit behind
+// branches: predicated, they kept the FP64 pipe busy in every warp (forced 512^3:
+// 1.87 -> 1.37 ms in stage 1, 2.53 -> 1.76 in stage 2).
 template <typename T, bool UNIT>
 __global__ void __launch_bounds__(256)
 k_update(typename Cx<T>::type *__restrict__ a, typename Cx<T>::type *__restrict__ a1,
@@ -260,7 +287,7 @@ k_update(typename Cx<T>::type *__restrict__ a, typename Cx<T>::type *__restrict_
         const T gdt = (T)ua.gdt, dt = (T)ua.dt, F = (T)ua.force_amp;
         const T rn = (T)ua.rn;   // the Coriolis factor in the units of nl
         const T kx = k.kx, ky = k.ky;
-        const bool every = all_kept(rc, ua.dealias);
+        const bool every = all_kept(rc, ua.dealias), forced = forced_row(q, ua);
         const int nk = rect_kz(rc, g);
         for (int z = threadIdx.x & 31; z < nk; z += 32) {
             const long m = q.m0 + z;
@@ -291,7 +318,7 @@ k_update(typename Cx<T>::type *__restrict__ a, typename Cx<T>::type *__restrict_
                     C t0 = mkc(f0.x + gdt * vx.x, f0.y + gdt * vx.y);
                     C t1 = mkc(f1.x + gdt * vy.x, f1.y + gdt * vy.y);
                     C t2 = mkc(f2.x + gdt * vz.x, f2.y + gdt * vz.y);
-                    abc_forcing(id, ua, F * dt, t0, t1, t2);
+                    if (__builtin_expect(forced, 0)) abc_forcing(id, ua, F * dt, t0, t1, t2);
                     o0 = cscale(t0, e);
                     o1 = cscale(t1, e);
                     o2 = cscale(t2, e);
@@ -300,10 +327,8 @@ k_update(typename Cx<T>::type *__restrict__ a, typename Cx<T>::type *__restrict_
                     o0 = mkc(e * f0.x + g0.x + gdt * vx.x, e * f0.y + g0.y + gdt * vx.y);
                     o1 = mkc(e * f1.x + g1.x + gdt * vy.x, e * f1.y + g1.y + gdt * vy.y);
                     o2 = mkc(e * f2.x + g2.x + gdt * vz.x, e * f2.y + g2.y + gdt * vz.y);
-                    abc_forcing(id, ua, F * dt, o0, o1, o2);
-                    o0 = mkc(halve(o0.x), halve(o0.y));
-                    o1 = mkc(halve(o1.x), halve(o1.y));
-                    o2 = mkc(halve(o2.x), halve(o2.y));
+                    if (__builtin_expect(forced, 0)) abc_forcing(id, ua, F * dt, o0, o1, o2);
+                    halve3(o0, o1, o2);
                 }
             }
             C *dst = ua.stage == 1 ? a1 : a;
@@ -317,7 +342,7 @@ k_update(typename Cx<T>::type *__restrict__ a, typename Cx<T>::type *__restrict_
                 a2 = fma((double)o1.y, (double)o1.y, a2);
                 a2 = fma((double)o2.x, (double)o2.x, a2);
                 a2 = fma((double)o2.y, (double)o2.y, a2);
-                if (z == 0 || 2 * z == g.nz) a2 = halve(a2);   // 1/2 * multiplicity
+                if ((z == 0 || 2 * z == g.nz) && __builtin_expect(!halves(a2), 0)) a2 *= 0.5;   // 1/2 * multiplicity
                 const double kz = UNIT ? (double)z : kmul(z, g.ilz);
                 er += a2;
                 zr = fma(kz * kz, a2, zr);
@@ -366,9 +391,10 @@ k_update_b(typename Cx<T>::type *__restrict__ b, typename Cx<T>::type *__restric
                 o2 = cscale(mkc(f2.x + gdt * nz.x, f2.y + gdt * nz.y), e);
             } else {
                 const C g0 = b1[m], g1 = b1[M + m], g2 = b1[2 * M + m];
-                o0 = mkc(halve(e * f0.x + g0.x + gdt * nx.x), halve(e * f0.y + g0.y + gdt * nx.y));
-                o1 = mkc(halve(e * f1.x + g1.x + gdt * ny.x), halve(e * f1.y + g1.y + gdt * ny.y));
-                o2 = mkc(halve(e * f2.x + g2.x + gdt * nz.x), halve(e * f2.y + g2.y + gdt * nz.y));
+                o0 = mkc(e * f0.x + g0.x + gdt * nx.x, e * f0.y + g0.y + gdt * nx.y);
+                o1 = mkc(e * f1.x + g1.x + gdt * ny.x, e * f1.y + g1.y + gdt * ny.y);
+                o2 = mkc(e * f2.x + g2.x + gdt * nz.x, e * f2.y + g2.y + gdt * nz.y);
+                halve3(o0, o1, o2);
             }
         }
         C *dst = stage == 1 ? b1 : b;
