@@ -1090,10 +1090,10 @@ template <typename T> ns_status plain_step(ns_ctx *c, Run &r, cudaStream_t s, Tr
         NS_CK(r2c_cross<T>(phys, phys + 3 * r.V, (C *)r.wn, g, f, s, fb, tr, &r.prune));
         if (r.p.dealias == 2) {   // the same on the grid shifted by half a spacing, averaged
             C *sh = (C *)r.sh, *sh2 = (C *)r.sh2;
-            NS_CK(NSK_TIMED(tr, "phase", plain_phase<T>(src, sh, (const C *)r.phtab, g, s)));
+            NS_CK(NSK_TIMED(tr, "phase", plain_phase<T>(src, sh, (const C *)r.phtab, g, rc, s)));
             NS_CK(c2r_both<T>(sh, sh2, (C *)r.work, phys, g, rc, f, s, fb, r.work_comps, tr, &r.prune));
             NS_CK(r2c_cross<T>(phys, phys + 3 * r.V, sh2, g, f, s, fb, tr, &r.prune));
-            NS_CK(NSK_TIMED(tr, "phase", plain_phase_avg<T>((C *)r.wn, sh2, (const C *)r.phtab, g, s)));
+            NS_CK(NSK_TIMED(tr, "phase", plain_phase_avg<T>((C *)r.wn, sh2, (const C *)r.phtab, g, rc, s)));
         }
         const UpdateArgs ua = update_args(r, stage);
         NS_CK(NSK_TIMED(tr, "update",

@@ -40,10 +40,10 @@ template <typename T> cudaError_t plain_cross_mhd(T *f, const Grid &g, cudaStrea
 // exp(i pi m / N_i) by array position, [N_x | N_y | N_z/2+1].
 template <typename T>
 cudaError_t plain_phase(const typename Cx<T>::type *src, typename Cx<T>::type *dst,
-                        const typename Cx<T>::type *ph, const Grid &g, cudaStream_t s);
+                        const typename Cx<T>::type *ph, const Grid &g, const Rect &rc, cudaStream_t s);
 template <typename T>
 cudaError_t plain_phase_avg(typename Cx<T>::type *acc, const typename Cx<T>::type *sh,
-                            const typename Cx<T>::type *ph, const Grid &g, cudaStream_t s);
+                            const typename Cx<T>::type *ph, const Grid &g, const Rect &rc, cudaStream_t s);
 // MHD induction update of b (stage 1: b1 = E (b + dt N_b); stage 2: b = E b/2 +
 // (b1 + dt N_b)/2) from nb = transform of u x b.  Factor tables (etab here,
 // and the update's): exp(-c k^2 dt) by integer |k|^2 on a unit box (the
