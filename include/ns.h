@@ -42,9 +42,10 @@
  * Precision: NS_FP64 is the plain form (unfused, FP64 arrays and pointwise
  *   arithmetic in the full half layout; its line transforms compute in 64-bit
  *   fixed point under one power-of-two scale per line, with a smaller error
- *   than FP64 arithmetic, and skip the lines the dealiasing rule zeroes or
- *   discards, with the same result bit for bit; a line with a NaN or an
- *   infinity comes out as NaN).  NS_FP32 is the
+ *   than FP64 arithmetic in the L2 norm and in the largest single mode or
+ *   point, and skip the lines the dealiasing rule zeroes or discards, with the
+ *   same result bit for bit; a line with a NaN or an infinity comes out as
+ *   NaN).  NS_FP32 is the
  *   fused form (pruned FP32 transforms and nonlinear term); its twiddle and
  *   integrating-factor tables are generated in FP64 and rounded once, and its
  *   energy, enstrophy and spectrum sums accumulate in FP64.

@@ -10,24 +10,39 @@
 // factors, so one power-of-two scale per line serves every intermediate value,
 // and 63 bits under that scale are more than the 53 of a double.  At 512^3
 // (three components) the passes went from 11.5 / 6.7 / 4.5 ms (z c2r, y, x)
-// in FP64 to 2.35 / 1.44 / 0.98 ms, bound by integer instruction issue.
+// in FP64 to 2.38 / 1.49 / 0.98 ms, most of it integer instruction issue.
 //
 // The scale: with S >= sum |x_j| over the line, every sub-transform of every
 // stage is bounded by S in modulus (it is a sum of x_j times unit factors), so
 // scaling S below 2^63 excludes overflow whatever the input, and the inputs
 // are known to 2^-62 S.  S lies between the line's 2-norm (one entry stands
 // out) and sqrt(n) times it (a flat line), so the relative error grows like
-// 2^-62 n at worst.  Against long double arithmetic, relative L2 error of one
-// line, worst over plans, signs and scales: 0.5-0.7e-16 for lines with a
-// decaying spectrum at any length, where FP64 gives 1.4-5e-16; for flat lines
-// 0.7e-16 (n = 128), 1.6e-16 (512), 2.9e-16 (1024; FP64: 3.4e-16 or more).
+// 2^-62 n at worst.  Against long double arithmetic, relative L2 error of one line
+// with its results as doubles (whose own rounding is 5e-17): 5-6e-17 for lines
+// with a decaying spectrum at any length, where FP64 gives 1.4-5e-16; for flat
+// lines 6e-17 (n = 256), 0.8e-16 (512), 1.5e-16 (1024; FP64: 3.4e-16 or more).
 //
-// Format: stage 0 works in |v| < 2^63.  The twiddle products of stage 1 take
-// their operand's upper 32 bits and next 30 bits and return v w / 4 (the
-// split that needs no shift), so from there |v| < 2^61 and a split at bit 30
-// makes the upper part fit 32 bits.  A twiddle is w = H 2^-30 + L 2^-60,
-// |H| <= 2^30, |L| <= 2^29 (balanced, so +-1 is exact and negation is exact).
-// The dropped terms and roundings of a product are about one unit.
+// Rounding: every shift here has a mean error of zero on either sign of its
+// operand (halves upwards where 2^-31 of the operands are halves; elsewhere to
+// even or by a bit of the data), and products split their operand into a high
+// word and a SIGNED low word, so that the partial product they drop has mean zero
+// too.  That matters more than the size of the errors: a loss of half a unit
+// with the same sign in every line adds up in phase over a transform's N^2 lines
+// where the data add up like noise.  With shifts that round down, the L2 error of
+// r2c on Gaussian 256^3 data was 1.1e-16, but that of the lowest modes 7.1e-14 of
+// the rms mode (3.9e-13 at 512^3), against 8e-16 in FP64 arithmetic (1.0e-15).  As
+// it is here no mode on the axes is off by more than 2.7e-16 (4.2e-16), for 2 %
+// of the 512^3 step (32.5 -> 33.2 ms).
+//
+// Format: stage 0 works in |v| < 2^63, the later ones in |v| < 2^61: the
+// twiddle products of stage 1 return v w / 4.  A twiddle is w = H 2^-30 + L 2^-62,
+// |H| <= 2^30, |L| < 2^31 (balanced, so +-1 is exact and negation is exact).
+// With v = xh 2^30 + xl / 4 (v / 4 in stage 1: the words of v themselves), v w =
+// xh H + (xl H + xh L) 2^-32 + (xl L) 2^-64, of which the last is dropped and the
+// middle one is the upper word of a sum that starts at 2^31.  To round xh to
+// nearest, the butterflies before a twiddled stage add 2^31 or 2^29 to
+// their input 0, which adds it to each of their outputs (fft_fix_line.cuh).
+// The sum stays below 2^63 while |v| < 0.914 of its range: fix_top's 1.1.
 #pragma once
 #include <stdint.h>
 
@@ -81,12 +96,12 @@ NSK_FIX i64 mulw(int a, int b) {
     return (i64)a * b;
 #endif
 }
-// Lower word of (hi:lo) shifted right by s < 32.
+// Lower word of (hi:lo) shifted right by s <= 32.
 NSK_FIX unsigned fshr(unsigned lo, unsigned hi, int s) {
 #ifdef __CUDA_ARCH__
-    return __funnelshift_r(lo, hi, s);
+    return __funnelshift_rc(lo, hi, s);
 #else
-    return s ? (lo >> s) | (hi << (32 - s)) : lo;
+    return s == 32 ? hi : s ? (lo >> s) | (hi << (32 - s)) : lo;
 #endif
 }
 // Upper word of (hi:lo) shifted left by s < 32.
@@ -98,7 +113,7 @@ NSK_FIX unsigned fshl(unsigned lo, unsigned hi, int s) {
 #endif
 }
 
-// A constant c in (0, 1) as add + H 2^-32 + L 2^-62.
+// A constant c in (0, 1) as add + H 2^-31 + L 2^-63, |H| <= 2^30.
 struct FixC {
     int add, H, L;
 };
@@ -107,26 +122,35 @@ struct FixC {
 // (values of the mathematical constants; sin key = cos (72 - key)).
 __host__ __device__ constexpr FixC fixcos(int key) {
     switch (key) {
-    case 8: return FixC{1, -65250204, 37236404};
-    case 16: return FixC{1, -259018221, -463849674};
-    case 18: return FixC{1, -326934918, -451244975};
-    case 24: return FixC{1, -575416509, -258386713};
-    case 32: return FixC{1, -1004831466, 513831524};
-    case 36: return FixC{1, -1257966796, -25716447};
-    case 40: return FixC{1, -1534215534, -131319465};
-    case 48: return FixC{0, 2147483647, 1073741824};   // 1/2; -H must not overflow
-    case 54: return FixC{0, 1643612827, -290889006};
-    case 56: return FixC{0, 1468965330, 168555869};
-    case 64: return FixC{0, 745813244, 96060625};
+    case 8: return FixC{1, -32625102, 74472808};
+    case 16: return FixC{1, -129509111, 1219784300};
+    case 18: return FixC{1, -163467459, -902489949};
+    case 24: return FixC{1, -287708255, 1630710223};
+    case 32: return FixC{1, -502415733, 1027663049};
+    case 36: return FixC{1, -628983398, -51432894};
+    case 40: return FixC{1, -767107767, -262638930};
+    case 48: return FixC{0, 1 << 30, 0};   // 1/2
+    case 54: return FixC{0, 821806413, 1565705635};
+    case 56: return FixC{0, 734482665, 337111738};
+    case 64: return FixC{0, 372906622, 192121251};
     default: return FixC{0, 0, 0};
     }
 }
 
+// x = xh 2^32 + xl with xl signed: x c = xh 2H + (xl H + xh L) 2^-31 + add x, the
+// middle term rounded (below 0.72 2^63 for every pair of constants of a rotation).
+NSK_FIX int xhi(i64 x) { return lhi(x) + (int)(llo(x) >> 31); }
+NSK_FIX i64 mad2h(int xh, int H, i64 c) {   // xh 2H + c; 2^31 is no int
+    if (H == 1 << 30) return c + (i64)((unsigned long long)(i64)xh << 31);
+    if (H == -(1 << 30)) return c - (i64)((unsigned long long)(i64)xh << 31);
+    return madw(xh, 2 * H, c);
+}
 // x c for a constant c, |x| < 2^63.
 NSK_FIX i64 mulc(i64 x, FixC c) {
-    const int xh = lhi(x), xl = (int)(llo(x) >> 2);
-    const i64 t = c.L ? madw(xh, c.L, mulw(xl, c.H)) : mulw(xl, c.H);
-    return madw(xh, c.H, (t >> 30) + (c.add ? x : 0));
+    const int xh = xhi(x), xl = (int)llo(x);
+    i64 t = madw(xl, c.H, 1LL << 30);
+    if (c.L) t = madw(xh, c.L, t);
+    return mad2h(xh, c.H, (t >> 31) + (c.add ? x : 0));
 }
 
 // v exp(DIR 2 pi i m / R), m and R compile-time constants once unrolled.
@@ -144,11 +168,11 @@ template <int R, int DIR> NSK_FIX L2 lrot(L2 v, int m) {
         return mkl(p - s, p + s);
     }
     const FixC c = fixcos(r), s = fixcos(72 - r);
-    const int xh = lhi(v.x), xl = (int)(llo(v.x) >> 2), yh = lhi(v.y), yl = (int)(llo(v.y) >> 2);
-    const i64 tx = madw(yh, -s.L, madw(yl, -s.H, madw(xh, c.L, mulw(xl, c.H))));
-    const i64 ty = madw(xh, s.L, madw(xl, s.H, madw(yh, c.L, mulw(yl, c.H))));
-    i64 rx = madw(xh, c.H, madw(yh, -s.H, tx >> 30));
-    i64 ry = madw(yh, c.H, madw(xh, s.H, ty >> 30));
+    const int xh = xhi(v.x), xl = (int)llo(v.x), yh = xhi(v.y), yl = (int)llo(v.y);
+    const i64 tx = madw(yh, -s.L, madw(yl, -s.H, madw(xh, c.L, madw(xl, c.H, 1LL << 30))));
+    const i64 ty = madw(xh, s.L, madw(xl, s.H, madw(yh, c.L, madw(yl, c.H, 1LL << 30))));
+    i64 rx = mad2h(xh, c.H, mad2h(yh, -s.H, tx >> 31));
+    i64 ry = mad2h(yh, c.H, mad2h(xh, s.H, ty >> 31));
     if (c.add) {
         rx += v.x;
         ry += v.y;
@@ -161,25 +185,29 @@ template <int R, int DIR> NSK_FIX L2 lrot(L2 v, int m) {
 }
 
 // v w (DIR < 0) or v conj(w) (DIR > 0) with w = (H, L) parts {re.H, re.L,
-// im.H, im.L}; first: v in stage 0's range, the result v w / 4.
-template <int DIR> NSK_FIX L2 cmul_w(L2 v, int4 w, bool first) {
-    int xh, yh;
-    unsigned xl, yl;
-    if (first) {
-        xh = lhi(v.x);
-        yh = lhi(v.y);
-        xl = llo(v.x) >> 2;
-        yl = llo(v.y) >> 2;
-    } else {
-        xh = (int)fshr(llo(v.x), (unsigned)lhi(v.x), 30);
-        yh = (int)fshr(llo(v.y), (unsigned)lhi(v.y), 30);
-        xl = llo(v.x) & 0x3fffffffu;
-        yl = llo(v.y) & 0x3fffffffu;
-    }
+// im.H, im.L}.  k2 = 2: v in stage 0's range, the result v w / 4; else k2 = 0.  v
+// carries the offset NSK_FIX_OFF << k2 in both parts, which its split takes off.
+// start = 2^31 rounds halves up, 2^31 - 1 down: v / 4 times +-1 or +-i is a half for
+// one v in four, so stage 1 takes either by turns (fix_tie).
+#define NSK_FIX_OFF (1 << 29)
+template <int DIR> NSK_FIX L2 cmul_w(L2 v, int4 w, int k2, i64 start) {
+    const int xh = (int)fshr(llo(v.x), (unsigned)lhi(v.x), 30 + k2), yh = (int)fshr(llo(v.y), (unsigned)lhi(v.y), 30 + k2);
+    const int xl = (int)((llo(v.x) << (2 - k2)) ^ 0x80000000u), yl = (int)((llo(v.y) << (2 - k2)) ^ 0x80000000u);
     const int ih = DIR < 0 ? w.z : -w.z, il = DIR < 0 ? w.w : -w.w;
-    const i64 tx = madw(yh, -il, madw((int)yl, -ih, madw(xh, w.y, mulw((int)xl, w.x))));
-    const i64 ty = madw(xh, il, madw((int)xl, ih, madw(yh, w.y, mulw((int)yl, w.x))));
-    return mkl(madw(xh, w.x, madw(yh, -ih, tx >> 30)), madw(yh, w.x, madw(xh, ih, ty >> 30)));
+    const i64 tx = madw(yh, -il, madw(yl, -ih, madw(xh, w.y, madw(xl, w.x, start))));
+    const i64 ty = madw(xh, il, madw(xl, ih, madw(yh, w.y, madw(yl, w.x, start))));
+    return mkl(madw(xh, w.x, madw(yh, -ih, (i64)lhi(tx))), madw(yh, w.x, madw(xh, ih, (i64)lhi(ty))));
+}
+
+// 0 or 1 with equal probability, from a value of the line: its lowest bit and its
+// sign, one of which at least varies from line to line (doubles as inputs end
+// in zero bits, a mean flow fixes the sign).
+NSK_FIX int fix_tie(i64 v) { return (int)((llo(v) ^ ((unsigned)lhi(v) >> 31)) & 1u); }
+
+// v / 2, halves to even.
+NSK_FIX i64 half_even(i64 v) {
+    const i64 h = v >> 1;
+    return h + (i64)(llo(v) & llo(h) & 1u);
 }
 
 // Register DFTs, the decompositions of fft_core.cuh in this arithmetic.
@@ -195,7 +223,7 @@ template <int DIR> struct LDft<3, DIR> {
     static NSK_FIX void run(L2 *a) {
         const FixC h = fixcos(24);   // sqrt(3)/2
         const L2 s = ladd(a[1], a[2]), d = lsub(a[1], a[2]);
-        const L2 t = mkl(a[0].x - (s.x >> 1), a[0].y - (s.y >> 1)), e = mkl(mulc(d.x, h), mulc(d.y, h));
+        const L2 t = mkl(a[0].x - half_even(s.x), a[0].y - half_even(s.y)), e = mkl(mulc(d.x, h), mulc(d.y, h));
         a[0] = ladd(a[0], s);
         a[1] = ladd_i<DIR>(t, e);
         a[2] = ladd_i<-DIR>(t, e);
@@ -273,7 +301,7 @@ NSK_FIX unsigned fix_f2u(float f) {
 // exponent field e - 896 is the FP32 field of the same power of two, and the
 // upper 20 mantissa bits follow.  Entries below 2^-126 count as zero and
 // those above 2^127 as that; lines whose sum leaves [kFixLow, kFixHigh] are
-// first multiplied by a power of two (line_scale in fft_fix.cu).
+// first multiplied by a power of two (line_scale in fft_fix_line.cuh).
 #define NSK_FIX_LOW 8.271806e-25f   // 2^-80
 #define NSK_FIX_HIGH 1.2676506e30f  // 2^100
 
@@ -289,10 +317,9 @@ NSK_FIX float fix_mag(int hx, int hy, unsigned &mx) {
     return fmaxf(a, b) + 0.41421360f * fminf(a, b);
 }
 
-// Power of two above S sqrt(2) (|z| <= sqrt(2) max) and the truncated
-// mantissas, as the biased double exponent of the range [2^e, 2^(e+1)) that
-// holds it: a double with this exponent maps to bit 62.
-NSK_FIX int fix_top(float S) { return S > 0.f ? (int)(fix_f2u(S * 1.001f) >> 23) + 896 : 1023; }
+// Exponent e (a double's biased one) with 1.1 S < 2^(e+1): a double with this
+// exponent maps to bit 62, so that a line with the sum S stays below 2^63 / 1.1.
+NSK_FIX int fix_top(float S) { return S > 0.f ? (int)(fix_f2u(S * 1.1f) >> 23) + 896 : 1023; }
 
 // The double with upper and lower words (hi, lo) times 2^(62 - (top - 1023)),
 // truncated towards zero; exponents above top do not occur.

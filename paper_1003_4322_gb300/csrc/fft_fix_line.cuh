@@ -79,7 +79,8 @@ template <class Op> NSK_DEV unsigned line_reduce(unsigned v, const LineGeo &g, u
 // instructions a value) at the end of one pass and one from it (17, and the
 // line sum) at the start of the next, for shifts, and two roundings to 53 bits
 // (512^3: x inverse 1.10 -> 0.98 ms, y inverse 1.60 -> 1.44, r2c with products
-// 2.84 -> 2.49, y forward 1.52 -> 1.32).  kZeroT: a line of zeros; kNanT: a line with a NaN or an
+// 2.84 -> 2.49, y forward 1.52 -> 1.32; with entries and products rounded to
+// nearest they take 0.98, 1.49, 2.54 and 1.39).  kZeroT: a line of zeros; kNanT: a line with a NaN or an
 // infinity; both stay beyond +-kEdgeT through the small steps the passes add.
 constexpr int kZeroT = -(1 << 20), kNanT = 1 << 20, kEdgeT = 1 << 19;
 
@@ -89,6 +90,10 @@ constexpr int kZeroT = -(1 << 20), kNanT = 1 << 20, kEdgeT = 1 << 19;
 struct LineScale {
     int top, t;
 };
+
+// Bits that a line's inputs leave free below 2^63: a plan of one stage has no
+// twiddle products that would return a quarter, so its inputs come in below 2^61.
+NSK_DEV int fix_room(const FixK &pl) { return pl.nst > 1 ? 0 : 2; }
 
 // The raw value x times the power of two f (a line outside the FP32 range).
 NSK_DEV i64 raw_scaled(i64 x, double f) { return __double_as_longlong(__longlong_as_double(x) * f); }
@@ -100,7 +105,7 @@ NSK_DEV i64 raw_scaled(i64 x, double f) { return __double_as_longlong(__longlong
 // entry; a line with a NaN or an infinity gets the factor NaN.  skip(i)
 // (CTA-uniform): v[i] is zero in the whole CTA.
 template <int NV, bool TWICE, class Skip>
-NSK_DEV LineScale line_scale(L2 (&v)[NV], const LineGeo &g, unsigned *sh, Skip skip) {
+NSK_DEV LineScale line_scale(L2 (&v)[NV], const LineGeo &g, unsigned *sh, int room, Skip skip) {
     auto sum = [&](unsigned &mx) {
         float s = 0.f;
         unsigned low = 0;   // the smallest subnormals have an empty upper word
@@ -137,7 +142,7 @@ NSK_DEV LineScale line_scale(L2 (&v)[NV], const LineGeo &g, unsigned *sh, Skip s
         if (odd) S = S2;
         __syncthreads();
     }
-    r.top = fix_top(S);
+    r.top = fix_top(S) + room;
     r.t = S == 0.f ? kZeroT : r.t + r.top;
     return r;
 }
@@ -145,9 +150,10 @@ NSK_DEV LineScale line_scale(L2 (&v)[NV], const LineGeo &g, unsigned *sh, Skip s
 // Scale of a line read in fixed point: v[i] with exponents t[i], brought to a
 // common one, which is returned.  The common exponent is at least the largest
 // t (an entry is not known below its own lines' unit), and leaves the line sum
-// below 2^63.  sh holds two words per thread.
+// below 2^63 / 1.1 (less the room's bits).  Entries are rounded to nearest, halves
+// by a bit of the data (the shift is one at least).  sh holds two words per thread.
 template <int NV, bool TWICE, class Skip>
-NSK_DEV int line_scale_fixed(L2 (&v)[NV], const int (&t)[NV], const LineGeo &g, unsigned *sh, Skip skip) {
+NSK_DEV int line_scale_fixed(L2 (&v)[NV], const int (&t)[NV], const LineGeo &g, unsigned *sh, int room, Skip skip) {
     int tm = kZeroT;
 #pragma unroll
     for (int i = 0; i < NV; i++)
@@ -165,12 +171,14 @@ NSK_DEV int line_scale_fixed(L2 (&v)[NV], const int (&t)[NV], const LineGeo &g, 
     }
     if (TWICE) s *= 2.f;
     const float S = __uint_as_float(line_reduce<OpAdd>(__float_as_uint(s), g, sh + blockDim.x));
-    const int R = max((int)(__float_as_uint(S * 1.001f) >> 23) + 32 - (127 + 62), 0);
+    const i64 down = -(i64)fix_tie(v[0].x);
+    const int R = max((int)(__float_as_uint(S * 1.1f) >> 23) + 32 - (127 + 62) + room, 1);
 #pragma unroll
     for (int i = 0; i < NV; i++) {
         if (skip(i)) continue;
         const int r = min(R + tm - t[i], 63);
-        v[i] = mkl(v[i].x >> r, v[i].y >> r);
+        const i64 h = (i64)(1ull << (r - 1));   // |v| < 2^62: no overflow
+        v[i] = mkl((v[i].x + h + down) >> r, (v[i].y + h + down) >> r);
     }
     return tm + R;
 }
@@ -245,15 +253,23 @@ template <int E> struct LineAt {
     static size_t entries(int n) { return (size_t)n + n / E; }
 };
 
-// Multiply by the stage twiddles and run the radix-R DFT of butterfly b.
+// Multiply by the stage twiddles and run the radix-R DFT of butterfly b, whose
+// inputs carry the offset NSK_FIX_OFF << k2 (k2: 2 in stage 1, else 0); the
+// outputs carry NSK_FIX_OFF, or none after the last stage.  tie: how this
+// thread's halves are rounded.
 template <int R, int E, int DIR>
-NSK_DEV void fix_butterfly(L2 (&v)[E], int b, int k, int p, const int4 *__restrict__ tab, bool first) {
-    const int sh = first ? 2 : 0;
-    v[b * R] = mkl(v[b * R].x >> sh, v[b * R].y >> sh);
+NSK_DEV void fix_butterfly(L2 (&v)[E], int b, int k, int p, const int4 *__restrict__ tab, int k2, int tie,
+                           bool last) {
+    if (k2 || last) {   // v / 4; the offset becomes the next one
+        const int add = (last ? -(NSK_FIX_OFF << k2) : 0) + (k2 ? 2 - tie : 0);
+        L2 &a = v[b * R];
+        a = mkl((a.x + (i64)add) >> k2, (a.y + (i64)add) >> k2);
+    }
     const int4 *w = tab + k;
+    const i64 start = (1ll << 31) - tie;
 #pragma unroll
     for (int q = 1; q < R; q++) {
-        v[b * R + q] = cmul_w<DIR>(v[b * R + q], __ldg(w + (q - 1) * p), first);
+        v[b * R + q] = cmul_w<DIR>(v[b * R + q], __ldg(w + (q - 1) * p), k2, start);
     }
     LDft<R, DIR>::run(&v[b * R]);
 }
@@ -263,7 +279,7 @@ NSK_DEV void fix_butterfly(L2 (&v)[E], int b, int k, int p, const int4 *__restri
 // order of the line: v[j] is element slot + j T.
 template <int R, int E, int DIR>
 NSK_DEV void fix_stage(L2 (&v)[E], bool active, int slot, int T, int p, const int4 *__restrict__ tab,
-                       bool first, bool last, const LineAt<E> &ln) {
+                       int k2, int tie, bool last, const LineAt<E> &ln) {
     constexpr int B = E / R;
     const int nR = T * B;
     const unsigned magic = 0xffffffffu / (unsigned)p + 1u;   // i / p for i p < 2^32
@@ -278,7 +294,7 @@ NSK_DEV void fix_stage(L2 (&v)[E], bool active, int slot, int T, int p, const in
 #pragma unroll
         for (int b = 0; b < B; b++) {
             const int i = slot + b * T;
-            fix_butterfly<R, E, DIR>(v, b, i - p * (int)__umulhi((unsigned)i, magic), p, tab, first);
+            fix_butterfly<R, E, DIR>(v, b, i - p * (int)__umulhi((unsigned)i, magic), p, tab, k2, tie, last);
         }
     }
     if (last) {   // p = n / R: butterfly i writes element i + q p = slot + (b + q B) T
@@ -311,8 +327,11 @@ NSK_DEV void fix_stage(L2 (&v)[E], bool active, int slot, int T, int p, const in
 // shared line, so a barrier must precede the first store.
 template <int E, int DIR>
 NSK_DEV void fix_line(L2 (&v)[E], bool active, int slot, int T, const FixK &pl, bool smem_read, const LineAt<E> &ln) {
-    const int nst = pl.nst;
-    if (active) LDft<E, DIR>::run(v);
+    const int nst = pl.nst, tie = fix_tie(v[0].x);
+    if (active) {
+        if (nst > 1) v[0] = ladd(v[0], mkl((i64)NSK_FIX_OFF << 2, (i64)NSK_FIX_OFF << 2));
+        LDft<E, DIR>::run(v);
+    }
     if (nst == 1) return;   // T = 1: element q is v[q]
     if (smem_read) __syncthreads();
     if (active) {
@@ -325,10 +344,11 @@ NSK_DEV void fix_line(L2 (&v)[E], bool active, int slot, int T, const FixK &pl, 
     const int4 *tab = pl.tab;
     for (int s = 1; s < nst; s++) {
         const bool last = s == nst - 1;
+        const int k2 = s == 1 ? 2 : 0;
         const int R = pl.rad(s);
 #define NSK_FIX_ST(RR)                                                                                  \
     case RR:                                                                                            \
-        if constexpr (E % RR == 0) fix_stage<RR, E, DIR>(v, active, slot, T, p, tab, s == 1, last, ln); \
+        if constexpr (E % RR == 0) fix_stage<RR, E, DIR>(v, active, slot, T, p, tab, k2, tie, last, ln); \
         break;
         switch (R) {
             NSK_FIX_ST(2)

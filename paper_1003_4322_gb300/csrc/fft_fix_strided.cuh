@@ -90,9 +90,9 @@ k_fix_strided(const longlong2 *in, longlong2 *out, FixK pl, StridedK k) {
     LineGeo g{kCols, cl, 0, c};
     int tl;
     if constexpr (IN == kIoFixed) {
-        tl = line_scale_fixed<E, false>(v, t, g, red, skip);
+        tl = line_scale_fixed<E, false>(v, t, g, red, fix_room(pl), skip);
     } else {
-        const LineScale sc = line_scale<E, false>(v, g, red, skip);
+        const LineScale sc = line_scale<E, false>(v, g, red, fix_room(pl), skip);
 #pragma unroll
         for (int q = 0; q < E; q++)
             if (!skip(q)) v[q] = fix_from_raw(v[q], sc.top);

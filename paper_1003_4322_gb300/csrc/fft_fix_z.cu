@@ -68,7 +68,7 @@ k_fix_r2c2(FixProduct in, longlong2 *__restrict__ out, int *__restrict__ tout, i
         v[q] = mkl(valid ? __double_as_longlong(product_at<KIND>(in, base, o1, o2, e)) : 0,
                    valid ? __double_as_longlong(product_at<KIND>(in, base + N, o1, o2, e)) : 0);
     }
-    const LineScale sc = line_scale<E, false>(v, z_geo(T, li), red, [](int) { return false; });
+    const LineScale sc = line_scale<E, false>(v, z_geo(T, li), red, fix_room(pl), [](int) { return false; });
 #pragma unroll
     for (int q = 0; q < E; q++) v[q] = fix_from_raw(v[q], sc.top);
     fix_line<E, -1>(v, true, slot, T, pl, false, ln);
@@ -78,16 +78,13 @@ k_fix_r2c2(FixProduct in, longlong2 *__restrict__ out, int *__restrict__ tout, i
     __syncthreads();
     if (!valid) return;
     longlong2 *d1 = out + l1 * (nh + 1), *d2 = out + l2 * (nh + 1);
-    // the halves of the pairing fall to the exponent; with one stage the
-    // values use all 63 bits, so that half is taken before the sum
-    const int pre = pl.nst > 1 ? 0 : 1;
-    if (slot < 2) tout[l1 + slot] = sc.t + (pl.nst > 1 ? 1 : 0);
-    if (T == 1) tout[l2] = sc.t + (pl.nst > 1 ? 1 : 0);
+    // the halves of the pairing fall to the exponent
+    if (slot < 2) tout[l1 + slot] = sc.t + (pl.nst > 1 ? 1 : -1);
+    if (T == 1) tout[l2] = sc.t + (pl.nst > 1 ? 1 : -1);
     for (int k = slot; k <= nh && k < kzk; k += T) {
         const L2 a = *ln.at(k), b = *ln.at(k == 0 ? 0 : N - k);
-        const i64 ax = a.x >> pre, ay = a.y >> pre, bx = b.x >> pre, by = b.y >> pre;
-        d1[k] = longlong2{ax + bx, ay - by};
-        d2[k] = longlong2{ay + by, bx - ax};
+        d1[k] = longlong2{a.x + b.x, a.y - b.y};
+        d2[k] = longlong2{a.y + b.y, b.x - a.x};
     }
 }
 
@@ -126,7 +123,7 @@ k_fix_c2r2(const longlong2 *__restrict__ in, const int *__restrict__ tin, int ny
         w[2 * j + 1] = mkl(b.x, b.y);
     }
     const int tz =
-        line_scale_fixed<2 * H, true>(w, t, z_geo(T, li), red, [&](int i) { return (i / 2) * T >= top_m; });
+        line_scale_fixed<2 * H, true>(w, t, z_geo(T, li), red, fix_room(pl), [&](int i) { return (i / 2) * T >= top_m; });
 #pragma unroll
     for (int j = 0; j < H; j++) {
         const int m = slot + j * T;

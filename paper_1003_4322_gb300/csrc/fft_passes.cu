@@ -147,16 +147,18 @@ template <typename T> typename Cx<T>::type *make_twiddles(int n, cudaError_t *er
 template float2 *make_twiddles<float>(int, cudaError_t *);
 template double2 *make_twiddles<double>(int, cudaError_t *);
 
-// exp(-2 pi i t / n) in the format of fft_fix.cuh, w = H 2^-30 + L 2^-60 per
+// exp(-2 pi i t / n) in the format of fft_fix.cuh, w = H 2^-30 + L 2^-62 per
 // part, from long double values (64 mantissa bits or more).
 static int4 fix_twiddle(int t, int n) {
-    const long double a = 6.283185307179586476925286766559005768L * t / n, one = 1073741824.0L;
+    const long double a = 6.283185307179586476925286766559005768L * t / n;
     const long double part[2] = {4 * t == n || 4 * t == 3 * n ? 0.0L : cosl(a),
                                  t == 0 || 2 * t == n ? 0.0L : -sinl(a)};
     int h[2], l[2];
     for (int i = 0; i < 2; i++) {
-        h[i] = (int)llroundl(part[i] * one);
-        l[i] = (int)llroundl((part[i] * one - h[i]) * one);
+        const long double v = part[i] * 1073741824.0L;   // 2^30
+        h[i] = (int)llroundl(v);
+        const long long r = llroundl((v - h[i]) * 4294967296.0L);
+        l[i] = (int)(r > 0x7fffffff ? 0x7fffffff : r < -0x7fffffff ? -0x7fffffff : r);   // -l is an int too
     }
     return make_int4(h[0], l[0], h[1], l[1]);
 }
