@@ -7,6 +7,7 @@
 // transpose ever touches HBM.
 #include <math.h>
 
+#include <algorithm>
 #include <map>
 #include <mutex>
 #include <set>
@@ -42,9 +43,9 @@ bool make_plan(int n, Plan *pl) {
 bool make_plan_e(int n, int E, Plan *pl) {
     int a, b, rest;
     if (n < 4) return false;
+    if (E != 4 && E != 6 && E != 8 && E != 9 && E != 12 && E != 16) return false;
     factor23(n, a, b, rest);
     if (rest != 1 || n % E != 0) return false;
-    if (E != 4 && E != 6 && E != 8 && E != 9 && E != 12 && E != 16) return false;
     static const int cand[] = {16, 12, 9, 8, 6, 4, 3, 2};
     pl->n = n;
     pl->E = E;
@@ -178,9 +179,9 @@ static const FixTables &fix_tables(int n) {
     std::vector<int4> base(n);
     for (int t = 0; t < n; t++) base[t] = fix_twiddle(t, n);
     FixTables f;
-    for (int E = 0; E <= 16; E++) {
+    std::fill(f.off, f.off + 17, -1L);
+    for (int E : {4, 6, 8, 9, 12, 16}) {
         Plan pl;
-        f.off[E] = -1;
         if (!make_plan_e(n, E, &pl)) continue;
         f.off[E] = (long)f.all.size();
         for (int s = 1, p = E; s < pl.nst; p *= pl.rad(s++)) {
