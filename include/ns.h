@@ -192,10 +192,11 @@ ns_status ns_step(ns_ctx *ctx, int nsteps);
  * overlap.  Asynchronous on the context's stream.  Errors: NS_ERR_ARG,
  * NS_ERR_UNSUPPORTED_N, NS_ERR_OOM (first call for a new n allocates its
  * tables), NS_ERR_CUDA.  An NS_FP64 context keeps the line exponents between
- * the passes (12 n (n/2+1) + 12 n^2 bytes for the largest n asked for, at most
- * four times that in all; where they cannot be had, as on a first call under
- * capture, the passes exchange doubles instead), so its transforms, captured
- * ones too, run one after the other. */
+ * the passes (12 n (n/2+1) + 12 n^2 bytes for the largest n asked for, or up to
+ * 4 MiB for more than three components, at most four times that in all; where
+ * they cannot be had, as on a first call under capture, the passes exchange
+ * doubles instead), so its transforms, captured ones too, run one after the
+ * other. */
 ns_status ns_fft_r2c(ns_ctx *ctx, int n, int ncomp, const void *in, void *out);
 
 /* Unnormalised inverse c2r transform of ncomp half-layout complex fields at

@@ -1213,16 +1213,26 @@ ns_status check_flags(ns_ctx *c) {
     return NS_OK;
 }
 
-// Line exponents for up to kFtxComp components of a standalone FP64 transform,
-// at least doubled for a larger grid; the outgrown buffers (together no larger)
-// live as long as the context, as a graph captured by the caller may hold them.
+// Components of a standalone FP64 r2c that share the passes: three, as the
+// large grids need no more to fill the GPU, or as many as have their line
+// exponents in kFtxInts (4 MiB).  Three at a time were 66 launches for 64 fields
+// of 16^3: 232 us where one launch per pass had taken 58 in FP64 arithmetic, and
+// takes 15 now; 200 fields of 32^3 881, 617 and 90 us, 12 of 128^3 397, 1749 and 377.
+const int kFtxComp = 3;
+const size_t kFtxInts = 1u << 20;
+int r2c_group(const Grid &g, int ncomp) {
+    return std::min(ncomp, std::max(kFtxComp, (int)(kFtxInts / FixBufs::ints(g, 1))));
+}
+
+// Line exponents for ncomp components of a standalone FP64 transform, at least
+// doubled for a larger need; the outgrown buffers (together no larger) live as
+// long as the context, as a graph captured by the caller may hold them.
 // Where they cannot be had (the stream is
 // being captured, or no memory is left), the transform keeps doubles between
 // its passes around the one-line z passes, which need none: *f3 then takes
 // `plain` for the z axis.
-const int kFtxComp = 3;
-FixBufs standalone_bufs(ns_ctx *c, const Grid &g, Fft3 *f3, PlainPlans *plain) {
-    size_t need = FixBufs::ints(g, kFtxComp);
+FixBufs standalone_bufs(ns_ctx *c, const Grid &g, int ncomp, Fft3 *f3, PlainPlans *plain) {
+    size_t need = FixBufs::ints(g, ncomp);
     if (c->ftx_ints < need) {
         need = std::max(need, 2 * c->ftx_ints);
         cudaStreamCaptureStatus cap = cudaStreamCaptureStatusActive;
@@ -1240,15 +1250,16 @@ FixBufs standalone_bufs(ns_ctx *c, const Grid &g, Fft3 *f3, PlainPlans *plain) {
             return FixBufs();
         }
     }
-    return FixBufs(c->ftx, g, kFtxComp);
+    return FixBufs(c->ftx, g, ncomp);
 }
 
-// r2c of any number of components, kFtxComp at a time.
+// r2c of any number of components, some at a time.
 cudaError_t standalone_r2c(ns_ctx *c, const double *in, double2 *out, const Grid &g, int ncomp, Fft3 f3) {
     PlainPlans plain;
-    const FixBufs fb = standalone_bufs(c, g, &f3, &plain);
-    for (int k = 0; k < ncomp; k += kFtxComp) {
-        const cudaError_t e = r2c_batch<double>(in + k * g.V(), out + k * g.M(), g, std::min(kFtxComp, ncomp - k), f3,
+    const int group = r2c_group(g, ncomp);
+    const FixBufs fb = standalone_bufs(c, g, group, &f3, &plain);
+    for (int k = 0; k < ncomp; k += group) {
+        const cudaError_t e = r2c_batch<double>(in + k * g.V(), out + k * g.M(), g, std::min(group, ncomp - k), f3,
                                                 c->stream, fb);
         if (e != cudaSuccess) return e;
     }
@@ -1258,7 +1269,7 @@ cudaError_t standalone_r2c(ns_ctx *c, const double *in, double2 *out, const Grid
 // c2r through tmp, one component at a time.
 cudaError_t standalone_c2r(ns_ctx *c, const double2 *in, double2 *tmp, double *out, const Grid &g, int ncomp, Fft3 f3) {
     PlainPlans plain;
-    const FixBufs fb = standalone_bufs(c, g, &f3, &plain);
+    const FixBufs fb = standalone_bufs(c, g, kFtxComp, &f3, &plain);
     for (int k = 0; k < ncomp; k++) {
         const cudaError_t e = c2r_batch<double>(in + k * g.M(), tmp, out + k * g.V(), g, 1, f3, c->stream, fb);
         if (e != cudaSuccess) return e;
