@@ -117,7 +117,6 @@ constexpr int ct_line_stride(int n, int E, int fields) {
 // Stage twiddles of one thread, kept in registers across many transforms of
 // the same length: W_{pR}^{q k} for stages s >= 1, k = (slot + b T) mod p.
 template <int n, int E, int NTAB> struct CtTwiddles {
-    static constexpr bool fm = false;
     static constexpr int offset(int s) {
         int o = 0;
         for (int i = 1; i < s; i++) o += (E / ct_radix(n, E, i)) * (ct_radix(n, E, i) - 1);

@@ -26,106 +26,12 @@
 
 namespace nsk {
 
-// Radix-R butterflies (R a power of two) in fused multiply-adds, the stage's
-// twiddles inside them.  Output j of a butterfly is the polynomial of its
-// inputs at z_j = e^{i theta} W_R^j (theta the thread's twiddle angle), and
-// even and odd inputs give P(z) = P_e(z^2) + z P_o(z^2) at z and -z:
-// a + w b in two multiply-adds per part and a - w b = 2 a - (a + w b) in one,
-// six instructions where twiddle, addition and subtraction take eight.  With
-// the roots of unity inside the twiddles, radix 16 with twiddles takes 192
-// instructions instead of 228 and 8 twiddles instead of 15 (R/2: those of the
-// second quarter of a level are the first's times +-i).  Pass C, bound by the
-// instructions it issues at 8 to 9 warps per SM: with the packing below 1043 ->
-// 976 us at 512^3 (bulk copies, one field parked: 236 -> 206 registers), 22.6
-// -> 19.6 us at 128^3.  The MHD pass C keeps CtTwiddles: its accumulators
-// leave no registers for the butterflies' halves (five 256^3 steps: 7.4 ms with
-// them, 6.9 without), as do the standalone transforms, bound by memory.
-template <int R> constexpr bool fm_radix = R == 2 || R == 4 || R == 8 || R == 16;
-constexpr int fm_count(int R) { return (R & (R - 1)) == 0 ? R / 2 : R - 1; }
-// Twiddles of level r (r points) of a butterfly start at r / 4 (r = 2: 0, the
-// others r/4 each).
-constexpr int fm_level(int r) { return r == 2 ? 0 : r / 4; }
-
-// a + w b and a - w b, w conjugated for DIR > 0; Q: w times DIR i.
-template <int DIR, bool Q> NSK_DEV void fm_bfly(float2 a, float2 b, float2 w, float2 &p, float2 &m) {
-    const float c = w.x, s = DIR < 0 ? w.y : -w.y;
-    const float wx = Q ? (DIR > 0 ? -s : s) : c, wy = Q ? (DIR > 0 ? c : -c) : s;
-    p = make_float2(fmaf(-wy, b.y, fmaf(wx, b.x, a.x)), fmaf(wy, b.x, fmaf(wx, b.y, a.y)));
-    m = make_float2(fmaf(2.f, a.x, -p.x), fmaf(2.f, a.y, -p.y));
-}
-// out[j] (j < r) = sum_i x[i STEP] z^i; w: the butterfly's twiddles, or
-// constants (TW false: theta = 0).
-template <int r, int STEP, int DIR, bool TW> NSK_DEV void fm_eval(const float2 *x, float2 *out, const float2 *w) {
-    if constexpr (r == 1) {
-        out[0] = x[0];
-    } else {
-        float2 e[r / 2], o[r / 2];
-        fm_eval<r / 2, 2 * STEP, DIR, TW>(x, e, w);
-        fm_eval<r / 2, 2 * STEP, DIR, TW>(x + STEP, o, w);
-#pragma unroll
-        for (int j = 0; j < r / 2; j++) {
-            constexpr int u = r >= 4 ? r / 4 : 1;
-            const bool q = r >= 4 && j >= u;
-            if (!TW && j % u == 0) {
-                const float2 b = q ? cmul_i<DIR>(o[j]) : o[j];
-                out[j] = cadd(e[j], b);
-                out[j + r / 2] = csub(e[j], b);
-            } else {
-                float2 v;
-                if constexpr (TW) {
-                    v = w[fm_level(r) + j % u];
-                } else {
-                    double c, sn;
-                    angle288((j % u) * (288 / r), c, sn);
-                    v = make_float2((float)c, (float)-sn);
-                }
-                if (q) fm_bfly<DIR, true>(e[j], o[j], v, out[j], out[j + r / 2]);
-                else fm_bfly<DIR, false>(e[j], o[j], v, out[j], out[j + r / 2]);
-            }
-        }
-    }
-}
-
-// Stage twiddles of one thread for ct_fft_reg, kept in registers.
-template <int n, int E, int NTAB> struct ZrTwiddles {
-    static constexpr int offset(int s) {
-        int o = 0;
-        for (int i = 1; i < s; i++) o += (E / ct_radix(n, E, i)) * fm_count(ct_radix(n, E, i));
-        return o;
-    }
-    static constexpr int count() { return offset(ct_nst(n, E)) > 0 ? offset(ct_nst(n, E)) : 1; }
-    static constexpr bool fm = true;
-    float2 w[count()];
-    template <int S = 1> NSK_DEV void load(int slot, const float2 *__restrict__ tw) {
-        if constexpr (S < ct_nst(n, E)) {
-            constexpr int R = ct_radix(n, E, S), p = ct_span(n, E, S), T = n / E, o = offset(S);
-            constexpr int tab = NTAB / (p * R);
-#pragma unroll
-            for (int b = 0; b < E / R; b++) {
-                const int k = (slot + b * T) % p;
-                float2 *wb = w + o + b * fm_count(R);
-                if constexpr (fm_radix<R>) {
-#pragma unroll
-                    for (int r = 2; r <= R; r *= 2)
-#pragma unroll
-                        for (int j = 0; j < (r >= 4 ? r / 4 : 1); j++)
-                            wb[fm_level(r) + j] = __ldg(tw + (R / r * k + p * R / r * j) * tab);
-                } else {
-#pragma unroll
-                    for (int q = 1; q < R; q++) wb[q - 1] = __ldg(tw + q * k * tab);
-                }
-            }
-            load<S + 1>(slot, tw);
-        }
-    }
-};
-
 // Length-n line FFT over the T = n/E threads of a line.  v enters holding
 // positions slot + j T (j < E) and leaves holding the transform at the same
 // positions; stages after the first exchange through the line's shared
-// buffer (sl/ss).  TW: CtTwiddles, or ZrTwiddles for the fused butterflies.
-template <int n, int E, int DIR, int NTAB, int S = 0, class TW, class SL, class SS>
-NSK_DEV void ct_fft_reg(float2 (&v)[E], int slot, const TW &twr, SL sl, SS ss) {
+// buffer (sl/ss).
+template <int n, int E, int DIR, int NTAB, int S = 0, class SL, class SS>
+NSK_DEV void ct_fft_reg(float2 (&v)[E], int slot, const CtTwiddles<n, E, NTAB> &twr, SL sl, SS ss) {
     constexpr int NST = ct_nst(n, E);
     constexpr int R = ct_radix(n, E, S), T = n / E, nR = n / R, p = ct_span(n, E, S);
     if constexpr (S > 0) {
@@ -138,20 +44,15 @@ NSK_DEV void ct_fft_reg(float2 (&v)[E], int slot, const TW &twr, SL sl, SS ss) {
     }
 #pragma unroll
     for (int b = 0; b < E / R; b++) {
-        const float2 *w = twr.w + TW::offset(S) + b * (TW::fm ? fm_count(R) : R - 1);
-        if constexpr (TW::fm && fm_radix<R>) {
-            float2 t[R];
-            fm_eval<R, 1, DIR, (S > 0)>(&v[b * R], t, w);
+        if constexpr (S > 0) {
+            constexpr int o = CtTwiddles<n, E, NTAB>::offset(S);
 #pragma unroll
-            for (int q = 0; q < R; q++) v[b * R + q] = t[q];
-        } else {
-            if constexpr (S > 0) {
-#pragma unroll
-                for (int q = 1; q < R; q++)
-                    v[b * R + q] = DIR < 0 ? cmul(v[b * R + q], w[q - 1]) : cmulc(v[b * R + q], w[q - 1]);
+            for (int q = 1; q < R; q++) {
+                const float2 w = twr.w[o + b * (R - 1) + q - 1];
+                v[b * R + q] = DIR < 0 ? cmul(v[b * R + q], w) : cmulc(v[b * R + q], w);
             }
-            Dft<R, DIR, float2>::run(&v[b * R]);
         }
+        Dft<R, DIR, float2>::run(&v[b * R]);
     }
     if constexpr (S + 1 < NST) {
         __syncwarp();
@@ -191,7 +92,10 @@ template <int N, int E_> struct ZrShape {
 
 // The even/odd packing of the real transforms (c2r_pack, r2c_unpack) with the
 // twiddle's products inside the additions: eight and ten instructions.  k, m:
-// whether X[k] and X[n-k] can be nonzero (constants once unrolled).
+// whether X[k] and X[n-k] can be nonzero (constants once unrolled).  Pass C at
+// 512^3 1043 -> 996 us, the nonlinear term's error 0.1-0.4 % smaller.  (The
+// butterflies in fused multiply-adds too, a - w b as 2 a - (a + w b), took 974 us
+// but made that error 5 to 8 % larger.)
 NSK_DEV float2 zr_pack(float2 a, float2 b, float2 w, bool k, bool m) {
     float2 f, g;
     if (k && m) {
@@ -317,7 +221,7 @@ k_fused_zr(float2 *buf, long fs, long nlines, long brun, const float2 *__restric
     auto sl = [&](int e) -> float2 { return L[ct_skew(e)]; };
     auto ss = [&](int e, float2 v) { L[ct_skew(e)] = v; };
 
-    ZrTwiddles<n, E, N> twr;
+    CtTwiddles<n, E, N> twr;
     twr.load(slot, tw);
     float2 wk[E];   // W^k = exp(-2 pi i k / N), k = slot + j T
 #pragma unroll
