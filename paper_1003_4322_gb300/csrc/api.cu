@@ -42,7 +42,7 @@ struct FftRes {
     Plan plN{}, plH{};
     PlainPlans pp;
     void *tw = nullptr;       // Cx<T>[n], exp(-2 pi i t / n)
-    int4 *ftab = nullptr;     // FP64: stage twiddles of every plan of length n,
+    int4 *ftab = nullptr;     // FP64: stage twiddles of every plan of length n (tw after them),
     const int4 *fix[17] = {}; // and where those of E elements per thread start
     FixPlan fixed(const Plan &pl) const { return FixPlan{pl, fix[pl.E]}; }
     void *scratch = nullptr;  // one half-layout field (c2r)
@@ -195,16 +195,13 @@ ns_status get_fft(ns_ctx *c, int n, FftRes **out) {
     f.pp.ct_inv = f.pp.ct_fwd = default_ct(n);
     cudaError_t e;
     if (c->prec == NS_FP64) {
-        f.tw = make_twiddles<double>(n, &e);
-        if (!f.tw) return fail_cuda(c, e);
-        if ((e = make_fix_tables(n, &f.ftab, f.fix)) != cudaSuccess) {
-            dev_free(f.tw);
+        if ((e = make_fix_tables(n, &f.ftab, f.fix, &f.tw)) != cudaSuccess) {
             if (f.ftab) dev_free(f.ftab);
             return fail_cuda(c, e);
         }
         f.pp = fix_defaults(n);
     } else {
-        f.tw = make_twiddles<float>(n, &e);
+        f.tw = make_twiddles(n, &e);
         if (!f.tw) return fail_cuda(c, e);
     }
     c->fft[n] = f;
@@ -913,35 +910,20 @@ static bool plain_prune_enabled() {
 // through the same launches, which takes a work buffer of six components
 // (32^3: 947 -> 747 us for ten steps with state transfer and spectrum, 96 x
 // 144 x 192: 0.95 -> 0.89 ms per step).  Larger ones fill the GPU with three and
-// keep the memory.  The buffers are widened once every run has its own, and
-// only within a sixteenth of the memory still free: a context that fits with
-// three components still fits.
+// keep the memory.  The buffers are that wide only if what this adds to all of
+// the context's runs is within a sixteenth of the memory that the three-component
+// buffers would leave free: a context that fits with three still fits.
 const long kBothModes = 256L * 256 * 129;
 
-void plain_widen(ns_ctx *c) {
-    size_t extra = 0, avail = 0, total = 0;
-    for (const Run &r : c->runs)
-        if (r.M <= kBothModes) extra += 3 * r.M * sizeof(double2);
-    if (!extra || cudaMemGetInfo(&avail, &total) != cudaSuccess || extra > avail / 16) return;
-    for (Run &r : c->runs) {
-        if (r.M > kBothModes) continue;
-        void *work = nullptr;
-        int *ftx = nullptr;
-        const size_t ints = FixBufs::ints(r.g, 6);
-        if (dalloc(&work, 6 * r.M * sizeof(double2)) != cudaSuccess ||
-            dalloc(&ftx, ints * sizeof(int)) != cudaSuccess ||
-            cudaMemsetAsync(ftx, 0, ints * sizeof(int), c->stream) != cudaSuccess) {
-            (void)cudaGetLastError();
-            if (work) dev_free(work);
-            if (ftx) dev_free(ftx);
-            return;
-        }
-        dev_free(r.work);   // nothing but the clearing of ftx has been queued on either
-        dev_free(r.ftx);
-        r.work = work;
-        r.ftx = ftx;
-        r.work_comps = 6;
+bool plain_both(const std::vector<Run> &runs) {
+    size_t need = 0, extra = 0, avail = 0, total = 0;
+    for (const Run &r : runs) {
+        const size_t half = (size_t)r.M * sizeof(double2), real = (size_t)r.V * sizeof(double);
+        const size_t nc = r.p.mhd ? 6 : 3;
+        need += (3 * nc + 3 + (r.p.dealias == 2 ? 6 : 0)) * half + 2 * nc * real + FixBufs::ints(r.g, 3) * sizeof(int);
+        if (r.M <= kBothModes) extra += 3 * half + (FixBufs::ints(r.g, 6) - FixBufs::ints(r.g, 3)) * sizeof(int);
     }
+    return extra && cudaMemGetInfo(&avail, &total) == cudaSuccess && avail > need && extra <= (avail - need) / 16;
 }
 
 template <typename T> ns_status plain_alloc(ns_ctx *c, Run &r) {
@@ -955,9 +937,13 @@ template <typename T> ns_status plain_alloc(ns_ctx *c, Run &r) {
     NS_CK(dalloc(&r.un, nc * half));
     NS_CK(dalloc(&r.u1, nc * half));
     NS_CK(dalloc(&r.wn, nc * half));
-    NS_CK(dalloc(&r.work, 3 * half));
+    if (r.work_comps == 6 && dalloc(&r.work, 6 * half) != cudaSuccess) {
+        (void)cudaGetLastError();
+        r.work_comps = 3;
+    }
+    if (!r.work) NS_CK(dalloc(&r.work, 3 * half));
     if (std::is_same<T, double>::value) {
-        const size_t ints = FixBufs::ints(r.g, 3);
+        const size_t ints = FixBufs::ints(r.g, r.work_comps);
         NS_CK(dalloc(&r.ftx, ints * sizeof(int)));
         NS_CK(cudaMemsetAsync(r.ftx, 0, ints * sizeof(int), c->stream));
     }
@@ -992,10 +978,10 @@ template <typename T> ns_status plain_alloc(ns_ctx *c, Run &r) {
     std::vector<T> h;
     factors(r.p.nu, h);
     if (r.g.unit) {   // pairs (factor, 1 / |k|^2)
-        std::vector<T> pairs;
+        std::vector<T> pairs(2 * h.size());
         for (size_t k2 = 0; k2 < h.size(); k2++) {
-            pairs.push_back(h[k2]);
-            pairs.push_back(k2 ? (T)1 / (T)k2 : (T)0);
+            pairs[2 * k2] = h[k2];
+            pairs[2 * k2 + 1] = k2 ? (T)1 / (T)k2 : (T)0;
         }
         h.swap(pairs);
     }
@@ -1177,11 +1163,7 @@ void free_run(Run &r) {
     void *ps[] = {r.un, r.u1, r.wn, r.work, r.ftx, r.phys, r.etab, r.etab_b, r.sh, r.sh2, r.phtab};
     for (void *p : ps)
         if (p) dev_free(p);
-    if (r.owns_diag) {
-        void *qs[] = {r.part, r.series, r.counter};
-        for (void *p : qs)
-            if (p) dev_free(p);
-    }
+    if (r.owns_diag) dev_free(r.series);   // part and counter lie behind it
 }
 
 // Entry check: a null context is an argument error; a context that already
@@ -1379,13 +1361,8 @@ ns_status ns_init(const ns_run_params *runs, int nruns, ns_prec prec, void *cuda
     cudaError_t e = cudaStreamCreateWithFlags(&c->cap, cudaStreamNonBlocking);
     if (e != cudaSuccess) return bail(fail_cuda(nullptr, e));
     if ((e = prepare_fft_kernels()) != cudaSuccess) return bail(fail_cuda(nullptr, e));
-    if ((e = cudaHostAlloc((void **)&c->hflags, sizeof(int), cudaHostAllocMapped)) != cudaSuccess)
-        return bail(fail_cuda(nullptr, e));
-    *c->hflags = 0;
-    if ((e = cudaHostGetDevicePointer((void **)&c->flags, c->hflags, 0)) != cudaSuccess)
-        return bail(fail_cuda(nullptr, e));
+    if ((e = error_word_take(&c->hflags, &c->flags)) != cudaSuccess) return bail(fail_cuda(nullptr, e));
     c->runs.resize(nruns);
-    int maxbins = 0;
     for (int i = 0; i < nruns; i++) {
         Run &r = c->runs[i];
         r.p = runs[i];
@@ -1395,6 +1372,12 @@ ns_status ns_init(const ns_run_params *runs, int nruns, ns_prec prec, void *cuda
                         axis_keep(r.g, 2, r.p.dealias)};
         r.M = r.g.M();
         r.V = r.g.V();
+    }
+    const bool both = prec == NS_FP64 && plain_both(c->runs);
+    int maxbins = 0;
+    for (int i = 0; i < nruns; i++) {
+        Run &r = c->runs[i];
+        r.work_comps = both && r.M <= kBothModes ? 6 : 3;
         const int nb = grid_nbins(r.g);
         maxbins = std::max(maxbins, nb);
         c->spec_slice = std::max(c->spec_slice, (size_t)nb * (1 + shell_parts(nb)));
@@ -1403,13 +1386,13 @@ ns_status ns_init(const ns_run_params *runs, int nruns, ns_prec prec, void *cuda
         if (use_fused(c)) continue;   // grouped below
         st = prec == NS_FP64 ? plain_alloc<double>(c, r) : plain_alloc<float>(c, r);
         if (st != NS_OK) return bail(st);
-        if ((e = dalloc(&r.part, sizeof(double) * 2 * kEnergyParts)) != cudaSuccess ||
-            (e = dalloc(&r.series, sizeof(double) * 2 * kSeriesCap)) != cudaSuccess ||
-            (e = dalloc(&r.counter, 2 * sizeof(unsigned long long))) != cudaSuccess)
+        // series, partial sums and counters in one allocation
+        if ((e = dalloc(&r.series, sizeof(double) * (2 * kSeriesCap + 2 * kEnergyParts + 2))) != cudaSuccess)
             return bail(fail_cuda(nullptr, e));
+        r.part = r.series + 2 * kSeriesCap;
+        r.counter = (unsigned long long *)(r.part + 2 * kEnergyParts);
         cudaMemset(r.counter, 0, 2 * sizeof(unsigned long long));   // steps recorded; finished blocks
     }
-    if (prec == NS_FP64) plain_widen(c);
     if (use_fused(c)) {
         // runs of the same grid, box and equations form one group (in order of
         // first appearance); an MHD group carries a magnetic block beside the
@@ -1474,11 +1457,10 @@ void ns_destroy(ns_ctx *c) {
     for (Run &r : c->runs) free_run(r);
     for (FusedRun &g : c->groups) fused_free(g);
     for (auto &kv : c->fft) {
-        if (kv.second.tw) dev_free(kv.second.tw);
-        if (kv.second.ftab) dev_free(kv.second.ftab);
+        dev_free(kv.second.ftab ? (void *)kv.second.ftab : kv.second.tw);
         if (kv.second.scratch) dev_free(kv.second.scratch);
     }
-    if (c->hflags) cudaFreeHost(c->hflags);
+    error_word_give(c->hflags);
     if (c->spec) dev_free(c->spec);
     if (c->staging) dev_free(c->staging);
     if (c->gscratch) dev_free(c->gscratch);

@@ -80,6 +80,54 @@ void dev_free(void *p) {
     live.erase(it);
 }
 
+// Error words come from one mapped page, allocated at the first context and kept
+// for the life of the process: a mapped allocation of its own took 119 us of every
+// ns_init and 165 of every ns_destroy, as much as the rest of either on a small
+// run.  Contexts beyond the page's words get such an allocation.
+namespace {
+const int kWords = 1024;
+std::mutex word_mu;
+int *word_page = nullptr;
+bool word_used[kWords];
+cudaError_t word_alloc(int **host, int count) {
+    return cudaHostAlloc((void **)host, count * sizeof(int), cudaHostAllocMapped | cudaHostAllocPortable);
+}
+}  // namespace
+
+cudaError_t error_word_take(int **host, int **dev) {
+    cudaError_t e;
+    *host = nullptr;
+    {
+        std::lock_guard<std::mutex> g(word_mu);
+        if (!word_page && (e = word_alloc(&word_page, kWords)) != cudaSuccess) {
+            word_page = nullptr;
+            return e;
+        }
+        for (int i = 0; i < kWords && !*host; i++)
+            if (!word_used[i]) {
+                word_used[i] = true;
+                *host = word_page + i;
+            }
+    }
+    if (!*host && (e = word_alloc(host, 1)) != cudaSuccess) {
+        *host = nullptr;
+        return e;
+    }
+    **host = 0;
+    if ((e = cudaHostGetDevicePointer((void **)dev, *host, 0)) != cudaSuccess) {
+        error_word_give(*host);
+        *host = nullptr;
+    }
+    return e;
+}
+
+void error_word_give(int *host) {
+    if (!host) return;
+    std::lock_guard<std::mutex> g(word_mu);
+    if (host >= word_page && host < word_page + kWords) word_used[host - word_page] = false;
+    else cudaFreeHost(host);
+}
+
 // Bytes of every live guard band that no longer hold the pattern.
 static cudaError_t scan_all(long long *bad) {
     unsigned long long *d = nullptr;

@@ -6,6 +6,7 @@
 // rows of contiguous columns (coalesced 128-byte rows), so no separate
 // transpose ever touches HBM.
 #include <math.h>
+#include <string.h>
 
 #include <algorithm>
 #include <map>
@@ -126,27 +127,26 @@ cudaError_t allow_smem(const void *kernel, size_t bytes) {
     return e;
 }
 
-template <typename T> typename Cx<T>::type *make_twiddles(int n, cudaError_t *err) {
-    typedef typename Cx<T>::type C;
-    std::vector<C> h(n);
-    const double two_pi = 6.283185307179586476925286766559;
+static double2 twiddle(int t, int n) {
+    const double a = 6.283185307179586476925286766559 * (double)t / (double)n;
+    return make_double2(cos(a), -sin(a));
+}
+float2 *make_twiddles(int n, cudaError_t *err) {
+    std::vector<float2> h(n);
     for (int t = 0; t < n; t++) {
-        const double a = two_pi * (double)t / (double)n;
-        h[t].x = (T)cos(a);
-        h[t].y = (T)(-sin(a));
+        const double2 w = twiddle(t, n);
+        h[t] = make_float2((float)w.x, (float)w.y);
     }
-    C *d = nullptr;
-    *err = dev_malloc((void **)&d, sizeof(C) * n);
+    float2 *d = nullptr;
+    *err = dev_malloc((void **)&d, sizeof(float2) * n);
     if (*err != cudaSuccess) return nullptr;
-    *err = cudaMemcpy(d, h.data(), sizeof(C) * n, cudaMemcpyHostToDevice);
+    *err = cudaMemcpy(d, h.data(), sizeof(float2) * n, cudaMemcpyHostToDevice);
     if (*err != cudaSuccess) {
         dev_free(d);
         return nullptr;
     }
     return d;
 }
-template float2 *make_twiddles<float>(int, cudaError_t *);
-template double2 *make_twiddles<double>(int, cudaError_t *);
 
 // exp(-2 pi i t / n) in the format of fft_fix.cuh, w = H 2^-30 + L 2^-62 per
 // part, from long double values (64 mantissa bits or more).
@@ -165,10 +165,12 @@ static int4 fix_twiddle(int t, int n) {
 }
 
 // Host side of make_fix_tables: computed once per length for the life of the
-// process (at most 16 (6 n) bytes for each supported length).
+// process (at most 16 (7 n) bytes for each supported length).  Behind the stage
+// twiddles sit the n doubles' twiddles of the one-line z passes, in one
+// allocation and copy (another of both is 32 us of an ns_init).
 struct FixTables {
     std::vector<int4> all;
-    long off[17];
+    long off[17], tw;
 };
 static const FixTables &fix_tables(int n) {
     static std::mutex mu;
@@ -190,16 +192,23 @@ static const FixTables &fix_tables(int n) {
                 for (int k = 0; k < p; k++) f.all.push_back(base[(long)q * k * stride]);
         }
     }
-    if (f.all.empty()) f.all.push_back(base[0]);   // single-stage plans read no twiddles
+    f.tw = (long)f.all.size();
+    for (int t = 0; t < n; t++) {
+        const double2 w = twiddle(t, n);
+        int4 bits;
+        memcpy(&bits, &w, sizeof bits);
+        f.all.push_back(bits);
+    }
     return done[n] = std::move(f);
 }
 
-cudaError_t make_fix_tables(int n, int4 **buf, const int4 *tab[17]) {
+cudaError_t make_fix_tables(int n, int4 **buf, const int4 *tab[17], void **tw) {
     const FixTables &f = fix_tables(n);
     cudaError_t e = dev_malloc((void **)buf, f.all.size() * sizeof(int4));
     if (e != cudaSuccess) return e;
     e = cudaMemcpy(*buf, f.all.data(), f.all.size() * sizeof(int4), cudaMemcpyHostToDevice);
     for (int E = 0; E <= 16; E++) tab[E] = f.off[E] >= 0 ? *buf + f.off[E] : nullptr;
+    *tw = *buf + f.tw;
     return e;
 }
 
@@ -527,6 +536,13 @@ cudaError_t fft_z_c2r(const typename Cx<T>::type *in, T *out, int N, long nlines
     return launch_z<T, false>(in, out, N, nlines, pl, tw, s, kzk);
 }
 cudaError_t prepare_fft_kernels() {
+    static std::mutex mu;
+    static std::set<int> ready;   // devices; asking again is a query and a look-up for each of some 130 kernels
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    std::lock_guard<std::mutex> g(mu);
+    if (ready.count(dev)) return cudaSuccess;
     const size_t big = 48 * 1024 + 1;
     const int Es[] = {4, 6, 8, 9, 12, 16};
     for (int E : Es) {
@@ -534,13 +550,12 @@ cudaError_t prepare_fft_kernels() {
                             z_kernel<float, true>(E), z_kernel<float, false>(E),
                             z_kernel<double, true>(E), z_kernel<double, false>(E),
                             z_kernel2<float, true>(E), z_kernel2<float, false>(E)};
-        for (const void *k : ks) {
-            cudaError_t e = allow_smem(k, big);
-            if (e != cudaSuccess) return e;
-        }
+        for (const void *k : ks)
+            if ((e = allow_smem(k, big)) != cudaSuccess) return e;
     }
-    const cudaError_t e = prepare_fix_strided();
-    return e != cudaSuccess ? e : prepare_fix_z();
+    if ((e = prepare_fix_strided()) != cudaSuccess || (e = prepare_fix_z()) != cudaSuccess) return e;
+    ready.insert(dev);
+    return cudaSuccess;
 }
 
 template cudaError_t fft_z_r2c<float>(const float *, float2 *, int, long, const Plan &,

@@ -83,9 +83,9 @@ bool make_plan_e(int n, int E, Plan *pl);
 // Is N a supported grid size (2^a 3^b, even, >= 8)?
 bool supported_n(int n);
 
-// Twiddle table exp(-2 pi i t / n), t < n, computed on the host in FP64 and
-// uploaded (rounded once to float for the FP32 path).
-template <typename T> typename Cx<T>::type *make_twiddles(int n, cudaError_t *err);
+// Twiddle table exp(-2 pi i t / n), t < n, computed on the host in FP64,
+// rounded once to float and uploaded.
+float2 *make_twiddles(int n, cudaError_t *err);
 
 // A subset of the columns and rows of a strided pass: the lines that the
 // dealiasing rule leaves zero (inverse) or whose result it discards
@@ -147,9 +147,10 @@ struct FixPlan {
     const int4 *tab = nullptr;
 };
 // The stage twiddles of length n for every E that suits it, in one device
-// array: tab[E] points at those of make_plan_e(n, E) (nullptr: no such plan).
-// *buf receives the array (freed with dev_free).
-cudaError_t make_fix_tables(int n, int4 **buf, const int4 *tab[17]);
+// array: tab[E] points at those of make_plan_e(n, E) (nullptr: no such plan), *tw
+// at a table of the n doubles exp(-2 pi i t / n).  *buf receives the array
+// (freed with dev_free).
+cudaError_t make_fix_tables(int n, int4 **buf, const int4 *tab[17], void **tw);
 
 // The FP64 passes (fft_fix_strided.cuh, fft_fix_z.cu).  Arrays of complex
 // values hold doubles, or fixed-point integers in the same 16 bytes with one
@@ -203,6 +204,10 @@ cudaError_t allow_smem(const void *kernel, size_t bytes);
 // guard bands when NS_GUARD=1.
 cudaError_t dev_malloc(void **p, size_t bytes);
 void dev_free(void *p);
+// A context's error word: zeroed host memory that kernels write through *dev.
+// Given back (nullptr is accepted) when nothing that could write it is queued.
+cudaError_t error_word_take(int **host, int **dev);
+void error_word_give(int *host);
 
 // Launch a kernel that begins with grid_dep(): it may become resident while
 // the kernel ahead of it in the stream drains (a programmatic dependency),
