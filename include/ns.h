@@ -193,16 +193,18 @@ ns_status ns_step(ns_ctx *ctx, int nsteps);
  * NS_ERR_UNSUPPORTED_N, NS_ERR_OOM (first call for a new n allocates its
  * tables), NS_ERR_CUDA.  An NS_FP64 context keeps the line exponents between
  * the passes (12 n (n/2+1) + 12 n^2 bytes for the largest n asked for, or up to
- * 4 MiB for more than three components, at most four times that in all; where
- * they cannot be had, as on a first call under capture, the passes exchange
- * doubles instead), so its transforms, captured ones too, run one after the
- * other. */
+ * 4 MiB for more than three components, at most four times that in all).
+ * Transforms under capture get a buffer of that size per captured graph (256 MiB
+ * in all, given back when the graph is destroyed), so that a graph may be
+ * replayed beside others and beside the context's own work, until ns_destroy.
+ * Where a buffer cannot be had, the passes exchange doubles instead. */
 ns_status ns_fft_r2c(ns_ctx *ctx, int n, int ncomp, const void *in, void *out);
 
 /* Unnormalised inverse c2r transform of ncomp half-layout complex fields at
  * device pointer in into real fields [ncomp][n][n][n] at device pointer out.
  * in is not modified; the context keeps one field of complex scratch per n
- * (allocated on the first call for that n).  Errors as ns_fft_r2c. */
+ * (allocated on the first call for that n), which captured calls use too.
+ * Errors as ns_fft_r2c. */
 ns_status ns_fft_c2r(ns_ctx *ctx, int n, int ncomp, const void *in, void *out);
 
 /* ns_fft_r2c / ns_fft_c2r on a grid of nx x ny x nz points (each 2^a 3^b,

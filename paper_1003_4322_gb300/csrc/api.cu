@@ -7,6 +7,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <atomic>
 #include <tuple>
 #include <type_traits>
 #include <map>
@@ -60,6 +61,16 @@ struct FixBufs {
     }
     FixBufs() = default;
     FixBufs(int *p, const Grid &g, int ncomp) : a(p), b(p ? p + a_ints(g, ncomp) : nullptr) {}
+};
+
+// Line exponents of the transforms of one graph that the caller captures.  The
+// graph may be replayed beside others and beside the context's own work, so it
+// shares them with neither; `free` turns true when the graph is gone.
+struct CaptureBuf {
+    unsigned long long id = 0;   // the capture
+    int *p = nullptr;
+    size_t ints = 0;
+    std::shared_ptr<std::atomic<bool>> free;
 };
 
 // The largest |m_i| per axis that a run's dealiasing rule keeps: the plain
@@ -125,7 +136,8 @@ struct ns_ctx {
     size_t gscratch_bytes = 0;
     int *ftx = nullptr;              // line exponents of the standalone FP64 transforms
     size_t ftx_ints = 0;
-    std::vector<int *> ftx_old;      // outgrown ones, which a graph captured by the caller may hold
+    std::vector<int *> ftx_old;      // outgrown ones, which queued work may still use
+    std::vector<CaptureBuf> ftx_cap; // those of transforms in the caller's graphs
     double *bspec = nullptr;         // batched spectra: per run nbins results + partials, twice
     size_t bspec_runs = 0;
     cudaGraphExec_t graph = nullptr;
@@ -1206,33 +1218,88 @@ int r2c_group(const Grid &g, int ncomp) {
     return std::min(ncomp, std::max(kFtxComp, (int)(kFtxInts / FixBufs::ints(g, 1))));
 }
 
-// Line exponents for ncomp components of a standalone FP64 transform, at least
-// doubled for a larger need; the outgrown buffers (together no larger) live as
-// long as the context, as a graph captured by the caller may hold them.
-// Where they cannot be had (the stream is
-// being captured, or no memory is left), the transform keeps doubles between
-// its passes around the one-line z passes, which need none: *f3 then takes
-// `plain` for the z axis.
-FixBufs standalone_bufs(ns_ctx *c, const Grid &g, int ncomp, Fft3 *f3, PlainPlans *plain) {
-    size_t need = FixBufs::ints(g, ncomp);
-    if (c->ftx_ints < need) {
-        need = std::max(need, 2 * c->ftx_ints);
-        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusActive;
-        int *p = nullptr;
-        if (cudaStreamIsCapturing(c->stream, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone &&
-            dalloc(&p, need * sizeof(int)) == cudaSuccess) {
-            if (c->ftx) c->ftx_old.push_back(c->ftx);
-            c->ftx = p;
-            c->ftx_ints = need;
-        } else {
+// Memory for the graphs' line exponents: 54 graphs of 512^3 transforms at a time.
+const size_t kCaptureInts = 64u << 20;
+
+// A buffer for the transforms of the capture `id` into `graph`: that of an earlier
+// call of the same capture (its transforms run one after the other), one whose
+// graph is gone, or a new one; nullptr: none to be had.
+int *capture_buf(ns_ctx *c, size_t need, unsigned long long id, cudaGraph_t graph) {
+    CaptureBuf *use = nullptr;
+    size_t held = 0;
+    for (CaptureBuf &b : c->ftx_cap) {
+        if (b.id == id && !*b.free && b.ints >= need) return b.p;
+        if (*b.free && b.ints >= need && (!use || b.ints < use->ints)) use = &b;
+        held += b.ints;
+    }
+    if (!use) {
+        if (held + need > kCaptureInts || dev_guards()) return nullptr;   // (guards are written by launches)
+        CaptureBuf b;
+        b.ints = need;
+        // an allocation is no part of the capture, whatever the capture's mode
+        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+        if (cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess) return nullptr;
+        const cudaError_t e = dalloc(&b.p, need * sizeof(int));
+        cudaThreadExchangeStreamCaptureMode(&mode);
+        if (e != cudaSuccess) {
             (void)cudaGetLastError();
-            *plain = *f3->pz;
-            plain->zc = plain->zr = f3->z->plH;
-            f3->pz = plain;
-            return FixBufs();
+            return nullptr;
+        }
+        c->ftx_cap.push_back(b);
+        use = &c->ftx_cap.back();
+    }
+    // the graph holds the flag, and raises it when the last of its executables goes
+    auto flag = std::make_shared<std::atomic<bool>>(false);
+    auto *held_flag = new std::shared_ptr<std::atomic<bool>>(flag);
+    cudaUserObject_t obj;
+    if (cudaUserObjectCreate(&obj, held_flag, [](void *p) {
+            auto *f = (std::shared_ptr<std::atomic<bool>> *)p;
+            **f = true;
+            delete f;
+        }, 1, cudaUserObjectNoDestructorSync) != cudaSuccess) {
+        delete held_flag;
+        (void)cudaGetLastError();
+    } else if (cudaGraphRetainUserObject(graph, obj, 1, cudaGraphUserObjectMove) != cudaSuccess) {
+        (void)cudaGetLastError();
+        cudaUserObjectRelease(obj, 1);
+        flag = std::make_shared<std::atomic<bool>>(false);   // stays with this graph for good
+    }
+    use->free = flag;
+    use->id = id;
+    return use->p;
+}
+
+// Line exponents for ncomp components of a standalone FP64 transform: the
+// context's, at least doubled for a larger need (the outgrown buffers, together
+// no larger, live as long as it), or the graph's under capture.  Where they cannot
+// be had, the transform keeps doubles between its passes around the one-line z
+// passes, which need none: *f3 then takes `plain` for the z axis.
+FixBufs standalone_bufs(ns_ctx *c, const Grid &g, int ncomp, Fft3 *f3, PlainPlans *plain) {
+    const size_t need = FixBufs::ints(g, ncomp);
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusInvalidated;
+    unsigned long long id = 0;
+    cudaGraph_t graph = nullptr;
+    int *p = nullptr;
+    if (cudaStreamGetCaptureInfo(c->stream, &cap, &id, &graph) == cudaSuccess) {
+        if (cap == cudaStreamCaptureStatusActive) {
+            p = capture_buf(c, need, id, graph);
+        } else if (cap == cudaStreamCaptureStatusNone && c->ftx_ints >= need) {
+            p = c->ftx;
+        } else if (cap == cudaStreamCaptureStatusNone) {
+            const size_t ints = std::max(need, 2 * c->ftx_ints);
+            if (dalloc(&p, ints * sizeof(int)) == cudaSuccess) {
+                if (c->ftx) c->ftx_old.push_back(c->ftx);
+                c->ftx = p;
+                c->ftx_ints = ints;
+            }
         }
     }
-    return FixBufs(c->ftx, g, ncomp);
+    if (p) return FixBufs(p, g, ncomp);
+    (void)cudaGetLastError();
+    *plain = *f3->pz;
+    plain->zc = plain->zr = f3->z->plH;
+    f3->pz = plain;
+    return FixBufs();
 }
 
 // r2c of any number of components, some at a time.
@@ -1466,6 +1533,7 @@ void ns_destroy(ns_ctx *c) {
     if (c->gscratch) dev_free(c->gscratch);
     if (c->ftx) dev_free(c->ftx);
     for (int *p : c->ftx_old) dev_free(p);
+    for (CaptureBuf &b : c->ftx_cap) dev_free(b.p);
     if (c->bspec) dev_free(c->bspec);
     if (c->cap) cudaStreamDestroy(c->cap);
     for (cudaStream_t q : c->par) cudaStreamDestroy(q);

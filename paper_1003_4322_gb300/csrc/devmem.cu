@@ -46,6 +46,8 @@ __global__ void k_guard_scan(const unsigned char *__restrict__ g, size_t n, unsi
 }
 }  // namespace
 
+bool dev_guards() { return guards(); }
+
 cudaError_t dev_malloc(void **p, size_t bytes) {
     *p = nullptr;
     if (bytes == 0) return cudaSuccess;

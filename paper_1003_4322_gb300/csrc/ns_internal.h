@@ -204,6 +204,7 @@ cudaError_t allow_smem(const void *kernel, size_t bytes);
 // guard bands when NS_GUARD=1.
 cudaError_t dev_malloc(void **p, size_t bytes);
 void dev_free(void *p);
+bool dev_guards();
 // A context's error word: zeroed host memory that kernels write through *dev.
 // Given back (nullptr is accepted) when nothing that could write it is queued.
 cudaError_t error_word_take(int **host, int **dev);
