@@ -196,6 +196,17 @@ PLAIN_KERNELS = ("fft_x_inverse", "fft_x_forward", "fft_y_inverse", "fft_y_forwa
                  "fft_z_r2c", "curl_x_inverse", "curl_x_inverse6", "fft_y_inverse6", "fft_z_c2r6",
                  "cross_z_r2c", "cross2_z_r2c")
 PLAIN_POINTWISE = ("curl", "update", "update_b", "energy_partials")
+DTYPE = {"fp64": "f64 (line transforms in 64-bit fixed point)", "fp32": "f32"}
+
+
+def fixed_point(name, desc):
+    """Does an FP64 kernel transform in 64-bit fixed point?  All transforms of the
+    plain form do but the z passes of one line per transform; desc (the run's
+    ns_describe_run) says which those are."""
+    z = {"fft_z_c2r": "z_c2r", "fft_z_r2c": "z_r2c"}.get(name)
+    if z:
+        return bool(desc) and desc.get(z, {}).get("lines_per_transform") == 2
+    return name in PLAIN_KERNELS
 
 
 def kernel_model(name, n, prec, keep=None):
@@ -250,7 +261,8 @@ def kernel_model(name, n, prec, keep=None):
         # pruned); reads the transformed product, the state (and the stage-1
         # state at stage 2: 7.5 components on average) of the kept modes only
         kept = (2 * ((nx - 1) // 3) + 1) * (2 * ((ny - 1) // 3) + 1) * ((nz - 1) // 3 + 1)
-        return (3 * rect + 7.5 * kept) * 2 * es, 3 * kept * 20
+        # (stage 2 of the update also sums energy and enstrophy: 15 flops a mode)
+        return (3 * rect + 7.5 * kept) * 2 * es, 3 * kept * 20 + (7.5 * kept if name == "update" else 0)
     # fused form (FP32 complex = 8 bytes; only the kept modes move): compact
     # state [ikx][iky][kz], A / D fields [iky][x][kz], B / C fields [y][x][kz]
     f_line, f_yline = 5 * nx * math.log2(nx), 5 * ny * math.log2(ny)
@@ -388,12 +400,11 @@ def time_form(w, prec, mem, steps, warmup, census_steps, dist, keep_states=True)
                 step_ms_median=statistics.median(per), step_ms_min=per[0])
 
 
-def roofline_of(census, w, prec, census_steps, peaks, sm_mhz, sizes=None):
+def roofline_of(census, w, prec, census_steps, peaks, sm_mhz, sizes=None, desc=None):
     """Dominant kernel (largest share of device time in the census) against
-    HBM or the FP64 ALU roof, whichever its algorithmic model says binds.  The
-    FP64 line transforms run in 64-bit fixed point on the integer pipes, and
-    pass the rate of the FP64 pipe: no roof there, so such a kernel is set
-    against HBM."""
+    HBM or the FP64 ALU roof, whichever its algorithmic model says binds.  A
+    transform in 64-bit fixed point (desc: the run's description) has no FP64
+    roof, its arithmetic being on the integer pipes: it is set against HBM."""
     if not census:
         return None, None
     total = sum(t for _, _, t in census)
@@ -427,7 +438,7 @@ def roofline_of(census, w, prec, census_steps, peaks, sm_mhz, sizes=None):
         tflops = flops / (per_launch_ms * 1e-3) / 1e12
         alu_frac = tflops * 1e12 / peak_flops
         roof["fp64_pipe_frac"] = alu_frac
-        if hbm_frac <= alu_frac <= 1.0:
+        if hbm_frac <= alu_frac and not fixed_point(name, desc):
             roof.update(bound="alu", achieved=tflops, peak=peak_flops / 1e12, unit="TFLOP/s",
                         frac=alu_frac, peak_source=src, hbm_frac=hbm_frac)
             return roof, total
@@ -712,7 +723,7 @@ def large_form(args, peaks, dist):
     mem = members(w)
     steps = min(args.steps, 5)
     t = time_form(w, "fp64", mem, steps, 3, 1, dist, keep_states=False)
-    roof, _ = roofline_of(t["census"], w, "fp64", 1, peaks, None, [dims_of(w)])
+    roof, _ = roofline_of(t["census"], w, "fp64", 1, peaks, None, [dims_of(w)], t["desc"])
     t["solver"].close()
     out["plain768_fp64"] = {"description": w["desc"], "value": steps / (t["ms"] * 1e-3),
                             "unit": "steps/s", "ms_per_step": t["ms"] / steps, "steps": steps,
@@ -772,14 +783,14 @@ def ours(args, w):
     clk = main["clocks"] or {}
     sizes = [dims_of(r) for r in mem[0]]
     roof, census_total = roofline_of(main["census"], w, w["prec"], census_steps, peaks,
-                                     clk.get("sm_mhz"), sizes)
+                                     clk.get("sm_mhz"), sizes, main["desc"])
     launches_per_step = sum(l for _, l, _ in main["census"]) / census_steps if main["census"] else 0
     main["solver"].close()
 
     comp = None
     if w.get("companion") and not args.no_companion:
         c = time_form(w, w["companion"], mem, args.steps, warmup, census_steps, dist)
-        croof, _ = roofline_of(c["census"], w, w["companion"], census_steps, peaks, None, sizes)
+        croof, _ = roofline_of(c["census"], w, w["companion"], census_steps, peaks, None, sizes, c["desc"])
         from oracle import rel_l2
         fp32, fp64 = (c["states"], main["states"]) if w["companion"] == "fp32" else \
             (main["states"], c["states"])
@@ -812,7 +823,7 @@ def ours(args, w):
         "steps": args.steps, "warmup": warmup, "ms_per_step": ms / args.steps,
         "ms_per_step_median": main["step_ms_median"], "ms_per_step_min": main["step_ms_min"],
         "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
-        "dtype": "f64" if w["prec"] == "fp64" else "f32",
+        "dtype": DTYPE[w["prec"]],
         "data": "synthetic (analytic / seeded initial condition, no dataset)",
         "config": config_of(args, w, world),
         "form": main["desc"]["form"], "execution": main["desc"],
