@@ -925,9 +925,12 @@ static bool plain_prune_enabled() {
 // keep the memory.  The buffers are that wide only if what this adds to all of
 // the context's runs is within a sixteenth of the memory that the three-component
 // buffers would leave free: a context that fits with three still fits.
+// NS_PLAIN_BOTH=0 keeps three (the results are the same bit for bit).
 const long kBothModes = 256L * 256 * 129;
 
 bool plain_both(const std::vector<Run> &runs) {
+    const char *v = getenv("NS_PLAIN_BOTH");
+    if (v && v[0] == '0') return false;
     size_t need = 0, extra = 0, avail = 0, total = 0;
     for (const Run &r : runs) {
         const size_t half = (size_t)r.M * sizeof(double2), real = (size_t)r.V * sizeof(double);
