@@ -321,16 +321,24 @@ NSK_FIX float fix_mag(int hx, int hy, unsigned &mx) {
 // exponent maps to bit 62, so that a line with the sum S stays below 2^63 / 1.1.
 NSK_FIX int fix_top(float S) { return S > 0.f ? (int)(fix_f2u(S * 1.1f) >> 23) + 896 : 1023; }
 
+// M shifted right by any number of bits: PTX's shift, unlike C++'s, is defined
+// beyond 63 (all zeros).
+NSK_FIX unsigned long long fix_shr(unsigned long long M, unsigned r) {
+#ifdef __CUDA_ARCH__
+    unsigned long long d;
+    asm("shr.u64 %0, %1, %2;" : "=l"(d) : "l"(M), "r"(r));
+    return d;
+#else
+    return r < 64u ? M >> r : 0;
+#endif
+}
+
 // The double with upper and lower words (hi, lo) times 2^(62 - (top - 1023)),
 // truncated towards zero; exponents above top do not occur.
 NSK_FIX i64 fix_from(int hi, unsigned lo, int top) {
     const unsigned e = ((unsigned)hi >> 20) & 0x7ffu, m = ((unsigned)hi & 0xfffffu) | 0x100000u;
     const unsigned long long M = ((unsigned long long)m << 42) | ((unsigned long long)lo << 10);
-    unsigned r = (unsigned)top - e;
-#ifndef __CUDA_ARCH__
-    r = r < 63u ? r : 63u;   // the device's shift yields zero beyond 63
-#endif
-    const i64 t = (i64)(M >> r), s = (i64)(hi >> 31);
+    const i64 t = (i64)fix_shr(M, (unsigned)top - e), s = (i64)(hi >> 31);
     return (t ^ s) - s;
 }
 

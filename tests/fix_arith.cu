@@ -132,5 +132,15 @@ int main() {
         for (int j = 0; j < 12; j++) bad += d[j].x != c[j].x + NSK_FIX_OFF || d[j].y != c[j].y + NSK_FIX_OFF;
     }
     printf("offset %d 0\n", bad);
+    // doubles of any exponent: below the line's unit they are zero
+    bad = 0;
+    for (int e = 0; e < 2046; e++)
+        for (int top = e; top < 2047; top += 1 + (top - e) / 8) {
+            const int hi = (e << 20) | 0x54321;
+            const i64 v = fix_from(hi, 0x9abcdef0u, top), n = fix_from(hi | (int)0x80000000, 0x9abcdef0u, top);
+            const long double want = ldexpl((long double)(0x154321ll << 32 | 0x9abcdef0ll), 10 - (top - e));
+            bad += v != (i64)want || n != -v;
+        }
+    printf("from %d 0\n", bad);
     return 0;
 }

@@ -36,3 +36,7 @@ def test_no_bias(report, name, worst):
 
 def test_offset_of_input_0_reaches_every_output(report):
     assert report["offset"][0] == 0
+
+
+def test_doubles_far_below_the_scale(report):
+    assert report["from"][0] == 0
