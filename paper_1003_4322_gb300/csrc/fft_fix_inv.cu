@@ -4,7 +4,8 @@
 
 namespace nsk {
 
-// Doubles on both sides serve the z passes that NS_PLAIN_Z=1 asks for.
+// Doubles on both sides go with the one-line z passes: those NS_PLAIN_Z=1 asks for,
+// and those of standalone transforms without a buffer for line exponents.
 const void *fix_inv_kernel(int E, int in, int out) {
     if (in == kIoFixed) return out == kIoFixed ? fix_kernel_of<1, kIoFixed, kIoFixed>(E) : nullptr;
     if (in == kIoCurl) return out == kIoFixed ? fix_kernel_of<1, kIoCurl, kIoFixed>(E) : nullptr;

@@ -80,8 +80,9 @@ template <class Op> NSK_DEV unsigned line_reduce(unsigned v, const LineGeo &g, u
 // line sum) at the start of the next, for shifts, and two roundings to 53 bits
 // (512^3: x inverse 1.10 -> 0.98 ms, y inverse 1.60 -> 1.44, r2c with products
 // 2.84 -> 2.49, y forward 1.52 -> 1.32; with entries and products rounded to
-// nearest they take 0.98, 1.49, 2.54 and 1.39).  kZeroT: a line of zeros; kNanT: a line with a NaN or an
-// infinity; both stay beyond +-kEdgeT through the small steps the passes add.
+// nearest they take 0.98, 1.49, 2.54 and 1.39).  kZeroT: a line of zeros; kNanT: a
+// line with a NaN or an infinity; both stay beyond +-kEdgeT through the small
+// steps the passes add.
 constexpr int kZeroT = -(1 << 20), kNanT = 1 << 20, kEdgeT = 1 << 19;
 
 // Scale of a line read as doubles: `top` for fix_from (of the entries, which

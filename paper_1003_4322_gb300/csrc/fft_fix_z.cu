@@ -25,8 +25,8 @@ NSK_DEV LineGeo z_geo(int T, int li) {
 // the fields as they are loaded (component c of f0 x f1, or of f0 x f1 + f2 x f3,
 // with f_i = 3 fields of V points).  A pass of products alone runs at the FP64
 // pipe's limit (two instructions a value: 1.45 ms at 512^3) while the
-// transform leaves that pipe idle; together they take 2.84 ms where the two took
-// 3.65.  The lines of a product's three components go to neighbouring
+// transform leaves that pipe idle; together they took 2.84 ms where the two took
+// 3.65 (2.54 with the spectra in fixed point).  The lines of a product's three components go to neighbouring
 // transforms, whose loads of the same lines meet in L1 and L2.
 template <int KIND>
 NSK_DEV double product_at(const FixProduct &f, long base, long o1, long o2, int e) {
@@ -154,8 +154,8 @@ k_fix_c2r2(const longlong2 *__restrict__ in, const int *__restrict__ tin, int ny
 
 // Threads per CTA (one line pair at least).  Smaller CTAs drift apart, so that
 // one's FP64 products and another's integer stages share an SM: 256 threads
-// took 3.25 ms for the product pass at 512^3, 128 take 2.84, 64 2.76 but more
-// elsewhere (c2r 2.36 / 2.26 / 2.28).
+// took 3.25 ms for the product pass at 512^3, 128 2.84, 64 2.76 but more elsewhere
+// (c2r 2.36 / 2.26 / 2.28; all with the spectra as doubles).
 static const int kThreads = 128;
 
 // kind: -1 c2r, else the r2c of that kind of input.
