@@ -65,3 +65,39 @@ def test_axis_modes_and_points(ns, dims):
         p[:len(s)] = s
         err = np.abs((_axis(v, ax) - _dft(p, +1)[0]).astype(float))
         assert err.max() < TOL * rms_point, (ax, int(err.argmax()))
+
+
+@pytest.mark.parametrize("dims", [(256, 16, 16), (144, 12, 8), (486, 8, 12), (1024, 8, 8), (16, 162, 8)])
+def test_coherent_lines_at_the_limit_of_the_range(ns, dims):
+    """A plane wave puts every entry of a line in phase at one output, which comes as
+    near to the largest representable value as the line's scale allows (amplitudes
+    between two powers of two): nothing overflows.  Error of the modes over that
+    output: the input's rounding, three passes and the result's, 2^-53 each at most;
+    eight of them."""
+    import torch
+    nx, ny, nz = dims
+    x, y = np.arange(nx)[:, None, None], np.arange(ny)[None, :, None]
+    nc = 32
+    amp = 2.0 ** (np.arange(nc) / nc)
+    u, want = np.empty((nc,) + dims), np.zeros((nc, nx, ny, nz // 2 + 1), dtype=complex)
+    for c in range(nc):
+        kx, ky = (7 * c + 1) % (nx // 2 - 1) + 1, (3 * c + 1) % (ny // 2 - 1) + 1
+        ph = 0.2 * c
+        turn = LD("6.283185307179586476925286766559005768") / LD(nx * ny)
+        wave = np.cos(((kx * x * ny + ky * y * nx) % (nx * ny)).astype(LD) * turn + LD(ph))
+        u[c] = (LD(amp[c]) * wave).astype(float)
+        a = 0.5 * amp[c] * np.prod(dims) * np.exp(1j * ph)
+        want[c, kx, ky, 0], want[c, -kx, -ky, 0] = a, np.conj(a)
+    ud = torch.from_numpy(u).cuda()
+    X, v = torch.empty((nc, nx, ny, nz // 2 + 1), dtype=torch.complex128, device="cuda"), torch.empty_like(ud)
+    ctx = ns.ns_init([dict(n=8, dt=1e-3)], ns.NS_FP64)
+    try:
+        ns.ns_fft_r2c_grid(ctx, *dims, nc, ud, X)
+        ns.ns_fft_c2r_grid(ctx, *dims, nc, torch.from_numpy(want).cuda(), v)
+        ns.ns_sync(ctx)
+    finally:
+        ns.ns_destroy(ctx)
+    peak = 0.5 * amp * np.prod(dims)
+    assert (np.abs(X.cpu().numpy() - want).max(axis=(1, 2, 3)) <= 8 * 2.0 ** -53 * peak).all()
+    back = v.cpu().numpy() / np.prod(dims)
+    assert (np.abs(back - u).max(axis=(1, 2, 3)) <= 8 * 2.0 ** -53 * amp).all()
